@@ -1,190 +1,333 @@
 // S2/S3 on plain fp32 ALUs: direct 3x3 convolution (pad 1, stride 1 or 2) with fused
 // bias + ReLU, or with the fused ConvLSTM gate math.  Used by the fp32 precision path and
-// for the first encoder layer of the bf16 path (3 input channels: too thin for a
-// tensor-core contraction, HBM/ALU bound).
+// for the first encoder layer of the bf16 path where the tensor-core kernel does not apply.
 //
-// Block = 32 x 8 output pixels x OCB output channels; 256 threads, one pixel each, OCB
-// accumulators per thread.  Input channels are consumed in chunks of CB: the haloed input
-// tile and the [CB][9][OCB] weight slice are staged in shared memory.
+// Bound by the fp32 pipe (128 FMA per clock and multiprocessor) where there is work for every
+// multiprocessor, by latency where there is not.  A thread holds 4 neighbouring pixels x 8 output
+// channels in registers, so that one channel's row of 3 taps costs 96 FMAs against 2 input loads and 6
+// broadcast weight loads from shared memory.  A warp covers 32 x 4 pixels of one group of 8 channels.
+// Blocks are made of WY warps along y, WO channel groups that share the input tile, and KS warps that share
+// out the input channels of a tile and add their sums up in shared memory at the end: small maps have too few
+// outputs to occupy the device otherwise.  Input tile (haloed; at stride 2 even and odd columns apart) and
+// weights of CB channels are copied asynchronously into one of two buffers while the other is used.
+//
+// Against one pixel x 16/32 channels per thread, 32 x 8 pixels per block and synchronous staging (stage times with
+// their event): ConvLSTM of one 64x64 map with 16 channels 51 -> 15 us, of three 80x60 maps with 32 channels 135 -> 70 us
+// (32 TFLOP/s, 43 % of the fp32 pipe: 16 warps per multiprocessor, two barriers per chunk and the last row and column
+// tiles' idle lanes).  The same tile as packed pairs of pixels (fma.rn.f32x2) took 94 us: more register moves to form
+// the pairs than FMAs saved.
+#include <algorithm>
+#include <climits>
+
 #include "tt_internal.h"
 
 namespace tt {
 namespace {
 
-constexpr int TW = 32, TH = 8, CB = 8;
+constexpr int TW = 32;          // pixels of a block along x: 8 lanes of 4
+constexpr int OC = 8;           // output channels per thread
 
-template <int OCB>
-__device__ __forceinline__ void store_bf16_vec(__nv_bfloat16* dst, const float* v, int n_valid) {
-  if (n_valid == OCB && ((uintptr_t)dst & 15) == 0) {
-#pragma unroll
-    for (int i = 0; i < OCB; i += 8) {
-      __nv_bfloat162 a = __floats2bfloat162_rn(v[i + 0], v[i + 1]);
-      __nv_bfloat162 b = __floats2bfloat162_rn(v[i + 2], v[i + 3]);
-      __nv_bfloat162 c = __floats2bfloat162_rn(v[i + 4], v[i + 5]);
-      __nv_bfloat162 d = __floats2bfloat162_rn(v[i + 6], v[i + 7]);
-      uint4 u;
-      u.x = *reinterpret_cast<uint32_t*>(&a);
-      u.y = *reinterpret_cast<uint32_t*>(&b);
-      u.z = *reinterpret_cast<uint32_t*>(&c);
-      u.w = *reinterpret_cast<uint32_t*>(&d);
-      *reinterpret_cast<uint4*>(dst + i) = u;
-    }
-  } else {
-    for (int i = 0; i < n_valid; ++i) dst[i] = __float2bfloat16_rn(v[i]);
-  }
+__device__ __forceinline__ uint32_t cs_smem(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// asynchronous copies; `ok` false writes zeros and reads nothing
+__device__ __forceinline__ void copy4(uint32_t dst, const float* src, bool ok) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(dst), "l"(src), "r"(ok ? 4 : 0) : "memory");
 }
+__device__ __forceinline__ void copy16(uint32_t dst, const float* src, bool ok) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(ok ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 
 __device__ __forceinline__ float sigmoid_acc(float z) { return 1.0f / (1.0f + expf(-z)); }
+// on the bf16 path every contraction takes bf16 operands, like the tensor-core layers
+__device__ __forceinline__ float round_bf16(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
-template <int STRIDE, int EPI, int OCB>
-__global__ void __launch_bounds__(TW* TH) conv3x3_simt_kernel(const __grid_constant__ ConvSimtParams p) {
-  constexpr int IN_W = TW * STRIDE + 2;
-  constexpr int IN_H = TH * STRIDE + 2;
-  constexpr int IN_WP = IN_W + 1;  // pad against bank conflicts
+template <int STRIDE, int WY, int WO, int KS>
+struct SimtCfg {
+  static constexpr int WARPS = WY * WO * KS, THREADS = 32 * WARPS;
+  static constexpr int TH = 4 * WY;
+  static constexpr int CB = STRIDE == 1 ? 8 : 4;                  // input channels per staged chunk
+  static constexpr int IN_W = (TW - 1) * STRIDE + 3, IN_H = (TH - 1) * STRIDE + 3;
+  static constexpr int ODD = 36;                                  // stride 2: where a row's odd columns begin (33 even ones before)
+  static constexpr int PITCH = STRIDE == 1 ? 36 : 68;             // floats per staged row, a multiple of 4
+  static constexpr int IN_FLOATS = CB * IN_H * PITCH;
+  static constexpr int W_FLOATS = CB * 9 * WO * OC;
+  static constexpr int BUF_FLOATS = IN_FLOATS + W_FLOATS;
+  static constexpr int SMEM_BYTES = 2 * BUF_FLOATS * 4;
+  static constexpr int N_POS = (IN_H * IN_W + THREADS - 1) / THREADS;   // positions of the input tile per thread
+  static constexpr int W_VECS = CB * 9 * WO * (OC / 4);                 // 16-byte vectors of weights per chunk
+  static_assert((KS - 1) * WY * WO * 32 * OC * 4 <= 2 * BUF_FLOATS, "the channel groups' partial sums reuse the staging buffers");
+};
+
+template <int STRIDE, int EPI, int WY, int WO, int KS>
+__global__ void __launch_bounds__(32 * WY * WO * KS) conv3x3_simt_kernel(const __grid_constant__ ConvSimtParams p) {
+  using Cfg = SimtCfg<STRIDE, WY, WO, KS>;
+  constexpr int CB = Cfg::CB, IN_H = Cfg::IN_H, IN_W = Cfg::IN_W, PITCH = Cfg::PITCH, NT = Cfg::THREADS;
   extern __shared__ __align__(16) float smem[];
-  float* s_in = smem;                       // [CB][IN_H][IN_WP]
-  float* s_w = smem + CB * IN_H * IN_WP;    // [CB][9][OCB]
+  pdl_launch_dependents();
 
   const int tiles_x = (p.Wo + TW - 1) / TW;
   const int tile_x = blockIdx.x % tiles_x, tile_y = blockIdx.x / tiles_x;
-  const int grp = blockIdx.y;  // output-channel group
   const int n = blockIdx.z;
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int tid = ty * TW + tx;
-  const int xo = tile_x * TW + tx, yo = tile_y * TH + ty;
-  const int x_in0 = tile_x * TW * STRIDE - 1, y_in0 = tile_y * TH * STRIDE - 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int wo = warp % WO, wy = (warp / WO) % WY, ks = warp / (WO * WY);
+  const int ly = wy * 4 + (lane >> 3), lx = (lane & 7) * 4;
+  const int xo = tile_x * TW + lx, yo = tile_y * Cfg::TH + ly;
+  const int grp = blockIdx.y * WO + wo;              // group of 8 packed output channels
   const int cin = p.C0 + p.C1;
   const size_t in_plane = (size_t)p.H * p.W;
   const float* base0 = p.in0 + (size_t)p.idx0.v[n] * p.img_stride0;
-  const float* base1 = p.C1 ? p.in1 + (size_t)p.idx1.v[n] * p.img_stride1 : nullptr;
+  const float* base1 = p.C1 ? p.in1 + (size_t)p.idx1.v[n] * p.img_stride1 : base0;
 
-  float acc[OCB];
+  // the input positions this thread copies, the same for every channel: offset in a channel's plane (-1: padding) and in a staged one
+  int g_off[Cfg::N_POS], s_off[Cfg::N_POS];
 #pragma unroll
-  for (int i = 0; i < OCB; ++i) acc[i] = 0.0f;
-
-  for (int c0 = 0; c0 < cin; c0 += CB) {
-    for (int i = tid; i < CB * IN_H * IN_W; i += TW * TH) {
-      const int c = i / (IN_H * IN_W);
-      const int r = (i / IN_W) % IN_H;
-      const int col = i % IN_W;
-      const int ci = c0 + c, yi = y_in0 + r, xi = x_in0 + col;
-      float v = 0.0f;
-      if (ci < cin && yi >= 0 && yi < p.H && xi >= 0 && xi < p.W) {
-        const float* src = ci < p.C0 ? base0 + (size_t)ci * in_plane : base1 + (size_t)(ci - p.C0) * in_plane;
-        v = __ldg(src + (size_t)yi * p.W + xi);
-        // on the bf16 path every contraction takes bf16 operands, like the tensor-core layers
-        if (EPI == EPI_RELU_BF16_NHWC) v = __bfloat162float(__float2bfloat16_rn(v));
-      }
-      s_in[(c * IN_H + r) * IN_WP + col] = v;
+  for (int j = 0; j < Cfg::N_POS; ++j) {
+    const int i = tid + j * NT, r = i / IN_W, col = i - r * IN_W;
+    const int yi = tile_y * Cfg::TH * STRIDE - 1 + r, xi = tile_x * TW * STRIDE - 1 + col;
+    g_off[j] = (yi >= 0 && yi < p.H && xi >= 0 && xi < p.W) ? yi * p.W + xi : -1;
+    s_off[j] = r * PITCH + (STRIDE == 1 ? col : (col & 1) * Cfg::ODD + (col >> 1));
+    if (r >= IN_H) s_off[j] = -1;
+  }
+  auto stage_weights = [&](int c0, float* buf) {
+    const uint32_t dst = cs_smem(buf + Cfg::IN_FLOATS);
+    for (int i = tid; i < Cfg::W_VECS; i += NT) {
+      const int row = i / (WO * 2), v = i - row * (WO * 2);      // row = channel * 9 + tap
+      const bool ok = c0 * 9 + row < cin * 9;
+      copy16(dst + i * 16, p.wgt + (ok ? (size_t)(c0 * 9 + row) * p.cout_packed + (size_t)blockIdx.y * WO * OC + v * 4 : 0), ok);
     }
-    for (int i = tid; i < CB * 9 * OCB; i += TW * TH) {
-      const int c = i / (9 * OCB);
-      const int rest = i % (9 * OCB);
+  };
+  auto stage_input = [&](int c0, float* buf) {
+    const uint32_t dst = cs_smem(buf);
+#pragma unroll
+    for (int c = 0; c < CB; ++c) {
       const int ci = c0 + c;
-      s_w[i] = ci < cin ? __ldg(p.wgt + ((size_t)ci * 9) * p.cout_packed + (size_t)(rest / OCB) * p.cout_packed +
-                                grp * OCB + (rest % OCB))
-                        : 0.0f;
+      const float* src = ci < p.C0 ? base0 + (size_t)ci * in_plane : base1 + (size_t)(ci - p.C0) * in_plane;
+      if (ci >= cin) src = base0;
+#pragma unroll
+      for (int j = 0; j < Cfg::N_POS; ++j) {
+        const bool ok = g_off[j] >= 0 && ci < cin;
+        if (s_off[j] >= 0) copy4(dst + (c * IN_H * PITCH + s_off[j]) * 4, src + (ok ? g_off[j] : 0), ok);
+      }
+    }
+  };
+
+  stage_weights(0, smem);
+  pdl_wait();   // the weights are nobody's output; from here on the previous kernel's results are read
+  stage_input(0, smem);
+  copies_commit();
+
+  // the old cell state is fetched now and used after the main loop
+  constexpr int HB = OC / 4;
+  float c_old[EPI == EPI_LSTM_F32_NCHW ? HB * 4 : 1];
+  const size_t out_plane = (size_t)p.Ho * p.Wo;
+  const size_t pix = (size_t)yo * p.Wo + xo;
+  if (EPI == EPI_LSTM_F32_NCHW && ks == 0) {
+    const float* c_img = p.c_state + (size_t)p.c_idx.v[n] * p.hidden * out_plane;
+#pragma unroll
+    for (int jj = 0; jj < HB; ++jj)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        c_old[jj * 4 + i] = (grp * HB + jj < p.hidden && yo < p.Ho && xo + i < p.Wo) ? c_img[(size_t)(grp * HB + jj) * out_plane + pix + i] : 0.0f;
+  }
+
+  float acc[OC][4];                                  // [channel][pixel]
+#pragma unroll
+  for (int i = 0; i < 4 * OC; ++i) acc[i >> 2][i & 3] = 0.0f;
+
+  int buf = 0;
+  for (int c0 = 0; c0 < cin; c0 += CB, buf ^= 1) {
+    const float* cur = smem + buf * Cfg::BUF_FLOATS;
+    if (c0 + CB < cin) {
+      float* nxt = smem + (buf ^ 1) * Cfg::BUF_FLOATS;
+      stage_weights(c0 + CB, nxt);
+      stage_input(c0 + CB, nxt);
+      copies_commit();
+      copies_wait<1>();
+    } else {
+      copies_wait<0>();
     }
     __syncthreads();
-#pragma unroll 2
-    for (int c = 0; c < CB; ++c) {
-      float v[9];
+    const int c_end = min(CB, cin - c0);
+#pragma unroll 1
+    for (int c = ks; c < c_end; c += KS) {
+      const float* in_c = cur + (c * IN_H + ly * STRIDE) * PITCH + lx;
+      const float* w_c = cur + Cfg::IN_FLOATS + (c * 9 * WO + wo) * OC;
 #pragma unroll
-      for (int ky = 0; ky < 3; ++ky)
+      for (int ky = 0; ky < 3; ++ky) {
+        // x[i]: input column lx * STRIDE + i of this row
+        float x[3 * STRIDE + 3];
+        const float* r = in_c + ky * PITCH;
+        if (STRIDE == 1) {
+          const float4 a = *reinterpret_cast<const float4*>(r);
+          const float2 b = *reinterpret_cast<const float2*>(r + 4);
+          x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y;
+        } else {
+          const float4 e = *reinterpret_cast<const float4*>(r);
+          const float4 o = *reinterpret_cast<const float4*>(r + Cfg::ODD);
+          x[0] = e.x; x[2] = e.y; x[4] = e.z; x[6] = e.w; x[8] = r[4];
+          x[1] = o.x; x[3] = o.y; x[5] = o.z; x[7] = o.w;
+        }
+        if (EPI == EPI_RELU_BF16_NHWC) {
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) v[ky * 3 + kx] = s_in[(c * IN_H + ty * STRIDE + ky) * IN_WP + tx * STRIDE + kx];
-      const float4* wv = reinterpret_cast<const float4*>(s_w + c * 9 * OCB);
+          for (int i = 0; i < 3 * STRIDE + 3; ++i) x[i] = round_bf16(x[i]);
+        }
 #pragma unroll
-      for (int t = 0; t < 9; ++t) {
+        for (int kx = 0; kx < 3; ++kx) {
+          const float4* w = reinterpret_cast<const float4*>(w_c + (ky * 3 + kx) * WO * OC);
 #pragma unroll
-        for (int o4 = 0; o4 < OCB / 4; ++o4) {
-          const float4 w4 = wv[t * (OCB / 4) + o4];
-          acc[o4 * 4 + 0] = fmaf(v[t], w4.x, acc[o4 * 4 + 0]);
-          acc[o4 * 4 + 1] = fmaf(v[t], w4.y, acc[o4 * 4 + 1]);
-          acc[o4 * 4 + 2] = fmaf(v[t], w4.z, acc[o4 * 4 + 2]);
-          acc[o4 * 4 + 3] = fmaf(v[t], w4.w, acc[o4 * 4 + 3]);
+          for (int o = 0; o < OC; o += 4) {
+            const float4 w4 = w[o >> 2];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float v = x[i * STRIDE + kx];
+              acc[o][i] = fmaf(v, w4.x, acc[o][i]);
+              acc[o + 1][i] = fmaf(v, w4.y, acc[o + 1][i]);
+              acc[o + 2][i] = fmaf(v, w4.z, acc[o + 2][i]);
+              acc[o + 3][i] = fmaf(v, w4.w, acc[o + 3][i]);
+            }
+          }
         }
       }
     }
     __syncthreads();
   }
 
-  if (xo >= p.Wo || yo >= p.Ho) return;
-  const size_t out_plane = (size_t)p.Ho * p.Wo;
-  const size_t pix = (size_t)yo * p.Wo + xo;
-  const float* bias = p.bias + grp * OCB;
+  if (KS > 1) {
+    // partial sums of the other channel groups, [group - 1][tile warp][value][lane], added in a fixed order
+    const int tw = warp % (WO * WY);
+    if (ks > 0) {
+#pragma unroll
+      for (int i = 0; i < 4 * OC; ++i) smem[(((ks - 1) * WO * WY + tw) * 4 * OC + i) * 32 + lane] = acc[i >> 2][i & 3];
+    }
+    __syncthreads();
+    if (ks > 0) return;
+#pragma unroll
+    for (int k = 0; k < KS - 1; ++k)
+#pragma unroll
+      for (int i = 0; i < 4 * OC; ++i) acc[i >> 2][i & 3] += smem[((k * WO * WY + tw) * 4 * OC + i) * 32 + lane];
+  }
+
+  if (yo >= p.Ho || xo >= p.Wo) return;
+  const int n_px = min(4, p.Wo - xo);
+  const float* bias = p.bias + grp * OC;
+  // four pixels of a planar map: one 128-bit store where the row length keeps them aligned
+  const bool vec = (p.Wo & 3) == 0;
+  auto store4 = [&](float* dst, const float (&v)[4]) {
+    if (vec) {
+      *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < n_px) dst[i] = v[i];
+    }
+  };
 
   if (EPI == EPI_RELU_F32_NCHW) {
     float* out = reinterpret_cast<float*>(p.out) + (size_t)n * p.out_img_stride;
 #pragma unroll
-    for (int i = 0; i < OCB; ++i) {
-      const int o = grp * OCB + i;
-      if (o < p.cout) out[(size_t)o * out_plane + pix] = fmaxf(acc[i] + __ldg(bias + i), 0.0f);
+    for (int o = 0; o < OC; ++o) {
+      if (grp * OC + o < p.cout) {
+        const float b = __ldg(bias + o);
+        const float v[4] = {fmaxf(acc[o][0] + b, 0.0f), fmaxf(acc[o][1] + b, 0.0f), fmaxf(acc[o][2] + b, 0.0f), fmaxf(acc[o][3] + b, 0.0f)};
+        store4(out + (size_t)(grp * OC + o) * out_plane + pix, v);
+      }
     }
   } else if (EPI == EPI_RELU_BF16_NHWC) {
-    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (size_t)n * p.out_img_stride;
+    // channels-last with a multiple of 8 channels: this thread's 8 are one aligned 16-byte piece of each pixel
+    __nv_bfloat16* out = reinterpret_cast<__nv_bfloat16*>(p.out) + (size_t)n * p.out_img_stride + pix * p.cout + grp * OC;
 #pragma unroll
-    for (int i = 0; i < OCB; ++i) acc[i] = fmaxf(acc[i] + __ldg(bias + i), 0.0f);
-    const int n_valid = min(OCB, p.cout - grp * OCB);
-    store_bf16_vec<OCB>(out + pix * p.cout + grp * OCB, acc, n_valid);
+    for (int i = 0; i < 4; ++i) {
+      if (i < n_px) {
+        uint32_t u[4];
+#pragma unroll
+        for (int o = 0; o < OC; o += 2) {
+          const __nv_bfloat162 h = __floats2bfloat162_rn(fmaxf(acc[o][i] + __ldg(bias + o), 0.0f), fmaxf(acc[o + 1][i] + __ldg(bias + o + 1), 0.0f));
+          u[o >> 1] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(out + (size_t)i * p.cout) = make_uint4(u[0], u[1], u[2], u[3]);
+      }
+    }
   } else {
-    // Packed order inside the group: local = gate*(OCB/4) + jj, hidden unit j = grp*(OCB/4) + jj.
-    constexpr int HB = OCB / 4;
+    // Packed order inside the group: local = gate*2 + jj, hidden unit j = grp*2 + jj.
     float* c_img = p.c_state + (size_t)p.c_idx.v[n] * p.hidden * out_plane;
     float* h_img = p.h_state + (size_t)p.h_out_idx.v[n] * p.hidden * out_plane;
 #pragma unroll
     for (int jj = 0; jj < HB; ++jj) {
       const int j = grp * HB + jj;
-      if (j >= p.hidden) break;
-      const float gi = acc[0 * HB + jj] + __ldg(bias + 0 * HB + jj);
-      const float gf = acc[1 * HB + jj] + __ldg(bias + 1 * HB + jj);
-      const float gg = acc[2 * HB + jj] + __ldg(bias + 2 * HB + jj);
-      const float go = acc[3 * HB + jj] + __ldg(bias + 3 * HB + jj);
-      const size_t idx = (size_t)j * out_plane + pix;
-      const float c_new = sigmoid_acc(gf) * c_img[idx] + sigmoid_acc(gi) * tanhf(gg);
-      c_img[idx] = c_new;
-      h_img[idx] = sigmoid_acc(go) * tanhf(c_new);
+      if (j < p.hidden) {
+        float c_new[4], h_new[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const float gi = acc[0 * HB + jj][i] + __ldg(bias + 0 * HB + jj);
+          const float gf = acc[1 * HB + jj][i] + __ldg(bias + 1 * HB + jj);
+          const float gg = acc[2 * HB + jj][i] + __ldg(bias + 2 * HB + jj);
+          const float go = acc[3 * HB + jj][i] + __ldg(bias + 3 * HB + jj);
+          c_new[i] = sigmoid_acc(gf) * c_old[jj * 4 + i] + sigmoid_acc(gi) * tanhf(gg);
+          h_new[i] = sigmoid_acc(go) * tanhf(c_new[i]);
+        }
+        store4(c_img + (size_t)j * out_plane + pix, c_new);
+        store4(h_img + (size_t)j * out_plane + pix, h_new);
+      }
     }
   }
 }
 
-template <int STRIDE, int EPI, int OCB>
+template <int STRIDE, int EPI, int WY, int WO, int KS>
 cudaError_t launch_one(const ConvSimtParams& p, cudaStream_t s) {
-  constexpr int IN_W = TW * STRIDE + 2, IN_H = TH * STRIDE + 2;
-  const size_t smem = (size_t)(CB * IN_H * (IN_W + 1) + CB * 9 * OCB) * sizeof(float);
-  auto kern = conv3x3_simt_kernel<STRIDE, EPI, OCB>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  using Cfg = SimtCfg<STRIDE, WY, WO, KS>;
+  auto kern = conv3x3_simt_kernel<STRIDE, EPI, WY, WO, KS>;
+  if (Cfg::SMEM_BYTES > 48 * 1024) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM_BYTES);
     if (e != cudaSuccess) return e;
   }
-  const int tiles = ((p.Wo + TW - 1) / TW) * ((p.Ho + TH - 1) / TH);
-  dim3 grid(tiles, p.cout_packed / OCB, p.K), block(TW, TH);
-  kern<<<grid, block, smem, s>>>(p);
-  return cudaGetLastError();
+  const int tiles = ((p.Wo + TW - 1) / TW) * ((p.Ho + Cfg::TH - 1) / Cfg::TH);
+  return launch_kernel(kern, dim3(tiles, p.cout_packed / (WO * OC), p.K), Cfg::THREADS, Cfg::SMEM_BYTES, s, p, p.pdl != 0);
 }
 
+// Estimated cycles on the busiest multiprocessor.  The warps of the blocks it gets share four schedulers (one warp alone
+// cannot use more than one of them); per chunk of input channels a warp takes its share of the channels (about 300
+// issue cycles each: 144 packed FMAs at two cycles, loads beside them) and its part of the staging (about 4 per
+// 4-byte copy, 6 per 16-byte copy), and every chunk costs a round trip to L2 once, whatever shares the multiprocessor.
+template <int STRIDE, int WY, int WO, int KS>
+long simt_cost(const ConvSimtParams& p) {
+  using Cfg = SimtCfg<STRIDE, WY, WO, KS>;
+  if (p.cout_packed % (WO * OC)) return LONG_MAX;
+  const int cin = p.C0 + p.C1;
+  const long blocks = (long)((p.Wo + TW - 1) / TW) * ((p.Ho + Cfg::TH - 1) / Cfg::TH) * (p.cout_packed / (WO * OC)) * p.K;
+  const long rounds = ((blocks + p.sm_count - 1) / p.sm_count * Cfg::WARPS + 3) / 4;
+  const long chunks = (cin + Cfg::CB - 1) / Cfg::CB, share = (std::min(cin, Cfg::CB) + KS - 1) / KS;
+  const long staging = 4 * Cfg::N_POS * Cfg::CB + 6 * Cfg::W_VECS / Cfg::THREADS;
+  return chunks * (rounds * (share * 300 + staging) + 500) + (KS > 1 ? 300 : 0);
+}
+
+// The block shape with the smallest estimate; among equals the one listed first (more reuse of the staged tile).  Splitting
+// the input channels only wins where the map is too small to give every scheduler a warp: 64x64 pixels x 64 channels from 32
+// input channels 25 us with 32 blocks of 8 warps, 15 us with 128 of 4; three maps of 80x60 x 128 channels from 64 70 us with
+// 288 of 8, 88 us with 2160 of 4, each on a quarter of the channels.
 template <int STRIDE, int EPI>
-cudaError_t launch_ocb(const ConvSimtParams& p, cudaStream_t s) {
-  if (p.ocb == 16) return launch_one<STRIDE, EPI, 16>(p, s);
-  if (p.ocb == 32) return launch_one<STRIDE, EPI, 32>(p, s);
-  return cudaErrorInvalidValue;
-}
-
-template <int STRIDE>
 cudaError_t launch_epi(const ConvSimtParams& p, cudaStream_t s) {
-  switch (p.epilogue) {
-    case EPI_RELU_F32_NCHW: return launch_ocb<STRIDE, EPI_RELU_F32_NCHW>(p, s);
-    case EPI_RELU_BF16_NHWC: return launch_ocb<STRIDE, EPI_RELU_BF16_NHWC>(p, s);
-    case EPI_LSTM_F32_NCHW: return launch_ocb<STRIDE, EPI_LSTM_F32_NCHW>(p, s);
+  const long cost[5] = {simt_cost<STRIDE, 2, 4, 1>(p), simt_cost<STRIDE, 4, 2, 1>(p), simt_cost<STRIDE, 4, 1, 1>(p),
+                        simt_cost<STRIDE, 1, 2, 2>(p), simt_cost<STRIDE, 1, 1, 4>(p)};
+  switch (std::min_element(cost, cost + 5) - cost) {
+    case 0: return launch_one<STRIDE, EPI, 2, 4, 1>(p, s);
+    case 1: return launch_one<STRIDE, EPI, 4, 2, 1>(p, s);
+    case 2: return launch_one<STRIDE, EPI, 4, 1, 1>(p, s);
+    case 3: return launch_one<STRIDE, EPI, 1, 2, 2>(p, s);
+    default: return launch_one<STRIDE, EPI, 1, 1, 4>(p, s);
   }
-  return cudaErrorInvalidValue;
 }
 
 }  // namespace
 
 cudaError_t launch_conv_simt(const ConvSimtParams& p, cudaStream_t s) {
-  if (p.stride == 1) return launch_epi<1>(p, s);
-  if (p.stride == 2) return launch_epi<2>(p, s);
+  if (p.stride != 1 && p.stride != 2) return cudaErrorInvalidValue;
+  switch (p.epilogue) {
+    case EPI_RELU_F32_NCHW: return p.stride == 1 ? launch_epi<1, EPI_RELU_F32_NCHW>(p, s) : launch_epi<2, EPI_RELU_F32_NCHW>(p, s);
+    case EPI_RELU_BF16_NHWC: return p.stride == 1 ? launch_epi<1, EPI_RELU_BF16_NHWC>(p, s) : launch_epi<2, EPI_RELU_BF16_NHWC>(p, s);
+    case EPI_LSTM_F32_NCHW: return p.stride == 1 ? launch_epi<1, EPI_LSTM_F32_NCHW>(p, s) : cudaErrorInvalidValue;
+  }
   return cudaErrorInvalidValue;
 }
 

@@ -95,6 +95,7 @@ __device__ __forceinline__ void finish_stream(const PostParams& p, int n, int nb
 
 __global__ void __launch_bounds__(POST_THREADS) post_tile_kernel(const __grid_constant__ PostParams p) {
   extern __shared__ __align__(16) float s_mem[];
+  pdl_launch_dependents();
   const int Ch = p.Ch, T = p.T;
   const int row = Ch + ROW_PAD;
   float* s_tile = s_mem;                     // [PIX][row]
@@ -111,6 +112,7 @@ __global__ void __launch_bounds__(POST_THREADS) post_tile_kernel(const __grid_co
   const float* h_img = p.h + (size_t)p.idx.v[n] * p.img_stride;
 
   for (int i = tid; i < T * Ch; i += POST_THREADS) s_w[i] = __ldg(p.head_w + i);
+  pdl_wait();   // the head weights are nobody's output; the hidden state is the previous kernel's
 
   if (p.channels_last) {
     const int row4 = Ch >> 2;
@@ -763,9 +765,8 @@ cudaError_t launch_postprocess(const PostParams& p, cudaStream_t s) {
     if (p.Ch == 256) return launch_kernel(post_stream_kernel<2>, grid, StreamCfg<2>::THREADS, StreamCfg<2>::SMEM_BYTES, s, p, pdl);
     return launch_kernel(post_stream_kernel<4>, grid, StreamCfg<4>::THREADS, StreamCfg<4>::SMEM_BYTES, s, p, pdl);
   } else {
-    post_tile_kernel<<<p.K * nb, POST_THREADS, post_smem_bytes(p.Ch), s>>>(p);
+    return launch_kernel(post_tile_kernel, p.K * nb, POST_THREADS, post_smem_bytes(p.Ch), s, p, p.pdl != 0);
   }
-  return cudaGetLastError();
 }
 
 }  // namespace tt

@@ -34,7 +34,7 @@ namespace {
 struct SimtLayer {
   float* w = nullptr;  // [Cin][9][CoutPacked]
   float* b = nullptr;
-  int cin = 0, cout = 0, cout_packed = 0, ocb = 16, stride = 1;
+  int cin = 0, cout = 0, cout_packed = 0, stride = 1;
 };
 
 struct TcLayer {
@@ -258,12 +258,12 @@ tt_status upload(tt_ctx* ctx, T** out, const std::vector<T>& host) {
   return TT_OK;
 }
 
-// OIHW fp32 -> [Cin][9][CoutPacked]; with lstm_hidden > 0 the packed output order groups, per
-// block of ocb outputs, the four gates of ocb/4 consecutive hidden units (gate-major inside).
-tt_status pack_simt(tt_ctx* ctx, SimtLayer* L, const float* w, const float* b, int cin, int cout, int stride, int ocb,
+// OIHW fp32 -> [Cin][9][CoutPacked]; with lstm_hidden > 0 the packed output order
+// groups, per block of 8 outputs, the four gates of 2 consecutive hidden units (gate-major inside).
+tt_status pack_simt(tt_ctx* ctx, SimtLayer* L, const float* w, const float* b, int cin, int cout, int stride,
                     int lstm_hidden, bool round_bf16) {
-  L->cin = cin; L->cout = cout; L->stride = stride; L->ocb = ocb;
-  const int hb = ocb / 4;
+  L->cin = cin; L->cout = cout; L->stride = stride;
+  constexpr int ocb = 8, hb = ocb / 4;
   const int packed = lstm_hidden ? round_up(lstm_hidden, hb) * 4 : round_up(cout, ocb);
   L->cout_packed = packed;
   std::vector<float> hw((size_t)cin * 9 * packed, 0.f), hbias((size_t)packed, 0.f);
@@ -551,11 +551,11 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
   if (!ctx->bf16) {
     for (int l = 0; l < c.n_enc; ++l)
       if ((st = pack_simt(ctx, &ctx->simt_enc[l], w->enc_w[l], w->enc_b[l], ctx->lay_c[l], ctx->lay_c[l + 1],
-                          c.enc_stride[l], ctx->lay_c[l + 1] > 16 ? 32 : 16, 0, false)) != TT_OK)
+                          c.enc_stride[l], 0, false)) != TT_OK)
         return st;
     if (!ctx->feed_forward &&
         (st = pack_simt(ctx, &ctx->simt_lstm, w->lstm_w, w->lstm_b, ctx->Cx + ctx->Ch, 4 * ctx->Ch, 1,
-                        ctx->Ch >= 8 ? 32 : 16, ctx->Ch, false)) != TT_OK)
+                        ctx->Ch, false)) != TT_OK)
       return st;
   } else {
     if (ctx->lay_c[1] % 8) return fail(ctx, TT_ERR_UNSUPPORTED, "bf16 path needs enc_cout[0] in multiples of 8");
@@ -595,7 +595,7 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
       f.scale = pre::norm_scale(1.0f / c.norm_div, 1.0f / c.norm_std);
       f.shift = pre::norm_shift(c.norm_mean, 1.0f / c.norm_std);
     } else if ((st = pack_simt(ctx, &ctx->simt_enc[0], w->enc_w[0], w->enc_b[0], 3, ctx->lay_c[1], c.enc_stride[0],
-                               ctx->lay_c[1] > 16 ? 32 : 16, 0, true)) != TT_OK) {
+                               0, true)) != TT_OK) {
       return st;
     }
     for (int l = 1; l < c.n_enc; ++l) {
@@ -744,7 +744,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       q.in0 = in; q.img_stride0 = (int64_t)ctx->lay_c[l] * ctx->lay_h[l] * ctx->lay_w[l]; q.idx0 = ident;
       q.C0 = ctx->lay_c[l]; q.C1 = 0;
       q.H = ctx->lay_h[l]; q.W = ctx->lay_w[l]; q.Ho = ctx->lay_h[l + 1]; q.Wo = ctx->lay_w[l + 1];
-      q.stride = L.stride; q.K = K; q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.ocb = L.ocb;
+      q.stride = L.stride; q.K = K; q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.sm_count = ctx->sm_count; q.pdl = ctx->profiling ? 0 : 1;
       q.epilogue = EPI_RELU_F32_NCHW; q.out = ctx->enc_out[l];
       q.out_img_stride = (int64_t)L.cout * q.Ho * q.Wo;
       TT_CUDA(ctx, launch_conv_simt(q, s));
@@ -757,7 +757,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     q.in0 = in; q.img_stride0 = (int64_t)ctx->Cx * plane; q.idx0 = ident; q.C0 = ctx->Cx;
     q.in1 = ctx->h_f32; q.img_stride1 = (int64_t)ctx->Ch * plane; q.idx1 = h_in; q.C1 = ctx->Ch;
     q.H = ctx->Hm; q.W = ctx->Wm; q.Ho = ctx->Hm; q.Wo = ctx->Wm; q.stride = 1; q.K = K;
-    q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.ocb = L.ocb;
+    q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.sm_count = ctx->sm_count; q.pdl = ctx->profiling ? 0 : 1;
     q.epilogue = EPI_LSTM_F32_NCHW; q.c_state = ctx->c_state; q.h_state = ctx->h_f32; q.c_idx = c_idx; q.h_out_idx = h_out;
     q.hidden = ctx->Ch;
     TT_CUDA(ctx, launch_conv_simt(q, s));
@@ -776,7 +776,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       ConvSimtParams q{};
       q.in0 = ctx->pre; q.img_stride0 = (int64_t)3 * c.net_h * c.net_w; q.idx0 = ident; q.C0 = 3; q.C1 = 0;
       q.H = c.net_h; q.W = c.net_w; q.Ho = ctx->lay_h[1]; q.Wo = ctx->lay_w[1];
-      q.stride = L.stride; q.K = K; q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.ocb = L.ocb;
+      q.stride = L.stride; q.K = K; q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.sm_count = ctx->sm_count; q.pdl = ctx->profiling ? 0 : 1;
       q.epilogue = EPI_RELU_BF16_NHWC; q.out = ctx->enc_out[0];
       q.out_img_stride = (int64_t)L.cout * q.Ho * q.Wo;
       TT_CUDA(ctx, launch_conv_simt(q, s));
@@ -852,7 +852,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   po.conf_mode = c.conf_mode; po.zthr = ctx->zthr;
   po.logits = ctx->logits; po.probs = ctx->probs; po.masks = ctx->masks; po.bits = ctx->bits;
   po.results = ctx->results_dev; po.scratch = ctx->post_scratch; po.status = ctx->status_dev; po.wait_limit = ctx->wait_limit;
-  po.pdl = (ctx->bf16 && !ctx->profiling) ? 1 : 0;
+  po.pdl = ctx->profiling ? 0 : 1;
   TT_CUDA(ctx, launch_postprocess(po, s));
   if ((ms_ = mark_stage(ctx, TT_STAGE_POSTPROCESS, 1)) != TT_OK) return ms_;
   }

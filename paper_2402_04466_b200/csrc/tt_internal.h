@@ -18,10 +18,10 @@ __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepc
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename Params>
-inline cudaError_t launch_kernel(void (*kern)(const Params), int grid, int block, size_t smem, cudaStream_t s, const Params& p,
+inline cudaError_t launch_kernel(void (*kern)(const Params), dim3 grid, int block, size_t smem, cudaStream_t s, const Params& p,
                                  bool pdl) {
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
@@ -69,7 +69,9 @@ struct ConvSimtParams {
   int32_t H, W, Ho, Wo, stride, K;
   const float* wgt;   // packed [Cin][9][CoutPacked]
   const float* bias;  // packed [CoutPacked]
-  int32_t cout, cout_packed, ocb;
+  int32_t cout, cout_packed;   // cout_packed: a multiple of 8
+  int32_t sm_count;
+  int32_t pdl;        // launch as a programmatic dependent of the previous kernel in the stream
   int32_t epilogue;
   // EPI_RELU_*: out; EPI_LSTM: c (in place), h_out
   void* out;
@@ -186,7 +188,7 @@ struct PostParams {
   void* scratch;
   int32_t* status;      // optional device word: set non-zero when a bounded wait ran out
   long long wait_limit; // SM cycles after which a wait for a copy gives up (0: the default)
-  int32_t pdl;          // launch as a programmatic dependent of the previous kernel in the stream (channels-last kernel only)
+  int32_t pdl;          // launch as a programmatic dependent of the previous kernel in the stream
 };
 size_t post_scratch_bytes(int K, int hm, int wm, int ch, int T);
 cudaError_t launch_postprocess(const PostParams& p, cudaStream_t s);
