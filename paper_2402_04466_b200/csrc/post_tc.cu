@@ -118,6 +118,7 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
 
+  int status_before = 0;   // thread 64: the status word as the kernels before this one left it
   if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------------------ producer
     // the packed weights first (they are not the previous kernel's output), then the tiles
@@ -171,6 +172,7 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
     // ------------------------------------------------------------------------ epilogue
     pdl_wait();
     const int et = threadIdx.x - 64;               // 0..127
+    if (et == 0) status_before = *(volatile int*)p.status;
     const int quarter = warp & 3;                  // tensor-memory lanes 32*quarter .. +31
     const int T = p.T;
     const int Ch = kslabs * 64;
@@ -312,6 +314,7 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
   }
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 64) report_status(status_before, *abort_flag != 0, p.status, p.status_out);
   if (warp == 1) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(32u) : "memory");

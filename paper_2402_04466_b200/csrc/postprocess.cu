@@ -9,6 +9,7 @@
 // forms confidence and centroid and re-zeroes the accumulators.
 #include <mutex>
 
+#include "tc_ptx.cuh"
 #include "tt_internal.h"
 
 namespace tt {
@@ -113,6 +114,7 @@ __global__ void __launch_bounds__(POST_THREADS) post_tile_kernel(const __grid_co
 
   for (int i = tid; i < T * Ch; i += POST_THREADS) s_w[i] = __ldg(p.head_w + i);
   pdl_wait();   // the head weights are nobody's output; the hidden state is the previous kernel's
+  if (blockIdx.x == 0 && tid == 0 && p.status) tc::report_status(*(volatile int*)p.status, false, p.status, p.status_out);
 
   if (p.channels_last) {
     const int row4 = Ch >> 2;
@@ -397,6 +399,7 @@ __global__ void __launch_bounds__(StreamCfg<NCHUNK>::THREADS, 1) post_stream_ker
   }
   __syncthreads();
   pdl_wait();   // head weights and barriers are set up; the hidden state is the previous kernel's output
+  if (blockIdx.x == 0 && tid == 0 && p.status) tc::report_status(*(volatile int*)p.status, false, p.status, p.status_out);
 
   const ScratchLayout sl = scratch_layout(p.K, plane, CH, T);
   uint8_t* scr = reinterpret_cast<uint8_t*>(p.scratch);
@@ -547,7 +550,10 @@ __global__ void __launch_bounds__(StreamCfg<NCHUNK>::THREADS, 1) post_stream_ker
         ok = __all_sync(0xffffffffu, ok);
         if (!ok) {
           // a copy never arrived: record it, give copies still in flight time to land, stop
-          if (lane == 0 && p.status) atomicCAS(p.status, 0, 0x700 + stage);
+          if (lane == 0 && p.status) {
+            atomicCAS(p.status, 0, 0x700 + stage);
+            tc::report_status(0x700 + stage, true, p.status, p.status_out);
+          }
           for (int w = 0; w < 64; ++w) __nanosleep(16000);
           break;
         }

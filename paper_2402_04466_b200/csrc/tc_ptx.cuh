@@ -62,6 +62,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The last kernel of a tick tells the host, through a mapped word, of a wait that ran out in it or before it: `before` is the
+// status word as it stood when the kernel's predecessors were done.  A healthy tick writes nothing.  One thread of every
+// block calls it after the block's last wait.
+__device__ __forceinline__ void report_status(int before, bool aborted, int* status, int* status_out) {
+  if (!status_out || (before == 0 && !aborted)) return;
+  const int code = before ? before : *(volatile int*)status;
+  *(volatile int*)status_out = code ? code : -1;
+}
+
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, uint32_t bar, int c0, int c1, int c2,
                                             int c3) {
   asm volatile(

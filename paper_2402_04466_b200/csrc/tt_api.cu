@@ -101,10 +101,9 @@ struct tt_ctx {
   __nv_bfloat16* h_bf16 = nullptr;    // bf16 path: [slots*2][plane][Ch]
   float *logits = nullptr, *probs = nullptr;
   uint8_t *masks = nullptr, *bits = nullptr, *overlay = nullptr;
-  tt_result* results_dev = nullptr;
-  tt_result* results_host = nullptr;  // pinned
+  tt_result* results_host = nullptr;  // pinned, mapped
   int32_t* status_dev = nullptr;
-  int32_t* status_host = nullptr;     // pinned
+  int32_t* status_host = nullptr;     // pinned, mapped
   void* post_scratch = nullptr;
   float* dbg_tmp = nullptr;
   size_t dbg_tmp_floats = 0;
@@ -130,8 +129,8 @@ struct tt_ctx {
     uint8_t* frames_stage = nullptr;
     float *logits = nullptr, *probs = nullptr;
     uint8_t *masks = nullptr, *bits = nullptr, *overlay = nullptr;
-    tt_result *results_dev = nullptr, *results_host = nullptr;
-    int32_t* status_host = nullptr;
+    tt_result* results_host = nullptr;   // mapped: the last kernel of a tick writes the records here itself
+    int32_t* status_host = nullptr;      // mapped: written by it when a wait has run out
     cudaEvent_t ev_start = nullptr, ev_stop = nullptr, ev_copy = nullptr;
     cudaEvent_t stage_ev[TT_STAGE_COUNT + 1] = {};
     bool stage_ran[TT_STAGE_COUNT] = {};
@@ -207,7 +206,7 @@ tt_status fail(tt_ctx* ctx, tt_status st, const char* fmt, ...) {
 void bind_slot(tt_ctx* ctx, int i) {
   const tt_ctx::Slot& sl = ctx->slots[i];
   ctx->frames_stage = sl.frames_stage; ctx->logits = sl.logits; ctx->probs = sl.probs; ctx->masks = sl.masks;
-  ctx->bits = sl.bits; ctx->overlay = sl.overlay; ctx->results_dev = sl.results_dev; ctx->results_host = sl.results_host;
+  ctx->bits = sl.bits; ctx->overlay = sl.overlay; ctx->results_host = sl.results_host;
   ctx->status_host = sl.status_host; ctx->ev_start = sl.ev_start; ctx->ev_stop = sl.ev_stop; ctx->ev_copy = sl.ev_copy;
   for (int k = 0; k <= TT_STAGE_COUNT; ++k) ctx->stage_ev[k] = sl.stage_ev[k];
   for (int k = 0; k < TT_STAGE_COUNT; ++k) ctx->stage_ran[k] = sl.stage_ran[k];
@@ -221,7 +220,7 @@ void bind_slot(tt_ctx* ctx, int i) {
 void save_slot(tt_ctx* ctx, int i) {
   tt_ctx::Slot& sl = ctx->slots[i];
   sl.frames_stage = ctx->frames_stage; sl.logits = ctx->logits; sl.probs = ctx->probs; sl.masks = ctx->masks;
-  sl.bits = ctx->bits; sl.overlay = ctx->overlay; sl.results_dev = ctx->results_dev; sl.results_host = ctx->results_host;
+  sl.bits = ctx->bits; sl.overlay = ctx->overlay; sl.results_host = ctx->results_host;
   sl.status_host = ctx->status_host; sl.ev_start = ctx->ev_start; sl.ev_stop = ctx->ev_stop; sl.ev_copy = ctx->ev_copy;
   for (int k = 0; k <= TT_STAGE_COUNT; ++k) sl.stage_ev[k] = ctx->stage_ev[k];
   for (int k = 0; k < TT_STAGE_COUNT; ++k) sl.stage_ran[k] = ctx->stage_ran[k];
@@ -512,9 +511,10 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
     if ((st = dev_alloc(ctx, &sl.masks, (size_t)S * ctx->T * plane)) != TT_OK) return st;
     if ((st = dev_alloc(ctx, &sl.bits, (size_t)S * plane)) != TT_OK) return st;
     if (c.overlay && (st = dev_alloc(ctx, &sl.overlay, (size_t)S * c.src_w * c.src_h * 4)) != TT_OK) return st;
-    if ((st = dev_alloc(ctx, &sl.results_dev, (size_t)S)) != TT_OK) return st;
-    TT_CUDA(ctx, cudaHostAlloc(reinterpret_cast<void**>(&sl.results_host), sizeof(tt_result) * S, cudaHostAllocDefault));
-    TT_CUDA(ctx, cudaHostAlloc(reinterpret_cast<void**>(&sl.status_host), sizeof(int32_t), cudaHostAllocDefault));
+    // written by the device through the unified address space: no copy behind the last kernel of a tick
+    TT_CUDA(ctx, cudaHostAlloc(reinterpret_cast<void**>(&sl.results_host), sizeof(tt_result) * S, cudaHostAllocMapped));
+    std::memset(sl.results_host, 0, sizeof(tt_result) * S);
+    TT_CUDA(ctx, cudaHostAlloc(reinterpret_cast<void**>(&sl.status_host), sizeof(int32_t), cudaHostAllocMapped));
     *sl.status_host = 0;
     {
       uint64_t* tab = nullptr;
@@ -835,7 +835,8 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   if (ctx->use_post_tc) {
     PostTcParams& q = ctx->post_tc;
     q.idx = ctx->feed_forward ? ident : h_out; q.K = K;
-    q.logits = ctx->logits; q.probs = ctx->probs; q.masks = ctx->masks; q.bits = ctx->bits; q.results = ctx->results_dev;
+    q.logits = ctx->logits; q.probs = ctx->probs; q.masks = ctx->masks; q.bits = ctx->bits; q.results = ctx->results_host;
+    q.status_out = ctx->status_host;
     q.pdl = ctx->profiling ? 0 : 1;
     TT_CUDA(ctx, launch_post_tc(q, ctx->sm_count, s));
     if ((ms_ = mark_stage(ctx, TT_STAGE_POSTPROCESS, 1)) != TT_OK) return ms_;
@@ -851,7 +852,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   po.head_w = ctx->head_w; po.head_b = ctx->head_b; po.conf_w = ctx->conf_w; po.conf_b = ctx->conf_b;
   po.conf_mode = c.conf_mode; po.zthr = ctx->zthr;
   po.logits = ctx->logits; po.probs = ctx->probs; po.masks = ctx->masks; po.bits = ctx->bits;
-  po.results = ctx->results_dev; po.scratch = ctx->post_scratch; po.status = ctx->status_dev; po.wait_limit = ctx->wait_limit;
+  po.results = ctx->results_host; po.scratch = ctx->post_scratch; po.status = ctx->status_dev; po.status_out = ctx->status_host; po.wait_limit = ctx->wait_limit;
   po.pdl = ctx->profiling ? 0 : 1;
   TT_CUDA(ctx, launch_postprocess(po, s));
   if ((ms_ = mark_stage(ctx, TT_STAGE_POSTPROCESS, 1)) != TT_OK) return ms_;
@@ -863,6 +864,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     ov.T = ctx->T; ov.Hm = ctx->Hm; ov.Wm = ctx->Wm; ov.masks = ctx->masks; ov.bits = ctx->bits;
     std::memcpy(ov.palette, c.palette, sizeof(ov.palette));
     ov.dst = ctx->overlay;
+    ov.pdl = ctx->profiling ? 0 : 1;
     TT_CUDA(ctx, launch_overlay(ov, s));
     if ((ms_ = mark_stage(ctx, TT_STAGE_OVERLAY, 1)) != TT_OK) return ms_;
   }
@@ -1120,16 +1122,12 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
     ctx->n_launches += tg->launches;
     ctx->n_ticks += 1;
   } else if (tg && (tg->seen >= 1 || family_warm)) {
-    // capture the sequence (kernels plus the two result copies), then launch it
+    // capture the sequence, then launch it
     const uint64_t launches_before = ctx->n_launches;
     cudaGraph_t graph = nullptr;
     cudaError_t ce = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (ce == cudaSuccess) {
       st = enqueue_tick(ctx, K, fp, states);
-      if (st == TT_OK) {
-        ce = cudaMemcpyAsync(ctx->results_host, ctx->results_dev, sizeof(tt_result) * K, cudaMemcpyDeviceToHost, s);
-        if (ce == cudaSuccess) ce = cudaMemcpyAsync(ctx->status_host, ctx->status_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-      }
       cudaError_t ee = cudaStreamEndCapture(s, &graph);
       if (ce == cudaSuccess) ce = ee;
     }
@@ -1145,8 +1143,6 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
       if ((st = refresh_table()) != TT_OK) return st;
       st = enqueue_tick(ctx, K, fp, states);
       if (st != TT_OK) return st;
-      TT_CUDA(ctx, cudaMemcpyAsync(ctx->results_host, ctx->results_dev, sizeof(tt_result) * K, cudaMemcpyDeviceToHost, s));
-      TT_CUDA(ctx, cudaMemcpyAsync(ctx->status_host, ctx->status_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     } else {
       tg->launches = ctx->n_launches - launches_before;
       if ((st = refresh_table()) != TT_OK) return st;
@@ -1156,8 +1152,6 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
     if ((st = refresh_table()) != TT_OK) return st;
     st = enqueue_tick(ctx, K, fp, states);
     if (st != TT_OK) return st;
-    TT_CUDA(ctx, cudaMemcpyAsync(ctx->results_host, ctx->results_dev, sizeof(tt_result) * K, cudaMemcpyDeviceToHost, s));
-    TT_CUDA(ctx, cudaMemcpyAsync(ctx->status_host, ctx->status_dev, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
     if (tg) tg->seen += 1;
   }
   TT_CUDA(ctx, cudaEventRecord(ctx->ev_stop, s));

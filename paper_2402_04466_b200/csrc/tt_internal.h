@@ -184,9 +184,10 @@ struct PostParams {
   float* probs;
   uint8_t* masks;
   uint8_t* bits;        // optional [K][plane], bit t = mask of tool t
-  tt_result* results;   // device, [K]
+  tt_result* results;   // device or host-mapped, [K]
   void* scratch;
   int32_t* status;      // optional device word: set non-zero when a bounded wait ran out
+  int32_t* status_out;  // with status: host-mapped word, written with the code when the status word is set, else left alone
   long long wait_limit; // SM cycles after which a wait for a copy gives up (0: the default)
   int32_t pdl;          // launch as a programmatic dependent of the previous kernel in the stream
 };
@@ -209,9 +210,10 @@ struct PostTcParams {
   float* probs;
   uint8_t* masks;
   uint8_t* bits;          // optional [K][plane]
-  tt_result* results;     // device, [K]
+  tt_result* results;     // device or host-mapped, [K]
   void* scratch;          // post_scratch_bytes(...) bytes, zero on entry, zero again on exit
   int32_t* status;
+  int32_t* status_out;    // as in PostParams
   long long wait_limit;
   int32_t pdl;
 };
@@ -227,6 +229,7 @@ struct OverlayParams {
   const uint8_t* bits;   // [K][plane] packed
   uint8_t palette[TT_MAX_TOOLS][3];
   uint8_t* dst;          // [K][src_h][src_w][4]
+  int32_t pdl;           // launch as a programmatic dependent of the previous kernel in the stream
 };
 cudaError_t launch_overlay(const OverlayParams& p, cudaStream_t s);
 
