@@ -66,9 +66,10 @@ typedef enum {
                                 (for A/B measurements) */
   TT_OPT_NO_HALO = 6,        /* ConvLSTM fetches one activation box per tap instead of one haloed patch per channel
                                 slab (for A/B measurements) */
-  TT_OPT_FUSED_PRE = 7,      /* bf16 path: run the preprocessing inside the first encoder layer instead of as a kernel of its
-                                own that writes the resized fp32 image (same bits; slower as measured, kept for A/B
-                                measurements; ignored where the layer or the resize factor does not allow it) */
+  TT_OPT_FUSED_PRE = 7,      /* bf16 path: the first encoder layer samples the frames itself in any case where its width and
+                                the resize factor allow; with this option it does not write the resized fp32 image on the way (same bits;
+                                tt_debug_tensor makes the image anew, from frame buffers that must then still be valid), not even
+                                as a separate kernel when stage events are on */
   TT_OPT_NO_POST_TC = 3      /* bf16 path: post-process from the fp32 hidden state, not from its bf16 copy on the
                                 tensor cores (for A/B measurements; not available for feed-forward models) */
 } tt_option;

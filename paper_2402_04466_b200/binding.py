@@ -159,7 +159,7 @@ def make_config(wl, max_streams: int = 1, device: int = 0, overlay: Optional[boo
     """Fill a tt_config from any object carrying the workload attributes (src_w, net_w, enc_cout, ...).
 
     plain_launches=True makes every tick launch its kernels one by one instead of replaying a CUDA graph.
-    fused_pre=True runs the preprocessing inside the first encoder layer (bf16 path; same bits, measured slower)."""
+    fused_pre=True: the first encoder layer, which samples the frames itself, does not write the resized image (bf16 path; same bits)."""
     cfg = tt_config()
     cfg.struct_size = C.sizeof(tt_config)
     cfg.abi_version = TT_ABI_VERSION

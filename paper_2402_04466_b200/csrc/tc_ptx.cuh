@@ -253,6 +253,12 @@ __device__ __forceinline__ void st_global_v8_b32(void* p, const uint32_t (&v)[8]
                : "memory");
 }
 
+// max(a, 0) and max(b, 0) as a pair of bf16, one instruction
+__device__ __forceinline__ uint32_t pack_relu_bf16(float a, float b) {
+  uint32_t r;
+  asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  return r;
+}
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
   __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
   return *reinterpret_cast<uint32_t*>(&v);

@@ -77,6 +77,19 @@ uint16_t f32_to_bf16_rne(float f) {
 }
 
 int conv_out(int n, int s) { return (n + 2 - 3) / s + 1; }
+
+// Sample position of output o of an axis resized from `in` to `out`: (scale * left source index, bits of the right
+// one's weight), the arithmetic of pre::axis_sample.
+int2 axis_entry(int o, int in, int out, int scale) {
+  const int den = 2 * out;
+  const int num = std::max(0, std::min((2 * o + 1) * in - out, (in - 1) * den));
+  const int i0 = num / den;
+  const float f = (float)(num - i0 * den) / (float)den;
+  int2 e;
+  e.x = scale * i0;
+  std::memcpy(&e.y, &f, 4);
+  return e;
+}
 int round_up(int a, int b) { return (a + b - 1) / b * b; }
 
 }  // namespace
@@ -114,7 +127,8 @@ struct tt_ctx {
   bool use_post_tc = false;
   ConvFirstTcParams first_tc{}; // bf16 path, first encoder layer on the tensor cores when its width (32 or 64) allows
   bool use_first_tc = false;
-  bool fuse_pre = false;        // the first layer samples the frames itself; no preprocess launch, ctx->pre is not written
+  bool fuse_first = false;      // the first layer samples the frames itself: one launch for preprocessing and first layer
+  bool fuse_pre = false;        // TT_OPT_FUSED_PRE: and it does not write the resized image (ctx->pre), not even with stage events on
   FramePtrs fp_inflight{};      // device frame pointers of the submit being described (saved per slot)
   SimtLayer simt_enc[TT_MAX_ENC];
   SimtLayer simt_lstm;
@@ -588,9 +602,18 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
         if ((st = encode_map_f32(ctx, &f.map_in, ctx->pre, 4, dims, str, box)) != TT_OK) return st;
       }
       ctx->use_first_tc = true;
-      ctx->fuse_pre = c.options[TT_OPT_FUSED_PRE] != 0 &&
-                      conv_first_tc_staging(f.stride, c.src_w, c.src_h, c.net_w, c.net_h, &f.src_rows_cap, &f.src_row_cap);
-      f.fused = ctx->fuse_pre ? 1 : 0;
+      ctx->fuse_first = conv_first_fused_staging(f.stride, c.src_w, c.src_h, c.net_w, c.net_h, &f.src_rows_cap, &f.src_row_cap);
+      ctx->fuse_pre = ctx->fuse_first && c.options[TT_OPT_FUSED_PRE] != 0;
+      if (ctx->fuse_first) {
+        std::vector<int2> xt((size_t)c.net_w), yt((size_t)c.net_h);
+        for (int o = 0; o < c.net_w; ++o) xt[o] = axis_entry(o, c.src_w, c.net_w, 3);
+        for (int o = 0; o < c.net_h; ++o) yt[o] = axis_entry(o, c.src_h, c.net_h, 1);
+        int2 *dx = nullptr, *dy = nullptr;
+        if ((st = upload(ctx, &dx, xt)) != TT_OK) return st;
+        if ((st = upload(ctx, &dy, yt)) != TT_OK) return st;
+        f.xtab = dx; f.ytab = dy; f.pre_out = ctx->pre;
+        f.one_row = std::all_of(yt.begin(), yt.end(), [](const int2& e) { return e.y == 0; }) ? 1 : 0;
+      }
       f.src_w = c.src_w; f.src_h = c.src_h; f.src_pitch = c.src_pitch;
       f.scale = pre::norm_scale(1.0f / c.norm_div, 1.0f / c.norm_std);
       f.shift = pre::norm_shift(c.norm_mean, 1.0f / c.norm_std);
@@ -731,7 +754,10 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     h_out.v[n] = slot * 2 + (1 - half);
   }
 
-  if (!ctx->fuse_pre) {
+  // With stage events on, preprocessing and first layer run as the two kernels they were, so that each has its time; the
+  // results are the same bits.
+  const bool fused = ctx->fuse_first && (ctx->fuse_pre || !ctx->profiling);
+  if (!fused) {
     TT_CUDA(ctx, launch_preprocess(preprocess_params(ctx, K, frames, ctx->cur_tab), s));
     if ((ms_ = mark_stage(ctx, TT_STAGE_PREPROCESS, 1)) != TT_OK) return ms_;
   }
@@ -766,10 +792,12 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   } else {
     if (ctx->use_first_tc) {
       ctx->first_tc.K = K;
-      // with the preprocessing inside it the kernel is the first of the tick and may follow a copy: launched normally
-      ctx->first_tc.pdl = (ctx->profiling || ctx->fuse_pre) ? 0 : 1;
+      ctx->first_tc.pdl = ctx->profiling ? 0 : 1;
       ctx->first_tc.src = frames; ctx->first_tc.src_tab = ctx->cur_tab;
-      TT_CUDA(ctx, launch_conv_first_tc(ctx->first_tc, ctx->sm_count, s));
+      ctx->first_tc.write_pre = ctx->fuse_pre ? 0 : 1;
+      // the fused kernel is the first of the tick and may follow a copy: launched normally
+      if (fused) TT_CUDA(ctx, launch_conv_first_fused(ctx->first_tc, ctx->sm_count, s));
+      else TT_CUDA(ctx, launch_conv_first_tc(ctx->first_tc, ctx->sm_count, s));
       if ((ms_ = mark_stage(ctx, TT_STAGE_ENC0, 1)) != TT_OK) return ms_;
     } else {
       const SimtLayer& L = ctx->simt_enc[0];

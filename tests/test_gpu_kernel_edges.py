@@ -31,3 +31,38 @@ def test_fp32_convolutions_at_the_edges_of_their_tiles(cuda_device, net, enc, st
         for k in range(K):
             _compare_frame(ctx, states[k], res[k], oras[k].step(frames[k][t]), 1e-4, 1e-3, tag=f"edges k={k} t={t}")
     ctx.destroy()
+
+
+@pytest.mark.parametrize("shape", [
+    dict(src_w=214, src_h=120, net_w=160, net_h=120),                                    # rows not resized
+    dict(src_w=300, src_h=233, net_w=132, net_h=70),                                     # both axes down, a last tile of 2 columns and 3 rows
+    dict(src_w=90, src_h=50, net_w=196, net_h=131, enc_stride=(1, 2, 2)),                # up-scaling, stride 1
+    dict(src_w=96, src_h=99, net_w=32, net_h=33, enc_cout=(64, 64), enc_stride=(1, 2)),  # every row on a frame row (a third), one tile wide
+    dict(src_w=640, src_h=700, net_w=260, net_h=192, enc_cout=(64, 128, 256), hidden=256),   # several tiles per block
+])
+def test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cuda_device, shape):
+    """One kernel resizes, normalises and convolves; with stage events on the two kernels it stands for run instead.  Same expressions, same
+    order of products: the resized image, the first layer's map, every result and the state are the same bits."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="first", **{"hidden": 64, **shape})
+    K, n = 3, 2
+    host = _frames(wl, K, n)
+    runs = []
+    for separate in (False, True):
+        ctx, states, _ = _make(wl, K)
+        ctx.set_profiling(separate)
+        out = []
+        for t in range(n):
+            # stream 1 at an odd address, the frame's last byte the buffer's last
+            bufs = [torch.empty(host[k][t].size + k, dtype=torch.uint8, device=cuda_device) for k in range(K)]
+            for k in range(K):
+                bufs[k][k:].copy_(torch.from_numpy(host[k][t]).reshape(-1))
+            ctx.submit_frames([bufs[k][k:] for k in range(K)], states, frame_index=t)
+            res = ctx.sync()
+            out += [a for i, r in enumerate(res) for a in (ctx.fetch_probs(r), ctx.fetch_masks(r), r["conf"], r["cx"], ctx.debug_tensor(states[i], "pre"),
+                                                           ctx.debug_tensor(states[i], "enc0"))]
+        if separate:
+            assert ctx.get_stage_times()["preprocess"] > 0
+        runs.append(out + [a for s in states for a in ctx.state_export(s)])
+        ctx.destroy()
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
