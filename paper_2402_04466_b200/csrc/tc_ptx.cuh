@@ -62,6 +62,36 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same wait for a whole warp whose control flow has to stay uniform: the usual case, the phase completing within a few
+// suspended tries, is a loop inside the assembly, so that the compiler sees straight-line code and can keep what the warp
+// works on in uniform registers.  Every lane gets the same answer.
+__device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code,
+                                                  long long limit) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+      "mov.u32 n, 8;\n"
+      "WAIT_%=:\n\t"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+      "@p bra DONE_%=;\n\t"
+      "sub.u32 n, n, 1;\n\t"
+      "setp.ne.u32 q, n, 0;\n\t"
+      "@q bra WAIT_%=;\n"
+      "DONE_%=:\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity), "r"(TRY_WAIT_SUSPEND_NS)
+      : "memory");
+  if (__builtin_expect(ok == 0u, 0)) ok = mbar_wait(bar, parity, abort_flag, status, code, limit) ? 1u : 0u;
+  return ok != 0u;
+}
+// true in one lane of a converged warp
+__device__ __forceinline__ bool elect_one() {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
+  return r != 0u;
+}
+
 // The last kernel of a tick tells the host, through a mapped word, of a wait that ran out in it or before it: `before` is the
 // status word as it stood when the kernel's predecessors were done.  A healthy tick writes nothing.  One thread of every
 // block calls it after the block's last wait.
@@ -219,6 +249,20 @@ __device__ __forceinline__ void umma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
+// as tmem_ld32, without the wait: the values may be used after tmem_wait_ld
+__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&v)[32]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+        "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+        "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+        "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+      : "r"(taddr)
+      : "memory");
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
@@ -253,10 +297,11 @@ __device__ __forceinline__ void st_global_v8_b32(void* p, const uint32_t (&v)[8]
                : "memory");
 }
 
-// max(a, 0) and max(b, 0) as a pair of bf16, one instruction
+// max(a, 0) and max(b, 0) as a pair of bf16: rounded first, then both compared in one instruction.  A NaN becomes 0, as
+// with fmaxf (the conversion's own .relu would keep it).
 __device__ __forceinline__ uint32_t pack_relu_bf16(float a, float b) {
   uint32_t r;
-  asm("cvt.rn.relu.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(b), "f"(a));
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n\tmax.bf16x2 %0, %0, %3;" : "=&r"(r) : "f"(b), "f"(a), "r"(0u));
   return r;
 }
 __device__ __forceinline__ uint32_t pack_bf16(float a, float b) {

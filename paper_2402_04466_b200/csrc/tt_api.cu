@@ -46,6 +46,7 @@ struct TcLayer {
   bool has_halo = false;
   TensorMap128 map_b[3];       // block_n = 64, 128, 256
   bool has_b[3] = {false, false, false};
+  ConvS2Params s2{};           // stride-2 layers that conv_s2 covers (s2.block_n > 0)
 };
 
 std::mutex g_err_mu;
@@ -627,6 +628,26 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
       if ((st = make_act_maps(ctx, &L.maps_a[0], reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l - 1]), S, ctx->lay_h[l],
                               ctx->lay_w[l], ctx->lay_c[l], c.enc_stride[l], L.slab_c)) != TT_OK)
         return st;
+      if (L.stride == 2 && conv_s2_block_n(L.slab_c, L.cin0, L.cout) > 0) {
+        const int H = ctx->lay_h[l], W = ctx->lay_w[l], C = ctx->lay_c[l];
+        ConvS2Params& q = L.s2;
+        for (int v = 0; v < 4; ++v) {
+          const int yp = v >> 1, xp = v & 1;
+          int bw, bh;
+          conv_s2_box(v, &bw, &bh);
+          const cuuint64_t dims[4] = {(cuuint64_t)C, (cuuint64_t)(xp ? W / 2 : (W + 1) / 2), (cuuint64_t)(yp ? H / 2 : (H + 1) / 2), (cuuint64_t)S};
+          const cuuint64_t str[3] = {(cuuint64_t)2 * C * 2, (cuuint64_t)2 * W * C * 2, (cuuint64_t)H * W * C * 2};
+          const cuuint32_t box[4] = {(cuuint32_t)L.slab_c, (cuuint32_t)bw, (cuuint32_t)bh, 1};
+          if ((st = encode_map(ctx, &q.map_v[v], reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l - 1]) + ((size_t)yp * W + xp) * C, 4, dims, str, box, L.slab_c * 2)) != TT_OK)
+            return st;
+        }
+        q.block_n = conv_s2_block_n(L.slab_c, L.cin0, L.cout);
+        q.map_b = L.map_b[0];
+        q.slab_c = L.slab_c; q.cout = L.cout; q.n_tiles_n = L.cout / q.block_n;
+        q.Ho = ctx->lay_h[l + 1]; q.Wo = ctx->lay_w[l + 1]; q.tiles_x = (q.Wo + 7) / 8; q.tiles_y = (q.Ho + 15) / 16;
+        q.bias = L.b; q.out = reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l]);
+        q.status = ctx->status_dev; q.wait_limit = ctx->wait_limit; q.one_per_sm = ctx->enc_two_per_sm ? 0 : 1;
+      }
     }
     TcLayer& L = ctx->tc_lstm;
     if (!ctx->feed_forward) {
@@ -835,6 +856,15 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     };
     for (int l = 1; l < ctx->n_enc; ++l) {
       const TcLayer& L = ctx->tc_enc[l];
+      // both kernels add up the same products in the same order: which one runs changes no bit
+      if (L.s2.block_n > 0 && conv_s2_pays(L.s2.slab_c, K * L.s2.tiles_x * L.s2.tiles_y * L.s2.n_tiles_n, ctx->sm_count)) {
+        ConvS2Params q = L.s2;
+        q.K = K;
+        q.pdl = ctx->profiling ? 0 : 1;
+        TT_CUDA(ctx, launch_conv_s2(q, ctx->sm_count, s));
+        if ((ms_ = mark_stage(ctx, TT_STAGE_ENC0 + l, 1)) != TT_OK) return ms_;
+        continue;
+      }
       ConvTcParams q{};
       tt_status st = fill_common(q, L, ctx->lay_h[l + 1], ctx->lay_w[l + 1], true);
       if (st != TT_OK) return st;

@@ -5,7 +5,7 @@ import torch
 
 import oracle
 import tt_synth
-from test_gpu_pipeline import _compare_frame, _frames, _make
+from test_gpu_pipeline import _compare_frame, _frames, _make, _run_bf16
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +66,43 @@ def test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cud
         ctx.destroy()
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("net,enc,stride,hidden,K", [
+    ((150, 110), (32, 128), (1, 2), 64, 2),            # 32 -> 128, 75 x 55 outputs: ragged in both directions
+    ((66, 66), (64, 64), (1, 2), 64, 1),               # 64 -> 64, a last tile of one column and one row
+    ((97, 131), (64, 64, 128, 128), (1, 2, 2, 2), 64, 3),   # odd inputs; 64 -> 128 resident, 128 -> 128 through the ring
+    ((130, 70), (32, 64, 128, 256), (1, 2, 2, 2), 64, 2),   # 128 -> 256 through the ring
+    ((128, 128), (64, 256), (2, 2), 64, 2),            # two groups of 128 resident outputs
+    ((16, 12), (32, 64), (2, 2), 64, 1),               # a map smaller than one tile
+])
+def test_bf16_stride2_layers_at_the_edges_of_their_tiles(cuda_device, net, enc, stride, hidden, K):
+    """The bounds of the other bf16 tests (_run_bf16): outputs 2e-2, intermediate maps 5e-2 of the oracle."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="s2", src_w=net[0] + 20, src_h=net[1] + 11, net_w=net[0], net_h=net[1], enc_cout=enc,
+                                              enc_stride=stride, hidden=hidden)
+    _run_bf16(cuda_device, wl, K, 2)
+
+
+def test_stride2_layer_kernels_give_the_same_bits_at_small_and_large_batches(cuda_device):
+    """One stream's strided layers run as a few tiles per block on views fetched with their halo, eight streams' as many tiles
+    per block with one box per tap: the same products in the same order, so a stream's maps, results and state must not change."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="s2-batch", src_w=800, src_h=500)
+    K = 8
+    host = [tt_synth.make_frames(wl.frame_kind, wl.stream_seed(s), 1, wl.src_w, wl.src_h)[0] for s in range(K)]
+    frames = [torch.from_numpy(f).to(cuda_device) for f in host]
+
+    def observe(ctx, st, r):
+        return [ctx.debug_tensor(st, "enc1"), ctx.debug_tensor(st, "enc2"), ctx.fetch_probs(r), r["conf"], r["cx"], *ctx.state_export(st)]
+
+    ctx, states, _ = _make(wl, K)
+    ctx.submit_frames(frames, states)
+    res = ctx.sync()
+    batch = {k: observe(ctx, states[k], res[k]) for k in (0, 7)}
+    ctx.destroy()
+    for k in (0, 7):
+        ctx, (st,), _ = _make(wl, 1)
+        ctx.submit_frames([frames[k]], [st])
+        (r,) = ctx.sync()
+        for a, b in zip(batch[k], observe(ctx, st, r)):
+            assert np.array_equal(a, b)
+        ctx.destroy()
