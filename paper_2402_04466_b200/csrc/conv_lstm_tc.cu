@@ -1,0 +1,347 @@
+// ConvLSTM step of the bf16 path on the tensor cores, 64-channel slabs, for launches whose units of 256 columns would leave
+// a good part of the last round of multiprocessors idle: the 3x3 convolution over [x, h] into i/f/g/o gates as an
+// implicit GEMM (M = output pixels, N = 4 x hidden, K = 9 taps x channels), gate math, c' and h' in the epilogue.
+//
+// Tiles and operands are those of the haloed form in conv_tc.cu (8 x 16 output pixels; one haloed patch of 18 x 10 pixels
+// per 64-channel slab, which the nine taps read in place; weights one tap and slab at a time through a ring of five stages,
+// the first fetched before the wait for the previous kernel), and the order of the sums is the same, so the results
+// are the same bits.
+//
+// Bound by rounds: a multiprocessor holds one block, and 80 units of 256 columns (one 854x480 stream) take as long as 148.  A unit
+// here is a tile x a group of columns of any multiple of 64 up to 256, grouped as the launch needs: by 192 where that
+// still fits the rounds, or by 256 with the last, partly filled round cut into halves.  M128 x N x K16 takes 128, 96 and 64
+// cycles at N = 256, 192 and 128; for a narrow group's slab to take less than a wide one's, the whole MMA warp
+// runs the issue loop and one elected lane issues (from a single lane's branch a slab takes about 600 cycles at any width).
+// ConvLSTM stage with its event, units of 256 -> this: one 854x480 stream 23.6 -> 20.5 us, one full-HD stream 105.5 -> 101.4 us.
+//
+// Warp roles (384 threads): 0 = patches by TMA; 10, 11 = weights by TMA, alternate iterations; 1 = tensor memory and MMA
+// issue; 2..9 = epilogue (TMEM lane quarter = warp mod 4, two warps per quarter sharing a unit's columns).  Two accumulators,
+// so the epilogue of a unit overlaps the next one's products.  All waits are bounded (see tc_ptx.cuh).
+#include <algorithm>
+
+#include "tt_internal.h"
+#include "tc_ptx.cuh"
+
+namespace tt {
+namespace {
+
+using namespace tc;
+
+constexpr int L_THREADS = 384;
+constexpr int L_EPI_WARPS = 8, L_EPI_WARP0 = 2;
+constexpr int L_PW = 8, L_PH = 16;                       // output tile
+constexpr int L_PITCH = 10, L_ROWS = 18;                 // haloed patch
+constexpr int L_A_TX = L_ROWS * L_PITCH * 128;
+constexpr int L_A_BYTES = (L_A_TX + 1023) / 1024 * 1024;
+constexpr int L_A_STAGES = 2;
+constexpr int L_B_BYTES = 256 * 128;                     // widest group: 256 rows of 64 channels
+constexpr int L_B_STAGES = 5;
+constexpr int L_MAX_COLS = 4 * 512;
+constexpr int L_SMEM = L_B_STAGES * L_B_BYTES + L_A_STAGES * L_A_BYTES + L_MAX_COLS * 4 + 256 + 1024 /*alignment slack*/;
+static_assert(L_SMEM <= 227 * 1024, "one block per multiprocessor");
+
+// One special-function instruction each: tanh.approx (relative error about 2^-11, far inside
+// the bf16 path's tolerance) and sigmoid(z) = 0.5 + 0.5 * tanh(z / 2).
+__device__ __forceinline__ float fast_tanh(float z) {
+  float y;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(z));
+  return y;
+}
+__device__ __forceinline__ float fast_sigmoid(float z) { return fmaf(0.5f, fast_tanh(0.5f * z), 0.5f); }
+
+struct Unit {
+  int m, col0, n;   // pixel tile, first column, columns
+};
+// Units in order of tile, then column group; from unit u_full on every group is cut into two.
+__device__ __forceinline__ Unit unit_at(const ConvLstmParams& p, int u) {
+  Unit t;
+  const int v = u - p.u_full, g = v < 0 ? u : p.u_full + (v >> 1);
+  t.m = g / p.groups;
+  t.col0 = (g - t.m * p.groups) * p.width;
+  t.n = min(p.width, p.cols - t.col0);
+  if (v >= 0) {
+    t.n >>= 1;
+    t.col0 += (v & 1) * t.n;
+  }
+  return t;
+}
+
+__global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_constant__ ConvLstmParams p) {
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t* s_b = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint8_t* s_a = s_b + L_B_STAGES * L_B_BYTES;
+  float* s_bias = reinterpret_cast<float*>(s_a + L_A_STAGES * L_A_BYTES);
+  uint64_t* bfull = reinterpret_cast<uint64_t*>(s_bias + L_MAX_COLS);   // [L_B_STAGES]
+  uint64_t* bempty = bfull + L_B_STAGES;                                // [L_B_STAGES]
+  uint64_t* afull = bempty + L_B_STAGES;                                // [2] patch landed
+  uint64_t* aempty = afull + 2;                                         // [2] all nine taps have read the patch
+  uint64_t* tfull = aempty + 2;                                         // [2]
+  uint64_t* tempty = tfull + 2;                                         // [2]
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  __shared__ int s_img[3][TT_MAX_STREAMS];                              // h in, c, h out
+
+  // broadcast, so that the compiler knows the roles below to be whole warps
+  const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
+  const long long wait_limit = p.wait_limit;
+  const int total = p.u_full + 2 * (p.tiles * p.groups - p.u_full);
+  const int slabs = p.slabs[0] + p.slabs[1];
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < L_B_STAGES; ++s) {
+      mbar_init(smem_u32(bfull + s), 1);
+      mbar_init(smem_u32(bempty + s), 1);
+    }
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(smem_u32(afull + a), 1);
+      mbar_init(smem_u32(aempty + a), 1);
+      mbar_init(smem_u32(tfull + a), 1);
+      mbar_init(smem_u32(tempty + a), L_EPI_WARPS);
+    }
+    *abort_flag = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b64) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.maps[0]) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.maps[1]) : "memory");
+  }
+  if (warp == 1) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  for (int i = threadIdx.x; i < p.cols; i += L_THREADS) s_bias[i] = __ldg(p.bias + i);
+  if (threadIdx.x < TT_MAX_STREAMS) {
+    s_img[0][threadIdx.x] = p.h_in.v[threadIdx.x];
+    s_img[1][threadIdx.x] = p.c_idx.v[threadIdx.x];
+    s_img[2][threadIdx.x] = p.h_out.v[threadIdx.x];
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_slot;
+  pdl_launch_dependents();   // behind the allocation: a dependent block must not take tensor memory that this grid still needs
+
+  const int tiles_per_img = p.tiles_x * p.tiles_y;
+  if (warp == 0 && lane == 0) {
+    // ----------------------------------------------------------------------- patches
+    pdl_wait();   // x is the previous kernel's output
+    uint32_t stage = 0, phase = 0;
+    bool ok = true;
+    for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
+      const int m = unit_at(p, u).m;
+      const int img = m / tiles_per_img, rem = m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
+      const int img_h = s_img[0][img];
+      for (int sg = 0; sg < slabs; ++sg) {
+        ok = mbar_wait(smem_u32(aempty + stage), phase ^ 1u, abort_flag, p.status, 0x900 + (int)stage, wait_limit);
+        if (!ok) break;
+        const int src = sg < p.slabs[0] ? 0 : 1;
+        mbar_arrive_expect_tx(smem_u32(afull + stage), L_A_TX);
+        tma_load_4d(smem_u32(s_a + stage * L_A_BYTES), &p.maps[src], smem_u32(afull + stage), (src ? sg - p.slabs[0] : sg) * 64,
+                    tx * L_PW - 1, ty * L_PH - 1, src ? img_h : img);
+        if (++stage == L_A_STAGES) { stage = 0; phase ^= 1u; }
+      }
+    }
+  } else if (warp >= L_EPI_WARP0 + L_EPI_WARPS && lane == 0) {
+    // ----------------------------------------------------------------------- weights
+    // producer j of two owns iterations j, j + 2, ... of the block's sequence (slab-major, tap inside)
+    const int j = warp - (L_EPI_WARP0 + L_EPI_WARPS);
+    const int iters = slabs * 9, cin = slabs * 64;
+    uint32_t stage = (uint32_t)j, phase = 0;
+    int it = j;
+    bool ok = true;
+    for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
+      const Unit t = unit_at(p, u);
+      for (; it < iters; it += 2) {
+        const int sg = it / 9, tap = it - sg * 9;
+        ok = mbar_wait(smem_u32(bempty + stage), phase ^ 1u, abort_flag, p.status, 0x100 + (int)stage, wait_limit);
+        if (!ok) break;
+        const uint32_t bar = smem_u32(bfull + stage), dst = smem_u32(s_b + stage * L_B_BYTES);
+        const int k0 = tap * cin + sg * 64;
+        mbar_arrive_expect_tx(bar, (uint32_t)t.n * 128u);
+        if (t.n == 256) {
+          tma_load_2d(dst, &p.map_b, bar, k0, t.col0);
+        } else {
+          for (int i = 0; i < t.n; i += 64) tma_load_2d(dst + i * 128, &p.map_b64, bar, k0, t.col0 + i);
+        }
+        stage += 2;
+        if (stage >= (uint32_t)L_B_STAGES) { stage -= L_B_STAGES; phase ^= 1u; }
+      }
+      it -= iters;
+    }
+  } else if (warp == 1) {
+    // -------------------------------------------------------------------- MMA issuer
+    const bool issuer = elect_one();
+    uint32_t stage = 0, phase = 0, acc_phase = 0, a_stage = 0, a_phase = 0;
+    int acc = 0;
+    bool ok = true;   // a wait that ran out ends the loop at the end of its unit
+    const uint64_t b_desc0 = make_smem_desc(smem_u32(s_b), 1024u, 2u);
+    for (int u = blockIdx.x; u < total; u += gridDim.x) {
+      // (no division in this loop where all groups are as wide)
+      const int n = p.even ? (u < p.u_full ? p.width : p.width >> 1) : unit_at(p, u).n;
+      const uint32_t idesc = make_idesc(128, 0) | ((uint32_t)(n >> 3) << 17);
+      ok &= mbar_wait_uniform(smem_u32(tempty + acc), acc_phase ^ 1u, abort_flag, p.status, 0x200 + acc, wait_limit);
+      tc_fence_after();   // the epilogue's reads of this accumulator come before the MMAs that overwrite it
+      const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
+      for (int sg = 0; sg < slabs; ++sg) {
+        ok &= mbar_wait_uniform(smem_u32(afull + a_stage), a_phase, abort_flag, p.status, 0xA00 + (int)a_stage, wait_limit);
+        const uint64_t a_patch = make_smem_desc(smem_u32(s_a + a_stage * L_A_BYTES), L_PITCH * 128u, 2u);
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap) {
+          ok &= mbar_wait_uniform(smem_u32(bfull + stage), phase, abort_flag, p.status, 0x300 + (int)stage, wait_limit);
+          const uint64_t a = a_patch + (uint64_t)(((tap / 3) * L_PITCH + tap % 3) * 128 >> 4);
+          const uint64_t b = b_desc0 + (uint64_t)stage * (uint64_t)(L_B_BYTES >> 4);
+          if (issuer) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units further on inside the swizzle atom
+              umma_bf16(d_tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, (tap == 0 && k == 0) ? (sg != 0 ? 1u : 0u) : 1u);
+            umma_commit(smem_u32(bempty + stage));
+            if (tap == 8) umma_commit(smem_u32(aempty + a_stage));
+          }
+          if (++stage == L_B_STAGES) { stage = 0; phase ^= 1u; }
+        }
+        if (++a_stage == L_A_STAGES) { a_stage = 0; a_phase ^= 1u; }
+      }
+      if (__any_sync(0xffffffffu, !ok)) break;
+      if (issuer) umma_commit(smem_u32(tfull + acc));
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+    }
+  } else if (warp >= L_EPI_WARP0 && warp < L_EPI_WARP0 + L_EPI_WARPS) {
+    // ---------------------------------------------------------------------- epilogue
+    pdl_wait();
+    const int quarter = warp & 3, half = (warp - L_EPI_WARP0) >> 2;
+    const int row = quarter * 32 + lane, py = row >> 3, px = row & 7;     // row of the 128-row tile = pixel of the patch
+    uint32_t acc_phase = 0;
+    int acc = 0;
+    for (int u = blockIdx.x; u < total; u += gridDim.x) {
+      const Unit t = unit_at(p, u);
+      const int img = t.m / tiles_per_img, rem = t.m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
+      const int x = tx * L_PW + px, y = ty * L_PH + py;
+      const bool valid = x < p.Wm && y < p.Hm;
+      const size_t pix = (size_t)y * p.Wm + x;
+      // chunks of 32 columns (8 hidden units x 4 gates): the first of the quarter's two warps takes 128 columns of a wide
+      // group and half of a narrow one, so that every pair of chunks starts on 32 bytes of h'
+      const int first = t.n > 128 ? 128 : t.n >> 1;
+      const int off = half ? first : 0, chunks = (half ? t.n - first : first) >> 5;
+      const int col0 = t.col0 + off;
+
+      // the old cell state of this thread's pixel is fetched before the accumulator is waited for: its latency hides under
+      // the unit's products
+      float c_old[4][8];
+      const size_t so = ((size_t)s_img[1][img] * p.Hm * p.Wm + pix) * p.hidden + (col0 >> 2);
+      const size_t ho = ((size_t)s_img[2][img] * p.Hm * p.Wm + pix) * p.hidden + (col0 >> 2);
+#pragma unroll
+      for (int ck = 0; ck < 4; ++ck)
+        if (valid && ck < chunks) ld_global_v8(p.c_state + so + ck * 8, c_old[ck]);
+
+      // the warp votes: its lanes leave the loop together or go on to the warp-collective TMEM loads together
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(tfull + acc), acc_phase, abort_flag, p.status, 0x400 + acc, wait_limit))) break;
+      tc_fence_after();
+      const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 256 + off);
+      uint32_t hb[8];
+#pragma unroll
+      for (int ck = 0; ck < 4; ++ck) {
+        if (ck < chunks) {
+          uint32_t v[32];
+          tmem_ld32(taddr + (uint32_t)(ck * 32), v);
+          if (valid) {
+            // packed column = 4 * unit + gate (i, f, g, o)
+            const float4* b4 = reinterpret_cast<const float4*>(s_bias + col0 + ck * 32);
+            float c_new[8], h_new[8];
+#pragma unroll
+            for (int jj = 0; jj < 8; ++jj) {
+              const float4 b = b4[jj];
+              const float gi = __uint_as_float(v[4 * jj + 0]) + b.x;
+              const float gf = __uint_as_float(v[4 * jj + 1]) + b.y;
+              const float gg = __uint_as_float(v[4 * jj + 2]) + b.z;
+              const float go = __uint_as_float(v[4 * jj + 3]) + b.w;
+              c_new[jj] = fast_sigmoid(gf) * c_old[ck][jj] + fast_sigmoid(gi) * fast_tanh(gg);
+              h_new[jj] = fast_sigmoid(go) * fast_tanh(c_new[jj]);
+            }
+            st_global_v8(p.c_state + so + ck * 8, c_new);
+            if (p.h_f32) st_global_v8(p.h_f32 + so + ck * 8, h_new);
+            // bf16 copy of h': 8 values are half a sector, so two neighbouring chunks leave together
+            const int hq = (ck & 1) * 4;
+            hb[hq + 0] = pack_bf16(h_new[0], h_new[1]);
+            hb[hq + 1] = pack_bf16(h_new[2], h_new[3]);
+            hb[hq + 2] = pack_bf16(h_new[4], h_new[5]);
+            hb[hq + 3] = pack_bf16(h_new[6], h_new[7]);
+            if (ck & 1) st_global_v8_b32(p.h_bf16 + ho + (ck - 1) * 8, hb);
+            else if (ck + 1 == chunks) *reinterpret_cast<uint4*>(p.h_bf16 + ho + ck * 8) = make_uint4(hb[0], hb[1], hb[2], hb[3]);
+          }
+        }
+      }
+      // hand the accumulator back to the MMA warp
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(tempty + acc));
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+    }
+  }
+
+  // ------------------------------------------------------------------------------- teardown
+  __syncwarp();
+  if (*abort_flag) {
+    // a wait ran out somewhere: give copies and MMAs in flight time to land before their memory is released
+    for (int i = 0; i < 64; ++i) __nanosleep(16000);
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 1) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+  }
+}
+
+// Time of a unit in units of one of 256 columns: tensor cycles per slab (512, 384, 256) but no less than the issue loop's
+// round of about 300, and the fixed parts.
+constexpr double L_COST_256 = 1.0, L_COST_192 = 0.77, L_COST_128 = 0.58;
+
+struct Grouping {
+  int width = 256, u_full = 0;
+  double cost = 0, plain = 0;   // rounds x time of a unit, as chosen and with groups of 256 throughout
+};
+Grouping group_columns(int tiles, int C, int sm_count) {
+  Grouping g;
+  auto rounds = [&](long units) { return (double)((units + sm_count - 1) / sm_count); };
+  const long g256 = (long)tiles * ((C + 255) / 256);
+  g.u_full = (int)g256;
+  g.cost = g.plain = rounds(g256) * L_COST_256;
+  // the last round cut into halves, if that leaves it one round
+  const long tail = g256 % sm_count;
+  if (C % 256 == 0 && tail > 0 && 2 * tail <= sm_count) {
+    g.cost = (double)(g256 / sm_count) * L_COST_256 + L_COST_128;
+    g.u_full = (int)(g256 - tail);
+  }
+  for (int w : {192, 128}) {
+    if (w >= C) continue;
+    const long units = (long)tiles * ((C + w - 1) / w);
+    const double t = rounds(units) * (w == 192 ? L_COST_192 : L_COST_128);
+    if (t < g.cost - 1e-9) { g.cost = t; g.width = w; g.u_full = (int)units; }
+  }
+  return g;
+}
+
+}  // namespace
+
+// Five per cent of the estimated time at least: 23 % for one 854x480 stream (80 units of 256 on 148 multiprocessors -> 120 of up
+// to 192), 10 % for one full-HD stream (480 -> 444 and 72 halves).  Where the rounds are full (eight full-HD streams)
+// conv_tc.cu's form is 2 % faster.
+bool conv_lstm_pays(int tiles, int cols, int sm_count) {
+  const Grouping g = group_columns(tiles, cols, sm_count);
+  return cols >= 256 && cols <= L_MAX_COLS && g.cost < 0.95 * g.plain;
+}
+
+cudaError_t launch_conv_lstm(const ConvLstmParams& p, int sm_count, cudaStream_t s) {
+  cudaError_t e = cudaFuncSetAttribute(conv_lstm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L_SMEM);
+  if (e != cudaSuccess) return e;
+  if (p.cols % 64 || p.cols < 256 || p.cols > L_MAX_COLS) return cudaErrorInvalidValue;
+  ConvLstmParams q = p;
+  const Grouping g = group_columns(p.tiles, p.cols, sm_count);
+  q.width = g.width;
+  q.u_full = g.u_full;
+  q.groups = (p.cols + q.width - 1) / q.width;
+  q.even = p.cols % q.width == 0;
+  const long total = q.u_full + 2L * ((long)q.tiles * q.groups - q.u_full);
+  return launch_kernel(conv_lstm_kernel, (int)std::min<long>(total, sm_count), L_THREADS, L_SMEM, s, q, p.pdl != 0);
+}
+
+}  // namespace tt

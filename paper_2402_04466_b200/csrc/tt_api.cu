@@ -880,12 +880,25 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     ConvTcParams q{};
     tt_status st = fill_common(q, L, ctx->Hm, ctx->Wm, false);
     if (st != TT_OK) return st;
-    q.n_src = 2; q.slabs[0] = L.cin0 / L.slab_c; q.slabs[1] = L.cin1 / L.slab_c; q.img0 = ident; q.img1 = h_in;
-    // with the heads on the tensor cores nothing on the path reads an fp32 copy of h': its consumers (the next
-    // step's convolution and the heads) take the bf16 copy, so only that copy is written
-    q.epilogue = TC_EPI_LSTM; q.c_state = ctx->c_state; q.h_f32 = ctx->use_post_tc ? nullptr : ctx->h_f32; q.h_bf16 = ctx->h_bf16;
-    q.c_idx = c_idx; q.h_out_idx = h_out; q.hidden = ctx->Ch;
-    TT_CUDA(ctx, launch_conv_tc(q, ctx->sm_count, s));
+    // both kernels add up the same products in the same order: which one runs changes no bit
+    if (q.halo && conv_lstm_pays(K * q.tiles_x * q.tiles_y, L.cout, ctx->sm_count)) {
+      ConvLstmParams w{};
+      w.maps[0] = L.maps_halo[0]; w.maps[1] = L.maps_halo[1];
+      w.map_b = L.map_b[2]; w.map_b64 = L.map_b[0];
+      w.slabs[0] = L.cin0 / 64; w.slabs[1] = L.cin1 / 64; w.cols = L.cout; w.hidden = ctx->Ch;
+      w.tiles_x = q.tiles_x; w.tiles_y = q.tiles_y; w.tiles = K * q.tiles_x * q.tiles_y;
+      w.Hm = ctx->Hm; w.Wm = ctx->Wm; w.h_in = h_in; w.c_idx = c_idx; w.h_out = h_out;
+      w.bias = L.b; w.c_state = ctx->c_state; w.h_f32 = ctx->use_post_tc ? nullptr : ctx->h_f32; w.h_bf16 = ctx->h_bf16;
+      w.status = ctx->status_dev; w.wait_limit = ctx->wait_limit; w.pdl = q.pdl;
+      TT_CUDA(ctx, launch_conv_lstm(w, ctx->sm_count, s));
+    } else {
+      q.n_src = 2; q.slabs[0] = L.cin0 / L.slab_c; q.slabs[1] = L.cin1 / L.slab_c; q.img0 = ident; q.img1 = h_in;
+      // with the heads on the tensor cores nothing on the path reads an fp32 copy of h': its consumers (the next
+      // step's convolution and the heads) take the bf16 copy, so only that copy is written
+      q.epilogue = TC_EPI_LSTM; q.c_state = ctx->c_state; q.h_f32 = ctx->use_post_tc ? nullptr : ctx->h_f32; q.h_bf16 = ctx->h_bf16;
+      q.c_idx = c_idx; q.h_out_idx = h_out; q.hidden = ctx->Ch;
+      TT_CUDA(ctx, launch_conv_tc(q, ctx->sm_count, s));
+    }
     if ((ms_ = mark_stage(ctx, TT_STAGE_CONVLSTM, 1)) != TT_OK) return ms_;
     }
   }

@@ -188,6 +188,28 @@ bool conv_s2_pays(int slab_c, int units, int sm_count);   // units: pixel tiles 
 void conv_s2_box(int view, int* w, int* h);
 cudaError_t launch_conv_s2(const ConvS2Params& p, int sm_count, cudaStream_t s);
 
+// ConvLSTM step on 64-channel slabs (x and h both multiples of 64 channels).
+struct ConvLstmParams {
+  TensorMap128 maps[2];     // x [K][Hm][Wm][Cx] and h [slots*2][Hm][Wm][Ch], box [64][10][18][1] (haloed patch of an 8 x 16 tile)
+  TensorMap128 map_b;       // packed weights [4*hidden][9*(Cx+Ch)] bf16, K-major, box [64][256]
+  TensorMap128 map_b64;     // the same, box [64][64]
+  int32_t slabs[2];         // 64-channel slabs of x and h
+  int32_t cols, hidden;     // 4 * hidden columns, a multiple of 64, at least 256
+  int32_t tiles, tiles_x, tiles_y, Hm, Wm;   // tiles = images x tiles_x x tiles_y
+  IdxMap h_in, c_idx, h_out;                 // image of h, slot of c, image of h' per batch position
+  int32_t width, groups, even, u_full;       // set by the launch: column groups, whether all are as wide, the unit from which they are cut in two
+  int32_t pdl;
+  const float* bias;        // packed order
+  float* c_state;           // [slots][Hm][Wm][Ch] in place
+  float* h_f32;             // [slots][Hm][Wm][Ch], or null: h' is written as its bf16 copy only
+  __nv_bfloat16* h_bf16;    // [slots*2][Hm][Wm][Ch]
+  int32_t* status;
+  long long wait_limit;
+};
+// whether grouping the columns otherwise than by 256 saves time on this many multiprocessors
+bool conv_lstm_pays(int tiles, int cols, int sm_count);
+cudaError_t launch_conv_lstm(const ConvLstmParams& p, int sm_count, cudaStream_t s);
+
 // Failure-path probe: one warp waits, through the same bounded wait as the tensor-core kernels, on
 // a barrier that nothing ever completes; when `limit_cycles` have passed it records `code` in
 // *status and returns normally.

@@ -5,6 +5,7 @@ import torch
 
 import oracle
 import tt_synth
+from paper_2402_04466_b200 import binding
 from test_gpu_pipeline import _compare_frame, _frames, _make, _run_bf16
 
 pytestmark = pytest.mark.gpu
@@ -106,3 +107,31 @@ def test_stride2_layer_kernels_give_the_same_bits_at_small_and_large_batches(cud
         for a, b in zip(batch[k], observe(ctx, st, r)):
             assert np.array_equal(a, b)
         ctx.destroy()
+
+
+@pytest.mark.parametrize("hidden,net", [
+    (64, (176, 136)),      # one group of 256 columns per tile: halves, or groups of 192 and 64
+    (128, (640, 480)),     # two groups: several rounds, the last cut into halves
+    (128, (400, 300)),     # a ragged map of few tiles: groups of 128
+    (256, (1280, 720)),    # four groups: 192 and a remainder of 64
+])
+def test_convlstm_column_groups_change_no_bit(cuda_device, hidden, net):
+    """How many multiprocessors there are decides how the gates' columns are grouped into units (or that the kernel of full rounds
+    runs): every grouping adds up the same products in the same order, so probabilities, confidences and state are the same bits."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="groups", src_w=net[0] + 30, src_h=net[1] + 20, net_w=net[0], net_h=net[1], hidden=hidden)
+    host = _frames(wl, 1, 2)[0]
+    w = tt_synth.make_weights(wl)
+    runs = []
+    for reserved in (0, 20, 48, 70):
+        ctx = binding.Context(binding.make_config(wl, reserved_sms=reserved), w)
+        st = ctx.state_create()
+        out = []
+        for t in range(2):
+            ctx.submit_frames([torch.from_numpy(host[t]).to(cuda_device)], [st], frame_index=t)
+            (r,) = ctx.sync()
+            out += [ctx.fetch_probs(r), r["conf"]]
+        runs.append(out + list(ctx.state_export(st)))
+        ctx.destroy()
+    for other in runs[1:]:
+        for a, b in zip(runs[0], other):
+            assert np.array_equal(a, b)
