@@ -16,9 +16,6 @@
 // (32 TFLOP/s, 43 % of the fp32 pipe: 16 warps per multiprocessor, two barriers per chunk and the last row and column
 // tiles' idle lanes).  The same tile as packed pairs of pixels (fma.rn.f32x2) took 94 us: more register moves to form
 // the pairs than FMAs saved.
-#include <algorithm>
-#include <climits>
-
 #include "tt_internal.h"
 
 namespace tt {
@@ -286,37 +283,41 @@ cudaError_t launch_one(const ConvSimtParams& p, cudaStream_t s) {
   return launch_kernel(kern, dim3(tiles, p.cout_packed / (WO * OC), p.K), Cfg::THREADS, Cfg::SMEM_BYTES, s, p, p.pdl != 0);
 }
 
-// Estimated cycles on the busiest multiprocessor.  The warps of the blocks it gets share four schedulers (one warp alone
-// cannot use more than one of them); per chunk of input channels a warp takes its share of the channels (about 300
-// issue cycles each: 144 packed FMAs at two cycles, loads beside them) and its part of the staging (about 4 per
-// 4-byte copy, 6 per 16-byte copy), and every chunk costs a round trip to L2 once, whatever shares the multiprocessor.
-template <int STRIDE, int WY, int WO, int KS>
-long simt_cost(const ConvSimtParams& p) {
-  using Cfg = SimtCfg<STRIDE, WY, WO, KS>;
-  if (p.cout_packed % (WO * OC)) return LONG_MAX;
-  const int cin = p.C0 + p.C1;
-  const long blocks = (long)((p.Wo + TW - 1) / TW) * ((p.Ho + Cfg::TH - 1) / Cfg::TH) * (p.cout_packed / (WO * OC)) * p.K;
-  const long rounds = ((blocks + p.sm_count - 1) / p.sm_count * Cfg::WARPS + 3) / 4;
-  const long chunks = (cin + Cfg::CB - 1) / Cfg::CB, share = (std::min(cin, Cfg::CB) + KS - 1) / KS;
-  const long staging = 4 * Cfg::N_POS * Cfg::CB + 6 * Cfg::W_VECS / Cfg::THREADS;
-  return chunks * (rounds * (share * 300 + staging) + 500) + (KS > 1 ? 300 : 0);
+// How many warps share out the input channels of a tile.  Their partial sums are added up in an order that depends on this number, so
+// it follows from the layer's shape for ONE stream: a stream's results must not change with the streams that share its tick, nor with
+// the multiprocessors left to another workload.  `warps` is what one stream's unsplit launch would have.  Below one per
+// multiprocessor four warps share a tile's channels, up to 400 two do (the line lies between the measured 256 and 540).  K = 1, 3, 8 streams, us
+// with 1 / 2 / 4 warps to a tile:
+//   40x30 x 128 channels from 64, stride 2 (64 warps)    25.9 25.9 26.3 / 17.4 17.4 25.8 / 12.9 18.0 28.7
+//   64x64 x 64 from 32 (256)                             14.1 20.0 34.2 / 10.4 17.4 36.1 /  9.9 23.4 43.7
+//   80x60 x 96 from 48 (540)                             19.9 39.5 95.8 / 18.7 45.1 103 / 19.7 52.6 124
+//   80x60 x 128 from 64 (720)                            36.5 64.0 157  / 30.9 73.5 177 / 30.2 82.8 208
+// Three input channels (a first layer) have little to share: two warps below the first line, else one; bf16 outputs are always one
+// warp's sums.
+int simt_split(const ConvSimtParams& p) {
+  const long warps = (long)((p.Wo + TW - 1) / TW) * ((p.Ho + 3) / 4) * (p.cout_packed / OC);
+  if (p.epilogue == EPI_RELU_BF16_NHWC) return 1;
+  if (p.C0 + p.C1 < 8) return warps < 148 ? 2 : 1;
+  return warps < 148 ? 4 : warps < 400 ? 2 : 1;
 }
 
-// The block shape with the smallest estimate; among equals the one listed first (more reuse of the staged tile).  Splitting
-// the input channels only wins where the map is too small to give every scheduler a warp: 64x64 pixels x 64 channels from 32
-// input channels 25 us with 32 blocks of 8 warps, 15 us with 128 of 4; three maps of 80x60 x 128 channels from 64 70 us with
-// 288 of 8, 88 us with 2160 of 4, each on a quarter of the channels.
+// The block shape, which changes no bit: as many channel groups on one staged input tile as divide the layer's, and twice the
+// output rows where the busiest multiprocessor gets no more to do by it (half the weight copies and less halo: 80x60 x 128 channels
+// from 64, three maps 64.0 against 65.6 us; at two maps the coarser blocks would take 64.1 against 51.1).
+template <int STRIDE, int EPI, int WY, int WO>
+cudaError_t launch_rows(const ConvSimtParams& p, cudaStream_t s) {
+  const long cols = (long)((p.Wo + TW - 1) / TW) * (p.cout_packed / (WO * OC)) * p.K;
+  const long fine = cols * ((p.Ho + 4 * WY - 1) / (4 * WY)), coarse = cols * ((p.Ho + 8 * WY - 1) / (8 * WY));
+  if (2 * ((coarse + p.sm_count - 1) / p.sm_count) <= (fine + p.sm_count - 1) / p.sm_count) return launch_one<STRIDE, EPI, 2 * WY, WO, 1>(p, s);
+  return launch_one<STRIDE, EPI, WY, WO, 1>(p, s);
+}
 template <int STRIDE, int EPI>
 cudaError_t launch_epi(const ConvSimtParams& p, cudaStream_t s) {
-  const long cost[5] = {simt_cost<STRIDE, 2, 4, 1>(p), simt_cost<STRIDE, 4, 2, 1>(p), simt_cost<STRIDE, 4, 1, 1>(p),
-                        simt_cost<STRIDE, 1, 2, 2>(p), simt_cost<STRIDE, 1, 1, 4>(p)};
-  switch (std::min_element(cost, cost + 5) - cost) {
-    case 0: return launch_one<STRIDE, EPI, 2, 4, 1>(p, s);
-    case 1: return launch_one<STRIDE, EPI, 4, 2, 1>(p, s);
-    case 2: return launch_one<STRIDE, EPI, 4, 1, 1>(p, s);
-    case 3: return launch_one<STRIDE, EPI, 1, 2, 2>(p, s);
-    default: return launch_one<STRIDE, EPI, 1, 1, 4>(p, s);
-  }
+  const int groups = p.cout_packed / OC, split = simt_split(p);
+  if (split == 4) return launch_one<STRIDE, EPI, 1, 1, 4>(p, s);
+  if (split == 2) return groups % 2 == 0 ? launch_one<STRIDE, EPI, 1, 2, 2>(p, s) : launch_one<STRIDE, EPI, 2, 1, 2>(p, s);
+  if (groups % 4 == 0) return launch_rows<STRIDE, EPI, 1, 4>(p, s);
+  return groups % 2 == 0 ? launch_rows<STRIDE, EPI, 2, 2>(p, s) : launch_one<STRIDE, EPI, 4, 1, 1>(p, s);
 }
 
 }  // namespace

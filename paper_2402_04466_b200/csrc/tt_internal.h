@@ -70,7 +70,7 @@ struct ConvSimtParams {
   const float* wgt;   // packed [Cin][9][CoutPacked]
   const float* bias;  // packed [CoutPacked]
   int32_t cout, cout_packed;   // cout_packed: a multiple of 8
-  int32_t sm_count;
+  int32_t sm_count;   // chooses between block shapes that give the same bits
   int32_t pdl;        // launch as a programmatic dependent of the previous kernel in the stream
   int32_t epilogue;
   // EPI_RELU_*: out; EPI_LSTM: c (in place), h_out

@@ -18,6 +18,9 @@ pytestmark = pytest.mark.gpu
     ((96, 64), (64,), (1,), 16, 3),          # large enough for the blocks of four channel groups
     ((200, 150), (32,), (1,), 32, 1),
     ((64, 64), (16,), (1,), 16, 1),          # small map, 32 input channels: shared out over the warps of a block
+    ((40, 38), (24,), (1,), 12, 2),          # an odd number of channel groups, channels shared out by four
+    ((130, 61), (8, 8), (1, 1), 20, 2),      # odd numbers of groups: shared out by two, and by nobody
+    ((320, 240), (16, 32), (2, 2), 32, 3),   # eight output rows per block instead of four, the last rows of a tile empty
 ])
 def test_fp32_convolutions_at_the_edges_of_their_tiles(cuda_device, net, enc, stride, hidden, K):
     """Bound as for the other fp32 tests: fp32 sums of up to 9 * 72 products against the oracle's double sums, 1e-4."""
@@ -32,6 +35,34 @@ def test_fp32_convolutions_at_the_edges_of_their_tiles(cuda_device, net, enc, st
         for k in range(K):
             _compare_frame(ctx, states[k], res[k], oras[k].step(frames[k][t]), 1e-4, 1e-3, tag=f"edges k={k} t={t}")
     ctx.destroy()
+
+
+@pytest.mark.parametrize("shape", [
+    dict(net_w=64, net_h=64, enc_cout=(16,), enc_stride=(1,), hidden=16),                # few warps: channels shared out
+    dict(net_w=320, net_h=240, enc_cout=(16, 32), enc_stride=(2, 2), hidden=32),         # last layer shared out, cell not
+    dict(net_w=158, net_h=120, enc_cout=(32, 64), enc_stride=(2, 2), hidden=64, precision="bf16"),   # bf16 model whose first layer runs here
+])
+def test_fp32_convolutions_give_a_stream_the_same_bits_whatever_shares_its_tick(cuda_device, shape):
+    """How many warps add up a tile's channels decides the order of the sums: it must not follow from the number of streams in the tick
+    or of multiprocessors left over.  Stream 0 alone against stream 0 among 2, 3, 5 and 8, and beside a reservation."""
+    wl = tt_synth.workload("cfg0-gain").with_(name="neighbours", src_w=shape["net_w"] + 7, src_h=shape["net_h"] + 5, frame_kind="endoscopy", **shape)
+    w = tt_synth.make_weights(wl)
+    host = _frames(wl, 2, 2)
+    frames = [[torch.from_numpy(f).to(cuda_device) for f in fs] for fs in host]
+    runs = []
+    for K, reserved in ((1, 0), (2, 0), (3, 0), (5, 0), (8, 0), (1, 60)):
+        ctx = binding.Context(binding.make_config(wl, max_streams=K, reserved_sms=reserved), w)
+        states = [ctx.state_create() for _ in range(K)]
+        out = []
+        for t in range(2):
+            ctx.submit_frames([frames[min(k, 1)][t] for k in range(K)], states, frame_index=t)
+            r = ctx.sync()[0]
+            out += [ctx.fetch_probs(r), r["conf"]] + [ctx.debug_tensor(states[0], f"enc{l}") for l in range(len(wl.enc_cout))]
+        runs.append(out + list(ctx.state_export(states[0])))
+        ctx.destroy()
+    for other in runs[1:]:
+        for a, b in zip(runs[0], other):
+            assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("shape", [
