@@ -70,7 +70,6 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
   uint64_t* p_full = t_empty + 2;           // [2] patch landed
   volatile int* abort_flag = &s_abort;
 
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wait_limit = p.wait_limit;
   if (threadIdx.x == 0) {
@@ -101,6 +100,7 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = s_tmem;
+  pdl_launch_dependents();   // behind the allocation: a dependent block must not take tensor memory that this grid still needs
   pdl_wait();   // the set-up above read weights only; the input tensor is the previous kernel's output
 
   const int tiles_per_img = p.tiles_x * p.tiles_y;

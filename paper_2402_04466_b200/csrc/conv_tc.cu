@@ -126,7 +126,6 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
   int4* s_tab = reinterpret_cast<int4*>(bar_mem + Cfg::BAR_BYTES);            // [k_iters] {map slot, channel offset, dx, dy}
   int* s_img = reinterpret_cast<int*>(s_tab + MAX_K_ITERS);                   // [4][TT_MAX_STREAMS]: img0, img1, c_idx, h_out_idx
 
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wait_limit = p.wait_limit;
   const int tiles_per_img = p.tiles_x * p.tiles_y;
@@ -212,6 +211,7 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
   if (PAIR) cluster_sync_all();   // the peer's barriers exist before anything is signalled across the pair
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_launch_dependents();   // behind the allocation: a dependent block must not take tensor memory that this grid still needs
   pdl_wait();   // everything above touched no activation; from here on the previous kernel's outputs are read
 
   const int n_prod = p.n_prod;

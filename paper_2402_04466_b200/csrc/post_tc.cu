@@ -81,7 +81,6 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   int* s_last = const_cast<int*>(abort_flag) + 1;
 
-  pdl_launch_dependents();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long wait_limit = p.wait_limit;
   const int plane = p.Hm * p.Wm;
@@ -117,6 +116,7 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  pdl_launch_dependents();   // behind the allocation: a dependent block must not take tensor memory that this grid still needs
 
   int status_before = 0;   // thread 64: the status word as the kernels before this one left it
   if (warp == 0 && lane == 0) {

@@ -1,0 +1,34 @@
+"""Rules of the device code that no run on a healthy device can show broken (no GPU needed)."""
+import glob
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2402_04466_b200", "csrc")
+
+
+def _code(path):
+    """Source without comments."""
+    return re.sub(r"/\*.*?\*/|//[^\n]*", "", open(path).read(), flags=re.S)
+
+
+SOURCES = {os.path.basename(f): _code(f) for f in sorted(glob.glob(os.path.join(CSRC, "*.cu")) + glob.glob(os.path.join(CSRC, "*.cuh")))}
+ALLOCATING = [n for n, c in SOURCES.items() if "tcgen05.alloc" in c]
+
+
+@pytest.mark.parametrize("name", ALLOCATING)
+def test_dependents_are_released_behind_the_tensor_memory_allocation(name):
+    """An allocation of tensor memory waits without a limit.  Once every block of a grid has released its dependents these may become
+    resident beside it, so a block that released first could find its columns taken by a block that waits for it in turn: every block
+    allocates, meets the others of its block at a barrier, and only then releases."""
+    code = SOURCES[name]
+    last_alloc, release = code.rindex("tcgen05.alloc"), code.index("pdl_launch_dependents()")
+    assert code.count("pdl_launch_dependents()") == 1
+    assert last_alloc < release and "__syncthreads()" in code[last_alloc:release]
+
+
+def test_the_rule_above_looks_at_every_allocating_kernel():
+    assert set(ALLOCATING) == {"conv_tc.cu", "conv_first_tc.cu", "conv_first_fused.cu", "conv_s2_tc.cu", "conv_lstm_tc.cu", "post_tc.cu"}
+    launched = [n for n in ALLOCATING if re.search(r"tcgen05\.alloc", SOURCES[n]) and SOURCES[n].count("__global__") == 1]
+    assert launched == ALLOCATING          # one kernel per file: an order in the file is an order in the kernel
