@@ -53,13 +53,13 @@ __device__ __forceinline__ void blend(uint32_t& rb, uint32_t& g, uint32_t k_rb, 
 }
 
 // Tools ascend from 0.  The loop runs over the tools that any lane of the warp needs, so that the colours are uniform
-// loads and lanes with other tools do not serialise.
+// loads and lanes with other tools do not serialise.  The whole warp takes part.
 template <int N>
 __device__ __forceinline__ void blend_all(uint32_t (&rb)[N], uint32_t (&g)[N], const uint32_t (&bits)[N], const OverlayArgs& a) {
   uint32_t some = 0;
 #pragma unroll
   for (int j = 0; j < N; ++j) some |= bits[j];
-  some = __reduce_or_sync(__activemask(), some);
+  some = __reduce_or_sync(0xffffffffu, some);
   while (some) {
     const int t = __ffs(some) - 1;
     some &= some - 1;
@@ -86,7 +86,6 @@ __global__ void __launch_bounds__(256) overlay_kernel(const __grid_constant__ Ov
   const uint32_t npx = (uint32_t)p.src_w * (uint32_t)p.src_h;           // at most 2^28
   uint8_t* dst = p.dst + (size_t)n * npx * 4;
   const uint32_t i0 = (blockIdx.x * blockDim.x + threadIdx.x) * 4;      // first of 4 pixels
-  if (i0 >= npx) return;
   int y = (int)div_by(i0, a.by_w), x = (int)i0 - y * p.src_w;
   // mask sample of (x, y) and the remainder of x * Wm / src_w, which the next pixel's sample follows from
   int mx = (int)div_by((uint32_t)(x * p.Wm), a.by_w), rem = x * p.Wm - mx * p.src_w;
@@ -100,13 +99,15 @@ __global__ void __launch_bounds__(256) overlay_kernel(const __grid_constant__ Ov
       my = (int)div_by((uint32_t)(y * p.Hm), a.by_h);
     }
   };
-  if (FLAT && i0 + 3 < npx) {
+  uint32_t bits[4] = {};
+  // the same for all lanes of a warp (its 128 pixels all exist): both branches vote with the whole warp
+  if (FLAT && (i0 & ~127u) + 128 <= npx) {
     const uint32_t* s32 = reinterpret_cast<const uint32_t*>(src) + (i0 >> 2) * 3;
     const uint32_t w0 = __ldg(s32), w1 = __ldg(s32 + 1), w2 = __ldg(s32 + 2);
     // bytes R0 G0 B0 R1 | G1 B1 R2 G2 | B2 R3 G3 B3
     uint32_t rb[4] = {w0 & 0x00FF00FFu, (w0 >> 24) | ((w1 & 0xFF00u) << 8), ((w1 >> 16) & 0xFFu) | ((w2 & 0xFFu) << 16), ((w2 >> 8) & 0xFFu) | ((w2 >> 24) << 16)};
     uint32_t g[4] = {(w0 >> 8) & 0xFFu, w1 & 0xFFu, w1 >> 24, (w2 >> 16) & 0xFFu};
-    uint32_t bits[4], out[4];
+    uint32_t out[4];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
       bits[j] = mask_bits<PACKED>(p, n, mx, my);
@@ -117,14 +118,24 @@ __global__ void __launch_bounds__(256) overlay_kernel(const __grid_constant__ Ov
     for (int j = 0; j < 4; ++j) out[j] = rgba(rb[j], g[j]);
     *reinterpret_cast<uint4*>(dst + (size_t)i0 * 4) = make_uint4(out[0], out[1], out[2], out[3]);
   } else {
-    for (uint32_t j = 0; j < 4 && i0 + j < npx; ++j) {
-      const uint8_t* s = src + (size_t)y * p.src_pitch + 3 * x;
-      uint32_t rb[1] = {(uint32_t)s[0] | ((uint32_t)s[2] << 16)}, g[1] = {s[1]};
-      const uint32_t bits[1] = {mask_bits<PACKED>(p, n, mx, my)};
-      blend_all<1>(rb, g, bits, a);
-      *reinterpret_cast<uint32_t*>(dst + (size_t)(i0 + j) * 4) = rgba(rb[0], g[0]);
-      if (i0 + j + 1 < npx) next();
+    // lanes behind the last pixel stay for the vote: they have no bits set, load and store nothing
+    const int live = i0 < npx ? (int)min(npx - i0, 4u) : 0;
+    uint32_t rb[4] = {}, g[4] = {};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      if (j < live) {
+        bits[j] = mask_bits<PACKED>(p, n, mx, my);
+        const uint8_t* s = src + (size_t)y * p.src_pitch + 3 * x;
+        rb[j] = (uint32_t)s[0] | ((uint32_t)s[2] << 16);
+        g[j] = s[1];
+      }
+      if (j < 3) next();
     }
+    blend_all<4>(rb, g, bits, a);
+    uint32_t* out = reinterpret_cast<uint32_t*>(dst + (size_t)i0 * 4);
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < live) out[j] = rgba(rb[j], g[j]);
   }
 }
 

@@ -110,7 +110,11 @@ def test_postprocess_threshold_and_empty_masks(cuda_device):
 
 
 @pytest.mark.parametrize("src_wh,grid,pad,K,T", [((854, 480), (60, 80), 0, 2, 7), ((50, 31), (7, 9), 3, 3, 4),
-                                                 ((128, 128), (64, 64), 0, 1, 4)])
+                                                 ((128, 128), (64, 64), 0, 1, 4),
+                                                 ((37, 23), (61, 95), 0, 1, 8),     # a mask grid larger than the frame; 851 pixels, the last word of 3
+                                                 ((3, 7), (9, 20), 0, 1, 2),        # 21 pixels, rows shorter than a thread's four
+                                                 ((1, 5), (4, 3), 2, 2, 3),         # one column, padded
+                                                 ((64, 33), (64, 64), 5, 3, 8)])    # as many samples as columns, padded rows
 def test_overlay_is_bit_exact(cuda_device, src_wh, grid, pad, K, T):
     (sw, sh), (hm, wm) = src_wh, grid
     frames = RNG.integers(0, 256, (K, sh, sw, 3), dtype=np.uint8)

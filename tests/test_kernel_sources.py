@@ -32,3 +32,8 @@ def test_the_rule_above_looks_at_every_allocating_kernel():
     assert set(ALLOCATING) == {"conv_tc.cu", "conv_first_tc.cu", "conv_first_fused.cu", "conv_s2_tc.cu", "conv_lstm_tc.cu", "post_tc.cu"}
     launched = [n for n in ALLOCATING if re.search(r"tcgen05\.alloc", SOURCES[n]) and SOURCES[n].count("__global__") == 1]
     assert launched == ALLOCATING          # one kernel per file: an order in the file is an order in the kernel
+
+
+def test_no_warp_vote_takes_whatever_lanes_happen_to_be_active():
+    """Nothing guarantees that the lanes __activemask() sees are those that reach the vote behind it together."""
+    assert [n for n, c in SOURCES.items() if "__activemask" in c] == []
