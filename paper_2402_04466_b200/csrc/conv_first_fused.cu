@@ -314,14 +314,14 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
   bool ok = true;
   for (int i = 0; i < n; ++i) {
     // this tile's rows have landed (the barrier at the end of the loop body: the patch has been gathered from)
-    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_landed[i & 1]), (uint32_t)(i >> 1) & 1u, abort_flag, p.status, 0x910 + (i & 1), p.wait_limit));
+    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_landed[i & 1]), (uint32_t)(i >> 1) & 1u, abort_flag, p.status, WAIT_CONV_FIRST_FUSED + (i & 1), p.wait_limit));
     if (p.one_row) sample(cur, i & 1, std::true_type{});
     else sample(cur, i & 1, std::false_type{});
     __syncthreads();                                  // the patch is complete, the frame rows have been read
     if (i + 2 < n) { stage(ahead, i & 1); advance(ahead); }
     if (i > 0) {
       // the MMAs of the tile before are done: its accumulator can be read and the operand overwritten
-      ok &= __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_bar), (uint32_t)(i - 1) & 1u, abort_flag, p.status, 0x900, p.wait_limit));
+      ok &= __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_bar), (uint32_t)(i - 1) & 1u, abort_flag, p.status, WAIT_CONV_FIRST_FUSED + 0x10, p.wait_limit));
       epilogue(last);
     }
     gather();
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     advance(cur);
   }
   if (ok && n > 0) {
-    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_bar), (uint32_t)(n - 1) & 1u, abort_flag, p.status, 0x901, p.wait_limit));
+    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_bar), (uint32_t)(n - 1) & 1u, abort_flag, p.status, WAIT_CONV_FIRST_FUSED + 0x11, p.wait_limit));
     if (ok) epilogue(last);
   }
   __syncwarp();

@@ -131,7 +131,7 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
       if (blockIdx.x + gridDim.x < total_tiles) fetch_patch(blockIdx.x + gridDim.x, 1);
     }
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-      if (!fail && !mbar_wait(smem_u32(p_full + buf), pphase, abort_flag, p.status, 0x900 + buf, wait_limit)) fail = true;
+      if (!fail && !mbar_wait(smem_u32(p_full + buf), pphase, abort_flag, p.status, WAIT_CONV_FIRST + buf, wait_limit)) fail = true;
       const float* patch = reinterpret_cast<const float*>(s_patch + buf * PATCH_STRIDE);
       float v[27];
 #pragma unroll
@@ -149,7 +149,7 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
       }
       if (buf) pphase ^= 1u;
       buf ^= 1;
-      if (!mbar_wait(smem_u32(a_empty + stage), phase ^ 1u, abort_flag, p.status, 0x500 + (int)stage, wait_limit)) {
+      if (!mbar_wait(smem_u32(a_empty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_FIRST + 0x10 + (int)stage, wait_limit)) {
         fail = true;
         continue;
       }
@@ -174,8 +174,8 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
       uint32_t stage = 0, phase = 0, acc_phase = 0;
       int acc = 0;
       for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
-        if (!mbar_wait(smem_u32(t_empty + acc), acc_phase ^ 1u, abort_flag, p.status, 0x600 + acc, wait_limit)) break;
-        if (!mbar_wait(smem_u32(a_full + stage), phase, abort_flag, p.status, 0x700 + (int)stage, wait_limit)) break;
+        if (!mbar_wait(smem_u32(t_empty + acc), acc_phase ^ 1u, abort_flag, p.status, WAIT_CONV_FIRST + 0x20 + acc, wait_limit)) break;
+        if (!mbar_wait(smem_u32(a_full + stage), phase, abort_flag, p.status, WAIT_CONV_FIRST + 0x30 + (int)stage, wait_limit)) break;
         tc_fence_after();
         const uint32_t a_addr = smem_u32(s_a + stage * F_A_BYTES), b_addr = smem_u32(s_b);
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 64);
@@ -204,7 +204,7 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
     int acc = 0;
     for (int tile = blockIdx.x; tile < total_tiles; tile += gridDim.x) {
       const TileAt t = tile_at(tile, p.tiles_x, tiles_per_img, inv_tiles_x, inv_tiles_per_img);
-      const bool fail = !mbar_wait(smem_u32(t_full + acc), acc_phase, abort_flag, p.status, 0x800 + acc, wait_limit);
+      const bool fail = !mbar_wait(smem_u32(t_full + acc), acc_phase, abort_flag, p.status, WAIT_CONV_FIRST + 0x40 + acc, wait_limit);
       // the previous tile's store must have finished reading s_out before it is overwritten
       if (leader) bulk_wait_group_read0();
       if (named_barrier_or(2, 128, fail)) break;   // all four warps stop together if any wait ran out

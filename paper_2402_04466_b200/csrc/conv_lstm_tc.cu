@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       const int img = m / tiles_per_img, rem = m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
       const int img_h = s_img[0][img];
       for (int sg = 0; sg < slabs; ++sg) {
-        ok = mbar_wait(smem_u32(aempty + stage), phase ^ 1u, abort_flag, p.status, 0x900 + (int)stage, wait_limit);
+        ok = mbar_wait(smem_u32(aempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x10 + (int)stage, wait_limit);
         if (!ok) break;
         const int src = sg < p.slabs[0] ? 0 : 1;
         mbar_arrive_expect_tx(smem_u32(afull + stage), L_A_TX);
@@ -152,7 +152,7 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       const Unit t = unit_at(p, u);
       for (; it < iters; it += 2) {
         const int sg = it / 9, tap = it - sg * 9;
-        ok = mbar_wait(smem_u32(bempty + stage), phase ^ 1u, abort_flag, p.status, 0x100 + (int)stage, wait_limit);
+        ok = mbar_wait(smem_u32(bempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + (int)stage, wait_limit);
         if (!ok) break;
         const uint32_t bar = smem_u32(bfull + stage), dst = smem_u32(s_b + stage * L_B_BYTES);
         const int k0 = tap * cin + sg * 64;
@@ -178,15 +178,15 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       // (no division in this loop where all groups are as wide)
       const int n = p.even ? (u < p.u_full ? p.width : p.width >> 1) : unit_at(p, u).n;
       const uint32_t idesc = make_idesc(128, 0) | ((uint32_t)(n >> 3) << 17);
-      ok &= mbar_wait_uniform(smem_u32(tempty + acc), acc_phase ^ 1u, abort_flag, p.status, 0x200 + acc, wait_limit);
+      ok &= mbar_wait_uniform(smem_u32(tempty + acc), acc_phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x30 + acc, wait_limit);
       tc_fence_after();   // the epilogue's reads of this accumulator come before the MMAs that overwrite it
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
       for (int sg = 0; sg < slabs; ++sg) {
-        ok &= mbar_wait_uniform(smem_u32(afull + a_stage), a_phase, abort_flag, p.status, 0xA00 + (int)a_stage, wait_limit);
+        ok &= mbar_wait_uniform(smem_u32(afull + a_stage), a_phase, abort_flag, p.status, WAIT_CONV_LSTM + 0x40 + (int)a_stage, wait_limit);
         const uint64_t a_patch = make_smem_desc(smem_u32(s_a + a_stage * L_A_BYTES), L_PITCH * 128u, 2u);
 #pragma unroll
         for (int tap = 0; tap < 9; ++tap) {
-          ok &= mbar_wait_uniform(smem_u32(bfull + stage), phase, abort_flag, p.status, 0x300 + (int)stage, wait_limit);
+          ok &= mbar_wait_uniform(smem_u32(bfull + stage), phase, abort_flag, p.status, WAIT_CONV_LSTM + 0x50 + (int)stage, wait_limit);
           const uint64_t a = a_patch + (uint64_t)(((tap / 3) * L_PITCH + tap % 3) * 128 >> 4);
           const uint64_t b = b_desc0 + (uint64_t)stage * (uint64_t)(L_B_BYTES >> 4);
           if (issuer) {
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
         if (valid && ck < chunks) ld_global_v8(p.c_state + so + ck * 8, c_old[ck]);
 
       // the warp votes: its lanes leave the loop together or go on to the warp-collective TMEM loads together
-      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(tfull + acc), acc_phase, abort_flag, p.status, 0x400 + acc, wait_limit))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(tfull + acc), acc_phase, abort_flag, p.status, WAIT_CONV_LSTM + 0x60 + acc, wait_limit))) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * 256 + off);
       uint32_t hb[8];

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(S2_THREADS, SLAB_C == 32 ? 2 : 1) conv_s2_kern
       for (int v = 3; v >= 0; --v) {   // in the order of their first taps
         const uint32_t buf = Cfg::bufs(v) == 2 ? seq & 1u : 0u, phase = Cfg::bufs(v) == 2 ? (seq >> 1) & 1u : seq & 1u;
         const uint32_t bar = smem_u32(vfull + 2 * v + buf);
-        ok = ok && mbar_wait(smem_u32(vempty + 2 * v + buf), phase ^ 1u, abort_flag, p.status, 0xC00 + v, wait_limit);
+        ok = ok && mbar_wait(smem_u32(vempty + 2 * v + buf), phase ^ 1u, abort_flag, p.status, WAIT_CONV_S2 + v, wait_limit);
         if (!ok) break;
         mbar_arrive_expect_tx(bar, Cfg::tx(v));
         tma_load_4d(smem_u32(smem + Cfg::v_off(v) + buf * Cfg::v_bytes(v)), &p.map_v[v], bar, 0, tx * S2_PW - (v & 1), ty * S2_PH - (v >> 1), img);
@@ -137,16 +137,16 @@ __global__ void __launch_bounds__(S2_THREADS, SLAB_C == 32 ? 2 : 1) conv_s2_kern
     int acc = 0;
     bool ok = true;
     const uint64_t b_desc0 = make_smem_desc(smem_u32(s_b), 8u * Cfg::ROW, LAYOUT);
-    ok &= mbar_wait_uniform(smem_u32(wfull), 0u, abort_flag, p.status, 0xC20, wait_limit);
+    ok &= mbar_wait_uniform(smem_u32(wfull), 0u, abort_flag, p.status, WAIT_CONV_S2 + 0x20, wait_limit);
     for (int m = worker; m < m_tiles; m += n_workers) {
-      ok &= mbar_wait_uniform(smem_u32(tempty + acc), acc_phase ^ 1u, abort_flag, p.status, 0xC30 + acc, wait_limit);
+      ok &= mbar_wait_uniform(smem_u32(tempty + acc), acc_phase ^ 1u, abort_flag, p.status, WAIT_CONV_S2 + 0x30 + acc, wait_limit);
       tc_fence_after();   // the epilogue's reads of this accumulator come before the MMAs that overwrite it
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * N);
 #pragma unroll
       for (int i = 0; i < 9; ++i) {
         const int v = s2_view(i), ky = i / 3, kx = i % 3;
         const uint32_t buf = Cfg::bufs(v) == 2 ? seq & 1u : 0u, phase = Cfg::bufs(v) == 2 ? (seq >> 1) & 1u : seq & 1u;
-        if (i == s2_first(v)) ok &= mbar_wait_uniform(smem_u32(vfull + 2 * v + buf), phase, abort_flag, p.status, 0xC40 + v, wait_limit);
+        if (i == s2_first(v)) ok &= mbar_wait_uniform(smem_u32(vfull + 2 * v + buf), phase, abort_flag, p.status, WAIT_CONV_S2 + 0x40 + v, wait_limit);
         const uint64_t a = make_smem_desc(smem_u32(smem + Cfg::v_off(v)), (uint32_t)(s2_view_w(v) * Cfg::ROW), LAYOUT) +
                            (uint64_t)(((ky == 2 ? s2_view_w(v) : 0) + (kx == 2 ? 1 : 0)) * Cfg::ROW >> 4) + (uint64_t)(buf * (Cfg::v_bytes(v) >> 4));
         const uint64_t b = b_desc0 + (uint64_t)(i * Cfg::B_BYTES >> 4);
@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(S2_THREADS, SLAB_C == 32 ? 2 : 1) conv_s2_kern
       // this lane writes piece lane % 4 of the pixels lane / 4 + 8 q of the warp's 32 (4 rows of 8)
       const int x = tx * S2_PW + (lane >> 2), y0 = ty * S2_PH + quarter * 4;
       __nv_bfloat16* out = p.out + (((size_t)img * p.Ho + y0) * p.Wo + x) * p.cout + nt * N + (lane & 3) * 8;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(tfull + acc), acc_phase, abort_flag, p.status, 0xC60 + acc, wait_limit));
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(tfull + acc), acc_phase, abort_flag, p.status, WAIT_CONV_S2 + 0x60 + acc, wait_limit));
       if (!ok) break;
       tc_fence_after();
       const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * N);

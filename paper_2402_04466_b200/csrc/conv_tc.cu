@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
           if (tap == 0) {
             const int seq = slab_seq0 + sg;
             const uint32_t a_stage = (uint32_t)seq & 1u, a_phase = ((uint32_t)seq >> 1) & 1u;
-            ok = mbar_wait(smem_u32(aempty_bar + a_stage), a_phase ^ 1u, abort_flag, p.status, 0x900 + (int)a_stage, wait_limit);
+            ok = mbar_wait(smem_u32(aempty_bar + a_stage), a_phase ^ 1u, abort_flag, p.status, WAIT_CONV_TC + 0x10 + (int)a_stage, wait_limit);
             if (!ok) break;
             const int src = sg < p.slabs[0] ? 0 : 1;
             const uint32_t ab = smem_u32(afull_bar + a_stage);
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
             tma_load_4d(smem_u32(smem_a + a_stage * Cfg::HALO_A_BYTES), &p.maps_halo[src], ab, (src ? sg - p.slabs[0] : sg) * SLAB_C,
                         tx * PW - 1, ty * PH - 1, src ? img_h : img_x);
           }
-          ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, 0x100 + (int)stage, wait_limit);
+          ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_TC + (int)stage, wait_limit);
           if (!ok) break;
           const uint32_t fb = smem_u32(full_bar + stage);
           mbar_arrive_expect_tx(fb, Cfg::B_BYTES);
@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
       const int img_x = s_img[img], img_h = s_img[TT_MAX_STREAMS + img];
       for (; it < k_iters; it += n_prod) {
         const int4 e = s_tab[it];
-        ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, 0x100 + (int)stage, wait_limit);
+        ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_TC + (int)stage, wait_limit);
         if (!ok) break;
         uint8_t* st = smem + stage * RING_STRIDE;
         if (PAIR) {
@@ -305,11 +305,11 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
     const uint64_t a_desc0 = make_smem_desc(smem_u32(smem), SBO, LAYOUT);
     constexpr uint64_t STAGE_UNITS = RING_STRIDE >> 4, B_UNITS = Cfg::A_BYTES >> 4;
     const uint64_t w_desc0 = make_smem_desc(smem_u32(smem_a), SBO, LAYOUT);   // WRES: first resident weight slab
-    if (WRES) ok = mbar_wait(smem_u32(afull_bar), 0u, abort_flag, p.status, 0xB00, wait_limit);
+    if (WRES) ok = mbar_wait(smem_u32(afull_bar), 0u, abort_flag, p.status, WAIT_CONV_TC + 0x20, wait_limit);
     const uint32_t full0 = smem_u32(full_bar), empty0 = smem_u32(empty_bar);
     uint64_t a_desc = a_desc0;
     for (int tile = worker; tile < total_tiles && ok; tile += n_workers) {
-      ok = mbar_wait(smem_u32(tempty_bar + acc), acc_phase ^ 1u, abort_flag, p.status, 0x200 + acc, wait_limit);
+      ok = mbar_wait(smem_u32(tempty_bar + acc), acc_phase ^ 1u, abort_flag, p.status, WAIT_CONV_TC + 0x30 + acc, wait_limit);
       if (!ok) break;
       tc_fence_after();   // the epilogue's TMEM reads of this buffer come before the MMAs that overwrite it
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BLOCK_N);
@@ -322,12 +322,12 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
         // pattern needs nothing but its start address.
         uint32_t first = 1;
         for (int sg = 0; sg < slabs_per_tap && ok; ++sg) {
-          ok = mbar_wait(smem_u32(afull_bar + a_stage), a_phase, abort_flag, p.status, 0xA00 + (int)a_stage, wait_limit);
+          ok = mbar_wait(smem_u32(afull_bar + a_stage), a_phase, abort_flag, p.status, WAIT_CONV_TC + 0x40 + (int)a_stage, wait_limit);
           if (!ok) break;
           const uint32_t a_base = smem_u32(smem_a + a_stage * Cfg::HALO_A_BYTES);
 #pragma unroll 1
           for (int tap = 0; tap < 9; ++tap) {
-            ok = mbar_wait(full0 + 8u * stage, phase, abort_flag, p.status, 0x300 + (int)stage, wait_limit);
+            ok = mbar_wait(full0 + 8u * stage, phase, abort_flag, p.status, WAIT_CONV_TC + 0x50 + (int)stage, wait_limit);
             if (!ok) break;
             const int ky = tap / 3, kx = tap - ky * 3;
             const uint64_t a_tap = make_smem_desc(a_base + (uint32_t)((ky * Cfg::HALO_PITCH + kx) * 128), Cfg::HALO_PITCH * 128u, LAYOUT);
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
       }
       for (int it = 0; it < k_iters && !HALO; ++it) {
         // the copies complete on the barrier through the async proxy, which the MMAs read through too
-        ok = mbar_wait(full0 + 8u * stage, phase, abort_flag, p.status, 0x300 + (int)stage, wait_limit);
+        ok = mbar_wait(full0 + 8u * stage, phase, abort_flag, p.status, WAIT_CONV_TC + 0x50 + (int)stage, wait_limit);
         if (!ok) break;
         const uint64_t b_desc = WRES ? w_desc0 + (uint64_t)it * (uint64_t)(Cfg::B_BYTES >> 4) : a_desc + B_UNITS;
         // advance along K inside the swizzle atom: 16 bf16 = 32 bytes = 2 descriptor units
@@ -411,7 +411,7 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
       }
 
       // the warp votes: its lanes leave the tile loop together or go on to the warp-collective TMEM loads together
-      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(tfull_bar + acc), acc_phase, abort_flag, p.status, 0x400 + acc, wait_limit));
+      ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(tfull_bar + acc), acc_phase, abort_flag, p.status, WAIT_CONV_TC + 0x60 + acc, wait_limit));
       if (!ok) break;
       tc_fence_after();
       const uint32_t t_addr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BLOCK_N + half * HALF_N);

@@ -131,7 +131,7 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
       const int n = tile / tpi, pix0 = (tile - n * tpi) << 7;
       const int img = p.idx.v[n];
       for (int k = 0; k < kslabs; ++k) {
-        ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, 0xB00 + (int)stage, wait_limit);
+        ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, WAIT_POST_TC + (int)stage, wait_limit);
         if (!ok) break;
         const uint32_t fb = smem_u32(full_bar + stage);
         mbar_arrive_expect_tx(fb, PT_SLAB_BYTES);
@@ -145,16 +145,16 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
     constexpr uint32_t IDESC = make_idesc(128, 16);
     uint32_t stage = 0, phase = 0, acc_phase = 0;
     int acc = 0;
-    bool ok = mbar_wait(smem_u32(w_bar), 0u, abort_flag, p.status, 0xB10, wait_limit);
+    bool ok = mbar_wait(smem_u32(w_bar), 0u, abort_flag, p.status, WAIT_POST_TC + 0x10, wait_limit);
     const uint64_t a_desc0 = make_smem_desc(smem_u32(smem), 1024u, 2u);
     const uint64_t b_desc0 = make_smem_desc(smem_u32(s_w), 1024u, 2u);
     for (int tile = t_begin; tile < t_end && ok; ++tile) {
-      ok = mbar_wait(smem_u32(tempty_bar + acc), acc_phase ^ 1u, abort_flag, p.status, 0xB20 + acc, wait_limit);
+      ok = mbar_wait(smem_u32(tempty_bar + acc), acc_phase ^ 1u, abort_flag, p.status, WAIT_POST_TC + 0x20 + acc, wait_limit);
       if (!ok) break;
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 16);
       for (int k = 0; k < kslabs; ++k) {
-        ok = mbar_wait(smem_u32(full_bar + stage), phase, abort_flag, p.status, 0xB30 + (int)stage, wait_limit);
+        ok = mbar_wait(smem_u32(full_bar + stage), phase, abort_flag, p.status, WAIT_POST_TC + 0x30 + (int)stage, wait_limit);
         if (!ok) break;
         const uint64_t a_desc = a_desc0 + (uint64_t)(stage * (PT_SLAB_BYTES >> 4));
         const uint64_t b_desc = b_desc0 + (uint64_t)(k * (PT_WSLAB_BYTES >> 4));
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
         tiles_done = 0;
       }
       // the four warps agree on whether to go on, so that they meet at the same barriers afterwards
-      ok = !named_barrier_or(2, 128, !mbar_wait(smem_u32(tfull_bar + acc), acc_phase, abort_flag, p.status, 0xB40 + acc, wait_limit));
+      ok = !named_barrier_or(2, 128, !mbar_wait(smem_u32(tfull_bar + acc), acc_phase, abort_flag, p.status, WAIT_POST_TC + 0x40 + acc, wait_limit));
       if (!ok) break;
       tc_fence_after();
       uint32_t v[16];

@@ -551,8 +551,8 @@ __global__ void __launch_bounds__(StreamCfg<NCHUNK>::THREADS, 1) post_stream_ker
         if (!ok) {
           // a copy never arrived: record it, give copies still in flight time to land, stop
           if (lane == 0 && p.status) {
-            atomicCAS(p.status, 0, 0x700 + stage);
-            tc::report_status(0x700 + stage, true, p.status, p.status_out);
+            atomicCAS(p.status, 0, tc::WAIT_POST_STREAM + stage);
+            tc::report_status(tc::WAIT_POST_STREAM + stage, true, p.status, p.status_out);
           }
           for (int w = 0; w < 64; ++w) __nanosleep(16000);
           break;

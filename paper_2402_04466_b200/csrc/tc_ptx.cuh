@@ -14,6 +14,10 @@ constexpr long long WAIT_LIMIT_CYCLES = 4000000000ll;  // default limit of a wai
 // "not yet": a suspended thread issues nothing, a thread that polls in a loop takes issue slots
 // from the warps that share its scheduler.
 constexpr uint32_t TRY_WAIT_SUSPEND_NS = 20000u;
+// What a kernel writes to the status word when one of its waits runs out: its own hundreds, in them the wait (its tens) and
+// the stage, buffer or view (ones).  The host prints the code.
+constexpr int WAIT_CONV_TC = 0x100, WAIT_CONV_LSTM = 0x200, WAIT_CONV_FIRST = 0x300, WAIT_CONV_FIRST_FUSED = 0x400, WAIT_CONV_S2 = 0x500,
+              WAIT_POST_TC = 0x600, WAIT_POST_STREAM = 0x700, WAIT_PROBE = 0xA00;
 
 // ------------------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

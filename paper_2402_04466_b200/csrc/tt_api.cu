@@ -17,6 +17,7 @@
 
 #include "tt_internal.h"
 #include "pre_math.cuh"
+#include "tc_ptx.cuh"
 
 using namespace tt;
 
@@ -1380,7 +1381,7 @@ tt_status tt_debug_expire_wait(tt_ctx* ctx, uint64_t limit_cycles) {
   if (limit_cycles == 0 || limit_cycles > (uint64_t)DEFAULT_WAIT_LIMIT_CYCLES)
     return fail(ctx, TT_ERR_INVALID_ARG, "limit_cycles must lie in [1, %lld]", DEFAULT_WAIT_LIMIT_CYCLES);
   TT_CUDA(ctx, cudaSetDevice(ctx->dev));
-  TT_CUDA(ctx, launch_wait_probe(ctx->status_dev, (long long)limit_cycles, 0xA00, ctx->stream));
+  TT_CUDA(ctx, launch_wait_probe(ctx->status_dev, (long long)limit_cycles, tc::WAIT_PROBE, ctx->stream));
   return TT_OK;
 }
 

@@ -37,3 +37,22 @@ def test_the_rule_above_looks_at_every_allocating_kernel():
 def test_no_warp_vote_takes_whatever_lanes_happen_to_be_active():
     """Nothing guarantees that the lanes __activemask() sees are those that reach the vote behind it together."""
     assert [n for n, c in SOURCES.items() if "__activemask" in c] == []
+
+
+def test_status_codes_name_the_kernel():
+    """Every bounded wait reports a code of its kernel's own hundreds."""
+    bases = dict(re.findall(r"(WAIT_[A-Z0-9_]+) = (0x[0-9A-F]+)", SOURCES["tc_ptx.cuh"]))
+    values = [int(v, 16) for v in bases.values()]
+    assert len(set(v >> 8 for v in values)) == len(values) and all(v & 0xFF == 0 for v in values)
+    of_file = {}
+    for name in [n for n in SOURCES if n.endswith(".cu") and n not in ("wait_probe.cu", "tt_api.cu")]:
+        code = SOURCES[name]
+        waits = re.findall(r"mbar_wait(?:_uniform)?\([^;]*?p\.status, ([^,]+), (?:p\.)?wait_limit\)", code) + re.findall(r"atomicCAS\(p\.status, 0, ([^)]+)\)", code)
+        assert len(waits) == code.count("mbar_wait(") + code.count("mbar_wait_uniform(") + code.count("atomicCAS(p.status")
+        for w in waits:
+            m = re.fullmatch(r"(?:tc::)?(WAIT_[A-Z0-9_]+)((?: \+ .*)?)", w)
+            assert m and m.group(1) in bases, (name, w)
+            of_file.setdefault(m.group(1), {}).setdefault(name, []).append(m.group(2))
+    for base, files in of_file.items():
+        assert len(files) == 1, f"{base} is used by {sorted(files)}"
+    assert set(of_file) == set(bases) - {"WAIT_PROBE"}
