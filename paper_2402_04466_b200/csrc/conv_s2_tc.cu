@@ -14,11 +14,11 @@
 // channels wide: their weights (9 x 64 x 32 or 64 bf16, 36 or 72 KB) stay in shared memory for the whole launch, fetched
 // before the wait for the previous kernel.  A block keeps its group of output channels and walks over the tiles.
 //
-// What it is for: launches of a few tiles per block, where a layer's time is start-up, first copies and barrier round
-// trips.  Per tile they fall from nine to four, and the bytes from 9 x 128 pixel rows and the weights to 561 rows.
-// With many tiles per block shared-memory bandwidth decides (an MMA of 64 columns reads 6 KB in its 48 cycles, all of
-// the 128 bytes a cycle there are; one of 128 columns 8 KB in 64), and the 128-wide tap-box form of conv_tc.cu does more per
-// byte read: 64 -> 128 channels at 8 full-HD frames take 78 us there and 132 us here.
+// Against one box per tap a tile's barrier round trips fall from nine to four, and its bytes from 9 x 128 pixel rows and the weights
+// to 561 rows.  At 32 channels that wins at every number of tiles.  At 64 it does while a launch has few tiles per block, where
+// its time is start-up, first copies and round trips; with many, shared-memory bandwidth decides (an MMA of 64 columns reads
+// 6 KB in its 48 cycles, all of the 128 bytes a cycle there are; one of 128 columns 8 KB in 64), and the 128-wide tap-box form of
+// conv_tc.cu does more per byte read: 64 -> 128 channels at 8 full-HD frames take 78 us there and 132 us here.
 //
 // Warp roles: 0 = views and weights by TMA, 1 = tensor memory and MMA issue, 2..5 = epilogue (TMEM lane quarter = warp
 // mod 4; results leave through 2 KB of shared memory per warp and 32 channels, so that four lanes write 64 bytes of a
@@ -243,9 +243,14 @@ cudaError_t launch_t(const ConvS2Params& p, int sm_count, cudaStream_t s) {
 // Output channels per tile, or 0 where this kernel does not apply: more than one channel slab.
 int conv_s2_block_n(int slab_c, int cin, int cout) { return cin == slab_c && cout % N == 0 ? N : 0; }
 
-// Up to four rounds of tiles: measured even or faster up to 2.7 rounds (five 854x480 streams), 10 % slower at 6.5 (one full-HD
-// stream, 64 -> 128 channels), 70 % slower at 52 (eight).
-bool conv_s2_pays(int slab_c, int units, int sm_count) { return units <= 4 * (slab_c == 32 ? 2 : 1) * sm_count; }
+// Against the tap-box form, whole ticks of a feed-forward model (us, mean of 360; `rounds` = units per block):
+//   32 input channels, two blocks per multiprocessor: never slower.  Rounds 0.5 -1.7, 1.6 -1.5, 2.7 -1.0, 4.3 -0.7, 6.5 -2.0, 9.7 -4.3,
+//   13 (eight full-HD streams) -7.6 of 166.  One block, which leaves half of the copies exposed: 1.1 -0.1, 3.2 -1.5, 4.3 +0.3, 7.3 +1.5, 26 +2.0.
+//   64 input channels, one block: 0.5 -1.5, 1.6 -1.0, 2.0 +1.9, 2.2 -2.0, 2.7 -1.4, 3.0 +0.4, 3.2 +1.2, 4.1 +2.4, 4.9 +0.4, 6.5 +2.6, 13 +6.1.
+bool conv_s2_pays(int slab_c, int units, int sm_count, bool one_per_sm) {
+  if (slab_c == 32 && !one_per_sm) return true;
+  return units <= (slab_c == 32 ? 4 : 3) * sm_count;
+}
 
 void conv_s2_box(int view, int* w, int* h) {
   *w = s2_view_w(view);

@@ -858,7 +858,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     for (int l = 1; l < ctx->n_enc; ++l) {
       const TcLayer& L = ctx->tc_enc[l];
       // both kernels add up the same products in the same order: which one runs changes no bit
-      if (L.s2.block_n > 0 && conv_s2_pays(L.s2.slab_c, K * L.s2.tiles_x * L.s2.tiles_y * L.s2.n_tiles_n, ctx->sm_count)) {
+      if (L.s2.block_n > 0 && conv_s2_pays(L.s2.slab_c, K * L.s2.tiles_x * L.s2.tiles_y * L.s2.n_tiles_n, ctx->sm_count, L.s2.one_per_sm != 0)) {
         ConvS2Params q = L.s2;
         q.K = K;
         q.pdl = ctx->profiling ? 0 : 1;

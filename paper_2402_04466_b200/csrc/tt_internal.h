@@ -184,7 +184,7 @@ struct ConvS2Params {
   long long wait_limit;
 };
 int conv_s2_block_n(int slab_c, int cin, int cout);
-bool conv_s2_pays(int slab_c, int units, int sm_count);   // units: pixel tiles x groups of block_n channels
+bool conv_s2_pays(int slab_c, int units, int sm_count, bool one_per_sm);   // units: pixel tiles x groups of block_n channels
 void conv_s2_box(int view, int* w, int* h);
 cudaError_t launch_conv_s2(const ConvS2Params& p, int sm_count, cudaStream_t s);
 

@@ -371,12 +371,13 @@ def test_bf16_preprocessing_inside_the_first_layer_changes_no_bit(cuda_device, s
         assert np.array_equal(h1, h2) and np.array_equal(c1, c2)
 
 
-def test_bf16_encoder_launch_shapes_change_no_bit(cuda_device):
-    """The tensor-core encoder layers run two blocks per multiprocessor by default, the 32 -> 64 channel layer with its
-    weights resident in shared memory; with one block per multiprocessor (weights streamed with the activations) the
-    products are accumulated in the same order, so every output and the state must be the same bits."""
-    wl = tt_synth.workload("cfg1-gain").with_(name="shapes", src_w=330, src_h=250, net_w=264, net_h=200, overlay=True)
-    K, n = 3, 3
+@pytest.mark.parametrize("shape,K,n", [(dict(src_w=330, src_h=250, net_w=264, net_h=200), 3, 3), (dict(src_w=660, src_h=500), 8, 2)])
+def test_bf16_encoder_launch_shapes_change_no_bit(cuda_device, shape, K, n):
+    """The tensor-core encoder layers run two blocks per multiprocessor by default, or one on request.  At the larger batch (1280 tiles of
+    the 32 -> 64 layer) that also takes this layer from the kernel with resident weights and whole views to the one that
+    streams a box and a weight slab per tap.  The products are accumulated in the same order, so every output and the state must
+    be the same bits."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="shapes", overlay=True, **shape)
     host = _frames(wl, K, n)
     runs = []
     for two in (True, False):
