@@ -8,7 +8,7 @@
 // are the same bits.
 //
 // Bound by rounds: a multiprocessor holds one block, and 80 units of 256 columns (one 854x480 stream) take as long as 148.  A unit
-// here is a tile x a group of columns of any multiple of 64 up to 256, grouped as the launch needs: by 192 where that
+// here is a tile x a group of columns, grouped as the launch needs: by 192 (with a remainder of 64 or 128) where that
 // still fits the rounds, or by 256 with the last, partly filled round cut into halves.  M128 x N x K16 takes 128, 96 and 64
 // cycles at N = 256, 192 and 128; for a narrow group's slab to take less than a wide one's, the whole MMA warp
 // runs the issue loop and one elected lane issues (from a single lane's branch a slab takes about 600 cycles at any width).
@@ -292,31 +292,30 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
 }
 
 // Time of a unit in units of one of 256 columns: tensor cycles per slab (512, 384, 256) but no less than the issue loop's
-// round of about 300, and the fixed parts.
+// round of about 300, and the fixed parts.  Units of 128 columns throughout are never the fewest rounds' worth (tried for all widths of up to
+// 2048 columns, 1 to 8000 tiles and 1 to 160 multiprocessors): 128 only appears as the half of a last round's units and as a remainder.
 constexpr double L_COST_256 = 1.0, L_COST_192 = 0.77, L_COST_128 = 0.58;
 
 struct Grouping {
   int width = 256, u_full = 0;
   double cost = 0, plain = 0;   // rounds x time of a unit, as chosen and with groups of 256 throughout
 };
+// C: a multiple of 256
 Grouping group_columns(int tiles, int C, int sm_count) {
   Grouping g;
   auto rounds = [&](long units) { return (double)((units + sm_count - 1) / sm_count); };
-  const long g256 = (long)tiles * ((C + 255) / 256);
+  const long g256 = (long)tiles * (C / 256);
   g.u_full = (int)g256;
   g.cost = g.plain = rounds(g256) * L_COST_256;
   // the last round cut into halves, if that leaves it one round
   const long tail = g256 % sm_count;
-  if (C % 256 == 0 && tail > 0 && 2 * tail <= sm_count) {
+  if (tail > 0 && 2 * tail <= sm_count) {
     g.cost = (double)(g256 / sm_count) * L_COST_256 + L_COST_128;
     g.u_full = (int)(g256 - tail);
   }
-  for (int w : {192, 128}) {
-    if (w >= C) continue;
-    const long units = (long)tiles * ((C + w - 1) / w);
-    const double t = rounds(units) * (w == 192 ? L_COST_192 : L_COST_128);
-    if (t < g.cost - 1e-9) { g.cost = t; g.width = w; g.u_full = (int)units; }
-  }
+  const long units = (long)tiles * ((C + 191) / 192);
+  const double t = rounds(units) * L_COST_192;
+  if (t < g.cost - 1e-9) { g.cost = t; g.width = 192; g.u_full = (int)units; }
   return g;
 }
 
@@ -326,14 +325,15 @@ Grouping group_columns(int tiles, int C, int sm_count) {
 // to 192), 10 % for one full-HD stream (480 -> 444 and 72 halves).  Where the rounds are full (eight full-HD streams)
 // conv_tc.cu's form is 2 % faster.
 bool conv_lstm_pays(int tiles, int cols, int sm_count) {
+  if (cols % 256 || cols > L_MAX_COLS) return false;
   const Grouping g = group_columns(tiles, cols, sm_count);
-  return cols >= 256 && cols <= L_MAX_COLS && g.cost < 0.95 * g.plain;
+  return g.cost < 0.95 * g.plain;
 }
 
 cudaError_t launch_conv_lstm(const ConvLstmParams& p, int sm_count, cudaStream_t s) {
   cudaError_t e = cudaFuncSetAttribute(conv_lstm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L_SMEM);
   if (e != cudaSuccess) return e;
-  if (p.cols % 64 || p.cols < 256 || p.cols > L_MAX_COLS) return cudaErrorInvalidValue;
+  if (p.cols < 256 || p.cols % 256 || p.cols > L_MAX_COLS) return cudaErrorInvalidValue;
   ConvLstmParams q = p;
   const Grouping g = group_columns(p.tiles, p.cols, sm_count);
   q.width = g.width;

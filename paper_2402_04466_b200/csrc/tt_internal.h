@@ -194,7 +194,7 @@ struct ConvLstmParams {
   TensorMap128 map_b;       // packed weights [4*hidden][9*(Cx+Ch)] bf16, K-major, box [64][256]
   TensorMap128 map_b64;     // the same, box [64][64]
   int32_t slabs[2];         // 64-channel slabs of x and h
-  int32_t cols, hidden;     // 4 * hidden columns, a multiple of 64, at least 256
+  int32_t cols, hidden;     // 4 * hidden columns, a multiple of 256
   int32_t tiles, tiles_x, tiles_y, Hm, Wm;   // tiles = images x tiles_x x tiles_y
   IdxMap h_in, c_idx, h_out;                 // image of h, slot of c, image of h' per batch position
   int32_t width, groups, even, u_full;       // set by the launch: column groups, whether all are as wide, the unit from which they are cut in two

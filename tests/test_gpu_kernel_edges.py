@@ -140,11 +140,13 @@ def test_stride2_layer_kernels_give_the_same_bits_at_small_and_large_batches(cud
         ctx.destroy()
 
 
+# units on 148, 128, 100 and 78 multiprocessors (0, 20, 48 and 70 reserved); "full": the kernel of full rounds
 @pytest.mark.parametrize("hidden,net", [
-    (64, (176, 136)),      # one group of 256 columns per tile: halves, or groups of 192 and 64
-    (128, (640, 480)),     # two groups: several rounds, the last cut into halves
-    (128, (400, 300)),     # a ragged map of few tiles: groups of 128
-    (256, (1280, 720)),    # four groups: 192 and a remainder of 64
+    (64, (640, 840)),      # 70 tiles of one group of 256: cut into halves on 148, else full
+    (128, (640, 480)),     # 40 tiles x 512 columns: 192, 192 and 128, but full on 100
+    (128, (400, 300)),     # 21 ragged tiles x 512: halves, but 192, 192 and 128 on 78
+    (256, (1280, 720)),    # 120 tiles x 1024: several rounds of 256, the last cut into halves; full on 128 and 100
+    (256, (368, 480)),     # 24 ragged tiles x 1024: five groups of 192 and one of 64 on 148 and 78, else full
 ])
 def test_convlstm_column_groups_change_no_bit(cuda_device, hidden, net):
     """How many multiprocessors there are decides how the gates' columns are grouped into units (or that the kernel of full rounds
