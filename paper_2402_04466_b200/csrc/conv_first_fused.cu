@@ -47,16 +47,6 @@ __device__ __forceinline__ void copy_row(uint32_t dst, uintptr_t src, uint32_t b
                ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
-// Six bytes starting at byte offset `b` of a word-aligned shared buffer: the RGB triples of two
-// neighbouring pixels.  lo = bytes b..b+3 (R0 G0 B0 R1), hi = bytes b+4..b+7 (G1 B1 . .).
-__device__ __forceinline__ void fetch_pair(const uint8_t* s, int b, uint32_t& lo, uint32_t& hi) {
-  const uint32_t* w = reinterpret_cast<const uint32_t*>(s) + (b >> 2);
-  const uint32_t sh = (uint32_t)(b & 3) * 8u;
-  const uint32_t w0 = w[0], w1 = w[1], w2 = w[2];
-  lo = __funnelshift_r(w0, w1, sh);
-  hi = __funnelshift_r(w1, w2, sh);
-}
-
 struct Tile {
   int img, tx, ty;
 };
@@ -140,7 +130,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
   // evaluate both sides.
   auto sample = [&](const Tile& t, int buf, auto one_row) {
     constexpr bool ONE_ROW = decltype(one_row)::value;
-    const uint8_t* rows = s_src + buf * src_bytes;
+    const uint32_t* rows = reinterpret_cast<const uint32_t*>(s_src + buf * src_bytes);
     const int b_lo = s_b_lo[buf], x0 = t.tx * FF_TW * STRIDE - 1;
     float* pre_img = p.pre_out + (size_t)t.img * 3 * plane;
     // the pixel of patch row e at byte offset xo of the staged rows -> patch entry q; `keep`: also to the resized image.

@@ -40,15 +40,6 @@ constexpr int L_MAX_COLS = 4 * 512;
 constexpr int L_SMEM = L_B_STAGES * L_B_BYTES + L_A_STAGES * L_A_BYTES + L_MAX_COLS * 4 + 256 + 1024 /*alignment slack*/;
 static_assert(L_SMEM <= 227 * 1024, "one block per multiprocessor");
 
-// One special-function instruction each: tanh.approx (relative error about 2^-11, far inside
-// the bf16 path's tolerance) and sigmoid(z) = 0.5 + 0.5 * tanh(z / 2).
-__device__ __forceinline__ float fast_tanh(float z) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(z));
-  return y;
-}
-__device__ __forceinline__ float fast_sigmoid(float z) { return fmaf(0.5f, fast_tanh(0.5f * z), 0.5f); }
-
 struct Unit {
   int m, col0, n;   // pixel tile, first column, columns
 };

@@ -258,8 +258,8 @@ void conv_s2_box(int view, int* w, int* h) {
 }
 
 cudaError_t launch_conv_s2(const ConvS2Params& p, int sm_count, cudaStream_t s) {
-  if (p.slab_c == 32 && p.block_n == 64) return launch_t<32>(p, sm_count, s);
-  if (p.slab_c == 64 && p.block_n == 64) return launch_t<64>(p, sm_count, s);
+  if (p.slab_c == 32) return launch_t<32>(p, sm_count, s);
+  if (p.slab_c == 64) return launch_t<64>(p, sm_count, s);
   return cudaErrorInvalidValue;
 }
 

@@ -76,15 +76,6 @@ struct TcCfg {
   static_assert(A_BYTES % 1024 == 0 && B_BYTES % 1024 == 0, "operand tiles must keep 1024-byte alignment");
 };
 
-// One special-function instruction each: tanh.approx (relative error about 2^-11, far inside
-// the bf16 path's tolerance) and sigmoid(z) = 0.5 + 0.5 * tanh(z / 2).
-__device__ __forceinline__ float fast_tanh(float z) {
-  float y;
-  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(z));
-  return y;
-}
-__device__ __forceinline__ float fast_sigmoid(float z) { return fmaf(0.5f, fast_tanh(0.5f * z), 0.5f); }
-
 
 // ------------------------------------------------------------------------------------ kernel
 // WRES (weights resident): a layer whose whole packed weight matrix is at most WRES_BYTES fetches it once per

@@ -41,17 +41,14 @@ __device__ __forceinline__ int div_by(int n, int d, float inv_d) {
   return q;
 }
 
-// axis_sample with the quotient from div_by: the same i0, i1 and f, bit for bit (inv_den = 1.0f / (2 * out)).
-__device__ __forceinline__ AxisSample axis_sample_fast(int o, int in, int out, float inv_den) {
-  int den = 2 * out;
-  int num = (2 * o + 1) * in - out;
-  int hi = (in - 1) * den;
-  num = max(0, min(num, hi));
-  AxisSample r;
-  r.i0 = div_by(num, den, inv_den);
-  r.i1 = min(r.i0 + 1, in - 1);
-  r.f = (float)(num - r.i0 * den) / (float)den;
-  return r;
+// Six bytes starting at byte offset `b` of a word-aligned shared buffer: the RGB triples of two
+// neighbouring pixels.  lo = bytes b..b+3 (R0 G0 B0 R1), hi = bytes b+4..b+7 (G1 B1 . .).
+__device__ __forceinline__ void fetch_pair(const uint32_t* s_words, int b, uint32_t& lo, uint32_t& hi) {
+  const uint32_t* w = s_words + (b >> 2);
+  const uint32_t sh = (uint32_t)(b & 3) * 8u;
+  const uint32_t w0 = w[0], w1 = w[1], w2 = w[2];
+  lo = __funnelshift_r(w0, w1, sh);
+  hi = __funnelshift_r(w1, w2, sh);
 }
 
 // byte k of x as the float 2^23 + b (exact)

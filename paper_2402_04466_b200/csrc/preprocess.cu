@@ -22,16 +22,6 @@ constexpr int PRE_OUT_W = PRE_TX * 4;
 constexpr int PRE_THREADS = PRE_TX * PRE_TY;
 constexpr int PRE_SMEM_BYTES = 44 * 1024;
 
-// Six bytes starting at byte offset `b` of a word-aligned shared buffer: the RGB triples of two
-// neighbouring pixels.  lo = bytes b..b+3 (R0 G0 B0 R1), hi = bytes b+4..b+7 (G1 B1 . .).
-__device__ __forceinline__ void fetch_pair(const uint32_t* s_words, int b, uint32_t& lo, uint32_t& hi) {
-  const int w = b >> 2;
-  const uint32_t sh = (uint32_t)(b & 3) * 8u;
-  const uint32_t w0 = s_words[w], w1 = s_words[w + 1], w2 = s_words[w + 2];
-  lo = __funnelshift_r(w0, w1, sh);
-  hi = __funnelshift_r(w1, w2, sh);
-}
-
 constexpr int PRE_ROWS = 16;          // output rows per block of the staged kernel: 2 per thread
 
 __global__ void __launch_bounds__(PRE_THREADS)

@@ -68,7 +68,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 
 // The same wait for a whole warp whose control flow has to stay uniform: the usual case, the phase completing within a few
 // suspended tries, is a loop inside the assembly, so that the compiler sees straight-line code and can keep what the warp
-// works on in uniform registers.  Every lane gets the same answer.
+// works on in uniform registers.  Each lane gets an answer of its own, and lanes may differ when the wait runs out: the caller votes
+// before its warp parts or goes on to something that takes the whole warp.
 __device__ __forceinline__ bool mbar_wait_uniform(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status, int code,
                                                   long long limit) {
   uint32_t ok;
@@ -95,6 +96,15 @@ __device__ __forceinline__ bool elect_one() {
   asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(r));
   return r != 0u;
 }
+
+// One special-function instruction each: tanh.approx (relative error about 2^-11, far inside
+// the bf16 path's tolerance) and sigmoid(z) = 0.5 + 0.5 * tanh(z / 2).
+__device__ __forceinline__ float fast_tanh(float z) {
+  float y;
+  asm("tanh.approx.f32 %0, %1;" : "=f"(y) : "f"(z));
+  return y;
+}
+__device__ __forceinline__ float fast_sigmoid(float z) { return fmaf(0.5f, fast_tanh(0.5f * z), 0.5f); }
 
 // The last kernel of a tick tells the host, through a mapped word, of a wait that ran out in it or before it: `before` is the
 // status word as it stood when the kernel's predecessors were done.  A healthy tick writes nothing.  One thread of every

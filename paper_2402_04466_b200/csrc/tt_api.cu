@@ -47,7 +47,7 @@ struct TcLayer {
   bool has_halo = false;
   TensorMap128 map_b[3];       // block_n = 64, 128, 256
   bool has_b[3] = {false, false, false};
-  ConvS2Params s2{};           // stride-2 layers that conv_s2 covers (s2.block_n > 0)
+  ConvS2Params s2{};           // stride-2 layers that conv_s2 covers (s2.n_tiles_n > 0)
 };
 
 std::mutex g_err_mu;
@@ -642,9 +642,8 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
           if ((st = encode_map(ctx, &q.map_v[v], reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l - 1]) + ((size_t)yp * W + xp) * C, 4, dims, str, box, L.slab_c * 2)) != TT_OK)
             return st;
         }
-        q.block_n = conv_s2_block_n(L.slab_c, L.cin0, L.cout);
         q.map_b = L.map_b[0];
-        q.slab_c = L.slab_c; q.cout = L.cout; q.n_tiles_n = L.cout / q.block_n;
+        q.slab_c = L.slab_c; q.cout = L.cout; q.n_tiles_n = L.cout / conv_s2_block_n(L.slab_c, L.cin0, L.cout);
         q.Ho = ctx->lay_h[l + 1]; q.Wo = ctx->lay_w[l + 1]; q.tiles_x = (q.Wo + 7) / 8; q.tiles_y = (q.Ho + 15) / 16;
         q.bias = L.b; q.out = reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l]);
         q.status = ctx->status_dev; q.wait_limit = ctx->wait_limit; q.one_per_sm = ctx->enc_two_per_sm ? 0 : 1;
@@ -858,7 +857,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     for (int l = 1; l < ctx->n_enc; ++l) {
       const TcLayer& L = ctx->tc_enc[l];
       // both kernels add up the same products in the same order: which one runs changes no bit
-      if (L.s2.block_n > 0 && conv_s2_pays(L.s2.slab_c, K * L.s2.tiles_x * L.s2.tiles_y * L.s2.n_tiles_n, ctx->sm_count, L.s2.one_per_sm != 0)) {
+      if (L.s2.n_tiles_n > 0 && conv_s2_pays(L.s2.slab_c, K * L.s2.tiles_x * L.s2.tiles_y * L.s2.n_tiles_n, ctx->sm_count, L.s2.one_per_sm != 0)) {
         ConvS2Params q = L.s2;
         q.K = K;
         q.pdl = ctx->profiling ? 0 : 1;

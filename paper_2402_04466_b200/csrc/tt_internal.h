@@ -172,10 +172,10 @@ constexpr long long DEFAULT_WAIT_LIMIT_CYCLES = 4000000000ll;   // about 2 s of 
 // Stride-2 layers of one channel slab (conv_s2_block_n > 0): parity views fetched once with their halo, weights resident.
 struct ConvS2Params {
   TensorMap128 map_v[4];    // views even/even, even rows/odd columns, odd/even, odd/odd; boxes [slab_c][conv_s2_box][1]
-  TensorMap128 map_b;       // packed weights [cout][9 * slab_c] bf16, K-major, box [slab_c][block_n]
+  TensorMap128 map_b;       // packed weights [cout][9 * slab_c] bf16, K-major, box [slab_c][64]
   int32_t slab_c;           // input channels: 32 or 64
   int32_t K, Ho, Wo, tiles_x, tiles_y;   // 8 x 16 pixel tiles
-  int32_t n_tiles_n, block_n, cout;
+  int32_t n_tiles_n, cout;  // groups of conv_s2_block_n output channels
   int32_t one_per_sm;       // one block per multiprocessor even where two fit
   int32_t pdl;
   const float* bias;
@@ -183,8 +183,8 @@ struct ConvS2Params {
   int32_t* status;
   long long wait_limit;
 };
-int conv_s2_block_n(int slab_c, int cin, int cout);
-bool conv_s2_pays(int slab_c, int units, int sm_count, bool one_per_sm);   // units: pixel tiles x groups of block_n channels
+int conv_s2_block_n(int slab_c, int cin, int cout);   // output channels of a tile, 0 where the kernel does not apply
+bool conv_s2_pays(int slab_c, int units, int sm_count, bool one_per_sm);   // units: pixel tiles x groups of channels
 void conv_s2_box(int view, int* w, int* h);
 cudaError_t launch_conv_s2(const ConvS2Params& p, int sm_count, cudaStream_t s);
 
