@@ -65,39 +65,52 @@ def test_fp32_convolutions_give_a_stream_the_same_bits_whatever_shares_its_tick(
             assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("shape", [
-    dict(src_w=214, src_h=120, net_w=160, net_h=120),                                    # rows not resized
-    dict(src_w=300, src_h=233, net_w=132, net_h=70),                                     # both axes down, a last tile of 2 columns and 3 rows
-    dict(src_w=90, src_h=50, net_w=196, net_h=131, enc_stride=(1, 2, 2)),                # up-scaling, stride 1
-    dict(src_w=96, src_h=99, net_w=32, net_h=33, enc_cout=(64, 64), enc_stride=(1, 2)),  # every row on a frame row (a third), one tile wide
-    dict(src_w=640, src_h=700, net_w=260, net_h=192, enc_cout=(64, 128, 256), hidden=256),   # several tiles per block
+@pytest.mark.parametrize("shape,K,pad", [
+    (dict(src_w=214, src_h=120, net_w=160, net_h=120), 3, 5),                                    # rows not resized; odd pitch
+    (dict(src_w=299, src_h=133, net_w=200, net_h=89), 3, 0),                                     # both axes down, a last tile of 4 columns and 5 rows
+    (dict(src_w=203, src_h=157, net_w=132, net_h=100), 2, 64),                                   # both axes down, wide padding
+    (dict(src_w=90, src_h=50, net_w=196, net_h=131, enc_stride=(1, 2, 2)), 3, 1),                # up-scaling, stride 1
+    (dict(src_w=96, src_h=99, net_w=32, net_h=33, enc_cout=(64, 64), enc_stride=(1, 2)), 3, 0),  # every row on a frame row (a third), one tile wide
+    (dict(src_w=960, src_h=720, enc_cout=(64, 128), enc_stride=(2, 2)), 8, 16),                  # 2400 tiles: five or six per block
 ])
-def test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cuda_device, shape):
+def test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cuda_device, shape, K, pad):
     """One kernel resizes, normalises and convolves; with stage events on the two kernels it stands for run instead.  Same expressions, same
-    order of products: the resized image, the first layer's map, every result and the state are the same bits."""
-    wl = tt_synth.workload("cfg1-gain").with_(name="first", **{"hidden": 64, **shape})
-    K, n = 3, 2
+    order of products: the resized image, the first layer's map, every result and the state are the same bits, from frames with padded
+    rows and from the same frames without padding."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="first", overlay=True, **{"hidden": 64, **shape})
+    w = tt_synth.make_weights(wl)
+    n = 2
     host = _frames(wl, K, n)
-    runs = []
-    for separate in (False, True):
-        ctx, states, _ = _make(wl, K)
+    runs, launches = [], []
+    for separate, extra in ((False, pad), (True, pad), (False, 0)):
+        cfg = binding.make_config(wl, max_streams=K)
+        cfg.src_pitch = pitch = 3 * wl.src_w + extra
+        ctx = binding.Context(cfg, w)
+        states = [ctx.state_create() for _ in range(K)]
         ctx.set_profiling(separate)
         out = []
         for t in range(n):
-            # stream 1 at an odd address, the frame's last byte the buffer's last
-            bufs = [torch.empty(host[k][t].size + k, dtype=torch.uint8, device=cuda_device) for k in range(K)]
+            # stream k at k bytes behind an aligned address, the frame's last byte the buffer's last
+            bufs = []
             for k in range(K):
-                bufs[k][k:].copy_(torch.from_numpy(host[k][t]).reshape(-1))
+                rows = np.full((wl.src_h, pitch), 201, np.uint8)
+                rows[:, :3 * wl.src_w] = host[k][t].reshape(wl.src_h, -1)
+                b = torch.empty(rows.size + k, dtype=torch.uint8, device=cuda_device)
+                b[k:].copy_(torch.from_numpy(rows.reshape(-1)))
+                bufs.append(b)
             ctx.submit_frames([bufs[k][k:] for k in range(K)], states, frame_index=t)
             res = ctx.sync()
-            out += [a for i, r in enumerate(res) for a in (ctx.fetch_probs(r), ctx.fetch_masks(r), r["conf"], r["cx"], ctx.debug_tensor(states[i], "pre"),
-                                                           ctx.debug_tensor(states[i], "enc0"))]
+            out += [a for i, r in enumerate(res) for a in (ctx.fetch_probs(r), ctx.fetch_masks(r), ctx.fetch_overlay(r), r["conf"], r["cx"],
+                                                           ctx.debug_tensor(states[i], "pre"), ctx.debug_tensor(states[i], "enc0"))]
         if separate:
             assert ctx.get_stage_times()["preprocess"] > 0
+        launches.append(ctx.get_counters()[0])
         runs.append(out + [a for s in states for a in ctx.state_export(s)])
         ctx.destroy()
-    for a, b in zip(*runs):
-        assert np.array_equal(a, b)
+    assert launches[0] == launches[2] == launches[1] - n          # one launch a tick fewer: the first layer did sample the frames itself
+    for other in runs[1:]:
+        for a, b in zip(runs[0], other):
+            assert np.array_equal(a, b)
 
 
 @pytest.mark.parametrize("net,enc,stride,hidden,K", [
@@ -105,7 +118,7 @@ def test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cud
     ((66, 66), (64, 64), (1, 2), 64, 1),               # 64 -> 64, a last tile of one column and one row
     ((97, 131), (64, 64, 128, 128), (1, 2, 2, 2), 64, 3),   # odd inputs; 64 -> 128 resident, 128 -> 128 through the ring
     ((130, 70), (32, 64, 128, 256), (1, 2, 2, 2), 64, 2),   # 128 -> 256 through the ring
-    ((128, 128), (64, 256), (2, 2), 64, 2),            # two groups of 128 resident outputs
+    ((128, 128), (64, 256), (2, 2), 64, 2),            # four groups of 64 resident outputs
     ((16, 12), (32, 64), (2, 2), 64, 1),               # a map smaller than one tile
 ])
 def test_bf16_stride2_layers_at_the_edges_of_their_tiles(cuda_device, net, enc, stride, hidden, K):
@@ -116,8 +129,9 @@ def test_bf16_stride2_layers_at_the_edges_of_their_tiles(cuda_device, net, enc, 
 
 
 def test_stride2_layer_kernels_give_the_same_bits_at_small_and_large_batches(cuda_device):
-    """One stream's strided layers run as a few tiles per block on views fetched with their halo, eight streams' as many tiles
-    per block with one box per tap: the same products in the same order, so a stream's maps, results and state must not change."""
+    """One stream's 64 -> 128 channel layer runs as a few tiles per block on views fetched with their halo, eight streams' as many
+    tiles per block with one box per tap: the same products in the same order, so a stream's maps, results and state must not
+    change.  (The 32 -> 64 channel layer runs on views in both.)"""
     wl = tt_synth.workload("cfg1-gain").with_(name="s2-batch", src_w=800, src_h=500)
     K = 8
     host = [tt_synth.make_frames(wl.frame_kind, wl.stream_seed(s), 1, wl.src_w, wl.src_h)[0] for s in range(K)]

@@ -334,9 +334,9 @@ def test_bf16_convlstm_one_box_per_tap_still_matches(cuda_device):
     dict(src_w=160, src_h=120, net_w=160, net_h=120, stride1=True),   # no resize, stride-1 first layer
 ])
 def test_bf16_preprocessing_inside_the_first_layer_changes_no_bit(cuda_device, shape):
-    """On request the first encoder layer samples the frames itself; against the preprocessing as a kernel of its own
-    (which writes the resized fp32 image the layer then reads) every output and the state must be the same bits.
-    Stream 1's frames sit at an odd address, and the last frame ends where its buffer ends."""
+    """The first encoder layer samples the frames itself, and on request does not write the resized fp32 image; against the
+    preprocessing as a kernel of its own (which runs with stage events on and writes the image the layer then reads) every output and
+    the state must be the same bits.  Stream 1's frames sit at an odd address, and the last frame ends where its buffer ends."""
     shape = dict(shape)
     stride1 = shape.pop("stride1", False)
     wl = tt_synth.workload("cfg1-gain").with_(name="fuse", overlay=True, **shape)
@@ -346,8 +346,9 @@ def test_bf16_preprocessing_inside_the_first_layer_changes_no_bit(cuda_device, s
     host = _frames(wl, K, n)
     nbytes = host[0][0].size
     runs = []
-    for fused in (True, False):
+    for fused, separate in ((True, False), (False, False), (False, True)):
         ctx, states, _ = _make(wl, K, overlay=True, fused_pre=fused)
+        ctx.set_profiling(separate)
         out = []
         for t in range(n):
             bufs = [torch.empty(nbytes + 1, dtype=torch.uint8, device=cuda_device) for _ in range(K)]
@@ -362,13 +363,14 @@ def test_bf16_preprocessing_inside_the_first_layer_changes_no_bit(cuda_device, s
                          ctx.debug_tensor(states[i], "pre"), ctx.debug_tensor(states[i], "enc0")) for i, r in enumerate(res)])
         runs.append((out, [ctx.state_export(s) for s in states]))
         ctx.destroy()
-    (a, ha), (b, hb) = runs
-    for ta, tb in zip(a, b):
-        for ra, rb in zip(ta, tb):
-            for va, vb in zip(ra, rb):
-                assert np.array_equal(va, vb)
-    for (h1, c1), (h2, c2) in zip(ha, hb):
-        assert np.array_equal(h1, h2) and np.array_equal(c1, c2)
+    a, ha = runs[0]
+    for b, hb in runs[1:]:
+        for ta, tb in zip(a, b):
+            for ra, rb in zip(ta, tb):
+                for va, vb in zip(ra, rb):
+                    assert np.array_equal(va, vb)
+        for (h1, c1), (h2, c2) in zip(ha, hb):
+            assert np.array_equal(h1, h2) and np.array_equal(c1, c2)
 
 
 @pytest.mark.parametrize("shape,K,n", [(dict(src_w=330, src_h=250, net_w=264, net_h=200), 3, 3), (dict(src_w=660, src_h=500), 8, 2)])
