@@ -277,7 +277,10 @@ tt_status tt_sched_stats(const tt_sched* s, uint64_t* batches, uint64_t* frames,
 /*
  * Measurement hooks (the paper times every operator's input and output, Section II-C, data
  * flow tracking; here CUDA events on the context's stream bracket each stage of a tick).
- * tt_set_profiling(on != 0) makes every following submit record stage events.
+ * tt_set_profiling(on != 0) makes every following submit record stage events.  Such a tick runs its stages as launches of
+ * their own, one behind the other: on the bf16 path preprocessing and first encoder layer, which a tick without events makes one
+ * launch where the layer and the resize factor allow, are two (same bits), so TT_STAGE_PREPROCESS and TT_STAGE_ENC0 are times of
+ * kernels that the unprofiled tick does not contain.  With TT_OPT_FUSED_PRE they stay one launch, timed as TT_STAGE_ENC0.
  * tt_get_stage_times fills ms[TT_STAGE_COUNT] (host) with the device time of each stage of
  * the last completed submit, -1 for stages that did not run or when profiling was off.
  * tt_get_counters reports how many of the library's kernels and ticks this context has
