@@ -17,8 +17,8 @@
 //   MMA      four tcgen05.mma M128 x COUT x K16, issued by one thread;
 //   epilogue of the tile before, while the next patch is already being built: bias, ReLU, 32-byte stores per lane.
 // A specialised form (eight sampling warps feeding four gather warps through patch buffers) had been 6 us slower per tick than
-// the two kernels at 5 streams of 854x480.  This one, alone under the profiler: 18 us against 10 + 14.6 us at that size, 9.0 against
-// 5.9 + 7.9 us for one stream, 97 against 38 + 62 us for 8 full-HD streams.
+// the two kernels at 5 streams of 854x480.  This one, alone under the profiler: 18.8 us against 10.1 + 14.4 us at that size, 9.8 against
+// 7.2 + 9.2 us for one stream, 100 against 38 + 61 us for 8 full-HD streams, where only the second launch's gap is won.
 #include <type_traits>
 
 #include "tt_internal.h"

@@ -17,13 +17,13 @@
 // Against one box per tap a tile's barrier round trips fall from nine to four, and its bytes from 9 x 128 pixel rows and the weights
 // to 561 rows.  At 32 channels that wins at every number of tiles.  At 64 it does while a launch has few tiles per block, where
 // its time is start-up, first copies and round trips; with many, shared-memory bandwidth decides (an MMA of 64 columns reads
-// 6 KB in its 48 cycles, all of the 128 bytes a cycle there are; one of 128 columns 8 KB in 64), and the 128-wide tap-box form of
-// conv_tc.cu does more per byte read: 64 -> 128 channels at 8 full-HD frames take 78 us there and 132 us here.
+// 6 KB, 48 cycles at 128 bytes a cycle for the 32 it keeps the tensor pipe busy; one of 128 columns 8 KB, 64 for 64), and the
+// 128-wide tap-box form of conv_tc.cu does more per byte read: 64 -> 128 channels at 8 full-HD frames take 78 us there and 132 us here.
 //
 // Warp roles: 0 = views and weights by TMA, 1 = tensor memory and MMA issue, 2..5 = epilogue (TMEM lane quarter = warp
 // mod 4; results leave through 2 KB of shared memory per warp and 32 channels, so that four lanes write 64 bytes of a
-// pixel).  The whole MMA warp runs the issue loop and one elected lane issues: with uniform control flow an MMA of
-// M128 x N x K16 takes 48 cycles at N = 64, 59 from a single lane's branch.
+// pixel).  The whole MMA warp runs the issue loop and one elected lane issues: with uniform control flow the
+// operand descriptors stay in uniform registers.
 // All waits are bounded (see tc_ptx.cuh).
 // Stage times with their event, tap-box form -> this one: one 854x480 stream 12.3 -> 10.3 us (32 -> 64 channels) and 12.3 -> 10.2 us
 // (64 -> 128), five 17.0 -> 17.1 and 15.4 -> 14.3 us.

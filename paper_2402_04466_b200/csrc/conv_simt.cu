@@ -8,13 +8,13 @@
 // broadcast weight loads from shared memory.  A warp covers 32 x 4 pixels of one group of 8 channels.
 // Blocks are made of WY warps along y, WO channel groups that share the input tile, and KS warps that share
 // out the input channels of a tile and add their sums up in shared memory at the end: small maps have too few
-// outputs to occupy the device otherwise.  Input tile (haloed; at stride 2 even and odd columns apart) and
+// outputs to occupy the device otherwise.  KS orders the sums and follows from the layer alone; WY and WO also from the batch.  Input tile (haloed; at stride 2 even and odd columns apart) and
 // weights of CB channels are copied asynchronously into one of two buffers while the other is used.
 //
 // Against one pixel x 16/32 channels per thread, 32 x 8 pixels per block and synchronous staging (stage times with
 // their event): ConvLSTM of one 64x64 map with 16 channels 51 -> 15 us, of three 80x60 maps with 32 channels 135 -> 70 us
-// (32 TFLOP/s, 43 % of the fp32 pipe: 16 warps per multiprocessor, two barriers per chunk and the last row and column
-// tiles' idle lanes).  The same tile as packed pairs of pixels (fma.rn.f32x2) took 94 us: more register moves to form
+// (32 TFLOP/s, 43 % of the fp32 pipe: 16 warps per multiprocessor and the last row and column tiles' idle lanes; one barrier per
+// chunk instead of two is worth 1 %).  The same tile as packed pairs of pixels (fma.rn.f32x2) took 94 us: more register moves to form
 // the pairs than FMAs saved.
 #include "tt_internal.h"
 

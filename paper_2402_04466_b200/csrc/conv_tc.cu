@@ -60,10 +60,8 @@ struct TcCfg {
   static constexpr int TAB_BYTES = MAX_K_ITERS * 16 + 4 * TT_MAX_STREAMS * 4;   // iteration table + image index maps
   static constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + BAR_BYTES + TAB_BYTES + 1024 /*alignment slack*/;
   // Halo mode (stride 1, 64-channel slabs): the activation ring holds haloed patches, one per
-  // channel slab: 18 rows x 16 pixels x 64 channels for an 8 x 16 output patch (10 of the 16
-  // columns are needed; a row pitch of 16 pixels = 2048 bytes keeps every 8-pixel operand group
-  // of every tap at the same phase of the 1024-byte swizzle pattern).  The weight ring holds one
-  // [BLOCK_N][64] slab per tap.
+  // channel slab: 18 rows x 10 pixels x 64 channels for an 8 x 16 output patch.  The weight ring holds
+  // one [BLOCK_N][64] slab per tap.
   static constexpr int HALO_PITCH = 10, HALO_ROWS = 18;
   static constexpr int HALO_A_BYTES = (HALO_ROWS * HALO_PITCH * SLAB_C * 2 + 1023) / 1024 * 1024;   // 23040 -> 23552
   static constexpr int HALO_A_TX = HALO_ROWS * HALO_PITCH * SLAB_C * 2;
@@ -306,10 +304,10 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BLOCK_N);
       if (HALO) {
         // Output pixel (py, px) of the 8 x 16 patch reads halo pixel (py + ky, px + kx): the A operand
-        // of a tap is the same shared-memory patch, entered (ky * 16 + kx) pixel rows of 128 bytes
+        // of a tap is the same shared-memory patch, entered (ky * 10 + kx) pixel rows of 128 bytes
         // further on.  The 8 pixels of one patch row are one 8-row operand group; groups are one halo
-        // row = 2048 bytes apart.  The 128-byte swizzle is a function of the shared-memory address
-        // (the TMA unit wrote the patch that way), so an operand that starts kx rows into a 1024-byte
+        // row = 1280 bytes apart.  The 128-byte swizzle is a function of the shared-memory address
+        // (the TMA unit wrote the patch that way), so an operand that starts in the middle of a 1024-byte
         // pattern needs nothing but its start address.
         uint32_t first = 1;
         for (int sg = 0; sg < slabs_per_tap && ok; ++sg) {

@@ -134,7 +134,7 @@ struct ConvTcParams {
   // A operand sources: up to two NHWC bf16 tensors (x then h); for stride 2 four parity
   // views of the single source.  maps_a[src*4 + parity] with parity = (ypar*2 + xpar).
   TensorMap128 maps_a[8];
-  TensorMap128 maps_halo[2];// halo mode: the two sources again with a box of [64 channels][16][18][1] (haloed patch of an 8 x 16 tile)
+  TensorMap128 maps_halo[2];// halo mode: the two sources again with a box of [64 channels][10][18][1] (haloed patch of an 8 x 16 tile)
   TensorMap128 map_b;       // packed weights [CoutPacked][Ktot] bf16, K-major
   int32_t n_src;            // 1 or 2
   int32_t slabs[2];         // channel slabs (of slab_c channels) per source
