@@ -1,13 +1,12 @@
 // S1: uint8 RGB interleaved frame -> bilinear resize -> normalise -> planar fp32.
 //
-// HBM-bound stage.  A block produces a 128 x 16 tile of the output.  The source rows it needs
-// are staged in shared memory with 128-bit loads of the aligned byte range that covers them
-// (row pitch 3*W is in general not a multiple of 16, so rows are treated as a byte stream and
-// indexed from the remainder).  The horizontal sample positions of the tile's 128 columns are
-// computed once per block into shared memory.  A thread produces 4 consecutive outputs of two
-// rows for all three channels: each bilinear tap pair (two neighbouring RGB pixels = 6 bytes) is
-// fetched as three 32-bit shared loads plus funnel shifts, bytes become floats by a byte
-// permute into the mantissa of 2^23, and the results leave as three 128-bit stores.
+// Bound by instruction issue (about 60 instructions per pixel of three channels where both axes are resized) and by HBM.  A block
+// works down a column of tiles of COLS output columns and `tile_rows` rows.  A thread keeps one output column, so the horizontal
+// sample position stays in its registers, neighbouring lanes read neighbouring bytes of a staged row (few bank conflicts; with
+// four neighbouring outputs per thread every fetch took four to five passes), and a warp's store is 128 contiguous bytes.
+// The frame rows under a tile are staged as a byte stream (row pitch 3*W is in general not a multiple of 16) by asynchronous 16-byte
+// copies of the aligned range that covers them, while the tile before is sampled.  A bilinear tap pair (two neighbouring RGB pixels = 6
+// bytes) is fetched as three 32-bit shared loads plus funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
 #include "tt_internal.h"
 #include "pre_math.cuh"
 
@@ -16,132 +15,143 @@ namespace {
 
 using namespace pre;
 
-constexpr int PRE_TX = 32;          // threads along x; each makes 4 outputs -> 128 outputs per block row
-constexpr int PRE_TY = 8;           // output rows per block
-constexpr int PRE_OUT_W = PRE_TX * 4;
-constexpr int PRE_THREADS = PRE_TX * PRE_TY;
-constexpr int PRE_SMEM_BYTES = 44 * 1024;
+constexpr int PRE_THREADS = 256, PRE_PER_SM = 4;
+constexpr int PRE_MAX_ROWS = 32;             // output rows of a tile
+constexpr int PRE_STAGE_BYTES = 26 * 1024;   // staged rows of a tile; two tiles of four blocks fit a multiprocessor
 
-constexpr int PRE_ROWS = 16;          // output rows per block of the staged kernel: 2 per thread
+struct PreprocessArgs {
+  PreprocessParams p;
+  float scale, shift;
+  int32_t tile_rows, tiles_x, tiles_y;
+  int32_t rows_cap, row_cap;                 // staged rows of a tile, bytes of one (a multiple of 16)
+  int32_t tiles_per_block, tiles_left;       // the first tiles_left blocks take one tile more
+};
 
-__global__ void __launch_bounds__(PRE_THREADS)
-preprocess_staged_kernel(const __grid_constant__ PreprocessParams p, int row_cap_bytes, float scale, float shift) {
-  extern __shared__ __align__(16) uint8_t s_mem[];
-  __shared__ __align__(16) int s_xoff[PRE_OUT_W];    // 3 * (i0 - sx_lo) per output column of the tile
-  __shared__ __align__(16) float s_fx[PRE_OUT_W];
-  __shared__ int s_y0[PRE_ROWS], s_y1[PRE_ROWS];     // source rows of every output row of the tile
-  __shared__ float s_fy[PRE_ROWS];
-  __shared__ int s_xlo, s_xhi;                       // source column range of the tile
+struct Tile {
+  int img, tx, ty;
+};
+
+// ONE_ROW: the height is not resized, so every sample sits on a source row (weight zero for the next one).
+template <int COLS, bool ONE_ROW>
+__global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_kernel(const __grid_constant__ PreprocessArgs a) {
+  constexpr int GROUPS = PRE_THREADS / COLS;         // rows sampled at a time
+  extern __shared__ __align__(16) uint8_t s_mem[];   // [2][rows_cap][row_cap]
+  __shared__ __align__(16) int4 s_row[2][PRE_MAX_ROWS];   // per tile row: byte offsets of its two source rows in the buffer, bits of the lower one's weight
   // the next kernel of the stream, if it was launched as a programmatic dependent, may start its set-up now;
   // it waits for this grid to finish before it reads the output
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int n = blockIdx.z;
-  const uint8_t* __restrict__ src = p.src_tab ? p.src_tab[n] : p.src.p[n];
-  const uint32_t src_lo = (uint32_t)(uintptr_t)src;  // only the low bits matter for 16-byte alignment
-  const int xo_blk = blockIdx.x * PRE_OUT_W;
-  const int yo_blk = blockIdx.y * PRE_ROWS;
-  const int tid = threadIdx.y * PRE_TX + threadIdx.x;
+  pdl_launch_dependents();
+  const PreprocessParams& p = a.p;
+  const int tid = threadIdx.x, col = tid % COLS, grp = tid / COLS;
+  const int buf_bytes = a.rows_cap * a.row_cap, vecs = a.row_cap >> 4;
+  const int t_begin = (int)blockIdx.x * a.tiles_per_block + min((int)blockIdx.x, a.tiles_left);
+  const int n = a.tiles_per_block + ((int)blockIdx.x < a.tiles_left ? 1 : 0);
+  const int step_r = PRE_THREADS / vecs, step_v = PRE_THREADS - step_r * vecs;   // from one of a thread's copies to its next
+  const int r_first = tid / vecs, v_first = tid - r_first * vecs;
+  // tiles in order of (image, tile column, tile row)
+  auto advance = [&](Tile& t) {
+    if (++t.ty == a.tiles_y) {
+      t.ty = 0;
+      if (++t.tx == a.tiles_x) { t.tx = 0; ++t.img; }
+    }
+  };
+  auto left_column = [&](int tx) { return axis_sample(tx * COLS, p.src_w, p.net_w).i0; };
 
-  // Phase 0: one sample position per thread (the only integer divisions of the kernel).
-  if (tid < PRE_OUT_W) {
-    const AxisSample sx = axis_sample(min(xo_blk + tid, p.net_w - 1), p.src_w, p.net_w);
-    s_xoff[tid] = 3 * sx.i0;
-    s_fx[tid] = sx.f;
-    if (tid == 0) s_xlo = sx.i0;
-    if (tid == PRE_OUT_W - 1) s_xhi = min(sx.i0 + 1, p.src_w - 1);
-  } else if (tid < PRE_OUT_W + PRE_ROWS) {
-    const int r = tid - PRE_OUT_W;
-    const AxisSample sy = axis_sample(min(yo_blk + r, p.net_h - 1), p.src_h, p.net_h);
-    s_y0[r] = sy.i0;
-    s_y1[r] = sy.i1;
-    s_fy[r] = sy.f;
+  // Byte b of a staged row is the frame's byte (aligned start of that row's range) + b.
+  auto stage = [&](const Tile& t, int buf, int sx_lo, int sx_hi) {
+    const uint8_t* src = p.src_tab ? p.src_tab[t.img] : p.src.p[t.img];
+    const int y0 = t.ty * a.tile_rows, y_last = min(y0 + a.tile_rows, p.net_h) - 1;
+    const int r_lo = axis_sample(y0, p.src_h, p.net_h).i0, rows = axis_sample(y_last, p.src_h, p.net_h).i1 - r_lo + 1;
+    if (tid < a.tile_rows) {
+      const AxisSample sy = axis_sample(min(y0 + tid, p.net_h - 1), p.src_h, p.net_h);
+      // low bits of the address of column sx_lo in source row 0: (that + row * pitch) & 15 is its position in the staged row
+      const uint32_t base_lo = (uint32_t)(uintptr_t)src + 3u * (uint32_t)sx_lo;
+      s_row[buf][tid] = make_int4((sy.i0 - r_lo) * a.row_cap + (int)((base_lo + (uint32_t)(sy.i0 * p.src_pitch)) & 15u),
+                                  (sy.i1 - r_lo) * a.row_cap + (int)((base_lo + (uint32_t)(sy.i1 * p.src_pitch)) & 15u), __float_as_int(sy.f), 0);
+    }
+    const uintptr_t first = (uintptr_t)src + (size_t)r_lo * p.src_pitch + 3 * sx_lo;
+    const int span = 3 * (sx_hi - sx_lo) + 2;          // last byte of a row, counted from its first
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_mem + buf * buf_bytes);
+    for (int r = r_first, v = v_first; r < rows;) {
+      const uintptr_t g = first + (size_t)r * p.src_pitch;
+      if (v * 16 <= (int)(g & 15) + span)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + r * a.row_cap + v * 16), "l"((g & ~(uintptr_t)15) + v * 16) : "memory");
+      r += step_r;
+      v += step_v;
+      if (v >= vecs) { v -= vecs; ++r; }
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+
+  Tile cur, ahead;
+  {
+    const int tiles_per_img = a.tiles_x * a.tiles_y;
+    cur.img = t_begin / tiles_per_img;
+    const int rem = t_begin - cur.img * tiles_per_img;
+    cur.tx = rem / a.tiles_y;
+    cur.ty = rem - cur.tx * a.tiles_y;
   }
-  __syncthreads();
-  const int sx_lo = s_xlo, sx_hi = s_xhi;
-  const int sy_lo = s_y0[0], sy_hi = s_y1[PRE_ROWS - 1];
-  const int n_rows = sy_hi - sy_lo + 1;
+  ahead = cur;
+  auto stage_ahead = [&](int buf) {
+    const int sx_lo = left_column(ahead.tx), sx_hi = axis_sample(min((ahead.tx + 1) * COLS, p.net_w) - 1, p.src_w, p.net_w).i1;
+    stage(ahead, buf, sx_lo, sx_hi);
+    advance(ahead);
+  };
+  if (n > 0) stage_ahead(0);
 
-  // Phase 1: row r of the footprint goes to s_mem[r*row_cap_bytes ...]; byte b of a staged row is
-  // the global byte (aligned start of that row's range) + b.  Warp w copies rows w, w+8, ...; its
-  // lanes copy 16-byte vectors lane, lane+32, ... of the row.
-  for (int r = threadIdx.y; r < n_rows; r += PRE_TY) {
-    const size_t g_first = (size_t)(sy_lo + r) * p.src_pitch + 3 * sx_lo;
-    const uintptr_t a_first = ((uintptr_t)src + g_first) & ~(uintptr_t)15;
-    const uintptr_t a_end = (((uintptr_t)src + g_first + 3 * (sx_hi - sx_lo) + 2) | 15) + 1;
-    const int n_vec = (int)((a_end - a_first) >> 4);
-    uint4* srow = reinterpret_cast<uint4*>(s_mem + (size_t)r * row_cap_bytes);
-    for (int i = threadIdx.x; i < n_vec; i += PRE_TX) srow[i] = __ldg(reinterpret_cast<const uint4*>(a_first) + i);
-  }
-  __syncthreads();
-
-  // Phase 2: 4 consecutive outputs of rows threadIdx.y and threadIdx.y + 8.
-  const int xl = threadIdx.x * 4;
-  const int xo0 = xo_blk + xl;
-  if (xo0 >= p.net_w) return;
-  const uint32_t* s_words = reinterpret_cast<const uint32_t*>(s_mem);
-  const int4 xoff4 = *reinterpret_cast<const int4*>(s_xoff + xl);
-  const float4 fx4 = *reinterpret_cast<const float4*>(s_fx + xl);
-  const int xoffs[4] = {xoff4.x - 3 * sx_lo, xoff4.y - 3 * sx_lo, xoff4.z - 3 * sx_lo, xoff4.w - 3 * sx_lo};
-  const float fxs[4] = {fx4.x, fx4.y, fx4.z, fx4.w};
   const size_t plane = (size_t)p.net_h * p.net_w;
-  // with a row length that is a multiple of 4 every row start is as aligned as the tensor itself
-  const bool vec_ok = ((p.net_w & 3) == 0) && (xo0 + 3 < p.net_w) && (((uintptr_t)p.dst & 15) == 0);
-
-#pragma unroll
-  for (int rr = 0; rr < 2; ++rr) {
-    const int r = threadIdx.y + rr * PRE_TY;
-    const int yo = yo_blk + r;
-    if (yo >= p.net_h) break;
-    const int y0 = s_y0[r], y1 = s_y1[r];
-    const float fy = s_fy[r];
-    // byte position of source column sx_lo inside the two staged rows
-    const int base0 = (y0 - sy_lo) * row_cap_bytes + (int)((src_lo + (uint32_t)(y0 * p.src_pitch + 3 * sx_lo)) & 15u);
-    const int base1 = (y1 - sy_lo) * row_cap_bytes + (int)((src_lo + (uint32_t)(y1 * p.src_pitch + 3 * sx_lo)) & 15u);
-    float o0[4], o1[4], o2[4];  // the three channels of the 4 outputs
-    if (fy == 0.0f) {
-      // The sample sits exactly on a source row (every row of an axis that is not resized): the
-      // lower row has weight zero, so top + 0 * (bot - top) = top and only one row is fetched.
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
+  int tx = -1, x = 0, xo = 0;
+  float fx = 0.f;
+  for (int i = 0; i < n; ++i) {
+    if (i + 1 < n) {
+      stage_ahead((i + 1) & 1);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
+    if (cur.tx != tx) {
+      tx = cur.tx;
+      x = tx * COLS + col;
+      const AxisSample sx = axis_sample(min(x, p.net_w - 1), p.src_w, p.net_w);
+      xo = 3 * (sx.i0 - left_column(tx));
+      fx = sx.f;
+    }
+    __syncthreads();                                   // this tile's rows and row table are complete
+    const uint32_t* words = reinterpret_cast<const uint32_t*>(s_mem + (i & 1) * buf_bytes);
+    const int y0 = cur.ty * a.tile_rows, rows = min(a.tile_rows, p.net_h - y0);
+    if (x < p.net_w) {
+      float* d = p.dst + (size_t)cur.img * 3 * plane + (size_t)(y0 + grp) * p.net_w + x;
+#pragma unroll 2
+      for (int r = grp; r < rows; r += GROUPS, d += GROUPS * p.net_w) {
+        const int4 e = s_row[i & 1][r];
+        float o0, o1, o2;
         uint32_t lo0, hi0;
-        fetch_pair(s_words, base0 + xoffs[j], lo0, hi0);
-        sample_row(lo0, hi0, fxs[j], scale, shift, o0[j], o1[j], o2[j]);
-      }
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        uint32_t lo0, hi0, lo1, hi1;
-        fetch_pair(s_words, base0 + xoffs[j], lo0, hi0);
-        fetch_pair(s_words, base1 + xoffs[j], lo1, hi1);
-        sample_rows(lo0, hi0, lo1, hi1, fxs[j], fy, scale, shift, o0[j], o1[j], o2[j]);
-      }
-    }
-    float* d0 = p.dst + (size_t)n * 3 * plane + (size_t)yo * p.net_w + xo0;
-    float* d1 = d0 + plane;
-    float* d2 = d1 + plane;
-    if (vec_ok) {
-      *reinterpret_cast<float4*>(d0) = make_float4(o0[0], o0[1], o0[2], o0[3]);
-      *reinterpret_cast<float4*>(d1) = make_float4(o1[0], o1[1], o1[2], o1[3]);
-      *reinterpret_cast<float4*>(d2) = make_float4(o2[0], o2[1], o2[2], o2[3]);
-    } else {
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        if (xo0 + j < p.net_w) {
-          d0[j] = o0[j];
-          d1[j] = o1[j];
-          d2[j] = o2[j];
+        fetch_pair(words, e.x + xo, lo0, hi0);
+        if (ONE_ROW) {
+          sample_row(lo0, hi0, fx, a.scale, a.shift, o0, o1, o2);
+        } else {
+          uint32_t lo1, hi1;
+          fetch_pair(words, e.y + xo, lo1, hi1);
+          sample_rows(lo0, hi0, lo1, hi1, fx, __int_as_float(e.z), a.scale, a.shift, o0, o1, o2);
         }
+        d[0] = o0;
+        d[plane] = o1;
+        d[2 * plane] = o2;
+      }
     }
+    __syncthreads();                                   // the buffer has been read
+    advance(cur);
   }
 }
 
+constexpr int DIR_TX = 32, DIR_TY = 8, DIR_OUT_W = DIR_TX * 4;   // threads of a block, 4 outputs each
+
 // Fallback for extreme down-scaling factors whose footprint does not fit in shared memory:
 // taps are read straight from global memory (L1-cached byte loads).
-__global__ void __launch_bounds__(PRE_THREADS) preprocess_direct_kernel(const __grid_constant__ PreprocessParams p, float scale, float shift) {
+__global__ void __launch_bounds__(DIR_TX * DIR_TY) preprocess_direct_kernel(const __grid_constant__ PreprocessParams p, float scale, float shift) {
   const int n = blockIdx.z;
   const uint8_t* __restrict__ src = p.src_tab ? p.src_tab[n] : p.src.p[n];
-  const int yo = blockIdx.y * PRE_TY + threadIdx.y;
-  const int xo0 = blockIdx.x * PRE_OUT_W + threadIdx.x * 4;
+  const int yo = blockIdx.y * DIR_TY + threadIdx.y;
+  const int xo0 = blockIdx.x * DIR_OUT_W + threadIdx.x * 4;
   if (yo >= p.net_h || xo0 >= p.net_w) return;
   const AxisSample sy = axis_sample(yo, p.src_h, p.net_h);
   const uint8_t* r0 = src + (size_t)sy.i0 * p.src_pitch;
@@ -161,24 +171,67 @@ __global__ void __launch_bounds__(PRE_THREADS) preprocess_direct_kernel(const __
   }
 }
 
+// Staged rows and bytes per row of a tile in the worst case: rows = ceil(tile_rows * sh/nh) + 2; bytes = 3 * (ceil(COLS * sw/nw) + 2) + 15
+// (alignment at the front) + 15 (at the end) + 12 (the tap fetch reads three whole words from its first byte), rounded up to 16.
+void staging(const PreprocessParams& p, int cols, int tile_rows, long* rows, long* row_cap) {
+  *rows = ((long)tile_rows * p.src_h + p.net_h - 1) / p.net_h + 2;
+  const long c = ((long)cols * p.src_w + p.net_w - 1) / p.net_w + 2;
+  *row_cap = ((3 * c + 48 + 15) / 16) * 16;
+}
+
+template <int COLS>
+cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits) {
+  constexpr int GROUPS = PRE_THREADS / COLS;
+  int sms = 0;
+  cudaError_t e = post_sm_count(&sms);
+  if (e != cudaSuccess) return e;
+  PreprocessArgs a;
+  a.p = p;
+  a.scale = pre::norm_scale(p.inv_div, p.inv_std);
+  a.shift = pre::norm_shift(p.mean, p.inv_std);
+  a.tiles_x = (p.net_w + COLS - 1) / COLS;
+  // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least.
+  const long slots = (long)PRE_PER_SM * sms;
+  long best = -1;
+  for (int rows = GROUPS; rows <= PRE_MAX_ROWS; rows += GROUPS) {
+    long cap_r, cap_b;
+    staging(p, COLS, rows, &cap_r, &cap_b);
+    if (cap_r * cap_b > PRE_STAGE_BYTES) break;
+    const long tiles = (long)p.K * a.tiles_x * ((p.net_h + rows - 1) / rows);
+    const long cost = (tiles + slots - 1) / slots * (rows + 2);
+    if (best >= 0 && cost >= best) continue;
+    best = cost;
+    a.tile_rows = rows;
+    a.rows_cap = (int)cap_r;
+    a.row_cap = (int)cap_b;
+  }
+  *fits = best >= 0;
+  if (!*fits) return cudaSuccess;
+  a.tiles_y = (p.net_h + a.tile_rows - 1) / a.tile_rows;
+  const long total = (long)p.K * a.tiles_x * a.tiles_y;
+  const int grid = (int)(total < slots ? total : slots);
+  a.tiles_per_block = (int)(total / grid);
+  a.tiles_left = (int)(total % grid);
+  const size_t smem = (size_t)2 * a.rows_cap * a.row_cap;
+  auto kern = p.src_h == p.net_h ? preprocess_staged_kernel<COLS, true> : preprocess_staged_kernel<COLS, false>;
+  if (smem > 48 * 1024) {
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * PRE_STAGE_BYTES);
+    if (e != cudaSuccess) return e;
+  }
+  kern<<<grid, PRE_THREADS, smem, s>>>(a);
+  return cudaGetLastError();
+}
+
 }  // namespace
 
 cudaError_t launch_preprocess(const PreprocessParams& p, cudaStream_t s) {
-  dim3 block(PRE_TX, PRE_TY);
-  const float scale = pre::norm_scale(p.inv_div, p.inv_std), shift = pre::norm_shift(p.mean, p.inv_std);
-  // Worst-case staged footprint of one block: rows = ceil(TY * sh/nh) + 2; bytes per row =
-  // 3 * (ceil(OUT_W * sw/nw) + 2) + 15 (alignment at the front) + 15 (at the end) + 12 (the tap
-  // fetch reads three whole words from its first byte), rounded up to 16.
-  const long rows = ((long)PRE_ROWS * p.src_h + p.net_h - 1) / p.net_h + 2;
-  const long cols = ((long)PRE_OUT_W * p.src_w + p.net_w - 1) / p.net_w + 2;
-  const long row_cap = ((3 * cols + 48 + 15) / 16) * 16;
-  if (rows * row_cap <= PRE_SMEM_BYTES) {
-    dim3 grid((p.net_w + PRE_OUT_W - 1) / PRE_OUT_W, (p.net_h + PRE_ROWS - 1) / PRE_ROWS, p.K);
-    preprocess_staged_kernel<<<grid, block, (size_t)(rows * row_cap), s>>>(p, (int)row_cap, scale, shift);
-  } else {
-    dim3 grid((p.net_w + PRE_OUT_W - 1) / PRE_OUT_W, (p.net_h + PRE_TY - 1) / PRE_TY, p.K);
-    preprocess_direct_kernel<<<grid, block, 0, s>>>(p, scale, shift);
-  }
+  bool fits = false;
+  // narrow tiles where the last wide one would be at most half full
+  const int over = p.net_w % 128;
+  cudaError_t e = over > 0 && over <= 64 ? launch_staged<64>(p, s, &fits) : launch_staged<128>(p, s, &fits);
+  if (e != cudaSuccess || fits) return e;
+  dim3 grid((p.net_w + DIR_OUT_W - 1) / DIR_OUT_W, (p.net_h + DIR_TY - 1) / DIR_TY, p.K);
+  preprocess_direct_kernel<<<grid, dim3(DIR_TX, DIR_TY), 0, s>>>(p, pre::norm_scale(p.inv_div, p.inv_std), pre::norm_shift(p.mean, p.inv_std));
   return cudaGetLastError();
 }
 

@@ -242,6 +242,7 @@ struct PostParams {
 size_t post_scratch_bytes(int K, int hm, int wm, int ch, int T);
 cudaError_t launch_postprocess(const PostParams& p, cudaStream_t s);
 cudaError_t post_prepare();
+cudaError_t post_sm_count(int* out);           // multiprocessors of the current device
 cudaError_t post_static_scratch(void** ptr);  // device address of the library's built-in scratch array
 
 // S4/S5 of the bf16 path on the tensor cores: reads the bf16 channels-last hidden state.

@@ -182,3 +182,24 @@ def test_convlstm_column_groups_change_no_bit(cuda_device, hidden, net):
     for other in runs[1:]:
         for a, b in zip(runs[0], other):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("src,net,pad,K", [
+    ((200, 150), (128, 64), 0, 1),       # one full tile column of 128
+    ((200, 150), (129, 65), 3, 2),       # a tile column of one output: narrow tiles
+    ((200, 150), (192, 90), 7, 3),       # half of the last wide tile: narrow tiles
+    ((200, 150), (193, 90), 1, 1),       # more than half: wide tiles
+    ((64, 40), (1, 1), 0, 8),
+    ((1600, 900), (160, 90), 2, 2),      # ten source rows and columns per output: few rows of a tile fit
+    ((2400, 1300), (40, 20), 0, 1),      # sixty: no tile fits, the kernel without staging
+    ((90, 700), (300, 700), 5, 2),       # height not resized
+])
+def test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, K):
+    """Bytes blended in fp32 by at most six roundings of values below 256, scaled to +-2: 2e-5 as in the stage tests."""
+    (sw, sh), (nw, nh) = src, net
+    frames = np.random.default_rng(5).integers(0, 256, (K, sh, sw, 3), dtype=np.uint8)
+    buf = np.full((K, sh, 3 * sw + pad), 201, np.uint8)
+    buf[:, :, :3 * sw] = frames.reshape(K, sh, 3 * sw)
+    out = binding.preprocess(torch.from_numpy(buf.reshape(K, -1)).to(cuda_device), sw, sh, 3 * sw + pad, nw, nh).cpu().numpy()
+    for k in range(K):
+        assert np.max(np.abs(out[k] - oracle.preprocess(frames[k], nw, nh))) < 2e-5
