@@ -14,7 +14,7 @@
 // warp 1 = tensor-memory allocation and MMA issue (one lane), warps 2..5 = epilogue, one thread per
 // pixel of the tile (tensor-memory lane = pixel).  Per tile every epilogue warp reduces its 32
 // pixels' statistics (mask count, sum x, sum y by integer warp reductions; probability or
-// confidence-head sums in a fixed shuffle order, then to fixed point); lane t keeps tool t's running
+// confidence-head sums in a fixed shuffle order, then to fixed point); lane 4 t keeps tool t's running
 // sums in registers.  When the block moves on to another stream or ends, the warps' sums meet in
 // shared memory and reach the per-stream accumulators in global memory through integer atomics;
 // the block that completes a stream forms its result record and zeroes the accumulators again.  Integer additions commute,
@@ -222,18 +222,19 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
       epi_bar();
     };
 
-    // Lane t < T of every epilogue warp carries tool t's running sums for the stream the block is
+    // Lane 4 t, t < T, of every epilogue warp carries tool t's running sums for the stream the block is
     // working on (mask count, sum x, sum y, and the fixed-point sum of probabilities or of the
     // confidence-head column); they meet in the block's shared accumulators only when the block
     // moves on to another stream or ends.
     long long r_cnt = 0, r_sx = 0, r_sy = 0, r_sum = 0;
     auto spill = [&]() {
-      if (lane < T) {
-        if (p.conf_mode == TT_CONF_MEAN_SIGMOID) atomicAdd(s_acc + 8 + lane * 4 + 3, (unsigned long long)r_sum);
-        else atomicAdd(s_acc + lane, (unsigned long long)r_sum);
-        atomicAdd(s_acc + 8 + lane * 4 + 0, (unsigned long long)r_cnt);
-        atomicAdd(s_acc + 8 + lane * 4 + 1, (unsigned long long)r_sx);
-        atomicAdd(s_acc + 8 + lane * 4 + 2, (unsigned long long)r_sy);
+      const int t = lane >> 2;
+      if ((lane & 3) == 0 && t < T) {
+        if (p.conf_mode == TT_CONF_MEAN_SIGMOID) atomicAdd(s_acc + 8 + t * 4 + 3, (unsigned long long)r_sum);
+        else atomicAdd(s_acc + t, (unsigned long long)r_sum);
+        atomicAdd(s_acc + 8 + t * 4 + 0, (unsigned long long)r_cnt);
+        atomicAdd(s_acc + 8 + t * 4 + 1, (unsigned long long)r_sx);
+        atomicAdd(s_acc + 8 + t * 4 + 2, (unsigned long long)r_sy);
       }
       r_cnt = r_sx = r_sy = r_sum = 0;
     };
@@ -266,36 +267,56 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
       const bool live = pix < plane;
       const int px = live ? pix % p.Wm : 0, py = live ? pix / p.Wm : 0;
       const size_t o0 = (size_t)n * T * plane + pix;     // tool t's element: + t * plane
+      // All eight tool slots take part (those behind T have zero weights and are masked out): without a branch per tool their
+      // votes and reductions overlap, where they had been eight chains one behind the other.
       uint32_t bits = 0;
+      float prob[TT_MAX_TOOLS];
 #pragma unroll
       for (int t = 0; t < TT_MAX_TOOLS; ++t) {
-        if (t < T) {
-          const float z = __uint_as_float(v[t]) + bias[t];
-          const float pr = sigmoid_fast(z);
-          const bool m = live && (z > p.zthr);
-          if (live) {
-            const size_t o = o0 + (size_t)t * plane;
-            p.logits[o] = z;
-            p.probs[o] = pr;
-            p.masks[o] = m ? 1 : 0;
-          }
-          bits |= (m ? 1u : 0u) << t;
-          const int c1 = __popc(__ballot_sync(0xffffffffu, m));
-          const int x1 = __reduce_add_sync(0xffffffffu, m ? px : 0);
-          const int y1 = __reduce_add_sync(0xffffffffu, m ? py : 0);
-          long long s1;
-          if (p.conf_mode == TT_CONF_MEAN_SIGMOID) {
-            // probabilities in units of 2^-26: 32 of them fit an unsigned 32-bit sum
-            s1 = (long long)__reduce_add_sync(0xffffffffu, live ? __float2uint_rn(pr * 67108864.0f) : 0u) << 4;
-          } else {
-            // this pixel's share of the confidence head; rows past the image end were zero-filled
-            float g = live ? __uint_as_float(v[8 + t]) : 0.0f;
-#pragma unroll
-            for (int d = 16; d > 0; d >>= 1) g += __shfl_xor_sync(0xffffffffu, g, d);
-            s1 = __float2ll_rn(g * PT_FIX_SCALE);
-          }
-          if (lane == t) { r_cnt += c1; r_sx += x1; r_sy += y1; r_sum += s1; }
+        const float z = __uint_as_float(v[t]) + bias[t];
+        const bool store = live && t < T, m = store && z > p.zthr;
+        prob[t] = sigmoid_fast(z);
+        if (store) {
+          const size_t o = o0 + (size_t)t * plane;
+          p.logits[o] = z;
+          p.probs[o] = prob[t];
+          p.masks[o] = m ? 1 : 0;
         }
+        bits |= (m ? 1u : 0u) << t;
+      }
+#pragma unroll
+      for (int t = 0; t < TT_MAX_TOOLS; ++t) {
+        const bool m = (bits >> t) & 1u;
+        const int c1 = __popc(__ballot_sync(0xffffffffu, m));
+        const int x1 = __reduce_add_sync(0xffffffffu, m ? px : 0);
+        const int y1 = __reduce_add_sync(0xffffffffu, m ? py : 0);
+        if (lane == 4 * t) { r_cnt += c1; r_sx += x1; r_sy += y1; }
+      }
+      if (p.conf_mode == TT_CONF_MEAN_SIGMOID) {
+#pragma unroll
+        for (int t = 0; t < TT_MAX_TOOLS; ++t) {
+          // probabilities in units of 2^-26: 32 of them fit an unsigned 32-bit sum
+          const uint32_t s1 = __reduce_add_sync(0xffffffffu, live ? __float2uint_rn(prob[t] * 67108864.0f) : 0u);
+          if (lane == 4 * t) r_sum += (long long)s1 << 4;
+        }
+      } else {
+        // this pixel's share of the confidence head (rows past the image end were zero-filled), summed over the warp: three rounds in
+        // which a lane hands on half of its tools, two of one value; lane l ends up with tool l / 4
+        float g[TT_MAX_TOOLS];
+#pragma unroll
+        for (int t = 0; t < TT_MAX_TOOLS; ++t) g[t] = live ? __uint_as_float(v[8 + t]) : 0.0f;
+#pragma unroll
+        for (int d = 16, half = 4; half >= 1; d >>= 1, half >>= 1) {
+          const bool upper = (lane & d) != 0;
+#pragma unroll
+          for (int j = 0; j < half; ++j) {
+            const float send = upper ? g[j] : g[j + half], keep = upper ? g[j + half] : g[j];
+            g[j] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+          }
+        }
+        g[0] += __shfl_xor_sync(0xffffffffu, g[0], 2);
+        g[0] += __shfl_xor_sync(0xffffffffu, g[0], 1);
+        r_sum += __float2ll_rn(g[0] * PT_FIX_SCALE);   // of lanes 4 t
       }
       if (p.bits && live) p.bits[(size_t)n * plane + pix] = (uint8_t)bits;
       tiles_done += 1;
