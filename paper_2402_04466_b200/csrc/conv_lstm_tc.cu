@@ -1,22 +1,31 @@
-// ConvLSTM step of the bf16 path on the tensor cores, 64-channel slabs, for launches whose units of 256 columns would leave
-// a good part of the last round of multiprocessors idle: the 3x3 convolution over [x, h] into i/f/g/o gates as an
+// ConvLSTM step of the bf16 path on the tensor cores, 64-channel slabs: the 3x3 convolution over [x, h] into i/f/g/o gates as an
 // implicit GEMM (M = output pixels, N = 4 x hidden, K = 9 taps x channels), gate math, c' and h' in the epilogue.
 //
-// Tiles and operands are those of the haloed form in conv_tc.cu (8 x 16 output pixels; one haloed patch of 18 x 10 pixels
-// per 64-channel slab, which the nine taps read in place; weights one tap and slab at a time through a ring of five stages,
-// the first fetched before the wait for the previous kernel), and the order of the sums is the same, so the results
-// are the same bits.
+// The output tile is an 8 x 16-pixel patch.  Per 64-channel slab ONE haloed patch (18 rows of 10 pixels, a 4-D TMA box in the ordinary
+// 128-byte swizzle) is fetched, and the nine taps read it in place: output pixel (py, px) of tap (ky, kx) is patch row
+// (py + ky) * 10 + px + kx, so a tap's A operand is the same shared memory entered (ky * 10 + kx) * 128 bytes further on, its groups of 8
+// rows 1280 bytes apart.  The swizzle is a function of the shared-memory address, so a start in the middle of its pattern needs
+// nothing but the address.  Weights come one tap and slab at a time through a ring, the first before the wait for the previous kernel.
 //
-// Bound by rounds: a multiprocessor holds one block, and 80 units of 256 columns (one 854x480 stream) take as long as 148.  A unit
-// here is a tile x a group of columns, grouped as the launch needs: by 192 (with a remainder of 64 or 128) where that
+// Bound by the tensor pipe where the rounds of units are full, and there by the clock that the power limit leaves; the bytes that travel from
+// L2 into the multiprocessors cost part of that power.  So beyond one round two blocks of a cluster work as a pair: one MMA of 256 rows
+// (cta_group::2) takes both blocks' tiles and half of the weight rows from each, 18.6 instead of 34.6 KB into a multiprocessor per 512
+// tensor cycles.  1.087 PFLOP of eight full-HD streams: 670 us on single blocks (1.62 PFLOP/s) -> 633 us (1.72 PFLOP/s), tick 1135 -> 1075 us;
+// one full-HD stream's tick 179 -> 170 us, five 854x480 streams' 115.3 -> 114.5 us.  One commit that signals both blocks, and the issue loop
+// below, make the difference to an earlier pair form (conv_tc.cu's, kept as an option) that was 11-15 % slower than single blocks.
+//
+// Bound by rounds where they are not full: a multiprocessor holds one block, and 80 units of 256 columns (one 854x480 stream) take as long as
+// 148.  A unit is a tile (or a pair's two) x a group of columns, grouped as the launch needs: by 192 (with a remainder of 64 or 128) where that
 // still fits the rounds, or by 256 with the last, partly filled round cut into halves.  M128 x N x K16 takes 128, 96 and 64
 // cycles at N = 256, 192 and 128; for a narrow group's slab to take less than a wide one's, the whole MMA warp
 // runs the issue loop and one elected lane issues (from a single lane's branch a slab takes about 600 cycles at any width).
 // ConvLSTM stage with its event, units of 256 -> this: one 854x480 stream 23.6 -> 20.5 us, one full-HD stream 105.5 -> 101.4 us.
+// The order of the sums is the same in all forms, so the results are the same bits.
 //
 // Warp roles (384 threads): 0 = patches by TMA; 10, 11 = weights by TMA, alternate iterations; 1 = tensor memory and MMA
-// issue; 2..9 = epilogue (TMEM lane quarter = warp mod 4, two warps per quarter sharing a unit's columns).  Two accumulators,
-// so the epilogue of a unit overlaps the next one's products.  All waits are bounded (see tc_ptx.cuh).
+// issue (of a pair: its first block's); 2..9 = epilogue (TMEM lane quarter = warp mod 4, two warps per quarter sharing a unit's columns).
+// Two accumulators, so the epilogue of a unit overlaps the next one's products.  A pair's copies complete on its first block's barriers, which
+// expect both blocks' bytes; "free" barriers are signalled in both blocks.  All waits are bounded (see tc_ptx.cuh).
 #include <algorithm>
 
 #include "tt_internal.h"
@@ -34,11 +43,18 @@ constexpr int L_PITCH = 10, L_ROWS = 18;                 // haloed patch
 constexpr int L_A_TX = L_ROWS * L_PITCH * 128;
 constexpr int L_A_BYTES = (L_A_TX + 1023) / 1024 * 1024;
 constexpr int L_A_STAGES = 2;
-constexpr int L_B_BYTES = 256 * 128;                     // widest group: 256 rows of 64 channels
-constexpr int L_B_STAGES = 5;
 constexpr int L_MAX_COLS = 4 * 512;
-constexpr int L_SMEM = L_B_STAGES * L_B_BYTES + L_A_STAGES * L_A_BYTES + L_MAX_COLS * 4 + 256 + 1024 /*alignment slack*/;
-static_assert(L_SMEM <= 227 * 1024, "one block per multiprocessor");
+
+template <bool PAIR>
+struct LCfg {
+  static constexpr int B_BYTES = (PAIR ? 128 : 256) * 128;   // a block's rows of the widest group, 64 channels each
+  static constexpr int B_STAGES = PAIR ? 10 : 5;
+  static constexpr int B_STEP = PAIR ? 32 : 64;              // rows of the small weight box
+  static constexpr int BAR_BYTES = 256;
+  static constexpr int SMEM = B_STAGES * B_BYTES + L_A_STAGES * L_A_BYTES + L_MAX_COLS * 4 + BAR_BYTES + 1024 /*alignment slack*/;
+  static_assert(SMEM <= 227 * 1024, "one block per multiprocessor");
+  static_assert((2 * B_STAGES + 8) * 8 + 8 <= BAR_BYTES, "barriers");
+};
 
 struct Unit {
   int m, col0, n;   // pixel tile, first column, columns
@@ -57,7 +73,11 @@ __device__ __forceinline__ Unit unit_at(const ConvLstmParams& p, int u) {
   return t;
 }
 
+template <bool PAIR>
 __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_constant__ ConvLstmParams p) {
+  using Cfg = LCfg<PAIR>;
+  constexpr int L_B_STAGES = Cfg::B_STAGES, L_B_BYTES = Cfg::B_BYTES;
+  constexpr int CTAS = PAIR ? 2 : 1;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* s_b = reinterpret_cast<uint8_t*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
   uint8_t* s_a = s_b + L_B_STAGES * L_B_BYTES;
@@ -75,7 +95,9 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
   // broadcast, so that the compiler knows the roles below to be whole warps
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
   const long long wait_limit = p.wait_limit;
-  const int total = p.u_full + 2 * (p.tiles * p.groups - p.u_full);
+  const int rank = PAIR ? (int)cluster_ctarank() : 0;
+  const int worker = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x, n_workers = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
+  const int total = p.u_full + 2 * (p.m_units * p.groups - p.u_full);
   const int slabs = p.slabs[0] + p.slabs[1];
   if (threadIdx.x == 0) {
     for (int s = 0; s < L_B_STAGES; ++s) {
@@ -86,18 +108,23 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       mbar_init(smem_u32(afull + a), 1);
       mbar_init(smem_u32(aempty + a), 1);
       mbar_init(smem_u32(tfull + a), 1);
-      mbar_init(smem_u32(tempty + a), L_EPI_WARPS);
+      mbar_init(smem_u32(tempty + a), CTAS * L_EPI_WARPS);
     }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b) : "memory");
-    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_b64) : "memory");
+    asm volatile("prefetch.tensormap [%0];" ::"l"(&p.map_bs) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&p.maps[0]) : "memory");
     asm volatile("prefetch.tensormap [%0];" ::"l"(&p.maps[1]) : "memory");
   }
   if (warp == 1) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
-    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    if (PAIR) {   // the same warp of both blocks allocates the pair's columns
+      asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    } else {
+      asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(512u) : "memory");
+      asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
   }
   for (int i = threadIdx.x; i < p.cols; i += L_THREADS) s_bias[i] = __ldg(p.bias + i);
   if (threadIdx.x < TT_MAX_STREAMS) {
@@ -107,6 +134,7 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
   }
   tc_fence_before();
   __syncthreads();
+  if (PAIR) cluster_sync_all();   // the peer's barriers exist before anything is signalled across the pair
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
   pdl_launch_dependents();   // behind the allocation: a dependent block must not take tensor memory that this grid still needs
@@ -117,17 +145,19 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
     pdl_wait();   // x is the previous kernel's output
     uint32_t stage = 0, phase = 0;
     bool ok = true;
-    for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
-      const int m = unit_at(p, u).m;
+    for (int u = worker; u < total && ok; u += n_workers) {
+      // a pair's second block takes the next tile; behind the last tile it computes that one again and stores nothing
+      const int m = min(CTAS * unit_at(p, u).m + rank, p.tiles - 1);
       const int img = m / tiles_per_img, rem = m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
       const int img_h = s_img[0][img];
       for (int sg = 0; sg < slabs; ++sg) {
         ok = mbar_wait(smem_u32(aempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x10 + (int)stage, wait_limit);
         if (!ok) break;
         const int src = sg < p.slabs[0] ? 0 : 1;
-        mbar_arrive_expect_tx(smem_u32(afull + stage), L_A_TX);
-        tma_load_4d(smem_u32(s_a + stage * L_A_BYTES), &p.maps[src], smem_u32(afull + stage), (src ? sg - p.slabs[0] : sg) * 64,
-                    tx * L_PW - 1, ty * L_PH - 1, src ? img_h : img);
+        const int c0 = (src ? sg - p.slabs[0] : sg) * 64, n_img = src ? img_h : img;
+        if (rank == 0) mbar_arrive_expect_tx(smem_u32(afull + stage), CTAS * L_A_TX);
+        if (PAIR) tma_load_4d_pair(smem_u32(s_a + stage * L_A_BYTES), &p.maps[src], map_to_cta(smem_u32(afull + stage), 0u), c0, tx * L_PW - 1, ty * L_PH - 1, n_img);
+        else tma_load_4d(smem_u32(s_a + stage * L_A_BYTES), &p.maps[src], smem_u32(afull + stage), c0, tx * L_PW - 1, ty * L_PH - 1, n_img);
         if (++stage == L_A_STAGES) { stage = 0; phase ^= 1u; }
       }
     }
@@ -139,36 +169,47 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
     uint32_t stage = (uint32_t)j, phase = 0;
     int it = j;
     bool ok = true;
-    for (int u = blockIdx.x; u < total && ok; u += gridDim.x) {
+    for (int u = worker; u < total && ok; u += n_workers) {
       const Unit t = unit_at(p, u);
       for (; it < iters; it += 2) {
         const int sg = it / 9, tap = it - sg * 9;
         ok = mbar_wait(smem_u32(bempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + (int)stage, wait_limit);
         if (!ok) break;
         const uint32_t bar = smem_u32(bfull + stage), dst = smem_u32(s_b + stage * L_B_BYTES);
-        const int k0 = tap * cin + sg * 64;
-        mbar_arrive_expect_tx(bar, (uint32_t)t.n * 128u);
-        if (t.n == 256) {
-          tma_load_2d(dst, &p.map_b, bar, k0, t.col0);
+        const int k0 = tap * cin + sg * 64, rows = t.n / CTAS, r0 = t.col0 + rank * rows;
+        if (rank == 0) mbar_arrive_expect_tx(bar, (uint32_t)t.n * 128u);
+        if (PAIR) {
+          const uint32_t bar0 = map_to_cta(bar, 0u);
+          if (t.n == 256) {
+            tma_load_2d_pair(dst, &p.map_b, bar0, k0, r0);
+          } else {
+            for (int i = 0; i < rows; i += Cfg::B_STEP) tma_load_2d_pair(dst + i * 128, &p.map_bs, bar0, k0, r0 + i);
+          }
+        } else if (t.n == 256) {
+          tma_load_2d(dst, &p.map_b, bar, k0, r0);
         } else {
-          for (int i = 0; i < t.n; i += 64) tma_load_2d(dst + i * 128, &p.map_b64, bar, k0, t.col0 + i);
+          for (int i = 0; i < rows; i += Cfg::B_STEP) tma_load_2d(dst + i * 128, &p.map_bs, bar, k0, r0 + i);
         }
         stage += 2;
         if (stage >= (uint32_t)L_B_STAGES) { stage -= L_B_STAGES; phase ^= 1u; }
       }
       it -= iters;
     }
-  } else if (warp == 1) {
-    // -------------------------------------------------------------------- MMA issuer
+  } else if (warp == 1 && rank == 0) {
+    // -------------------------------------------------------------------- MMA issuer (of a pair: its first block)
     const bool issuer = elect_one();
+    auto commit = [](uint64_t* bar) {
+      if (PAIR) umma_commit_both(smem_u32(bar));
+      else umma_commit(smem_u32(bar));
+    };
     uint32_t stage = 0, phase = 0, acc_phase = 0, a_stage = 0, a_phase = 0;
     int acc = 0;
     bool ok = true;   // a wait that ran out ends the loop at the end of its unit
     const uint64_t b_desc0 = make_smem_desc(smem_u32(s_b), 1024u, 2u);
-    for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    for (int u = worker; u < total; u += n_workers) {
       // (no division in this loop where all groups are as wide)
       const int n = p.even ? (u < p.u_full ? p.width : p.width >> 1) : unit_at(p, u).n;
-      const uint32_t idesc = make_idesc(128, 0) | ((uint32_t)(n >> 3) << 17);
+      const uint32_t idesc = make_idesc(128 * CTAS, 0) | ((uint32_t)(n >> 3) << 17);
       ok &= mbar_wait_uniform(smem_u32(tempty + acc), acc_phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x30 + acc, wait_limit);
       tc_fence_after();   // the epilogue's reads of this accumulator come before the MMAs that overwrite it
       const uint32_t d_tmem = tmem_base + (uint32_t)(acc * 256);
@@ -182,17 +223,20 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
           const uint64_t b = b_desc0 + (uint64_t)stage * (uint64_t)(L_B_BYTES >> 4);
           if (issuer) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k)   // 16 bf16 = 32 bytes = 2 descriptor units further on inside the swizzle atom
-              umma_bf16(d_tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, (tap == 0 && k == 0) ? (sg != 0 ? 1u : 0u) : 1u);
-            umma_commit(smem_u32(bempty + stage));
-            if (tap == 8) umma_commit(smem_u32(aempty + a_stage));
+            for (int k = 0; k < 4; ++k) {  // 16 bf16 = 32 bytes = 2 descriptor units further on inside the swizzle atom
+              const uint32_t more = (tap == 0 && k == 0) ? (sg != 0 ? 1u : 0u) : 1u;
+              if (PAIR) umma_bf16_pair(d_tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, more);
+              else umma_bf16(d_tmem, a + (uint64_t)(2 * k), b + (uint64_t)(2 * k), idesc, more);
+            }
+            commit(bempty + stage);
+            if (tap == 8) commit(aempty + a_stage);
           }
           if (++stage == L_B_STAGES) { stage = 0; phase ^= 1u; }
         }
         if (++a_stage == L_A_STAGES) { a_stage = 0; a_phase ^= 1u; }
       }
       if (__any_sync(0xffffffffu, !ok)) break;
-      if (issuer) umma_commit(smem_u32(tfull + acc));
+      if (issuer) commit(tfull + acc);
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
   } else if (warp >= L_EPI_WARP0 && warp < L_EPI_WARP0 + L_EPI_WARPS) {
@@ -202,11 +246,12 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
     const int row = quarter * 32 + lane, py = row >> 3, px = row & 7;     // row of the 128-row tile = pixel of the patch
     uint32_t acc_phase = 0;
     int acc = 0;
-    for (int u = blockIdx.x; u < total; u += gridDim.x) {
+    for (int u = worker; u < total; u += n_workers) {
       const Unit t = unit_at(p, u);
-      const int img = t.m / tiles_per_img, rem = t.m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
+      const int m_own = CTAS * t.m + rank, m = min(m_own, p.tiles - 1);
+      const int img = m / tiles_per_img, rem = m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
       const int x = tx * L_PW + px, y = ty * L_PH + py;
-      const bool valid = x < p.Wm && y < p.Hm;
+      const bool valid = x < p.Wm && y < p.Hm && m_own < p.tiles;
       const size_t pix = (size_t)y * p.Wm + x;
       // chunks of 32 columns (8 hidden units x 4 gates): the first of the quarter's two warps takes 128 columns of a wide
       // group and half of a narrow one, so that every pair of chunks starts on 32 bytes of h'
@@ -263,7 +308,10 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       // hand the accumulator back to the MMA warp
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(tempty + acc));
+      if (lane == 0) {
+        if (PAIR) mbar_arrive_cluster(map_to_cta(smem_u32(tempty + acc), 0u));
+        else mbar_arrive(smem_u32(tempty + acc));
+      }
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
     }
   }
@@ -276,9 +324,12 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
   }
   tc_fence_before();
   __syncthreads();
+  // neither block of a pair may go while the other can still signal its barriers or have its shared memory read by the pair's MMAs
+  if (PAIR) cluster_sync_all();
   if (warp == 1) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    if (PAIR) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
+    else asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
 }
 
@@ -289,50 +340,54 @@ constexpr double L_COST_256 = 1.0, L_COST_192 = 0.77, L_COST_128 = 0.58;
 
 struct Grouping {
   int width = 256, u_full = 0;
-  double cost = 0, plain = 0;   // rounds x time of a unit, as chosen and with groups of 256 throughout
 };
-// C: a multiple of 256
-Grouping group_columns(int tiles, int C, int sm_count) {
+// m_units: tiles (or pairs of tiles) to be shared out over `workers` blocks (or pairs); C: a multiple of 256
+Grouping group_columns(int m_units, int C, int workers) {
   Grouping g;
-  auto rounds = [&](long units) { return (double)((units + sm_count - 1) / sm_count); };
-  const long g256 = (long)tiles * (C / 256);
+  auto rounds = [&](long units) { return (double)((units + workers - 1) / workers); };
+  const long g256 = (long)m_units * (C / 256);
   g.u_full = (int)g256;
-  g.cost = g.plain = rounds(g256) * L_COST_256;
+  double cost = rounds(g256) * L_COST_256;
   // the last round cut into halves, if that leaves it one round
-  const long tail = g256 % sm_count;
-  if (tail > 0 && 2 * tail <= sm_count) {
-    g.cost = (double)(g256 / sm_count) * L_COST_256 + L_COST_128;
+  const long tail = g256 % workers;
+  if (tail > 0 && 2 * tail <= workers) {
+    cost = (double)(g256 / workers) * L_COST_256 + L_COST_128;
     g.u_full = (int)(g256 - tail);
   }
-  const long units = (long)tiles * ((C + 191) / 192);
-  const double t = rounds(units) * L_COST_192;
-  if (t < g.cost - 1e-9) { g.cost = t; g.width = 192; g.u_full = (int)units; }
+  const long units = (long)m_units * ((C + 191) / 192);
+  if (rounds(units) * L_COST_192 < cost - 1e-9) { g.width = 192; g.u_full = (int)units; }
   return g;
+}
+
+template <bool PAIR>
+cudaError_t launch_form(const ConvLstmParams& p, const TensorMap128& whole, const TensorMap128& step, int workers, cudaStream_t s) {
+  constexpr int CTAS = PAIR ? 2 : 1;
+  auto kern = conv_lstm_kernel<PAIR>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LCfg<PAIR>::SMEM);
+  if (e != cudaSuccess) return e;
+  ConvLstmParams q = p;
+  q.map_b = whole;
+  q.map_bs = step;
+  q.m_units = (q.tiles + CTAS - 1) / CTAS;
+  const Grouping g = group_columns(q.m_units, q.cols, workers);
+  q.width = g.width;
+  q.u_full = g.u_full;
+  q.groups = (q.cols + q.width - 1) / q.width;
+  q.even = q.cols % q.width == 0;
+  const long total = q.u_full + 2L * ((long)q.m_units * q.groups - q.u_full);
+  return launch_kernel(kern, CTAS * (int)std::min<long>(total, workers), L_THREADS, LCfg<PAIR>::SMEM, s, q, q.pdl != 0, CTAS);
 }
 
 }  // namespace
 
-// Five per cent of the estimated time at least: 23 % for one 854x480 stream (80 units of 256 on 148 multiprocessors -> 120 of up
-// to 192), 10 % for one full-HD stream (480 -> 444 and 72 halves).  Where the rounds are full (eight full-HD streams)
-// conv_tc.cu's form is 2 % faster.
-bool conv_lstm_pays(int tiles, int cols, int sm_count) {
-  if (cols % 256 || cols > L_MAX_COLS) return false;
-  const Grouping g = group_columns(tiles, cols, sm_count);
-  return g.cost < 0.95 * g.plain;
-}
-
-cudaError_t launch_conv_lstm(const ConvLstmParams& p, int sm_count, cudaStream_t s) {
-  cudaError_t e = cudaFuncSetAttribute(conv_lstm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, L_SMEM);
-  if (e != cudaSuccess) return e;
+// Pairs where the units of one tile take more than one round.  ConvLSTM stage with its event, single blocks -> pairs (us): one, two, five and eight
+// full-HD streams 100.5 -> 94.2, 172 -> 162, 430 -> 397, 686 -> 633; four, six and eight 854x480 streams 45.1 -> 43.0, 57.3 -> 55.3, 71.1 -> 67.6,
+// two and three (1.1 and 1.6 rounds) the same.  Within one round copies are not what a block waits for, and the pair's start and
+// hand-overs show: one 854x480 stream 65.1 -> 65.3 us a tick.
+cudaError_t launch_conv_lstm(const ConvLstmParams& p, const TensorMap128 (&rows)[4], int sm_count, cudaStream_t s) {
   if (p.cols < 256 || p.cols % 256 || p.cols > L_MAX_COLS) return cudaErrorInvalidValue;
-  ConvLstmParams q = p;
-  const Grouping g = group_columns(p.tiles, p.cols, sm_count);
-  q.width = g.width;
-  q.u_full = g.u_full;
-  q.groups = (p.cols + q.width - 1) / q.width;
-  q.even = p.cols % q.width == 0;
-  const long total = q.u_full + 2L * ((long)q.tiles * q.groups - q.u_full);
-  return launch_kernel(conv_lstm_kernel, (int)std::min<long>(total, sm_count), L_THREADS, L_SMEM, s, q, p.pdl != 0);
+  if ((long)p.tiles * (p.cols / 256) > sm_count && sm_count >= 2) return launch_form<true>(p, rows[1], rows[3], sm_count / 2, s);
+  return launch_form<false>(p, rows[0], rows[2], sm_count, s);
 }
 
 }  // namespace tt

@@ -187,6 +187,11 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(map_to_cta(bar, 1u)) : "memory");
 }
 
+// the same with one commit that signals both blocks of the pair
+__device__ __forceinline__ void umma_commit_both(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3) : "memory");
+}
+
 // Named barrier over `count` threads that also ORs a flag across them: every participant learns
 // whether any of them wants to stop, so a group of warps leaves a loop together and nobody is
 // left waiting at the barrier for a warp that has gone.

@@ -47,6 +47,7 @@ struct TcLayer {
   bool has_halo = false;
   TensorMap128 map_b[3];       // block_n = 64, 128, 256
   bool has_b[3] = {false, false, false};
+  TensorMap128 map_b32;        // the ConvLSTM's: boxes of 32 rows
   ConvS2Params s2{};           // stride-2 layers that conv_s2 covers (s2.n_tiles_n > 0)
 };
 
@@ -382,6 +383,13 @@ tt_status pack_tc(tt_ctx* ctx, TcLayer* L, const float* w, const float* b, int c
   L->w = reinterpret_cast<__nv_bfloat16*>(dw);
   st = upload(ctx, &L->b, hb);
   if (st != TT_OK) return st;
+  if (lstm_hidden) {
+    const cuuint64_t dims[2] = {(cuuint64_t)ktot, (cuuint64_t)cout};
+    const cuuint64_t str[1] = {(cuuint64_t)ktot * 2};
+    const cuuint32_t box[2] = {(cuuint32_t)L->slab_c, 32};
+    st = encode_map(ctx, &L->map_b32, L->w, 2, dims, str, box, L->slab_c * 2);
+    if (st != TT_OK) return st;
+  }
   const int bns[3] = {64, 128, 256};
   for (int i = 0; i < 3; ++i) {
     L->has_b[i] = (cout % bns[i] == 0) && !(L->slab_c == 32 && bns[i] == 256);
@@ -843,12 +851,6 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       q.pair = (bi == 2 && L.slab_c == 64 && L.has_b[1] && ctx->cta_pairs && K * q.tiles_x * q.tiles_y >= 2) ? 1 : 0;
       if (q.pair) q.map_b = L.map_b[1];
       q.two_per_sm = (encoder && ctx->enc_two_per_sm) ? 1 : 0;
-      if (!encoder && L.has_halo && !q.pair && (bi == 2 || bi == 1)) {
-        q.halo = 1;
-        q.maps_halo[0] = L.maps_halo[0];
-        q.maps_halo[1] = L.maps_halo[1];
-        q.tiles_x = (Wo + 7) / 8; q.tiles_y = (Ho + 15) / 16;
-      }
       q.cout = L.cout; q.bias = L.b; q.status = ctx->status_dev; q.wait_limit = ctx->wait_limit;
       q.n_prod = 3;
       q.pdl = ctx->profiling ? 0 : 1;
@@ -880,17 +882,16 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     ConvTcParams q{};
     tt_status st = fill_common(q, L, ctx->Hm, ctx->Wm, false);
     if (st != TT_OK) return st;
-    // both kernels add up the same products in the same order: which one runs changes no bit
-    if (q.halo && conv_lstm_pays(K * q.tiles_x * q.tiles_y, L.cout, ctx->sm_count)) {
+    if (L.has_halo && !q.pair) {
       ConvLstmParams w{};
       w.maps[0] = L.maps_halo[0]; w.maps[1] = L.maps_halo[1];
-      w.map_b = L.map_b[2]; w.map_b64 = L.map_b[0];
       w.slabs[0] = L.cin0 / 64; w.slabs[1] = L.cin1 / 64; w.cols = L.cout; w.hidden = ctx->Ch;
-      w.tiles_x = q.tiles_x; w.tiles_y = q.tiles_y; w.tiles = K * q.tiles_x * q.tiles_y;
+      w.tiles_x = (ctx->Wm + 7) / 8; w.tiles_y = (ctx->Hm + 15) / 16; w.tiles = K * w.tiles_x * w.tiles_y;
       w.Hm = ctx->Hm; w.Wm = ctx->Wm; w.h_in = h_in; w.c_idx = c_idx; w.h_out = h_out;
       w.bias = L.b; w.c_state = ctx->c_state; w.h_f32 = ctx->use_post_tc ? nullptr : ctx->h_f32; w.h_bf16 = ctx->h_bf16;
       w.status = ctx->status_dev; w.wait_limit = ctx->wait_limit; w.pdl = q.pdl;
-      TT_CUDA(ctx, launch_conv_lstm(w, ctx->sm_count, s));
+      const TensorMap128 rows[4] = {L.map_b[2], L.map_b[1], L.map_b[0], L.map_b32};
+      TT_CUDA(ctx, launch_conv_lstm(w, rows, ctx->sm_count, s));
     } else {
       q.n_src = 2; q.slabs[0] = L.cin0 / L.slab_c; q.slabs[1] = L.cin1 / L.slab_c; q.img0 = ident; q.img1 = h_in;
       // with the heads on the tensor cores nothing on the path reads an fp32 copy of h': its consumers (the next

@@ -19,17 +19,26 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 
 template <typename Params>
 inline cudaError_t launch_kernel(void (*kern)(const Params), dim3 grid, int block, size_t smem, cudaStream_t s, const Params& p,
-                                 bool pdl) {
+                                 bool pdl, int cluster = 1) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchAttribute attr[2];
+  int n = 0;
+  if (pdl) {
+    attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[n].id = cudaLaunchAttributeClusterDimension;
+    attr[n].val.clusterDim.x = (unsigned)cluster;
+    attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+    ++n;
+  }
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 1 : 0;
+  cfg.numAttrs = (unsigned)n;
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
@@ -134,7 +143,6 @@ struct ConvTcParams {
   // A operand sources: up to two NHWC bf16 tensors (x then h); for stride 2 four parity
   // views of the single source.  maps_a[src*4 + parity] with parity = (ypar*2 + xpar).
   TensorMap128 maps_a[8];
-  TensorMap128 maps_halo[2];// halo mode: the two sources again with a box of [64 channels][10][18][1] (haloed patch of an 8 x 16 tile)
   TensorMap128 map_b;       // packed weights [CoutPacked][Ktot] bf16, K-major
   int32_t n_src;            // 1 or 2
   int32_t slabs[2];         // channel slabs (of slab_c channels) per source
@@ -149,7 +157,6 @@ struct ConvTcParams {
   int32_t n_prod;           // producer warps that issue loads, 1..3
   int32_t two_per_sm;       // encoder layers with tiles up to 128 wide: two blocks per multiprocessor, half the ring each
   int32_t wres;             // two_per_sm layer of 64 outputs and 32-channel slabs whose weights fit in 40 KB: fetched once per block
-  int32_t halo;             // stride-1 layer of 64-channel slabs: one haloed patch per channel slab, 8 x 16 output patches
   int32_t pair;             // run as CTA pairs (cta_group::2): block_n 256, map_b's box then holds 128 rows
   int32_t pdl;              // launch as a programmatic dependent of the previous kernel in the stream
   int32_t cout;             // real output channels (RELU) or 4*hidden (LSTM)
@@ -191,13 +198,13 @@ cudaError_t launch_conv_s2(const ConvS2Params& p, int sm_count, cudaStream_t s);
 // ConvLSTM step on 64-channel slabs (x and h both multiples of 64 channels).
 struct ConvLstmParams {
   TensorMap128 maps[2];     // x [K][Hm][Wm][Cx] and h [slots*2][Hm][Wm][Ch], box [64][10][18][1] (haloed patch of an 8 x 16 tile)
-  TensorMap128 map_b;       // packed weights [4*hidden][9*(Cx+Ch)] bf16, K-major, box [64][256]
-  TensorMap128 map_b64;     // the same, box [64][64]
+  TensorMap128 map_b;       // packed weights [4*hidden][9*(Cx+Ch)] bf16, K-major; set by the launch: box of a whole group's rows ...
+  TensorMap128 map_bs;      // ... and of a step of rows that every narrower group is a multiple of
   int32_t slabs[2];         // 64-channel slabs of x and h
   int32_t cols, hidden;     // 4 * hidden columns, a multiple of 256
   int32_t tiles, tiles_x, tiles_y, Hm, Wm;   // tiles = images x tiles_x x tiles_y
   IdxMap h_in, c_idx, h_out;                 // image of h, slot of c, image of h' per batch position
-  int32_t width, groups, even, u_full;       // set by the launch: column groups, whether all are as wide, the unit from which they are cut in two
+  int32_t m_units, width, groups, even, u_full;   // set by the launch: tiles or pairs of tiles, column groups, whether all are as wide, the unit from which they are cut in two
   int32_t pdl;
   const float* bias;        // packed order
   float* c_state;           // [slots][Hm][Wm][Ch] in place
@@ -206,9 +213,8 @@ struct ConvLstmParams {
   int32_t* status;
   long long wait_limit;
 };
-// whether grouping the columns otherwise than by 256 saves time on this many multiprocessors
-bool conv_lstm_pays(int tiles, int cols, int sm_count);
-cudaError_t launch_conv_lstm(const ConvLstmParams& p, int sm_count, cudaStream_t s);
+// `rows`: maps of the weights with boxes of 256, 128, 64 and 32 rows of 64 channels
+cudaError_t launch_conv_lstm(const ConvLstmParams& p, const TensorMap128 (&rows)[4], int sm_count, cudaStream_t s);
 
 // Failure-path probe: one warp waits, through the same bounded wait as the tensor-core kernels, on
 // a barrier that nothing ever completes; when `limit_cycles` have passed it records `code` in

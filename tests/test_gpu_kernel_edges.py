@@ -184,6 +184,32 @@ def test_convlstm_column_groups_change_no_bit(cuda_device, hidden, net):
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("hidden,net,K", [
+    (128, (400, 300), 5),     # 105 tiles: the last pair has no second tile
+    (64, (400, 300), 8),      # one group of columns
+    (256, (368, 480), 3),     # 72 ragged tiles x 1024 columns: several rounds, the last cut into halves
+])
+def test_convlstm_on_pairs_of_blocks_changes_no_bit(cuda_device, hidden, net, K):
+    """Beyond one round of units the ConvLSTM runs on pairs of blocks: every stream must get the bits it gets alone, on single blocks."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="pairs", src_w=net[0] + 30, src_h=net[1] + 20, net_w=net[0], net_h=net[1], hidden=hidden)
+    frames = _frames(wl, K, 2)
+    ctx, states, _ = _make(wl, K)
+    for t in range(2):
+        ctx.submit_frames([torch.from_numpy(frames[k][t]).to(cuda_device) for k in range(K)], states)
+        res = ctx.sync()
+    batch = [(*ctx.state_export(states[k]), ctx.fetch_probs(res[k])) for k in range(K)]
+    ctx.destroy()
+    ctx, (st,), _ = _make(wl, 1)
+    for k in (0, K - 2, K - 1):
+        ctx.state_reset(st)
+        for t in range(2):
+            ctx.submit_frames([torch.from_numpy(frames[k][t]).to(cuda_device)], [st])
+            (r,) = ctx.sync()
+        for a, b in zip(batch[k], (*ctx.state_export(st), ctx.fetch_probs(r))):
+            assert np.array_equal(a, b)
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("src,net,pad,K", [
     ((200, 150), (128, 64), 0, 1),       # one full tile column of 128
     ((200, 150), (129, 65), 3, 2),       # a tile column of one output: narrow tiles
