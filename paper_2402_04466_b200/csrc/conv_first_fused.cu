@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     constexpr bool ONE_ROW = decltype(one_row)::value;
     const uint32_t* rows = reinterpret_cast<const uint32_t*>(s_src + buf * src_bytes);
     const int b_lo = s_b_lo[buf], x0 = t.tx * FF_TW * STRIDE - 1;
-    float* pre_img = p.pre_out + (size_t)t.img * 3 * plane;
+    float* pre_img = p.pre_out + (size_t)(p.img0 + t.img) * 3 * plane;
     // the pixel of patch row e at byte offset xo of the staged rows -> patch entry q; `keep`: also to the resized image.
     // A column outside the image comes with scale and shift zero.
     auto pixel = [&](const int4& e, int xo, float fx, float scale, float shift, __nv_bfloat16* q, bool keep, int x) {
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     tc_fence_after();
     const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * COUT);
     const int y = t.ty * FF_TH + warp, x0 = t.tx * FF_TW;
-    __nv_bfloat16* out = p.out + (((size_t)t.img * p.Ho + y) * p.Wo + x0) * COUT;
+    __nv_bfloat16* out = p.out + (((size_t)(p.img0 + t.img) * p.Ho + y) * p.Wo + x0) * COUT;
     // The warp's 32 pixels x 32 channels pass through the 2 KB of the operand that its own gather fills next, so that four
     // lanes write the 64 bytes of a pixel: as 32-byte pieces of one pixel per lane the stores took a third of the kernel's time.
     // 16-byte piece c of pixel i lies at piece c ^ (i / 2 % 4).

@@ -122,7 +122,7 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
       const uint32_t bar = smem_u32(p_full + b);
       mbar_arrive_expect_tx(bar, PATCH_BYTES);
       // column tx*16*STRIDE - 1 is the halo; the box starts 3 columns earlier, on a 16-byte boundary
-      tma_load_4d(smem_u32(s_patch + b * PATCH_STRIDE), &p.map_in, bar, tx * 16 * STRIDE - 4, ty * 8 * STRIDE - 1, 0, img);
+      tma_load_4d(smem_u32(s_patch + b * PATCH_STRIDE), &p.map_in, bar, tx * 16 * STRIDE - 4, ty * 8 * STRIDE - 1, 0, p.img0 + img);
     };
 
     bool fail = false;   // a bounded wait ran out; the four warps learn of it together at the barrier
@@ -235,7 +235,7 @@ conv_first_tc_kernel(const __grid_constant__ ConvFirstTcParams p) {
       fence_proxy_async_smem();
       asm volatile("bar.sync 3, 128;" ::: "memory");
       if (leader) {
-        tma_store_4d(&p.map_out, smem_u32(s_out), 0, t.tx * 16, t.ty * 8, t.img);
+        tma_store_4d(&p.map_out, smem_u32(s_out), 0, t.tx * 16, t.ty * 8, p.img0 + t.img);
         bulk_commit_group();
       }
       if (++acc == 2) { acc = 0; acc_phase ^= 1u; }

@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
   uint64_t* tempty = tfull + 2;                                         // [2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tempty + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  __shared__ int s_img[3][TT_MAX_STREAMS];                              // h in, c, h out
+  __shared__ int s_img[4][TT_MAX_STREAMS];                              // h in, c, h out, x in
 
   // broadcast, so that the compiler knows the roles below to be whole warps
   const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
@@ -131,6 +131,7 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
     s_img[0][threadIdx.x] = p.h_in.v[threadIdx.x];
     s_img[1][threadIdx.x] = p.c_idx.v[threadIdx.x];
     s_img[2][threadIdx.x] = p.h_out.v[threadIdx.x];
+    s_img[3][threadIdx.x] = p.x_in.v[threadIdx.x];
   }
   tc_fence_before();
   __syncthreads();
@@ -149,12 +150,12 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       // a pair's second block takes the next tile; behind the last tile it computes that one again and stores nothing
       const int m = min(CTAS * unit_at(p, u).m + rank, p.tiles - 1);
       const int img = m / tiles_per_img, rem = m - img * tiles_per_img, ty = rem / p.tiles_x, tx = rem - ty * p.tiles_x;
-      const int img_h = s_img[0][img];
+      const int img_h = s_img[0][img], img_x = s_img[3][img];
       for (int sg = 0; sg < slabs; ++sg) {
         ok = mbar_wait(smem_u32(aempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x10 + (int)stage, wait_limit);
         if (!ok) break;
         const int src = sg < p.slabs[0] ? 0 : 1;
-        const int c0 = (src ? sg - p.slabs[0] : sg) * 64, n_img = src ? img_h : img;
+        const int c0 = (src ? sg - p.slabs[0] : sg) * 64, n_img = src ? img_h : img_x;
         if (rank == 0) mbar_arrive_expect_tx(smem_u32(afull + stage), CTAS * L_A_TX);
         if (PAIR) tma_load_4d_pair(smem_u32(s_a + stage * L_A_BYTES), &p.maps[src], map_to_cta(smem_u32(afull + stage), 0u), c0, tx * L_PW - 1, ty * L_PH - 1, n_img);
         else tma_load_4d(smem_u32(s_a + stage * L_A_BYTES), &p.maps[src], smem_u32(afull + stage), c0, tx * L_PW - 1, ty * L_PH - 1, n_img);

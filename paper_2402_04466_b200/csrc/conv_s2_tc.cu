@@ -126,7 +126,7 @@ __global__ void __launch_bounds__(S2_THREADS, SLAB_C == 32 ? 2 : 1) conv_s2_kern
         ok = ok && mbar_wait(smem_u32(vempty + 2 * v + buf), phase ^ 1u, abort_flag, p.status, WAIT_CONV_S2 + v, wait_limit);
         if (!ok) break;
         mbar_arrive_expect_tx(bar, Cfg::tx(v));
-        tma_load_4d(smem_u32(smem + Cfg::v_off(v) + buf * Cfg::v_bytes(v)), &p.map_v[v], bar, 0, tx * S2_PW - (v & 1), ty * S2_PH - (v >> 1), img);
+        tma_load_4d(smem_u32(smem + Cfg::v_off(v) + buf * Cfg::v_bytes(v)), &p.map_v[v], bar, 0, tx * S2_PW - (v & 1), ty * S2_PH - (v >> 1), p.img0 + img);
       }
     }
   } else if (warp == 1) {

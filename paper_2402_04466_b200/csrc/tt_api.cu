@@ -71,6 +71,22 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
+// Whether two host pointers lie in one pinned allocation (pageable memory: no).
+bool same_pinned_range(const void* a, const void* b) {
+  typedef CUresult (*AttributeFn)(void*, CUpointer_attribute, CUdeviceptr);
+  static AttributeFn fn = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<AttributeFn>(p);
+  });
+  CUdeviceptr ra = 0, rb = 0;
+  return fn && fn(&ra, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)(uintptr_t)a) == CUDA_SUCCESS &&
+         fn(&rb, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, (CUdeviceptr)(uintptr_t)b) == CUDA_SUCCESS && ra == rb;
+}
+
 uint16_t f32_to_bf16_rne(float f) {
   uint32_t u;
   std::memcpy(&u, &f, 4);
@@ -164,7 +180,7 @@ struct tt_ctx {
   // Frame pointers may change every tick, so the kernels read them from a small device table; a table that
   // does not yet hold the tick's pointers is refreshed by a 64-byte copy in front of the graph launch.
   struct TickGraph {
-    int K = 0, slot = 0, flat = 0, tab = 0;
+    int K = 0, n0 = 0, slot = 0, flat = 0, tab = 0;   // n0: first batch position, of a tick launched in parts
     int sig[TT_MAX_STREAMS] = {};   // state slot * 2 + half of every batch position
     int seen = 0;                   // direct executions of this key so far (capture happens on the second)
     uint64_t launches = 0;          // kernels inside the graph
@@ -184,7 +200,6 @@ struct tt_ctx {
   const uint8_t* frame_tab_last[TT_MAX_IN_FLIGHT][FRAME_TABS][TT_MAX_STREAMS] = {};   // what each device table holds
   bool frame_tab_valid[TT_MAX_IN_FLIGHT][FRAME_TABS] = {};
   uint64_t frame_tab_used[TT_MAX_IN_FLIGHT][FRAME_TABS] = {};             // tick at which the table was last used (the oldest is replaced)
-  const uint8_t* const* cur_tab = nullptr;                  // table the tick being enqueued reads
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_copy = nullptr;
   bool tick_profiled = false;
@@ -758,25 +773,26 @@ tt_status mark_stage(tt_ctx* ctx, int stage, int launches) {
   return TT_OK;
 }
 
-PreprocessParams preprocess_params(const tt_ctx* ctx, int K, const FramePtrs& frames, const uint8_t* const* tab) {
+PreprocessParams preprocess_params(const tt_ctx* ctx, int n0, int K, const FramePtrs& frames, const uint8_t* const* tab) {
   const tt_config& c = ctx->cfg;
   PreprocessParams pp;
   pp.src = frames; pp.src_tab = tab; pp.K = K; pp.src_w = c.src_w; pp.src_h = c.src_h; pp.src_pitch = c.src_pitch;
   pp.net_w = c.net_w; pp.net_h = c.net_h;
   pp.inv_div = 1.0f / c.norm_div; pp.mean = c.norm_mean; pp.inv_std = 1.0f / c.norm_std;
-  pp.dst = ctx->pre;
+  pp.dst = ctx->pre + (size_t)n0 * 3 * c.net_h * c.net_w;
   return pp;
 }
 
-// Launch sequence of one tick.  Everything is enqueued on ctx->stream.
-tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* const* states) {
+// Launch sequence of batch positions n0 .. n0 + K - 1 of a tick (all of them, or a part whose frames have arrived); `frames`, `tab`
+// and `states` are those of the part.  Everything is enqueued on ctx->stream.
+tt_status enqueue_tick(tt_ctx* ctx, int n0, int K, const FramePtrs& frames, const uint8_t* const* tab, tt_state* const* states) {
   const tt_config& c = ctx->cfg;
   cudaStream_t s = ctx->stream;
   tt_status ms_;
   const size_t plane = (size_t)ctx->Hm * ctx->Wm;
   IdxMap ident, c_idx, h_in, h_out;
   for (int n = 0; n < TT_MAX_STREAMS; ++n) {
-    ident.v[n] = n;
+    ident.v[n] = n0 + n;
     const int slot = n < K ? states[n]->slot : 0, half = n < K ? states[n]->half : 0;
     c_idx.v[n] = slot;
     h_in.v[n] = slot * 2 + half;
@@ -787,7 +803,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   // results are the same bits.
   const bool fused = ctx->fuse_first && (ctx->fuse_pre || !ctx->profiling);
   if (!fused) {
-    TT_CUDA(ctx, launch_preprocess(preprocess_params(ctx, K, frames, ctx->cur_tab), s));
+    TT_CUDA(ctx, launch_preprocess(preprocess_params(ctx, n0, K, frames, tab), s));
     if ((ms_ = mark_stage(ctx, TT_STAGE_PREPROCESS, 1)) != TT_OK) return ms_;
   }
 
@@ -800,8 +816,8 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       q.C0 = ctx->lay_c[l]; q.C1 = 0;
       q.H = ctx->lay_h[l]; q.W = ctx->lay_w[l]; q.Ho = ctx->lay_h[l + 1]; q.Wo = ctx->lay_w[l + 1];
       q.stride = L.stride; q.K = K; q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.sm_count = ctx->sm_count; q.pdl = ctx->profiling ? 0 : 1;
-      q.epilogue = EPI_RELU_F32_NCHW; q.out = ctx->enc_out[l];
       q.out_img_stride = (int64_t)L.cout * q.Ho * q.Wo;
+      q.epilogue = EPI_RELU_F32_NCHW; q.out = reinterpret_cast<float*>(ctx->enc_out[l]) + n0 * q.out_img_stride;
       TT_CUDA(ctx, launch_conv_simt(q, s));
       if ((ms_ = mark_stage(ctx, TT_STAGE_ENC0 + l, 1)) != TT_OK) return ms_;
       in = reinterpret_cast<const float*>(ctx->enc_out[l]);
@@ -821,8 +837,9 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   } else {
     if (ctx->use_first_tc) {
       ctx->first_tc.K = K;
+      ctx->first_tc.img0 = n0;
       ctx->first_tc.pdl = ctx->profiling ? 0 : 1;
-      ctx->first_tc.src = frames; ctx->first_tc.src_tab = ctx->cur_tab;
+      ctx->first_tc.src = frames; ctx->first_tc.src_tab = tab;
       ctx->first_tc.write_pre = ctx->fuse_pre ? 0 : 1;
       // the fused kernel is the first of the tick and may follow a copy: launched normally
       if (fused) TT_CUDA(ctx, launch_conv_first_fused(ctx->first_tc, ctx->sm_count, s));
@@ -834,8 +851,8 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       q.in0 = ctx->pre; q.img_stride0 = (int64_t)3 * c.net_h * c.net_w; q.idx0 = ident; q.C0 = 3; q.C1 = 0;
       q.H = c.net_h; q.W = c.net_w; q.Ho = ctx->lay_h[1]; q.Wo = ctx->lay_w[1];
       q.stride = L.stride; q.K = K; q.wgt = L.w; q.bias = L.b; q.cout = L.cout; q.cout_packed = L.cout_packed; q.sm_count = ctx->sm_count; q.pdl = ctx->profiling ? 0 : 1;
-      q.epilogue = EPI_RELU_BF16_NHWC; q.out = ctx->enc_out[0];
       q.out_img_stride = (int64_t)L.cout * q.Ho * q.Wo;
+      q.epilogue = EPI_RELU_BF16_NHWC; q.out = reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[0]) + n0 * q.out_img_stride;
       TT_CUDA(ctx, launch_conv_simt(q, s));
       if ((ms_ = mark_stage(ctx, TT_STAGE_ENC0, 1)) != TT_OK) return ms_;
     }
@@ -861,7 +878,8 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       // both kernels add up the same products in the same order: which one runs changes no bit
       if (L.s2.n_tiles_n > 0 && conv_s2_pays(L.s2.slab_c, K * L.s2.tiles_x * L.s2.tiles_y * L.s2.n_tiles_n, ctx->sm_count, L.s2.one_per_sm != 0)) {
         ConvS2Params q = L.s2;
-        q.K = K;
+        q.K = K; q.img0 = n0;
+        q.out += (size_t)n0 * q.Ho * q.Wo * q.cout;
         q.pdl = ctx->profiling ? 0 : 1;
         TT_CUDA(ctx, launch_conv_s2(q, ctx->sm_count, s));
         if ((ms_ = mark_stage(ctx, TT_STAGE_ENC0 + l, 1)) != TT_OK) return ms_;
@@ -873,7 +891,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       q.n_src = 1; q.slabs[0] = L.cin0 / L.slab_c; q.slabs[1] = 0; q.img0 = ident; q.img1 = ident;
       // a weight matrix of at most 40 KB (64 outputs, up to 32 inputs x 9 taps) stays in shared memory for the whole launch
       q.wres = (q.two_per_sm && q.block_n == 64 && L.slab_c == 32 && q.n_tiles_n == 1 && 9 * q.slabs[0] * 64 * 32 * 2 <= 40 * 1024) ? 1 : 0;
-      q.epilogue = TC_EPI_RELU_BF16; q.out = reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l]);
+      q.epilogue = TC_EPI_RELU_BF16; q.out = reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[l]) + (size_t)n0 * q.Ho * q.Wo * q.cout;
       TT_CUDA(ctx, launch_conv_tc(q, ctx->sm_count, s));
       if ((ms_ = mark_stage(ctx, TT_STAGE_ENC0 + l, 1)) != TT_OK) return ms_;
     }
@@ -887,7 +905,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
       w.maps[0] = L.maps_halo[0]; w.maps[1] = L.maps_halo[1];
       w.slabs[0] = L.cin0 / 64; w.slabs[1] = L.cin1 / 64; w.cols = L.cout; w.hidden = ctx->Ch;
       w.tiles_x = (ctx->Wm + 7) / 8; w.tiles_y = (ctx->Hm + 15) / 16; w.tiles = K * w.tiles_x * w.tiles_y;
-      w.Hm = ctx->Hm; w.Wm = ctx->Wm; w.h_in = h_in; w.c_idx = c_idx; w.h_out = h_out;
+      w.Hm = ctx->Hm; w.Wm = ctx->Wm; w.x_in = ident; w.h_in = h_in; w.c_idx = c_idx; w.h_out = h_out;
       w.bias = L.b; w.c_state = ctx->c_state; w.h_f32 = ctx->use_post_tc ? nullptr : ctx->h_f32; w.h_bf16 = ctx->h_bf16;
       w.status = ctx->status_dev; w.wait_limit = ctx->wait_limit; w.pdl = q.pdl;
       const TensorMap128 rows[4] = {L.map_b[2], L.map_b[1], L.map_b[0], L.map_b32};
@@ -904,10 +922,11 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
     }
   }
 
+  const size_t out0 = (size_t)n0 * ctx->T * plane;
   if (ctx->use_post_tc) {
     PostTcParams& q = ctx->post_tc;
     q.idx = ctx->feed_forward ? ident : h_out; q.K = K;
-    q.logits = ctx->logits; q.probs = ctx->probs; q.masks = ctx->masks; q.bits = ctx->bits; q.results = ctx->results_host;
+    q.logits = ctx->logits + out0; q.probs = ctx->probs + out0; q.masks = ctx->masks + out0; q.bits = ctx->bits + n0 * plane; q.results = ctx->results_host + n0;
     q.status_out = ctx->status_host;
     q.pdl = ctx->profiling ? 0 : 1;
     TT_CUDA(ctx, launch_post_tc(q, ctx->sm_count, s));
@@ -923,8 +942,8 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
   po.K = K; po.Hm = ctx->Hm; po.Wm = ctx->Wm; po.Ch = ctx->Ch; po.T = ctx->T;
   po.head_w = ctx->head_w; po.head_b = ctx->head_b; po.conf_w = ctx->conf_w; po.conf_b = ctx->conf_b;
   po.conf_mode = c.conf_mode; po.zthr = ctx->zthr;
-  po.logits = ctx->logits; po.probs = ctx->probs; po.masks = ctx->masks; po.bits = ctx->bits;
-  po.results = ctx->results_host; po.scratch = ctx->post_scratch; po.status = ctx->status_dev; po.status_out = ctx->status_host; po.wait_limit = ctx->wait_limit;
+  po.logits = ctx->logits + out0; po.probs = ctx->probs + out0; po.masks = ctx->masks + out0; po.bits = ctx->bits + n0 * plane;
+  po.results = ctx->results_host + n0; po.scratch = ctx->post_scratch; po.status = ctx->status_dev; po.status_out = ctx->status_host; po.wait_limit = ctx->wait_limit;
   po.pdl = ctx->profiling ? 0 : 1;
   TT_CUDA(ctx, launch_postprocess(po, s));
   if ((ms_ = mark_stage(ctx, TT_STAGE_POSTPROCESS, 1)) != TT_OK) return ms_;
@@ -932,15 +951,117 @@ tt_status enqueue_tick(tt_ctx* ctx, int K, const FramePtrs& frames, tt_state* co
 
   if (c.overlay) {
     OverlayParams ov{};
-    ov.src = frames; ov.src_tab = ctx->cur_tab; ov.K = K; ov.src_w = c.src_w; ov.src_h = c.src_h; ov.src_pitch = c.src_pitch;
-    ov.T = ctx->T; ov.Hm = ctx->Hm; ov.Wm = ctx->Wm; ov.masks = ctx->masks; ov.bits = ctx->bits;
+    ov.src = frames; ov.src_tab = tab; ov.K = K; ov.src_w = c.src_w; ov.src_h = c.src_h; ov.src_pitch = c.src_pitch;
+    ov.T = ctx->T; ov.Hm = ctx->Hm; ov.Wm = ctx->Wm; ov.masks = ctx->masks + out0; ov.bits = ctx->bits + n0 * plane;
     std::memcpy(ov.palette, c.palette, sizeof(ov.palette));
-    ov.dst = ctx->overlay;
+    ov.dst = ctx->overlay + (size_t)n0 * c.src_w * c.src_h * 4;
     ov.pdl = ctx->profiling ? 0 : 1;
     TT_CUDA(ctx, launch_overlay(ov, s));
     if ((ms_ = mark_stage(ctx, TT_STAGE_OVERLAY, 1)) != TT_OK) return ms_;
   }
-  ctx->n_ticks += 1;
+  return TT_OK;
+}
+
+// Streams per part of a tick of K host frames: the part size for which the estimated time from the first copy to the last launch's end is
+// least, K where cutting saves less than a tenth.  A frame takes its bytes at 45 GB/s (pinned memory); k streams compute for 30 us (launches,
+// start-up, latency chains) and their operations at 1.3 PFLOP/s (fp32 path: 25 TFLOP/s).  One 854x480 stream: 27 us to copy, 30 + 10 to
+// compute, so parts of two streams hide behind the next part's copy; one full-HD stream: 138 and 30 + 118, parts of one.
+int part_size(const tt_ctx* ctx, int K) {
+  double ops = 0;
+  for (int l = 0; l < ctx->n_enc; ++l) ops += 18.0 * ctx->lay_c[l] * ctx->lay_c[l + 1] * ctx->lay_h[l + 1] * ctx->lay_w[l + 1];
+  if (!ctx->feed_forward) ops += 72.0 * (ctx->Cx + ctx->Ch) * ctx->Ch * ctx->Hm * ctx->Wm;
+  const double copy = (double)ctx->frame_bytes / 45e9, fixed = 30e-6, stream = ops / (ctx->bf16 ? 1.3e15 : 25e12);
+  int best = K;
+  double best_t = 0.9 * (K * copy + fixed + K * stream);
+  for (int k = 1; k < K; ++k) {
+    double arrived = 0, done = 0;
+    for (int n0 = 0, n1; n0 < K; n0 = n1) {
+      n1 = n0 == 0 && K % k ? K % k : n0 + k;
+      arrived += (n1 - n0) * copy;
+      done = std::max(done, arrived) + fixed + (n1 - n0) * stream;
+    }
+    if (done < best_t) { best_t = done; best = k; }
+  }
+  return best;
+}
+
+// Launches batch positions n0 .. n0 + K - 1 of the tick being submitted (fp, table and states are the whole tick's).
+//
+// The launch sequence is replayed from a CUDA graph.  Which kernel variants it launches depends
+// on the stream count and the frames' alignment alone, so the first launch of such a family runs as plain
+// launches (modules load, attributes are set outside any capture); after it, every new (positions, slot, pointer
+// table, state placement) of the family is captured the first time it shows up.  With stage events
+// requested the tick always runs as plain launches.
+template <typename Refresh>
+tt_status launch_part(tt_ctx* ctx, int slot, int tab, int n0, int K, const FramePtrs& tick_fp, const uint8_t* const* table, tt_state* const* tick_states,
+                      Refresh refresh_table) {
+  cudaStream_t s = ctx->stream;
+  tt_status st = TT_OK;
+  FramePtrs fp{};
+  for (int n = 0; n < K; ++n) fp.p[n] = tick_fp.p[n0 + n];
+  table += n0;
+  tt_state* const* states = tick_states + n0;
+  tt_ctx::TickGraph* tg = nullptr;
+  bool family_warm = false;
+  if (!ctx->graphs_off && !ctx->profiling) {
+    int flat = 1;
+    // the overlay launch picks its word-wise variant from the frames' 4-byte alignment: part of the key
+    for (int n = 0; n < K; ++n) flat &= (((uintptr_t)fp.p[n] & 3) == 0) ? 1 : 0;
+    for (auto& g : ctx->graphs) {
+      family_warm |= g.K == K && g.flat == flat && (g.seen >= 1 || g.exec);
+      bool same = g.K == K && g.n0 == n0 && g.slot == slot && g.flat == flat && g.tab == tab;
+      for (int n = 0; n < K && same; ++n) same = g.sig[n] == states[n]->slot * 2 + states[n]->half;
+      if (same) { tg = &g; break; }
+    }
+    if (!tg) {
+      if (ctx->graphs.size() >= 256) {            // bounded cache: drop everything and start over
+        for (auto& g : ctx->graphs)
+          if (g.exec) cudaGraphExecDestroy(g.exec);
+        ctx->graphs.clear();
+      }
+      tt_ctx::TickGraph g;
+      g.K = K; g.n0 = n0; g.slot = slot; g.flat = flat; g.tab = tab;
+      for (int n = 0; n < K; ++n) g.sig[n] = states[n]->slot * 2 + states[n]->half;
+      ctx->graphs.push_back(g);
+      tg = &ctx->graphs.back();
+    }
+  }
+  if (tg && tg->exec) {
+    if ((st = refresh_table()) != TT_OK) return st;
+    TT_CUDA(ctx, cudaGraphLaunch(tg->exec, s));
+    ctx->n_launches += tg->launches;
+  } else if (tg && (tg->seen >= 1 || family_warm)) {
+    // capture the sequence, then launch it
+    const uint64_t launches_before = ctx->n_launches;
+    cudaGraph_t graph = nullptr;
+    cudaError_t ce = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
+    if (ce == cudaSuccess) {
+      st = enqueue_tick(ctx, n0, K, fp, table, states);
+      cudaError_t ee = cudaStreamEndCapture(s, &graph);
+      if (ce == cudaSuccess) ce = ee;
+    }
+    if (st == TT_OK && ce == cudaSuccess && graph) ce = cudaGraphInstantiate(&tg->exec, graph, 0);
+    if (graph) cudaGraphDestroy(graph);
+    if (st != TT_OK || ce != cudaSuccess || !tg->exec) {
+      // capture is an optimisation only: clear the error, switch it off and run this tick directly
+      cudaGetLastError();
+      tg->exec = nullptr;
+      ctx->graphs_off = true;
+      ctx->n_launches = launches_before;
+      if ((st = refresh_table()) != TT_OK) return st;
+      st = enqueue_tick(ctx, n0, K, fp, table, states);
+      if (st != TT_OK) return st;
+    } else {
+      tg->launches = ctx->n_launches - launches_before;
+      if ((st = refresh_table()) != TT_OK) return st;
+      TT_CUDA(ctx, cudaGraphLaunch(tg->exec, s));
+    }
+  } else {
+    if ((st = refresh_table()) != TT_OK) return st;
+    st = enqueue_tick(ctx, n0, K, fp, table, states);
+    if (st != TT_OK) return st;
+    if (tg) tg->seen += 1;
+  }
   return TT_OK;
 }
 
@@ -1113,21 +1234,8 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
   FramePtrs fp{};
   bool any_h2d = false;
   for (int n = 0; n < K; ++n) {
-    if (frames[n].on_device) {
-      fp.p[n] = frames[n].data;
-    } else {
-      // host frames go over a copy stream of their own, so the copy of this tick can run while the
-      // previous tick still computes; the compute stream waits for the copy below
-      uint8_t* dst = ctx->frames_stage + (size_t)n * ctx->frame_bytes;
-      TT_CUDA(ctx, cudaMemcpyAsync(dst, frames[n].data, ctx->frame_bytes, cudaMemcpyHostToDevice, ctx->copy_stream));
-      fp.p[n] = dst;
-      any_h2d = true;
-    }
-  }
-  tt_status st = TT_OK;
-  if (any_h2d) {
-    TT_CUDA(ctx, cudaEventRecord(ctx->ev_copy, ctx->copy_stream));
-    TT_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_copy, 0));
+    any_h2d |= !frames[n].on_device;
+    fp.p[n] = frames[n].on_device ? frames[n].data : ctx->frames_stage + (size_t)n * ctx->frame_bytes;
   }
   // frame pointers of this tick -> the slot's device table (the kernels read them from there).  The copy is
   // skipped when the table already holds these pointers: always the case for host frames (they are staged in
@@ -1142,90 +1250,48 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
   const bool tab_miss = tab < 0;
   if (tab_miss) tab = oldest;
   ctx->frame_tab_used[slot][tab] = ctx->n_ticks + 1;
-  ctx->cur_tab = ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS;
-  // refreshes the chosen table; called in front of the tick's launch (a graph capture, which enqueues nothing,
-  // comes before it, so that its host time stays outside the interval between the tick's events)
-  auto refresh_table = [&]() -> tt_status {
-    TT_CUDA(ctx, record_start());
-    if (tab_miss) {
-      for (int n = 0; n < TT_MAX_STREAMS; ++n) ctx->frame_tab_last[slot][tab][n] = ctx->frame_tab_host[slot][n] = n < K ? fp.p[n] : nullptr;
-      ctx->frame_tab_valid[slot][tab] = false;   // stays so if the copy cannot be enqueued
-      TT_CUDA(ctx, cudaMemcpyAsync(ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS, ctx->frame_tab_host[slot],
-                                   sizeof(void*) * TT_MAX_STREAMS, cudaMemcpyHostToDevice, s));
-      ctx->frame_tab_valid[slot][tab] = true;
+  const uint8_t* const* const table = ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS;
+  // With nothing else in flight a tick of host frames is cut into parts, each launched when its frames have arrived (submits behind
+  // others need no cut: their copies run while those compute).  A stream's results do not depend on what shares its launches.
+  const int part = any_h2d && !ctx->profiling && ctx->q_count == 0 ? part_size(ctx, K) : K;
+  tt_status st = TT_OK;
+  for (int n0 = 0, n1; n0 < K; n0 = n1) {
+    n1 = n0 == 0 && K % part ? K % part : n0 + part;   // the odd part first
+    bool copied = false;
+    for (int n = n0; n < n1;) {
+      if (frames[n].on_device) { ++n; continue; }
+      // host frames go over a copy stream of their own, so the copy can run while an earlier part or tick still
+      // computes; the compute stream waits for the copy below.  Frames that lie one behind the other in one pinned buffer travel as one
+      // copy (six of 854x480: 180 us as six, 153 us as one)
+      int m = n + 1;
+      while (m < n1 && !frames[m].on_device && frames[m].data == frames[m - 1].data + ctx->frame_bytes && same_pinned_range(frames[n].data, frames[m].data)) ++m;
+      TT_CUDA(ctx, cudaMemcpyAsync(ctx->frames_stage + (size_t)n * ctx->frame_bytes, frames[n].data, (size_t)(m - n) * ctx->frame_bytes, cudaMemcpyHostToDevice, ctx->copy_stream));
+      copied = true;
+      n = m;
     }
-    // everything that moves host data to the device (frames, pointer table) counts as the H2D stage
-    return mark_stage(ctx, TT_STAGE_H2D, 0);
-  };
-
-  // The launch sequence of a tick is replayed from a CUDA graph.  Which kernel variants a tick launches depends
-  // on the stream count and the frames' alignment alone, so the first tick of such a family runs as plain
-  // launches (modules load, attributes are set outside any capture); after it, every new (slot, pointer
-  // table, state placement) of the family is captured the first time it shows up.  With stage events
-  // requested the tick always runs as plain launches.
-  tt_ctx::TickGraph* tg = nullptr;
-  bool family_warm = false;
-  if (!ctx->graphs_off && !ctx->profiling) {
-    int flat = 1;
-    // the overlay launch picks its word-wise variant from the frames' 4-byte alignment: part of the key
-    for (int n = 0; n < K; ++n) flat &= (((uintptr_t)fp.p[n] & 3) == 0) ? 1 : 0;
-    for (auto& g : ctx->graphs) {
-      family_warm |= g.K == K && g.flat == flat && (g.seen >= 1 || g.exec);
-      bool same = g.K == K && g.slot == slot && g.flat == flat && g.tab == tab;
-      for (int n = 0; n < K && same; ++n) same = g.sig[n] == states[n]->slot * 2 + states[n]->half;
-      if (same) { tg = &g; break; }
+    if (copied) {
+      // recorded anew for every part: a wait keeps the record it was enqueued behind
+      TT_CUDA(ctx, cudaEventRecord(ctx->ev_copy, ctx->copy_stream));
+      TT_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_copy, 0));
     }
-    if (!tg) {
-      if (ctx->graphs.size() >= 256) {            // bounded cache: drop everything and start over
-        for (auto& g : ctx->graphs)
-          if (g.exec) cudaGraphExecDestroy(g.exec);
-        ctx->graphs.clear();
+    // refreshes the chosen table; called in front of the tick's first launch (a graph capture, which enqueues nothing,
+    // comes before it, so that its host time stays outside the interval between the tick's events)
+    auto refresh_table = [&]() -> tt_status {
+      TT_CUDA(ctx, record_start());
+      if (n0 > 0) return TT_OK;
+      if (tab_miss) {
+        for (int n = 0; n < TT_MAX_STREAMS; ++n) ctx->frame_tab_last[slot][tab][n] = ctx->frame_tab_host[slot][n] = n < K ? fp.p[n] : nullptr;
+        ctx->frame_tab_valid[slot][tab] = false;   // stays so if the copy cannot be enqueued
+        TT_CUDA(ctx, cudaMemcpyAsync(ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS, ctx->frame_tab_host[slot],
+                                     sizeof(void*) * TT_MAX_STREAMS, cudaMemcpyHostToDevice, s));
+        ctx->frame_tab_valid[slot][tab] = true;
       }
-      tt_ctx::TickGraph g;
-      g.K = K; g.slot = slot; g.flat = flat; g.tab = tab;
-      for (int n = 0; n < K; ++n) g.sig[n] = states[n]->slot * 2 + states[n]->half;
-      ctx->graphs.push_back(g);
-      tg = &ctx->graphs.back();
-    }
+      // everything that moves host data to the device (frames, pointer table) counts as the H2D stage
+      return mark_stage(ctx, TT_STAGE_H2D, 0);
+    };
+    if ((st = launch_part(ctx, slot, tab, n0, n1 - n0, fp, table, states, refresh_table)) != TT_OK) return st;
   }
-  if (tg && tg->exec) {
-    if ((st = refresh_table()) != TT_OK) return st;
-    TT_CUDA(ctx, cudaGraphLaunch(tg->exec, s));
-    ctx->n_launches += tg->launches;
-    ctx->n_ticks += 1;
-  } else if (tg && (tg->seen >= 1 || family_warm)) {
-    // capture the sequence, then launch it
-    const uint64_t launches_before = ctx->n_launches;
-    cudaGraph_t graph = nullptr;
-    cudaError_t ce = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
-    if (ce == cudaSuccess) {
-      st = enqueue_tick(ctx, K, fp, states);
-      cudaError_t ee = cudaStreamEndCapture(s, &graph);
-      if (ce == cudaSuccess) ce = ee;
-    }
-    if (st == TT_OK && ce == cudaSuccess && graph) ce = cudaGraphInstantiate(&tg->exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    if (st != TT_OK || ce != cudaSuccess || !tg->exec) {
-      // capture is an optimisation only: clear the error, switch it off and run this tick directly
-      cudaGetLastError();
-      tg->exec = nullptr;
-      ctx->graphs_off = true;
-      ctx->n_launches = launches_before;
-      ctx->n_ticks -= (st == TT_OK) ? 1 : 0;
-      if ((st = refresh_table()) != TT_OK) return st;
-      st = enqueue_tick(ctx, K, fp, states);
-      if (st != TT_OK) return st;
-    } else {
-      tg->launches = ctx->n_launches - launches_before;
-      if ((st = refresh_table()) != TT_OK) return st;
-      TT_CUDA(ctx, cudaGraphLaunch(tg->exec, s));
-    }
-  } else {
-    if ((st = refresh_table()) != TT_OK) return st;
-    st = enqueue_tick(ctx, K, fp, states);
-    if (st != TT_OK) return st;
-    if (tg) tg->seen += 1;
-  }
+  ctx->n_ticks += 1;
   TT_CUDA(ctx, cudaEventRecord(ctx->ev_stop, s));
   for (int n = 0; n < TT_MAX_STREAMS; ++n) ctx->states[n].last_pos = -1;
   for (int n = 0; n < K; ++n) {
@@ -1330,7 +1396,7 @@ tt_status tt_debug_tensor(tt_ctx* ctx, tt_state* st, int32_t which, float* host_
     n = (size_t)3 * ctx->cfg.net_h * ctx->cfg.net_w;
     if (ctx->fuse_pre) {
       // the resized image never reached memory: make it now, from the frame buffers of that submit
-      TT_CUDA(ctx, launch_preprocess(preprocess_params(ctx, ctx->K_inflight, ctx->fp_inflight, nullptr), s));
+      TT_CUDA(ctx, launch_preprocess(preprocess_params(ctx, 0, ctx->K_inflight, ctx->fp_inflight, nullptr), s));
     }
     src = ctx->pre + (size_t)pos * n;
   } else if (which >= TT_TENSOR_ENC0 && which < TT_TENSOR_ENC0 + ctx->n_enc) {

@@ -105,6 +105,7 @@ struct ConvFirstTcParams {
   const float* in;            // [K][3][H][W] fp32
   __nv_bfloat16* out;         // [K][Ho][Wo][cout] bf16
   int32_t H, W, Ho, Wo, stride, K, cout, tiles_x, tiles_y;
+  int32_t img0;               // image of batch position 0 inside the input and output tensors
   int32_t pdl;                // launch as a programmatic dependent of the previous kernel in the stream
   const uint16_t* w_packed;   // device, cout*32 bf16 in the MMA operand layout
   const float* bias;          // device, [cout]
@@ -183,6 +184,7 @@ struct ConvS2Params {
   int32_t slab_c;           // input channels: 32 or 64
   int32_t K, Ho, Wo, tiles_x, tiles_y;   // 8 x 16 pixel tiles
   int32_t n_tiles_n, cout;  // groups of conv_s2_block_n output channels
+  int32_t img0;             // input image of batch position 0 (`out` starts at its output)
   int32_t one_per_sm;       // one block per multiprocessor even where two fit
   int32_t pdl;
   const float* bias;
@@ -203,7 +205,7 @@ struct ConvLstmParams {
   int32_t slabs[2];         // 64-channel slabs of x and h
   int32_t cols, hidden;     // 4 * hidden columns, a multiple of 256
   int32_t tiles, tiles_x, tiles_y, Hm, Wm;   // tiles = images x tiles_x x tiles_y
-  IdxMap h_in, c_idx, h_out;                 // image of h, slot of c, image of h' per batch position
+  IdxMap x_in, h_in, c_idx, h_out;           // images of x and h, slot of c, image of h' per batch position
   int32_t m_units, width, groups, even, u_full;   // set by the launch: tiles or pairs of tiles, column groups, whether all are as wide, the unit from which they are cut in two
   int32_t pdl;
   const float* bias;        // packed order

@@ -229,3 +229,40 @@ def test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, K):
     out = binding.preprocess(torch.from_numpy(buf.reshape(K, -1)).to(cuda_device), sw, sh, 3 * sw + pad, nw, nh).cpu().numpy()
     for k in range(K):
         assert np.max(np.abs(out[k] - oracle.preprocess(frames[k], nw, nh))) < 2e-5
+
+
+@pytest.mark.parametrize("shape,K", [
+    (dict(src_w=854, src_h=480, net_w=640, net_h=480, hidden=128), 5),                        # parts of 1, 2 and 2 streams
+    (dict(src_w=854, src_h=480, net_w=642, net_h=480, hidden=128), 6),                        # parts of 2; first layer on the fp32 kernel
+    (dict(src_w=854, src_h=480, net_w=320, net_h=240, hidden=32, enc_cout=(16, 32), enc_stride=(2, 2), precision="fp32"), 6),
+])
+def test_a_tick_of_host_frames_in_parts_changes_nothing(cuda_device, shape, K):
+    """Streams of large host frames are launched in parts as their frames arrive: results, maps, overlay, intermediate tensors and state
+    are those of the same frames on the device, whose tick is not cut, and a tick counts once.  The middle stream's frame is on the device."""
+    wl = tt_synth.workload("cfg1-gain").with_(name="parts", overlay=True, **shape)
+    w = tt_synth.make_weights(wl)
+    frames = _frames(wl, K, 3)
+    runs, launches = [], []
+    for host in (True, False):
+        ctx = binding.Context(binding.make_config(wl, max_streams=K), w)
+        states = [ctx.state_create() for _ in range(K)]
+        out = []
+        for t in range(3):
+            fr = [torch.from_numpy(frames[k][t]) for k in range(K)]
+            fr = [f.pin_memory() if host and k != K // 2 else f.to(cuda_device) for k, f in enumerate(fr)]
+            before = ctx.get_counters()[0]
+            ctx.submit_frames(fr, states, frame_index=t)
+            res = ctx.sync()
+            launches.append(ctx.get_counters()[0] - before)
+            for k in range(K):
+                out += [res[k][n] for n in ("conf", "cx", "cy", "count")] + [ctx.fetch_probs(res[k]), ctx.fetch_masks(res[k]), ctx.fetch_overlay(res[k])]
+                out += [ctx.debug_tensor(states[k], n) for n in ["pre", "prob"] + [f"enc{l}" for l in range(len(wl.enc_cout))]]
+        if wl.recurrent:
+            for k in range(K):
+                out += list(ctx.state_export(states[k]))
+        assert ctx.get_counters()[1] == 3
+        runs.append(out)
+        ctx.destroy()
+    assert launches[0] == launches[2] >= 2 * launches[3]        # the host ticks were cut
+    for a, b in zip(*runs):
+        assert np.array_equal(a, b)
