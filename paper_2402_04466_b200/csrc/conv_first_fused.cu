@@ -3,8 +3,8 @@
 // The resized fp32 image is an observable tensor of the context and is still written (unless the caller does not
 // want it), but nothing reads it back, and one launch with its start-up and drain is gone.
 //
-// Bound by instruction issue in the resize (about 60 instructions per pixel of three channels where both axes are
-// resized) and by HBM (8 full-HD frames: 50 MB in, 88 + 236 MB out).  A block of 8 warps takes tiles of 32 x 8 outputs in
+// Bound by the load/store pipe (at two full-HD frames 72 % of the active cycles, of which 72 % passes through shared memory, against 30 % of
+// the issue slots), the chain of phases below, and by HBM (8 full-HD frames: 50 MB in, 88 + 236 MB out).  A block of 8 warps takes tiles of 32 x 8 outputs in
 // turn, down a column of tiles, and every warp takes part in every phase, so the sampling has all the warps of
 // the multiprocessor (three blocks) at its disposal and the phases of different blocks overlap:
 //   stage    the 16-byte aligned byte range of every frame row under the tile's input patch, by bulk copies two
@@ -15,10 +15,13 @@
 //   gather   a thread per output pixel packs its 27 taps into one 64-byte row of the operand (no-swizzle core-matrix
 //            layout, two tiles of 128 rows);
 //   MMA      four tcgen05.mma M128 x COUT x K16, issued by one thread;
-//   epilogue of the tile before, while the next patch is already being built: bias, ReLU, 32-byte stores per lane.
+//   epilogue of the tile before, while the next patch is already being built: bias, ReLU, tile stores by the TMA unit.
 // A specialised form (eight sampling warps feeding four gather warps through patch buffers) had been 6 us slower per tick than
 // the two kernels at 5 streams of 854x480.  This one, alone under the profiler: 18.8 us against 10.1 + 14.4 us at that size, 9.8 against
-// 7.2 + 9.2 us for one stream, 100 against 38 + 61 us for 8 full-HD streams, where only the second launch's gap is won.
+// 7.2 + 9.2 us for one stream, 100 against 38 + 61 us for 8 full-HD streams, where only the second launch's gap is won.  All that with the
+// output read back from shared memory and stored by the warps, and the resized image stored one column off its 128-byte lines; with tile
+// stores and whole lines (both sides in one call): a tick of eight full-HD streams 1049 -> 1034 us, of one 168.4 -> 166.9, of five 854x480 streams
+// 111.6 -> 110.7, of one 64.15 -> 63.9.
 #include <type_traits>
 
 #include "tt_internal.h"
@@ -54,12 +57,13 @@ struct Tile {
 template <int COUT, int STRIDE>
 __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel(const __grid_constant__ ConvFirstTcParams p) {
   constexpr int PW = ff_patch_w(STRIDE), PH = ff_patch_h(STRIDE), PITCH = ff_pitch(STRIDE);
-  constexpr int FULL = PW / 32, EXTRA = PW - 32 * FULL;       // whole warps of patch columns, and the columns behind them
+  constexpr int FULL = PW / 32, EXTRA = PW - 32 * FULL;       // whole warps of patch columns, from the tile's first own column on, and the rest
   constexpr int GROUPS = FF_WARPS / FULL;                     // patch rows sampled at a time
   constexpr int A_BYTES = 2 * 128 * 64;
-  extern __shared__ __align__(128) uint8_t smem[];
+  extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* s_a = smem;                                        // operand: two tiles of [128 rows][32] bf16
-  uint8_t* s_b = s_a + A_BYTES;                               // weights in operand layout
+  uint8_t* s_out = s_a + A_BYTES;                             // per warp 32 pixels x 32 channels on their way out
+  uint8_t* s_b = s_out + FF_WARPS * 2048;                     // weights in operand layout
   float* s_bias = reinterpret_cast<float*>(s_b + COUT * 64);
   __nv_bfloat16* s_patch = reinterpret_cast<__nv_bfloat16*>(s_bias + COUT);      // [3][PH][PITCH]
   uint8_t* s_src = reinterpret_cast<uint8_t*>(s_patch) + ((3 * PH * PITCH * 2 + 15) & ~15);   // [2][src_rows_cap][src_row_cap]
@@ -158,12 +162,13 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     };
     auto zero = [&](__nv_bfloat16* q) { q[0] = q[PH * PITCH] = q[2 * PH * PITCH] = __float2bfloat16_rn(0.f); };
     {
-      const int j = (warp % FULL) * 32 + lane, x = x0 + j;
-      const bool in_x = x >= 0 && x < p.W;
-      const int2 xe = __ldg(&p.xtab[min(max(x, 0), p.W - 1)]);
+      // the tile's own columns (patch columns 1 .. 32 FULL), so that the 128 bytes a warp stores of the resized image are one line
+      const int j = 1 + (warp % FULL) * 32 + lane, x = x0 + j;
+      const bool in_x = x < p.W;
+      const int2 xe = __ldg(&p.xtab[min(x, p.W - 1)]);
       const int xo = in_x ? xe.x - b_lo : 0;
       const float scale = in_x ? p.scale : 0.f, shift = in_x ? p.shift : 0.f;
-      const bool own = p.write_pre && in_x && j >= 1 && j <= FF_TW * STRIDE;   // of this tile, not of its halo
+      const bool own = p.write_pre && in_x;
 #pragma unroll
       for (int k = 0; k < (PH + GROUPS - 1) / GROUPS; ++k) {
         const int r = warp / FULL + k * GROUPS;
@@ -176,12 +181,13 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
       }
     }
     if (warp == FF_WARPS - 1 && lane < EXTRA * PH) {   // a warp with one row less than the first ones
-      const int r = lane / EXTRA, j = 32 * FULL + lane % EXTRA, x = x0 + j;
+      // halo columns: the one in front, at stride 1 also the one behind
+      const int r = lane / EXTRA, j = lane % EXTRA ? 32 * FULL + 1 : 0, x = x0 + j;
       const int4 e = s_row[buf][r];
       __nv_bfloat16* q = s_patch + r * PITCH + j;
-      if (x < p.W && e.w >= 0) {
+      if (x >= 0 && x < p.W && e.w >= 0) {
         const int2 xe = __ldg(&p.xtab[x]);
-        pixel(e, xe.x - b_lo, __int_as_float(xe.y), p.scale, p.shift, q, p.write_pre && j <= FF_TW * STRIDE && r >= 1 && r <= FF_TH * STRIDE, x);
+        pixel(e, xe.x - b_lo, __int_as_float(xe.y), p.scale, p.shift, q, false, x);
       } else {
         zero(q);
       }
@@ -236,16 +242,18 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     tc_fence_after();
     const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * COUT);
     const int y = t.ty * FF_TH + warp, x0 = t.tx * FF_TW;
-    __nv_bfloat16* out = p.out + (((size_t)(p.img0 + t.img) * p.Ho + y) * p.Wo + x0) * COUT;
-    // The warp's 32 pixels x 32 channels pass through the 2 KB of the operand that its own gather fills next, so that four
-    // lanes write the 64 bytes of a pixel: as 32-byte pieces of one pixel per lane the stores took a third of the kernel's time.
-    // 16-byte piece c of pixel i lies at piece c ^ (i / 2 % 4).
-    uint8_t* mine = s_a + warp * 2048;
+    // 32 channels of the warp's row of 32 pixels leave as one tile store, which clips what lies outside the map.  They wait for it in 2 KB of
+    // the warp's own, the first half of 64 channels in the part of the operand that the warp's own gather fills next.
+    // 16-byte piece c of pixel i lies at piece c ^ (i / 2 % 4), the swizzle of the store's map.
 #pragma unroll
     for (int ck = 0; ck < COUT / 32; ++ck) {
+      uint8_t* mine = (ck + 1 < COUT / 32 ? s_a : s_out) + warp * 2048;
       uint32_t v[32];
       tmem_ld32(taddr + (uint32_t)(ck * 32), v);
-      if (ck > 0) __syncwarp();
+      if (ck == 0) {   // the stores of the tile before have been read
+        if (lane == 0) bulk_wait_group_read0();
+        __syncwarp();
+      }
 #pragma unroll
       for (int i = 0; i < 32; i += 8) {
         uint32_t u[4];
@@ -257,17 +265,17 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
         }
         *reinterpret_cast<uint4*>(mine + lane * 64 + (((i >> 3) ^ ((lane >> 1) & 3)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
       }
+      fence_proxy_async_smem();
       __syncwarp();
-      if (y < p.Ho) {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int px = q * 8 + (lane >> 2), c = lane & 3;
-          const uint4 u = *reinterpret_cast<const uint4*>(mine + px * 64 + ((c ^ ((px >> 1) & 3)) << 4));
-          if (x0 + px < p.Wo) *reinterpret_cast<uint4*>(out + px * COUT + ck * 32 + c * 8) = u;
-        }
+      if (lane == 0) {
+        if (y < p.Ho) tma_store_4d(&p.map_rows, smem_u32(mine), ck * 32, x0, y, p.img0 + t.img);
+        bulk_commit_group();
       }
     }
-    __syncwarp();
+    if (COUT > 32) {   // the operand's part has been read
+      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+      __syncwarp();
+    }
   };
 
   Tile cur, ahead, last;
@@ -336,6 +344,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&s_bar), (uint32_t)(n - 1) & 1u, abort_flag, p.status, WAIT_CONV_FIRST_FUSED + 0x11, p.wait_limit));
     if (ok) epilogue(last);
   }
+  if (lane == 0) bulk_wait_group0();
   __syncwarp();
   if (*abort_flag) {
     for (int i = 0; i < 64; ++i) __nanosleep(16000);
@@ -350,7 +359,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
 
 template <int COUT, int STRIDE>
 cudaError_t launch_t(const ConvFirstTcParams& p, int sm_count, cudaStream_t s) {
-  const int smem = 2 * 128 * 64 + COUT * 64 + COUT * 4 + ((3 * ff_patch_h(STRIDE) * ff_pitch(STRIDE) * 2 + 15) & ~15) + 2 * p.src_rows_cap * p.src_row_cap;
+  const int smem = 2 * 128 * 64 + FF_WARPS * 2048 + COUT * 64 + COUT * 4 + ((3 * ff_patch_h(STRIDE) * ff_pitch(STRIDE) * 2 + 15) & ~15) + 2 * p.src_rows_cap * p.src_row_cap;
   auto kern = conv_first_fused_kernel<COUT, STRIDE>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;

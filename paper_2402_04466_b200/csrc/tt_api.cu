@@ -619,6 +619,8 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
         const cuuint64_t str[3] = {(cuuint64_t)co * 2, (cuuint64_t)f.Wo * co * 2, (cuuint64_t)f.Ho * f.Wo * co * 2};
         const cuuint32_t box[4] = {(cuuint32_t)co, 16, 8, 1};
         if ((st = encode_map(ctx, &f.map_out, ctx->enc_out[0], 4, dims, str, box, co * 2)) != TT_OK) return st;
+        const cuuint32_t row_box[4] = {32, 32, 1, 1};
+        if ((st = encode_map(ctx, &f.map_rows, ctx->enc_out[0], 4, dims, str, row_box, 64)) != TT_OK) return st;
       }
       {
         const cuuint64_t dims[4] = {(cuuint64_t)f.W, (cuuint64_t)f.H, 3, (cuuint64_t)S};

@@ -111,6 +111,7 @@ struct ConvFirstTcParams {
   const float* bias;          // device, [cout]
   int32_t* status;
   long long wait_limit;       // SM cycles after which a barrier wait gives up
+  TensorMap128 map_rows;      // conv_first_fused: output again, box [32][32][1][1], 64B swizzle
   // conv_first_fused only: the kernel samples the uint8 RGB frames itself (resize to W x H, then v * scale + shift)
   // and neither `in` nor the maps are used
   FramePtrs src;                   // frame pointers by value ...
