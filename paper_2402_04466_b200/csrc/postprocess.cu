@@ -272,19 +272,6 @@ struct StreamCfg {
   static_assert(SMEM_BYTES + 2560 <= 227 * 1024, "dynamic plus static shared memory must fit one block per multiprocessor");
 };
 
-// Two fp32 values in one 64-bit register, and the packed fused multiply-add acc += a * b on both halves.
-__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
-  unsigned long long r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
-}
-__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
-  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
-}
-
 __device__ __forceinline__ uint32_t sw_smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // Bounded wait on a warp-private mbarrier; false when the limit ran out (the caller gives up).
@@ -583,16 +570,16 @@ __global__ void __launch_bounds__(StreamCfg<NCHUNK>::THREADS, 1) post_stream_ker
           for (int c = 0; c < 4; ++c) {
             const float4 wa = s_w[(k * 8 + c * 2 + 0) * 32 + lane];    // tools 0..3
             const float4 wb = s_w[(k * 8 + c * 2 + 1) * 32 + lane];    // tools 4..7
-            const unsigned long long w01 = pack2(wa.x, wa.y), w23 = pack2(wa.z, wa.w);
-            const unsigned long long w45 = pack2(wb.x, wb.y), w67 = pack2(wb.z, wb.w);
+            const unsigned long long w01 = tc::pack2(wa.x, wa.y), w23 = tc::pack2(wa.z, wa.w);
+            const unsigned long long w45 = tc::pack2(wb.x, wb.y), w67 = tc::pack2(wb.z, wb.w);
 #pragma unroll
             for (int qq = 0; qq < SW_ROUND_PIX; ++qq) {
               const float hc = c == 0 ? hv[qq][k].x : c == 1 ? hv[qq][k].y : c == 2 ? hv[qq][k].z : hv[qq][k].w;
-              const unsigned long long h2 = pack2(hc, hc);
-              fma2(v2[qq][0], h2, w01);
-              fma2(v2[qq][1], h2, w23);
-              fma2(v2[qq][2], h2, w45);
-              fma2(v2[qq][3], h2, w67);
+              const unsigned long long h2 = tc::pack2(hc, hc);
+              tc::fma2(v2[qq][0], h2, w01);
+              tc::fma2(v2[qq][1], h2, w23);
+              tc::fma2(v2[qq][2], h2, w45);
+              tc::fma2(v2[qq][3], h2, w67);
             }
           }
           if (p.conf_mode == TT_CONF_GAP_LINEAR) {
@@ -606,7 +593,7 @@ __global__ void __launch_bounds__(StreamCfg<NCHUNK>::THREADS, 1) post_stream_ker
 #pragma unroll
         for (int qq = 0; qq < SW_ROUND_PIX; ++qq)
 #pragma unroll
-          for (int tp = 0; tp < 4; ++tp) unpack2(v2[qq][tp], v[qq * 8 + 2 * tp], v[qq * 8 + 2 * tp + 1]);
+          for (int tp = 0; tp < 4; ++tp) tc::unpack2(v2[qq][tp], v[qq * 8 + 2 * tp], v[qq * 8 + 2 * tp + 1]);
         // transposing butterfly: after the round with offset d a lane keeps the half of its values
         // selected by its own bit d; five rounds leave value index == lane
 #pragma unroll

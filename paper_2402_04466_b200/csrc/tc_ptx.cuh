@@ -316,6 +316,19 @@ __device__ __forceinline__ void st_global_v8_b32(void* p, const uint32_t (&v)[8]
                : "memory");
 }
 
+// Two fp32 values in one 64-bit register, and the packed fused multiply-add acc += a * b on both halves.
+__device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ void fma2(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
 // max(a, 0) and max(b, 0) as a pair of bf16: rounded first, then both compared in one instruction.  A NaN becomes 0, as
 // with fmaxf (the conversion's own .relu would keep it).
 __device__ __forceinline__ uint32_t pack_relu_bf16(float a, float b) {
