@@ -126,7 +126,6 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
   }
-  for (int i = threadIdx.x; i < p.cols; i += L_THREADS) s_bias[i] = __ldg(p.bias + i);
   if (threadIdx.x < TT_MAX_STREAMS) {
     s_img[0][threadIdx.x] = p.h_in.v[threadIdx.x];
     s_img[1][threadIdx.x] = p.c_idx.v[threadIdx.x];
@@ -242,6 +241,9 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
     }
   } else if (warp >= L_EPI_WARP0 && warp < L_EPI_WARP0 + L_EPI_WARPS) {
     // ---------------------------------------------------------------------- epilogue
+    // the biases are fetched here and not in front of the block's first barrier, where the copies would wait for them
+    for (int i = threadIdx.x - 32 * L_EPI_WARP0; i < p.cols; i += 32 * L_EPI_WARPS) s_bias[i] = __ldg(p.bias + i);
+    asm volatile("bar.sync 1, 256;" ::: "memory");
     pdl_wait();
     const int quarter = warp & 3, half = (warp - L_EPI_WARP0) >> 2;
     const int row = quarter * 32 + lane, py = row >> 3, px = row & 7;     // row of the 128-row tile = pixel of the patch
@@ -254,10 +256,8 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
       const int x = tx * L_PW + px, y = ty * L_PH + py;
       const bool valid = x < p.Wm && y < p.Hm && m_own < p.tiles;
       const size_t pix = (size_t)y * p.Wm + x;
-      // chunks of 32 columns (8 hidden units x 4 gates): the first of the quarter's two warps takes 128 columns of a wide
-      // group and half of a narrow one, so that every pair of chunks starts on 32 bytes of h'
-      const int first = t.n > 128 ? 128 : t.n >> 1;
-      const int off = half ? first : 0, chunks = (half ? t.n - first : first) >> 5;
+      // chunks of 32 columns (8 hidden units x 4 gates), half of them for either of the quarter's two warps
+      const int off = half ? t.n >> 1 : 0, chunks = t.n >> 6, odd = (off >> 5) & 1;
       const int col0 = t.col0 + off;
 
       // the old cell state of this thread's pixel is fetched before the accumulator is waited for: its latency hides under
@@ -295,14 +295,17 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
             }
             st_global_v8(p.c_state + so + ck * 8, c_new);
             if (p.h_f32) st_global_v8(p.h_f32 + so + ck * 8, h_new);
-            // bf16 copy of h': 8 values are half a sector, so two neighbouring chunks leave together
-            const int hq = (ck & 1) * 4;
-            hb[hq + 0] = pack_bf16(h_new[0], h_new[1]);
-            hb[hq + 1] = pack_bf16(h_new[2], h_new[3]);
-            hb[hq + 2] = pack_bf16(h_new[4], h_new[5]);
-            hb[hq + 3] = pack_bf16(h_new[6], h_new[7]);
-            if (ck & 1) st_global_v8_b32(p.h_bf16 + ho + (ck - 1) * 8, hb);
-            else if (ck + 1 == chunks) *reinterpret_cast<uint4*>(p.h_bf16 + ho + ck * 8) = make_uint4(hb[0], hb[1], hb[2], hb[3]);
+            // bf16 copy of h': 8 values are half a sector, so an even chunk of the unit waits for the odd one behind it
+            const uint4 hv = make_uint4(pack_bf16(h_new[0], h_new[1]), pack_bf16(h_new[2], h_new[3]), pack_bf16(h_new[4], h_new[5]), pack_bf16(h_new[6], h_new[7]));
+            if (((ck + odd) & 1) == 0) {
+              hb[0] = hv.x; hb[1] = hv.y; hb[2] = hv.z; hb[3] = hv.w;
+              if (ck + 1 == chunks) *reinterpret_cast<uint4*>(p.h_bf16 + ho + ck * 8) = hv;
+            } else if (ck == 0) {
+              *reinterpret_cast<uint4*>(p.h_bf16 + ho) = hv;
+            } else {
+              hb[4] = hv.x; hb[5] = hv.y; hb[6] = hv.z; hb[7] = hv.w;
+              st_global_v8_b32(p.h_bf16 + ho + (ck - 1) * 8, hb);
+            }
           }
         }
       }
