@@ -1,7 +1,7 @@
 // S4 + S5: mask head (1x1 conv hidden -> tools), sigmoid, threshold, per-tool confidence
 // and mask centroid.  HBM-bound: the hidden state is read exactly once.
 //
-// Generic kernel (post_tile_kernel): a block stages 64 pixels x Ch hidden values in shared
+// Planar state (post_planar_kernel, below): a thread per pixel.  Channels-last state of any width (post_tile_kernel): a block stages 64 pixels x Ch hidden values in shared
 // memory with coalesced 128-bit loads, four threads per pixel form the T dot products, and the
 // masks, logits and probabilities are written.
 // The block's partial sums go into per-stream accumulators with integer atomics (fixed point for
@@ -116,17 +116,12 @@ __global__ void __launch_bounds__(POST_THREADS) post_tile_kernel(const __grid_co
   pdl_wait();   // the head weights are nobody's output; the hidden state is the previous kernel's
   if (blockIdx.x == 0 && tid == 0 && p.status) tc::report_status(*(volatile int*)p.status, false, p.status, p.status_out);
 
-  if (p.channels_last) {
+  {
     const int row4 = Ch >> 2;
     const float4* g = reinterpret_cast<const float4*>(h_img + (size_t)pix0 * Ch);
     for (int i = tid; i < npix * row4; i += POST_THREADS) {
       const int pp = i / row4, c4 = i % row4;
       *reinterpret_cast<float4*>(s_tile + pp * row + 4 * c4) = __ldg(g + i);
-    }
-  } else {
-    for (int i = tid; i < Ch * PIX; i += POST_THREADS) {
-      const int c = i / PIX, pp = i % PIX;
-      if (pp < npix) s_tile[pp * row + c] = __ldg(h_img + (size_t)c * plane + pix0 + pp);
     }
   }
   __syncthreads();
@@ -230,6 +225,182 @@ __global__ void __launch_bounds__(POST_THREADS) post_tile_kernel(const __grid_co
     }
   }
   finish_stream(p, n, nb, tid);
+}
+
+// Planar state (the fp32 path's): a thread per pixel, whose channels are coalesced loads across the warp, 16 in flight, against head weights in
+// shared memory, two tools to an FMA.  Bound by latency: loads, then the chain from a block's sums to the stream's record.  A thread sums the channels up in
+// the order of post_tile_kernel's four threads, so the logits are the same bits; the pooled-state confidence is, by linearity, one more dot product per
+// pixel, summed over the pixels.  Against staging 64 pixels x channels in shared memory for four threads a pixel, in a tick: three streams of
+// 80x60 x 32 channels 11 -> 6.4 us, one 64x64 x 16 6.8 -> 4.9 us; a call on planar state of the caller's 156 -> 112 us.
+constexpr int PLANAR_THREADS = 128;
+
+template <bool GAP>
+__global__ void __launch_bounds__(PLANAR_THREADS) post_planar_kernel(const __grid_constant__ PostParams p) {
+  extern __shared__ __align__(16) float s_mem[];
+  __shared__ unsigned long long s_acc[TT_MAX_TOOLS * 4];   // [tool][count, sum x, sum y, sum of probabilities or of the confidence head]
+  __shared__ int s_last;
+  pdl_launch_dependents();
+  const int Ch = p.Ch, T = p.T, tid = threadIdx.x, lane = tid & 31;
+  const int plane = p.Hm * p.Wm, nb = (plane + PLANAR_THREADS - 1) / PLANAR_THREADS;
+  const int n = blockIdx.x / nb, pix = (blockIdx.x - n * nb) * PLANAR_THREADS + tid;
+  const bool live = pix < plane;
+  // [channel][8 tools], then the confidence head's
+  for (int i = tid; i < Ch * 8; i += PLANAR_THREADS) {
+    const int c = i >> 3, t = i & 7;
+    s_mem[i] = t < T ? __ldg(p.head_w + t * Ch + c) : 0.0f;
+    if (GAP) s_mem[Ch * 8 + i] = t < T ? __ldg(p.conf_w + t * Ch + c) : 0.0f;
+  }
+  float bias[TT_MAX_TOOLS];
+#pragma unroll
+  for (int t = 0; t < TT_MAX_TOOLS; ++t) bias[t] = t < T ? __ldg(p.head_b + t) : 0.0f;
+  if (tid < TT_MAX_TOOLS * 4) s_acc[tid] = 0ull;
+  __syncthreads();
+  pdl_wait();   // the weights are nobody's output; the hidden state is the previous kernel's
+  if (blockIdx.x == 0 && tid == 0 && p.status) tc::report_status(*(volatile int*)p.status, false, p.status, p.status_out);
+
+  const float* h = p.h + (size_t)p.idx.v[n] * p.img_stride + (live ? pix : plane - 1);
+  // sums of the channels whose fours are 0, 1, 2, 3 mod 4, for pairs of tools
+  unsigned long long z2[4][4], g2[GAP ? 4 : 1][4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      z2[q][k] = 0ull;
+      if (GAP) g2[q][k] = 0ull;
+    }
+  for (int c0 = 0; c0 < Ch; c0 += 16) {
+    float v[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = c0 + j < Ch ? __ldg(h + (size_t)(c0 + j) * plane) : 0.0f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (c0 + 4 * q < Ch) {   // the number of channels is a multiple of 4
+#pragma unroll
+        for (int j = 4 * q; j < 4 * q + 4; ++j) {
+          const unsigned long long x = tc::pack2(v[j], v[j]);
+          const ulonglong2* w = reinterpret_cast<const ulonglong2*>(s_mem + (c0 + j) * 8);
+          const ulonglong2 wa = w[0], wb = w[1];
+          tc::fma2(z2[q][0], x, wa.x);
+          tc::fma2(z2[q][1], x, wa.y);
+          tc::fma2(z2[q][2], x, wb.x);
+          tc::fma2(z2[q][3], x, wb.y);
+          if (GAP) {
+            const ulonglong2 ca = w[2 * Ch], cb = w[2 * Ch + 1];
+            tc::fma2(g2[q][0], x, ca.x);
+            tc::fma2(g2[q][1], x, ca.y);
+            tc::fma2(g2[q][2], x, cb.x);
+            tc::fma2(g2[q][3], x, cb.y);
+          }
+        }
+      }
+    }
+  }
+  auto combine = [](const unsigned long long (&a)[4][4], int k, float& lo, float& hi) {
+    float l[4], u[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) tc::unpack2(a[q][k], l[q], u[q]);
+    lo = (l[0] + l[1]) + (l[2] + l[3]);
+    hi = (u[0] + u[1]) + (u[2] + u[3]);
+  };
+
+  const int px = live ? pix % p.Wm : 0, py = live ? pix / p.Wm : 0;
+  const size_t o0 = (size_t)n * T * plane + pix;           // tool t's element: + t * plane
+  uint32_t bits = 0;
+  float prob[TT_MAX_TOOLS];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    float dot[2];
+    combine(z2, k, dot[0], dot[1]);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const int t = 2 * k + i;
+      const float z = dot[i] + bias[t];
+      const bool store = live && t < T, m = store && z > p.zthr;
+      prob[t] = sigmoid_acc(z);
+      if (store) {
+        const size_t o = o0 + (size_t)t * plane;
+        p.logits[o] = z;
+        p.probs[o] = prob[t];
+        p.masks[o] = m ? 1 : 0;
+      }
+      bits |= (m ? 1u : 0u) << t;
+    }
+  }
+  if (p.bits && live) p.bits[(size_t)n * plane + pix] = (uint8_t)bits;
+
+  // the warp's sums of its 32 pixels, tool t's in lane 4 t; what is a float is summed in a fixed tree and turned into fixed point
+  long long cnt = 0, sx = 0, sy = 0, sum = 0;
+#pragma unroll
+  for (int t = 0; t < TT_MAX_TOOLS; ++t) {
+    const bool m = (bits >> t) & 1u;
+    const int c1 = __popc(__ballot_sync(0xffffffffu, m));
+    const int x1 = __reduce_add_sync(0xffffffffu, m ? px : 0);
+    const int y1 = __reduce_add_sync(0xffffffffu, m ? py : 0);
+    if (lane == 4 * t) { cnt = c1; sx = x1; sy = y1; }
+  }
+  float g[TT_MAX_TOOLS];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    if (GAP) {
+      combine(reinterpret_cast<const unsigned long long (&)[4][4]>(g2), k, g[2 * k], g[2 * k + 1]);
+    } else {
+      g[2 * k] = prob[2 * k];
+      g[2 * k + 1] = prob[2 * k + 1];
+    }
+  }
+#pragma unroll
+  for (int t = 0; t < TT_MAX_TOOLS; ++t) g[t] = live ? g[t] : 0.0f;
+  // three rounds in which a lane hands on half of its tools, two of one value
+#pragma unroll
+  for (int d = 16, half = 4; half >= 1; d >>= 1, half >>= 1) {
+    const bool upper = (lane & d) != 0;
+#pragma unroll
+    for (int j = 0; j < half; ++j) {
+      const float send = upper ? g[j] : g[j + half], keep = upper ? g[j + half] : g[j];
+      g[j] = keep + __shfl_xor_sync(0xffffffffu, send, d);
+    }
+  }
+  g[0] += __shfl_xor_sync(0xffffffffu, g[0], 2);
+  g[0] += __shfl_xor_sync(0xffffffffu, g[0], 1);
+  sum = to_fixed(g[0]);
+  if ((lane & 3) == 0 && (lane >> 2) < T) {
+    unsigned long long* a = s_acc + lane;                  // 4 * tool
+    atomicAdd(a + 0, (unsigned long long)cnt);
+    atomicAdd(a + 1, (unsigned long long)sx);
+    atomicAdd(a + 2, (unsigned long long)sy);
+    atomicAdd(a + 3, (unsigned long long)sum);
+  }
+  __syncthreads();
+
+  // into the stream's accumulators; the block that completes the stream forms its record and zeroes them again
+  const ScratchLayout sl = scratch_layout(p.K, plane, Ch, T);
+  uint8_t* scr = reinterpret_cast<uint8_t*>(p.scratch);
+  unsigned int* counter = reinterpret_cast<unsigned int*>(scr + sl.off_counter) + n;
+  long long* acc = reinterpret_cast<long long*>(scr + sl.off_acc + (size_t)n * sl.acc_stride) + Ch;
+  if (tid < T * 4) {
+    const unsigned long long v = s_acc[tid];
+    if (v) atomicAdd(reinterpret_cast<unsigned long long*>(acc + tid), v);
+  }
+  __threadfence();
+  __syncthreads();
+  if (tid == 0) s_last = (atomicAdd(counter, 1u) == (unsigned int)(nb - 1));
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  if (tid < T) {
+    const float inv_plane = 1.0f / (float)plane;
+    const long long* st = acc + tid * 4;
+    const long long c = __ldcg(st + 0), x = __ldcg(st + 1), y = __ldcg(st + 2), f = __ldcg(st + 3);
+    const float mean = (float)((double)f * (double)FIX_INV) * inv_plane;
+    tt_result* r = p.results + n;
+    r->conf[tid] = GAP ? sigmoid_acc(mean + __ldg(p.conf_b + tid)) : mean;
+    r->count[tid] = (int32_t)c;
+    r->cx[tid] = c ? (float)((double)x / (double)c) : -1.0f;
+    r->cy[tid] = c ? (float)((double)y / (double)c) : -1.0f;
+  }
+  __syncthreads();
+  if (tid < T * 4) acc[tid] = 0;
+  if (tid == 0) *counter = 0u;
 }
 
 // Channels-last fast path (hidden a multiple of 128): a persistent kernel of independent warps.
@@ -757,6 +928,10 @@ cudaError_t launch_postprocess(const PostParams& p, cudaStream_t s) {
     if (p.Ch == 128) return launch_kernel(post_stream_kernel<1>, grid, StreamCfg<1>::THREADS, StreamCfg<1>::SMEM_BYTES, s, p, pdl);
     if (p.Ch == 256) return launch_kernel(post_stream_kernel<2>, grid, StreamCfg<2>::THREADS, StreamCfg<2>::SMEM_BYTES, s, p, pdl);
     return launch_kernel(post_stream_kernel<4>, grid, StreamCfg<4>::THREADS, StreamCfg<4>::SMEM_BYTES, s, p, pdl);
+  } else if (!p.channels_last) {
+    const int blocks = p.K * ((plane + PLANAR_THREADS - 1) / PLANAR_THREADS);
+    if (p.conf_mode == TT_CONF_GAP_LINEAR) return launch_kernel(post_planar_kernel<true>, blocks, PLANAR_THREADS, (size_t)p.Ch * 64, s, p, p.pdl != 0);
+    return launch_kernel(post_planar_kernel<false>, blocks, PLANAR_THREADS, (size_t)p.Ch * 32, s, p, p.pdl != 0);
   } else {
     return launch_kernel(post_tile_kernel, p.K * nb, POST_THREADS, post_smem_bytes(p.Ch), s, p, p.pdl != 0);
   }

@@ -266,3 +266,35 @@ def test_a_tick_of_host_frames_in_parts_changes_nothing(cuda_device, shape, K):
     assert launches[0] == launches[2] >= 2 * launches[3]        # the host ticks were cut
     for a, b in zip(*runs):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("conf_mode", ["mean_sigmoid", "gap_linear"])
+@pytest.mark.parametrize("K,ch,hm,wm,T", [
+    (1, 4, 1, 1, 1),         # one pixel, four channels, one tool
+    (2, 20, 9, 15, 8),       # 135 pixels: a second block of seven; channels in a partial chunk
+    (3, 16, 8, 16, 5),       # one full block
+    (8, 36, 16, 20, 7),      # ten full warps
+    (2, 512, 13, 10, 3),     # widest state
+])
+def test_heads_of_a_planar_state_at_the_edges_of_their_blocks(cuda_device, K, ch, hm, wm, T, conf_mode):
+    """fp32 sums of up to 512 products and fixed-point sums of 2^-30 against the oracle's double sums: 1e-4 as in the stage tests; sizes and
+    centroids exactly those of the mask.  The second call finds the accumulators zeroed."""
+    rng = np.random.default_rng(9)
+    h = (rng.standard_normal((K, ch, hm, wm)) * 0.5).astype(np.float32)
+    hw, cw = ((rng.standard_normal((T, ch)) * 2 / np.sqrt(ch)).astype(np.float32) for _ in range(2))
+    hb, cb = ((rng.standard_normal(T) * 0.3).astype(np.float32) for _ in range(2))
+    dev = [torch.from_numpy(a).to(cuda_device) for a in (hw, hb, cw, cb)]
+    out = binding.postprocess(torch.from_numpy(h).to(cuda_device), False, *dev, conf_mode)
+    again = binding.postprocess(torch.from_numpy(h).to(cuda_device), False, *dev, conf_mode)
+    for k in range(K):
+        z, p, m = oracle.head(h[k], hw, hb, 0.5)
+        got = {n: out[n][k].cpu().numpy() for n in ("logits", "probs", "masks")}
+        assert np.max(np.abs(got["logits"] - z)) < 1e-4 and np.max(np.abs(got["probs"] - p)) < 1e-4
+        assert np.array_equal(got["masks"] != 0, got["logits"] > 0)
+        r = out["results"][k]
+        conf = oracle.conf_mean_sigmoid(p) if conf_mode == "mean_sigmoid" else oracle.conf_gap_linear(h[k], cw, cb)
+        assert np.max(np.abs(r["conf"] - conf)) < 1e-4
+        cx, cy, n = oracle.centroids(got["masks"])
+        assert np.array_equal(r["count"], n) and np.array_equal(r["cx"], cx) and np.array_equal(r["cy"], cy)
+        for f in ("conf", "cx", "cy", "count"):
+            assert np.array_equal(r[f], again["results"][k][f])
