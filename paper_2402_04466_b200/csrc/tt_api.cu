@@ -965,16 +965,19 @@ tt_status enqueue_tick(tt_ctx* ctx, int n0, int K, const FramePtrs& frames, cons
 }
 
 // Streams per part of a tick of K host frames: the part size for which the estimated time from the first copy to the last launch's end is
-// least, K where cutting saves less than a tenth.  A frame takes its bytes at 45 GB/s (pinned memory); k streams compute for 30 us (launches,
-// start-up, latency chains) and their operations at 1.3 PFLOP/s (fp32 path: 25 TFLOP/s).  One 854x480 stream: 27 us to copy, 30 + 10 to
-// compute, so parts of two streams hide behind the next part's copy; one full-HD stream: 138 and 30 + 118, parts of one.
+// least, K where cutting saves less than a twentieth.  A frame takes its bytes at 50 GB/s (pinned memory); a part computes for 45 us (launches,
+// start-up, latency chains, and what copies lose beside kernels) and its streams' operations at 1.3 PFLOP/s (fp32 path: 25 TFLOP/s).  A 854x480 stream:
+// 25 us to copy, 10 to compute; a full-HD one 124 and 118.  Measured, us a tick uncut / in parts of 1 / 2 / 3 / 4 streams (* chosen): 854x480 with
+// overlay, three streams 164* 199 160 164, four 198 265 190 193* 198, six 266 344 271 254* 247, eight without overlay 322 432 322 285* 286; full-HD, two
+// 492 416*, four 937 722* 729 831, eight 1822 1336 1289* 1313 1406; six feed-forward 854x480 206* 232 200 200 205; eight 428x240 on the fp32
+// path 247* 488 344 295 263.
 int part_size(const tt_ctx* ctx, int K) {
   double ops = 0;
   for (int l = 0; l < ctx->n_enc; ++l) ops += 18.0 * ctx->lay_c[l] * ctx->lay_c[l + 1] * ctx->lay_h[l + 1] * ctx->lay_w[l + 1];
   if (!ctx->feed_forward) ops += 72.0 * (ctx->Cx + ctx->Ch) * ctx->Ch * ctx->Hm * ctx->Wm;
-  const double copy = (double)ctx->frame_bytes / 45e9, fixed = 30e-6, stream = ops / (ctx->bf16 ? 1.3e15 : 25e12);
+  const double copy = (double)ctx->frame_bytes / 50e9, fixed = 45e-6, stream = ops / (ctx->bf16 ? 1.3e15 : 25e12);
   int best = K;
-  double best_t = 0.9 * (K * copy + fixed + K * stream);
+  double best_t = 0.95 * (K * copy + fixed + K * stream);
   for (int k = 1; k < K; ++k) {
     double arrived = 0, done = 0;
     for (int n0 = 0, n1; n0 < K; n0 = n1) {

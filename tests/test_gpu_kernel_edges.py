@@ -232,8 +232,8 @@ def test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, K):
 
 
 @pytest.mark.parametrize("shape,K", [
-    (dict(src_w=854, src_h=480, net_w=640, net_h=480, hidden=128), 5),                        # parts of 1, 2 and 2 streams
-    (dict(src_w=854, src_h=480, net_w=642, net_h=480, hidden=128), 6),                        # parts of 2; first layer on the fp32 kernel
+    (dict(src_w=854, src_h=480, net_w=640, net_h=480, hidden=128), 5),                        # parts of 2 and 3 streams
+    (dict(src_w=854, src_h=480, net_w=642, net_h=480, hidden=128), 6),                        # parts of 3; first layer on the fp32 kernel
     (dict(src_w=854, src_h=480, net_w=320, net_h=240, hidden=32, enc_cout=(16, 32), enc_stride=(2, 2), precision="fp32"), 6),
 ])
 def test_a_tick_of_host_frames_in_parts_changes_nothing(cuda_device, shape, K):
