@@ -56,8 +56,9 @@ typedef enum {
   TT_OPT_FEED_FORWARD = 1,   /* the model has no recurrent cell: encoder -> mask/confidence heads (the paper's second
                                 workload class, a feed-forward segmentation network, Section V-B); `hidden` must equal the
                                 last encoder width, lstm_w/lstm_b are ignored, states carry nothing */
-  TT_OPT_CTA_PAIRS = 2,      /* run 256-wide tensor-core tiles on CTA pairs (cta_group::2).  Off by default: measured
-                                11-15 % slower than single-CTA tiles on the benchmark shapes */
+  TT_OPT_CTA_PAIRS = 2,      /* run 256-wide tensor-core tiles of one activation box per tap on CTA pairs (cta_group::2).  Off by
+                                default: measured 11-15 % slower than such tiles on single CTAs on the benchmark shapes (the ConvLSTM's own
+                                form on haloed patches uses pairs by itself where they pay) */
   TT_OPT_RESERVED_SMS = 4,   /* value = number of multiprocessors left free for another workload (at most half of the
                                 device): the persistent tensor-core and post-processing kernels size their grids for the
                                 rest.  With tt_render_layers' carved-out form this gives the visualisation load its own
@@ -199,7 +200,7 @@ tt_status tt_state_import(tt_ctx* ctx, tt_state* st, const float* h_host, const 
  * Asynchronous: returns once the work is enqueued.  Up to TT_MAX_IN_FLIGHT submits may be in flight (the
  * host->device copies of the later ones overlap the compute of the first: with three, the copy engine
  * need not wait for the host between ticks; ticks execute in submit order, so a state may be used by
- * all of them); tt_sync returns them oldest first.  frames[k].data must
+ * all of them; with none, a tick of host frames may be launched in parts as its frames arrive); tt_sync returns them oldest first.  frames[k].data must
  * stay valid until the tt_sync of its submit returns.  Errors: K < 1 or null/duplicate/foreign states -> TT_ERR_INVALID_ARG;
  * K > max_streams -> TT_ERR_ADMISSION; TT_MAX_IN_FLIGHT submits already in flight -> TT_ERR_NOT_READY.
  * Nothing is enqueued when one of these argument errors is returned.

@@ -268,7 +268,8 @@ __global__ void __launch_bounds__(PT_THREADS, 3) post_tc_kernel(const __grid_con
       const int px = live ? pix % p.Wm : 0, py = live ? pix / p.Wm : 0;
       const size_t o0 = (size_t)n * T * plane + pix;     // tool t's element: + t * plane
       // All eight tool slots take part (those behind T have zero weights and are masked out): without a branch per tool their
-      // votes and reductions overlap, where they had been eight chains one behind the other.
+      // votes and reductions overlap, where they had been eight chains one behind the other: one 854x480 stream 6.4 -> 5.3 us in a tick, five
+      // 7.7 -> 6.7, eight full-HD streams 20 -> 18.
       uint32_t bits = 0;
       float prob[TT_MAX_TOOLS];
 #pragma unroll
