@@ -48,7 +48,7 @@ def load_peaks():
         return dict(FALLBACK_PEAKS), "fallback"
 
 
-KERNEL_SOURCES = {"convlstm": ["conv_tc.cu", "conv_lstm_tc.cu", "tc_ptx.cuh"], "enc1": ["conv_tc.cu", "conv_s2_tc.cu", "tc_ptx.cuh"],
+KERNEL_SOURCES = {"convlstm": ["conv_lstm_tc.cu", "tc_ptx.cuh"], "enc1": ["conv_tc.cu", "conv_s2_tc.cu", "tc_ptx.cuh"],
                   "enc2": ["conv_tc.cu", "conv_s2_tc.cu", "tc_ptx.cuh"],
                   "enc0": ["conv_first_tc.cu", "conv_first_fused.cu", "tc_ptx.cuh", "pre_math.cuh"], "preprocess": ["preprocess.cu", "pre_math.cuh"],
                   "postprocess": ["post_tc.cu", "tc_ptx.cuh"], "overlay": ["overlay.cu"]}
