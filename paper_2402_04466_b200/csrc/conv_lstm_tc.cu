@@ -161,6 +161,12 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
         if (++stage == L_A_STAGES) { stage = 0; phase ^= 1u; }
       }
     }
+    // The last "free" signals of both buffers, which the MMAs' commits send into both blocks of a pair, arrive before either block leaves:
+    // a later commit's signal (an accumulator's) says nothing about when an earlier one's reaches the other block.
+    for (int i = 0; PAIR && i < L_A_STAGES && ok; ++i) {
+      ok = mbar_wait(smem_u32(aempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x18 + (int)stage, wait_limit);
+      if (++stage == L_A_STAGES) { stage = 0; phase ^= 1u; }
+    }
   } else if (warp >= L_EPI_WARP0 + L_EPI_WARPS && lane == 0) {
     // ----------------------------------------------------------------------- weights
     // producer j of two owns iterations j, j + 2, ... of the block's sequence (slab-major, tap inside)
@@ -194,6 +200,12 @@ __global__ void __launch_bounds__(L_THREADS, 1) conv_lstm_kernel(const __grid_co
         if (stage >= (uint32_t)L_B_STAGES) { stage -= L_B_STAGES; phase ^= 1u; }
       }
       it -= iters;
+    }
+    // the last "free" signals of this producer's share of the ring: those its next iterations would wait for, one turn of the ring on
+    for (; PAIR && it < L_B_STAGES && ok; it += 2) {
+      ok = mbar_wait(smem_u32(bempty + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_LSTM + 0x20 + (int)stage, wait_limit);
+      stage += 2;
+      if (stage >= (uint32_t)L_B_STAGES) { stage -= L_B_STAGES; phase ^= 1u; }
     }
   } else if (warp == 1 && rank == 0) {
     // -------------------------------------------------------------------- MMA issuer (of a pair: its first block)

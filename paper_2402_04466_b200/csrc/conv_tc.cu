@@ -229,6 +229,14 @@ __global__ void __launch_bounds__(TC_THREADS, CTAS) conv_tc_kernel(const __grid_
       }
       it -= k_iters;
     }
+    // The last "free" signals of this producer's share of the ring arrive before either block of a pair leaves: those its next iterations
+    // would wait for, one turn of the ring on.  The MMAs' commits send them into both blocks, and a later commit's signal (an
+    // accumulator's) says nothing about when they reach the other one.
+    for (; PAIR && it < STAGES && ok; it += n_prod) {
+      ok = mbar_wait(smem_u32(empty_bar + stage), phase ^ 1u, abort_flag, p.status, WAIT_CONV_TC + 0x70 + (int)stage, wait_limit);
+      stage += (uint32_t)n_prod;
+      if (stage >= (uint32_t)STAGES) { stage -= STAGES; phase ^= 1u; }
+    }
   } else if (warp == MMA_WARP && lane == 0 && rank == 0) {
     // -------------------------------------------------------------------- MMA issuer
     // This loop is one thread's chain of dependent instructions and sets the pace of the whole

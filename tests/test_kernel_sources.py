@@ -56,3 +56,41 @@ def test_status_codes_name_the_kernel():
     for base, files in of_file.items():
         assert len(files) == 1, f"{base} is used by {sorted(files)}"
     assert set(of_file) == set(bases) - {"WAIT_PROBE"}
+
+
+@pytest.mark.parametrize("name", [n for n, c in SOURCES.items() if "__global__" in c and re.search(r"umma_commit_(both|pair)\(", c)])
+def test_producers_of_a_pair_wait_for_their_last_free_signals(name):
+    """The commits that free a ring's stages signal barriers in both blocks of a pair.  The second block must still be there when the last of
+    them arrive: every producer takes a turn of its ring behind its loop, as if it had something left to load, before the blocks meet."""
+    body = SOURCES[name].split("__global__", 1)[1].rsplit("if (PAIR) cluster_sync_all();", 1)[0]
+    waits = re.findall(r"mbar_wait\(smem_u32\((\w*empty\w*) \+ stage\), phase \^ 1u", body)
+    rings = re.findall(r"commit(?:_pair)?\((\w*empty\w*) \+", body)      # freed by commits ("empty0": the address of empty_bar)
+    assert rings and sorted(waits) == sorted(2 * [{"empty0": "empty_bar"}.get(r, r) for r in dict.fromkeys(rings) if r in waits or r == "empty0"])
+    tails = re.findall(r"for \([^;]*; PAIR && (\w+) < (\w+) && ok;", body)
+    assert len(tails) == len(waits) // 2
+
+
+@pytest.mark.parametrize("producers,stages", [(2, 10), (2, 5), (1, 2), (3, 4), (3, 8)])
+def test_a_turn_of_the_ring_waits_for_each_stages_last_use_once(producers, stages):
+    """The index arithmetic of that turn: producer j owns iterations j, j + producers, ...; the wait in front of iteration g is for the use
+    `stages` iterations before it.  All producers' turns together wait for the last use of every stage, and for nothing that never comes."""
+    for per_unit in (1, 9, 18, 27, 36):
+        for units in (0, 1, 2, 5):
+            total, waited = per_unit * units, []
+            for j in range(producers):
+                stage, phase, it = j % stages, 0, j
+                g = j
+                for _ in range(units):
+                    while it < per_unit:
+                        assert (stage, phase) == (g % stages, g // stages & 1)
+                        it, g, stage = it + producers, g + producers, stage + producers
+                        if stage >= stages:
+                            stage, phase = stage - stages, phase ^ 1
+                    it -= per_unit
+                while it < stages:
+                    assert (stage, phase) == (g % stages, g // stages & 1)
+                    waited.append(g - stages)
+                    it, g, stage = it + producers, g + producers, stage + producers
+                    if stage >= stages:
+                        stage, phase = stage - stages, phase ^ 1
+            assert sorted(waited) == list(range(total - stages, total))     # negative: never used, the wait returns at once
