@@ -203,7 +203,9 @@ tt_status tt_state_import(tt_ctx* ctx, tt_state* st, const float* h_host, const 
  * all of them; with none, a tick of host frames may be launched in parts as its frames arrive); tt_sync returns them oldest first.  frames[k].data must
  * stay valid until the tt_sync of its submit returns.  Errors: K < 1 or null/duplicate/foreign states -> TT_ERR_INVALID_ARG;
  * K > max_streams -> TT_ERR_ADMISSION; TT_MAX_IN_FLIGHT submits already in flight -> TT_ERR_NOT_READY.
- * Nothing is enqueued when one of these argument errors is returned.
+ * Nothing is enqueued when one of these argument errors is returned.  Any other error (TT_ERR_CUDA, TT_ERR_OOM) leaves nothing of the
+ * submit in flight.  A frame that cannot be copied leaves every stream as it was; when a launch is refused, each stream has taken its frame or
+ * has not (tt_last_error says which).
  */
 tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_state* const* states);
 

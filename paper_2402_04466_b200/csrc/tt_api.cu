@@ -164,7 +164,8 @@ struct tt_ctx {
     uint8_t *masks = nullptr, *bits = nullptr, *overlay = nullptr;
     tt_result* results_host = nullptr;   // mapped: the last kernel of a tick writes the records here itself
     int32_t* status_host = nullptr;      // mapped: written by it when a wait has run out
-    cudaEvent_t ev_start = nullptr, ev_stop = nullptr, ev_copy = nullptr;
+    cudaEvent_t ev_start = nullptr, ev_stop = nullptr;
+    cudaEvent_t ev_copy[TT_MAX_STREAMS] = {};   // the host frames of a tick's part have arrived
     cudaEvent_t stage_ev[TT_STAGE_COUNT + 1] = {};
     bool stage_ran[TT_STAGE_COUNT] = {};
     FramePtrs fp{};
@@ -201,8 +202,8 @@ struct tt_ctx {
   bool frame_tab_valid[TT_MAX_IN_FLIGHT][FRAME_TABS] = {};
   uint64_t frame_tab_used[TT_MAX_IN_FLIGHT][FRAME_TABS] = {};             // tick at which the table was last used (the oldest is replaced)
   cudaStream_t copy_stream = nullptr;
-  cudaEvent_t ev_copy = nullptr;
   bool tick_profiled = false;
+  int n_stepped = 0;                // batch positions of the submit being enqueued whose recurrent step has been enqueued
   int K_inflight = 0;
   tt_frame frames_inflight[TT_MAX_STREAMS];
   tt_state* states_inflight[TT_MAX_STREAMS];
@@ -239,7 +240,7 @@ void bind_slot(tt_ctx* ctx, int i) {
   const tt_ctx::Slot& sl = ctx->slots[i];
   ctx->frames_stage = sl.frames_stage; ctx->logits = sl.logits; ctx->probs = sl.probs; ctx->masks = sl.masks;
   ctx->bits = sl.bits; ctx->overlay = sl.overlay; ctx->results_host = sl.results_host;
-  ctx->status_host = sl.status_host; ctx->ev_start = sl.ev_start; ctx->ev_stop = sl.ev_stop; ctx->ev_copy = sl.ev_copy;
+  ctx->status_host = sl.status_host; ctx->ev_start = sl.ev_start; ctx->ev_stop = sl.ev_stop;
   for (int k = 0; k <= TT_STAGE_COUNT; ++k) ctx->stage_ev[k] = sl.stage_ev[k];
   for (int k = 0; k < TT_STAGE_COUNT; ++k) ctx->stage_ran[k] = sl.stage_ran[k];
   ctx->tick_profiled = sl.profiled;
@@ -253,7 +254,7 @@ void save_slot(tt_ctx* ctx, int i) {
   tt_ctx::Slot& sl = ctx->slots[i];
   sl.frames_stage = ctx->frames_stage; sl.logits = ctx->logits; sl.probs = ctx->probs; sl.masks = ctx->masks;
   sl.bits = ctx->bits; sl.overlay = ctx->overlay; sl.results_host = ctx->results_host;
-  sl.status_host = ctx->status_host; sl.ev_start = ctx->ev_start; sl.ev_stop = ctx->ev_stop; sl.ev_copy = ctx->ev_copy;
+  sl.status_host = ctx->status_host; sl.ev_start = ctx->ev_start; sl.ev_stop = ctx->ev_stop;
   for (int k = 0; k <= TT_STAGE_COUNT; ++k) sl.stage_ev[k] = ctx->stage_ev[k];
   for (int k = 0; k < TT_STAGE_COUNT; ++k) sl.stage_ran[k] = ctx->stage_ran[k];
   sl.profiled = ctx->tick_profiled;
@@ -563,7 +564,7 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
     }
     TT_CUDA(ctx, cudaEventCreate(&sl.ev_start));
     TT_CUDA(ctx, cudaEventCreate(&sl.ev_stop));
-    TT_CUDA(ctx, cudaEventCreateWithFlags(&sl.ev_copy, cudaEventDisableTiming));
+    for (int k = 0; k < S; ++k) TT_CUDA(ctx, cudaEventCreateWithFlags(&sl.ev_copy[k], cudaEventDisableTiming));
     for (int k = 0; k <= TT_STAGE_COUNT; ++k) TT_CUDA(ctx, cudaEventCreate(&sl.stage_ev[k]));
   }
   bind_slot(ctx, 0);
@@ -748,7 +749,8 @@ void release(tt_ctx* ctx) {
     if (sl.status_host) cudaFreeHost(sl.status_host);
     if (sl.ev_start) cudaEventDestroy(sl.ev_start);
     if (sl.ev_stop) cudaEventDestroy(sl.ev_stop);
-    if (sl.ev_copy) cudaEventDestroy(sl.ev_copy);
+    for (cudaEvent_t e : sl.ev_copy)
+      if (e) cudaEventDestroy(e);
     for (int k = 0; k <= TT_STAGE_COUNT; ++k)
       if (sl.stage_ev[k]) cudaEventDestroy(sl.stage_ev[k]);
   }
@@ -834,6 +836,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int n0, int K, const FramePtrs& frames, cons
     q.epilogue = EPI_LSTM_F32_NCHW; q.c_state = ctx->c_state; q.h_state = ctx->h_f32; q.c_idx = c_idx; q.h_out_idx = h_out;
     q.hidden = ctx->Ch;
     TT_CUDA(ctx, launch_conv_simt(q, s));
+    ctx->n_stepped = n0 + K;
     if ((ms_ = mark_stage(ctx, TT_STAGE_CONVLSTM, 1)) != TT_OK) return ms_;
     }
   } else {
@@ -920,6 +923,7 @@ tt_status enqueue_tick(tt_ctx* ctx, int n0, int K, const FramePtrs& frames, cons
       q.c_idx = c_idx; q.h_out_idx = h_out; q.hidden = ctx->Ch;
       TT_CUDA(ctx, launch_conv_tc(q, ctx->sm_count, s));
     }
+    ctx->n_stepped = n0 + K;
     if ((ms_ = mark_stage(ctx, TT_STAGE_CONVLSTM, 1)) != TT_OK) return ms_;
     }
   }
@@ -1034,10 +1038,12 @@ tt_status launch_part(tt_ctx* ctx, int slot, int tab, int n0, int K, const Frame
   if (tg && tg->exec) {
     if ((st = refresh_table()) != TT_OK) return st;
     TT_CUDA(ctx, cudaGraphLaunch(tg->exec, s));
+    ctx->n_stepped = n0 + K;
     ctx->n_launches += tg->launches;
   } else if (tg && (tg->seen >= 1 || family_warm)) {
     // capture the sequence, then launch it
     const uint64_t launches_before = ctx->n_launches;
+    const int stepped_before = ctx->n_stepped;
     cudaGraph_t graph = nullptr;
     cudaError_t ce = cudaStreamBeginCapture(s, cudaStreamCaptureModeThreadLocal);
     if (ce == cudaSuccess) {
@@ -1047,6 +1053,7 @@ tt_status launch_part(tt_ctx* ctx, int slot, int tab, int n0, int K, const Frame
     }
     if (st == TT_OK && ce == cudaSuccess && graph) ce = cudaGraphInstantiate(&tg->exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
+    ctx->n_stepped = stepped_before;
     if (st != TT_OK || ce != cudaSuccess || !tg->exec) {
       // capture is an optimisation only: clear the error, switch it off and run this tick directly
       cudaGetLastError();
@@ -1060,6 +1067,7 @@ tt_status launch_part(tt_ctx* ctx, int slot, int tab, int n0, int K, const Frame
       tg->launches = ctx->n_launches - launches_before;
       if ((st = refresh_table()) != TT_OK) return st;
       TT_CUDA(ctx, cudaGraphLaunch(tg->exec, s));
+      ctx->n_stepped = n0 + K;
     }
   } else {
     if ((st = refresh_table()) != TT_OK) return st;
@@ -1259,45 +1267,67 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
   // With nothing else in flight a tick of host frames is cut into parts, each launched when its frames have arrived (submits behind
   // others need no cut: their copies run while those compute).  A stream's results do not depend on what shares its launches.
   const int part = any_h2d && !ctx->profiling && ctx->q_count == 0 ? part_size(ctx, K) : K;
-  tt_status st = TT_OK;
-  for (int n0 = 0, n1; n0 < K; n0 = n1) {
-    n1 = n0 == 0 && K % part ? K % part : n0 + part;   // the odd part first
-    bool copied = false;
+  const auto part_end = [&](int n0) { return n0 == 0 && K % part ? K % part : n0 + part; };   // the odd part first
+  ctx->n_stepped = 0;
+  bool launching = false;
+  // An error behind this point leaves nothing of the submit in flight, so that the caller's frames are its own again and the slot's buffers may
+  // be written anew.  Streams whose step had been enqueued have taken their frame, whole (c in place, h in the other half), and the error says so.
+  const auto give_up = [&](tt_status st) -> tt_status {
+    const std::string why = ctx->err;
+    cudaStreamSynchronize(ctx->copy_stream);
+    cudaStreamSynchronize(s);
+    cudaGetLastError();   // so that a later launch does not find it
+    for (int n = 0; n < ctx->n_stepped; ++n) states[n]->half ^= 1;
+    if (launching)
+      for (tt_state& x : ctx->states) x.last_pos = -1;   // the intermediate tensors are no completed submit's
+    if (!ctx->n_stepped) return fail(ctx, st, "%s; no stream has taken its frame", why.c_str());
+    return fail(ctx, st, "%s; the streams of frames[0..%d] have taken theirs, the others have not", why.c_str(), ctx->n_stepped - 1);
+  };
+  // Every copy is accepted before anything is launched: a frame that cannot be copied leaves all streams as they were.  Host frames go over a copy
+  // stream of their own, so the copies can run while an earlier part or tick still computes.  Frames that lie one behind the other in
+  // one pinned buffer travel as one copy (six of 854x480: 180 us as six, 153 us as one).
+  const auto copy_part = [&](int n0, int n1, bool* copied) -> tt_status {
     for (int n = n0; n < n1;) {
       if (frames[n].on_device) { ++n; continue; }
-      // host frames go over a copy stream of their own, so the copy can run while an earlier part or tick still
-      // computes; the compute stream waits for the copy below.  Frames that lie one behind the other in one pinned buffer travel as one
-      // copy (six of 854x480: 180 us as six, 153 us as one)
       int m = n + 1;
       while (m < n1 && !frames[m].on_device && frames[m].data == frames[m - 1].data + ctx->frame_bytes && same_pinned_range(frames[n].data, frames[m].data)) ++m;
       TT_CUDA(ctx, cudaMemcpyAsync(ctx->frames_stage + (size_t)n * ctx->frame_bytes, frames[n].data, (size_t)(m - n) * ctx->frame_bytes, cudaMemcpyHostToDevice, ctx->copy_stream));
-      copied = true;
+      *copied = true;
       n = m;
     }
-    if (copied) {
-      // recorded anew for every part: a wait keeps the record it was enqueued behind
-      TT_CUDA(ctx, cudaEventRecord(ctx->ev_copy, ctx->copy_stream));
-      TT_CUDA(ctx, cudaStreamWaitEvent(s, ctx->ev_copy, 0));
+    if (*copied) TT_CUDA(ctx, cudaEventRecord(ctx->slots[slot].ev_copy[n0], ctx->copy_stream));
+    return TT_OK;
+  };
+  // refreshes the chosen table; called in front of the tick's first launch (a graph capture, which enqueues nothing,
+  // comes before it, so that its host time stays outside the interval between the tick's events)
+  const auto refresh_table = [&]() -> tt_status {
+    TT_CUDA(ctx, record_start());
+    if (tab_miss) {
+      for (int n = 0; n < TT_MAX_STREAMS; ++n) ctx->frame_tab_last[slot][tab][n] = ctx->frame_tab_host[slot][n] = n < K ? fp.p[n] : nullptr;
+      ctx->frame_tab_valid[slot][tab] = false;   // stays so if the copy cannot be enqueued
+      TT_CUDA(ctx, cudaMemcpyAsync(ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS, ctx->frame_tab_host[slot],
+                                   sizeof(void*) * TT_MAX_STREAMS, cudaMemcpyHostToDevice, s));
+      ctx->frame_tab_valid[slot][tab] = true;
     }
-    // refreshes the chosen table; called in front of the tick's first launch (a graph capture, which enqueues nothing,
-    // comes before it, so that its host time stays outside the interval between the tick's events)
-    auto refresh_table = [&]() -> tt_status {
-      TT_CUDA(ctx, record_start());
-      if (n0 > 0) return TT_OK;
-      if (tab_miss) {
-        for (int n = 0; n < TT_MAX_STREAMS; ++n) ctx->frame_tab_last[slot][tab][n] = ctx->frame_tab_host[slot][n] = n < K ? fp.p[n] : nullptr;
-        ctx->frame_tab_valid[slot][tab] = false;   // stays so if the copy cannot be enqueued
-        TT_CUDA(ctx, cudaMemcpyAsync(ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS, ctx->frame_tab_host[slot],
-                                     sizeof(void*) * TT_MAX_STREAMS, cudaMemcpyHostToDevice, s));
-        ctx->frame_tab_valid[slot][tab] = true;
-      }
-      // everything that moves host data to the device (frames, pointer table) counts as the H2D stage
-      return mark_stage(ctx, TT_STAGE_H2D, 0);
-    };
-    if ((st = launch_part(ctx, slot, tab, n0, n1 - n0, fp, table, states, refresh_table)) != TT_OK) return st;
-  }
+    // everything that moves host data to the device (frames, pointer table) counts as the H2D stage
+    return mark_stage(ctx, TT_STAGE_H2D, 0);
+  };
+  const auto run_part = [&](int n0, int n1, bool copied) -> tt_status {
+    if (copied) TT_CUDA(ctx, cudaStreamWaitEvent(s, ctx->slots[slot].ev_copy[n0], 0));
+    return launch_part(ctx, slot, tab, n0, n1 - n0, fp, table, states, [&]() -> tt_status { return n0 > 0 ? TT_OK : refresh_table(); });
+  };
+  const auto finish = [&]() -> tt_status {
+    TT_CUDA(ctx, cudaEventRecord(ctx->ev_stop, s));
+    return TT_OK;
+  };
+  tt_status st = TT_OK;
+  bool copied[TT_MAX_STREAMS] = {};
+  for (int n0 = 0; n0 < K && st == TT_OK; n0 = part_end(n0)) st = copy_part(n0, part_end(n0), &copied[n0]);
+  launching = st == TT_OK;
+  for (int n0 = 0; n0 < K && st == TT_OK; n0 = part_end(n0)) st = run_part(n0, part_end(n0), copied[n0]);
+  if (st == TT_OK) st = finish();
+  if (st != TT_OK) return give_up(st);
   ctx->n_ticks += 1;
-  TT_CUDA(ctx, cudaEventRecord(ctx->ev_stop, s));
   for (int n = 0; n < TT_MAX_STREAMS; ++n) ctx->states[n].last_pos = -1;
   for (int n = 0; n < K; ++n) {
     ctx->frames_inflight[n] = frames[n];

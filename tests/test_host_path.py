@@ -1,0 +1,152 @@
+"""Host code of tt_submit_frames against a CUDA runtime that only writes down what it is asked for (no GPU needed)."""
+import ctypes as C
+import glob
+import os
+import re
+import subprocess
+
+import numpy as np
+import pytest
+
+import tt_synth
+from paper_2402_04466_b200 import binding
+from paper_2402_04466_b200 import build as build_mod
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def fake_path(tmp_path_factory):
+    """The library's own objects, linked with fake_cudart.c in the place of the CUDA runtime."""
+    build_mod.build()
+    objs = sorted(glob.glob(os.path.join(build_mod.OBJ_DIR, "*.o")))
+    if not objs:                      # a checkout that came with the library alone
+        build_mod.build(force=True)
+        objs = sorted(glob.glob(os.path.join(build_mod.OBJ_DIR, "*.o")))
+    d = tmp_path_factory.mktemp("fake")
+    include = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(build_mod._nvcc()))), "include")
+    subprocess.run(["gcc", "-O1", "-fPIC", "-I", include, "-c", os.path.join(HERE, "fake_cudart.c"), "-o", str(d / "fake.o")], check=True)
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-Wl,-z,defs", "-o", str(d / "libtt_fake.so"), *objs, str(d / "fake.o")], check=True)
+    return str(d / "libtt_fake.so")
+
+
+@pytest.fixture
+def fake(fake_path, monkeypatch):
+    monkeypatch.setattr(binding, "_LIB", None)
+    monkeypatch.setattr(binding, "LIB_PATH", fake_path)
+    lib = binding.load_library(build_if_missing=False)
+    lib.fake_log.restype = C.c_char_p
+    lib.fake_fail.argtypes = [C.c_char_p, C.c_int]
+    lib.fake_pinned.argtypes = [C.c_void_p, C.c_size_t]
+    lib.fake_reset()
+    return lib
+
+
+# copies of 124 us and 31 us of operations a stream, by the estimate: a tick of host frames runs in parts of one stream
+WORKLOAD = dict(src_w=1920, src_h=1080, net_w=320, net_h=240, enc_cout=(16, 32), enc_stride=(2, 2), hidden=32, n_tools=3)
+
+
+class Streams:
+    """A context of K streams, each with a frame in pinned host memory of its own."""
+
+    def __init__(self, lib, K, pad=0, workload=WORKLOAD, **options):
+        wl = tt_synth.workload("cfg0-gain").with_(name="host-path", **workload)
+        cfg = binding.make_config(wl, max_streams=K, **options)
+        cfg.src_pitch = 3 * wl.src_w + pad
+        self.lib, self.K, self.wl, self.bytes = lib, K, wl, wl.src_h * cfg.src_pitch
+        self.ctx = binding.Context(cfg, tt_synth.make_weights(wl))
+        self.states = [self.ctx.state_create() for _ in range(K)]
+        self.frames = [np.full(self.bytes, 10 + k, np.uint8) for k in range(K)]
+        for f in self.frames:
+            lib.fake_pinned(f.ctypes.data, f.size)
+        self.addr = [f.ctypes.data for f in self.frames]
+
+    def submit(self, on_device=()):
+        """Status and log of one tt_submit_frames."""
+        fr = (binding.tt_frame * self.K)()
+        for k in range(self.K):
+            fr[k].data, fr[k].on_device = self.addr[k], int(k in on_device)
+        status = self.ctx.submit_raw(self.K, fr, (C.c_void_p * self.K)(*[s.value for s in self.states]))
+        log = self.lib.fake_log().decode().splitlines()
+        self.lib.fake_reset()
+        return status, log
+
+    def sync(self):
+        self.ctx.sync()
+        self.lib.fake_reset()
+
+    def mark(self):
+        """Puts a value of its own into every stream's state: a stream that has taken a frame shows the other half of h, which holds another."""
+        self.base = getattr(self, "base", 0.0) + 100.0
+        for k, s in enumerate(self.states):
+            x = np.full((self.wl.hidden, self.ctx.hm, self.ctx.wm), self.base + k, np.float32)
+            self.ctx.state_import(s, x, x)
+        self.lib.fake_reset()
+
+    def advanced(self):
+        return [k for k, s in enumerate(self.states) if self.ctx.state_export(s)[0].flat[0] != self.base + k]
+
+
+def _first(log, *words):
+    return next((i for i, line in enumerate(log) if line.startswith(words)), len(log))
+
+
+def _copies(log):
+    """[(from, bytes, to)] of the copies into device memory, pointer tables apart."""
+    found = [re.match(r"copy in (\d+) from (0x\w+) to (0x\w+)", line) for line in log]
+    return [(int(m[2], 16), int(m[1]), int(m[3], 16)) for m in found if m and int(m[1]) != 8 * binding.TT_MAX_STREAMS]
+
+
+@pytest.mark.parametrize("warm", [0, 8])
+@pytest.mark.parametrize("nth", [1, 2, 4])
+def test_a_frame_that_cannot_be_copied_leaves_every_stream_as_it_was(fake, nth, warm):
+    """A tick in parts launches nothing before all of its frames have been accepted, neither plainly nor from graphs."""
+    s = Streams(fake, 4)
+    for _ in range(warm):
+        assert s.submit()[0] == binding.TT_OK
+        s.sync()
+    s.mark()
+    fake.fake_fail(b"cudaMemcpyAsync", nth)
+    status, log = s.submit()
+    assert status == 4 and "failed cudaMemcpyAsync" in log       # TT_ERR_CUDA
+    assert _first(log, "launch", "replay", "capture") == len(log) and log.count("drain") == 2
+    assert "no stream has taken its frame" in s.ctx.last_error() and "cudaMemcpyAsync" in s.ctx.last_error()
+    assert s.advanced() == []
+    fake.fake_reset()
+    status, log = s.submit()                                     # the caller tries again
+    assert status == binding.TT_OK and [c[0] for c in _copies(log)] == s.addr
+    last_copy = max(i for i, line in enumerate(log) if line.startswith("copy in") and " 64 " not in line)
+    assert last_copy < _first(log, "launch", "replay", "capture")
+    assert sum(line.startswith("wait") for line in log) == 4     # ... and was cut into four parts
+    s.sync()
+    assert s.advanced() == [0, 1, 2, 3]
+
+
+@pytest.mark.parametrize("call,nth,taken", [
+    ("cudaGraphLaunch", 1, 0), ("cudaGraphLaunch", 3, 2), ("cudaStreamWaitEvent", 2, 1), ("cudaEventRecord", 6, 4),   # the tick's last event
+    ("cudaLaunchKernel", 5 + 3, 1),       # an encoder layer of the second part
+    ("cudaLaunchKernel", 5 + 4, 1),       # its recurrent step
+    ("cudaLaunchKernel", 5 + 5, 2),       # the heads behind it
+])
+def test_a_launch_that_fails_leaves_every_stream_before_or_behind_its_frame(fake, call, nth, taken):
+    """Streams whose recurrent step had been enqueued have taken their frame, the others have not, the error names them, and nothing is left in
+    flight: the next submit works on either."""
+    s = Streams(fake, 4, plain_launches=call == "cudaLaunchKernel")
+    for _ in range(8):
+        assert s.submit()[0] == binding.TT_OK
+        s.sync()
+    s.mark()
+    fake.fake_fail(call.encode(), nth)
+    status, log = s.submit()
+    assert status == 4 and f"failed {call}" in log and log[-2:] == ["drain", "drain"]
+    error = s.ctx.last_error()
+    assert (f"frames[0..{taken - 1}] have taken" if taken else "no stream has taken") in error
+    assert s.advanced() == list(range(taken))
+    with pytest.raises(binding.TTError):
+        s.ctx.debug_tensor(s.states[0], "prob")                  # no completed submit's
+    assert s.ctx.query() is False                                # nothing in flight
+    s.mark()
+    fake.fake_reset()
+    assert s.submit()[0] == binding.TT_OK
+    s.sync()
+    assert s.advanced() == [0, 1, 2, 3]
