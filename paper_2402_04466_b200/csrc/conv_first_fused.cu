@@ -54,7 +54,8 @@ struct Tile {
   int img, tx, ty;
 };
 
-template <int COUT, int STRIDE>
+// OWN_OUT: output waits for its tile stores in shared memory of its own and not in the operand's.
+template <int COUT, int STRIDE, bool OWN_OUT>
 __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel(const __grid_constant__ ConvFirstTcParams p) {
   constexpr int PW = ff_patch_w(STRIDE), PH = ff_patch_h(STRIDE), PITCH = ff_pitch(STRIDE);
   constexpr int FULL = PW / 32, EXTRA = PW - 32 * FULL;       // whole warps of patch columns, from the tile's first own column on, and the rest
@@ -62,8 +63,8 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
   constexpr int A_BYTES = 2 * 128 * 64;
   extern __shared__ __align__(1024) uint8_t smem[];
   uint8_t* s_a = smem;                                        // operand: two tiles of [128 rows][32] bf16
-  uint8_t* s_out = s_a + A_BYTES;                             // per warp 32 pixels x 32 channels on their way out
-  uint8_t* s_b = s_out + FF_WARPS * 2048;                     // weights in operand layout
+  uint8_t* s_out = s_a + A_BYTES;                             // OWN_OUT: per warp 32 pixels x 32 channels on their way out
+  uint8_t* s_b = s_out + (OWN_OUT ? FF_WARPS * 2048 : 0);     // weights in operand layout
   float* s_bias = reinterpret_cast<float*>(s_b + COUT * 64);
   __nv_bfloat16* s_patch = reinterpret_cast<__nv_bfloat16*>(s_bias + COUT);      // [3][PH][PITCH]
   uint8_t* s_src = reinterpret_cast<uint8_t*>(s_patch) + ((3 * PH * PITCH * 2 + 15) & ~15);   // [2][src_rows_cap][src_row_cap]
@@ -243,14 +244,14 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     const uint32_t taddr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * COUT);
     const int y = t.ty * FF_TH + warp, x0 = t.tx * FF_TW;
     // 32 channels of the warp's row of 32 pixels leave as one tile store, which clips what lies outside the map.  They wait for it in 2 KB of
-    // the warp's own, the first half of 64 channels in the part of the operand that the warp's own gather fills next.
-    // 16-byte piece c of pixel i lies at piece c ^ (i / 2 % 4), the swizzle of the store's map.
+    // the warp's own (OWN_OUT), the first half of 64 channels in the part of the operand that the warp's own gather fills next; without memory of
+    // their own all wait there, one half behind the other.  16-byte piece c of pixel i lies at piece c ^ (i / 2 % 4), the swizzle of the store's map.
 #pragma unroll
     for (int ck = 0; ck < COUT / 32; ++ck) {
-      uint8_t* mine = (ck + 1 < COUT / 32 ? s_a : s_out) + warp * 2048;
+      uint8_t* mine = (OWN_OUT && ck + 1 == COUT / 32 ? s_out : s_a) + warp * 2048;
       uint32_t v[32];
       tmem_ld32(taddr + (uint32_t)(ck * 32), v);
-      if (ck == 0) {   // the stores of the tile before have been read
+      if (OWN_OUT ? ck == 0 : ck > 0) {   // the stores of the tile before (the half before) have been read
         if (lane == 0) bulk_wait_group_read0();
         __syncwarp();
       }
@@ -272,8 +273,11 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
         bulk_commit_group();
       }
     }
-    if (COUT > 32) {   // the operand's part has been read
-      if (lane == 0) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+    if (COUT > 32 || !OWN_OUT) {          // the operand's part has been read
+      if (lane == 0) {
+        if (OWN_OUT) asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory");
+        else bulk_wait_group_read0();
+      }
       __syncwarp();
     }
   };
@@ -357,19 +361,45 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
   }
 }
 
-template <int COUT, int STRIDE>
-cudaError_t launch_t(const ConvFirstTcParams& p, int sm_count, cudaStream_t s) {
-  const int smem = 2 * 128 * 64 + FF_WARPS * 2048 + COUT * 64 + COUT * 4 + ((3 * ff_patch_h(STRIDE) * ff_pitch(STRIDE) * 2 + 15) & ~15) + 2 * p.src_rows_cap * p.src_row_cap;
-  auto kern = conv_first_fused_kernel<COUT, STRIDE>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+// Dynamic shared memory of a block whose two buffers of frame rows take src_bytes.
+template <int COUT, int STRIDE, bool OWN_OUT>
+constexpr int ff_smem(int src_bytes) {
+  return 2 * 128 * 64 + (OWN_OUT ? FF_WARPS * 2048 : 0) + COUT * 64 + COUT * 4 + ((3 * ff_patch_h(STRIDE) * ff_pitch(STRIDE) * 2 + 15) & ~15) + src_bytes;
+}
+
+// Blocks of a form that a multiprocessor holds, by shared memory: a block takes 1 KB beside its own, and its static variables' up to the
+// alignment of the dynamic part.
+template <int COUT, int STRIDE, bool OWN_OUT>
+constexpr int ff_per_sm(int src_bytes) {
+  constexpr int SMEM_SM = 228 * 1024, BESIDE = 1024 + 1024;
+  const int n = SMEM_SM / (ff_smem<COUT, STRIDE, OWN_OUT>(src_bytes) + BESIDE);
+  return n < FF_PER_SM ? n : FF_PER_SM;
+}
+
+template <int COUT, int STRIDE, bool OWN_OUT>
+cudaError_t launch_form(const ConvFirstTcParams& p, int src_bytes, int sm_count, cudaStream_t s) {
+  auto kern = conv_first_fused_kernel<COUT, STRIDE, OWN_OUT>;
+  // the most the form ever takes: the same value whichever context launches
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, ff_smem<COUT, STRIDE, OWN_OUT>(FF_SRC_BUDGET));
   if (e != cudaSuccess) return e;
   ConvFirstTcParams q = p;
   q.tiles_x = (p.Wo + FF_TW - 1) / FF_TW;
   q.tiles_y = (p.Ho + FF_TH - 1) / FF_TH;
-  const int total = p.K * q.tiles_x * q.tiles_y, slots = FF_PER_SM * sm_count, grid = total < slots ? total : slots;
+  const int total = p.K * q.tiles_x * q.tiles_y, slots = ff_per_sm<COUT, STRIDE, OWN_OUT>(src_bytes) * sm_count, grid = total < slots ? total : slots;
   q.tiles_per_block = total / grid;
   q.tiles_left = total % grid;
-  return launch_kernel(kern, grid, FF_THREADS, (size_t)smem, s, q, false);
+  return launch_kernel(kern, grid, FF_THREADS, (size_t)ff_smem<COUT, STRIDE, OWN_OUT>(src_bytes), s, q, false);
+}
+
+// The frame rows under a patch grow with the resize factor: the output has memory of its own where that costs no block.  Full-HD frames, this layer, one
+// more and heads, five / eight streams, us a tick, two blocks with and three without such memory: to 960x540 with 64 channels 116 / 161 and 101 / 135, to
+// 856x480 with 32 channels 92 / 117 and 80 / 100.  Where two fit either way (to 768x432, 64 channels) a grid cut for three took 120, cut for two 107.5.
+template <int COUT, int STRIDE>
+cudaError_t launch_t(const ConvFirstTcParams& p, int sm_count, cudaStream_t s) {
+  const int src_bytes = 2 * p.src_rows_cap * p.src_row_cap;
+  static_assert(ff_per_sm<COUT, STRIDE, true>(FF_SRC_BUDGET) >= 1, "any staging leaves room for a block");
+  if (ff_per_sm<COUT, STRIDE, true>(src_bytes) >= ff_per_sm<COUT, STRIDE, false>(src_bytes)) return launch_form<COUT, STRIDE, true>(p, src_bytes, sm_count, s);
+  return launch_form<COUT, STRIDE, false>(p, src_bytes, sm_count, s);
 }
 
 }  // namespace

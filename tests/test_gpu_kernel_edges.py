@@ -113,6 +113,17 @@ def test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cud
             assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("shape,K,pad", [
+    (dict(src_w=640, src_h=480, net_w=320, net_h=240, enc_cout=(64, 64), enc_stride=(2, 2)), 8, 3),     # 600 tiles; 2 x 64 output channels
+    (dict(src_w=420, src_h=310, net_w=200, net_h=140), 3, 7),
+    (dict(src_w=402, src_h=258, net_w=100, net_h=65, enc_stride=(1, 2, 2)), 2, 1),
+    (dict(src_w=400, src_h=260, net_w=100, net_h=65, enc_cout=(64, 64), enc_stride=(1, 2)), 2, 0),
+])
+def test_first_layer_whose_output_waits_in_the_operand_changes_no_bit(cuda_device, shape, K, pad):
+    """Resize factors of 2 and more: the staged frame rows leave no room for the output beside three blocks."""
+    test_first_layer_kernel_equals_preprocessing_and_convolution_bit_for_bit(cuda_device, shape, K, pad)
+
+
 @pytest.mark.parametrize("net,enc,stride,hidden,K", [
     ((150, 110), (32, 128), (1, 2), 64, 2),            # 32 -> 128, 75 x 55 outputs: ragged in both directions
     ((66, 66), (64, 64), (1, 2), 64, 1),               # 64 -> 64, a last tile of one column and one row

@@ -150,3 +150,27 @@ def test_a_launch_that_fails_leaves_every_stream_before_or_behind_its_frame(fake
     assert s.submit()[0] == binding.TT_OK
     s.sync()
     assert s.advanced() == [0, 1, 2, 3]
+
+
+@pytest.mark.parametrize("src,net,cout,stride", [
+    ((854, 480), (640, 480), 32, 2), ((1920, 1080), (1280, 720), 64, 2),       # memory of its own for the output
+    ((1920, 1080), (960, 540), 64, 2), ((1280, 960), (640, 480), 64, 2),       # twice the network's size
+    ((1920, 1080), (856, 480), 32, 2), ((1920, 1080), (800, 448), 64, 2),
+    ((1280, 720), (320, 180), 32, 1), ((1280, 720), (320, 180), 64, 1),
+    ((1920, 1080), (768, 432), 64, 2),                                         # almost as much staging as the kernel takes
+])
+def test_the_first_layers_blocks_fit_and_its_grid_is_theirs(fake, src, net, cout, stride):
+    """Three blocks to a multiprocessor unless the frame rows under their patches alone leave room for two, and as many blocks as fit at once."""
+    w = dict(src_w=src[0], src_h=src[1], net_w=net[0], net_h=net[1], enc_cout=(cout, 64), enc_stride=(stride, 2), hidden=64, n_tools=3, precision="bf16")
+    s = Streams(fake, 2, workload=w)
+    log = s.submit(on_device=(0, 1))[1]
+    (m,) = [m for m in (re.match(r"launch \S*conv_first_fused_kernelILi(\d+)ELi(\d)E(?:Lb([01])E)?\S* grid (\d+) 1 1 smem (\d+)", line) for line in log) if m]
+    assert (int(m[1]), int(m[2])) == (cout, stride)
+    own, grid, smem = int(m[3] or 1), int(m[4]), int(m[5])
+    least = smem - own * 8 * 2048
+    fits, could = (min(3, 228 * 1024 // (b + 2048)) for b in (smem, least))
+    assert fits == could and (own or min(3, 228 * 1024 // (least + 8 * 2048 + 2048)) < could)
+    assert could == 3 or least + 2048 > 228 * 1024 // 3
+    ho, wo = ((n - 1) // stride + 1 for n in (net[1], net[0]))
+    assert grid == min(2 * ((wo + 31) // 32) * ((ho + 7) // 8), fits * 148)
+    s.sync()
