@@ -968,25 +968,27 @@ tt_status enqueue_tick(tt_ctx* ctx, int n0, int K, const FramePtrs& frames, cons
   return TT_OK;
 }
 
-// Streams per part of a tick of K host frames: the part size for which the estimated time from the first copy to the last launch's end is
+// Streams per part of a tick of K frames, some of them host frames (the others need no copy): the part size for which the estimated time from the first copy to the last launch's end is
 // least, K where cutting saves less than a twentieth.  A frame takes its bytes at 50 GB/s (pinned memory); a part computes for 45 us (launches,
 // start-up, latency chains, and what copies lose beside kernels) and its streams' operations at 1.3 PFLOP/s (fp32 path: 25 TFLOP/s).  A 854x480 stream:
 // 25 us to copy, 10 to compute; a full-HD one 124 and 118.  Measured, us a tick uncut / in parts of 1 / 2 / 3 / 4 streams (* chosen): 854x480 with
 // overlay, three streams 164* 199 160 164, four 198 265 190 193* 198, six 266 344 271 254* 247, eight without overlay 322 432 322 285* 286; full-HD, two
 // 492 416*, four 937 722* 729 831, eight 1822 1336 1289* 1313 1406; six feed-forward 854x480 206* 232 200 200 205; eight 428x240 on the fp32
 // path 247* 488 344 295 263.
-int part_size(const tt_ctx* ctx, int K) {
+int part_size(const tt_ctx* ctx, int K, const tt_frame* frames) {
   double ops = 0;
   for (int l = 0; l < ctx->n_enc; ++l) ops += 18.0 * ctx->lay_c[l] * ctx->lay_c[l + 1] * ctx->lay_h[l + 1] * ctx->lay_w[l + 1];
   if (!ctx->feed_forward) ops += 72.0 * (ctx->Cx + ctx->Ch) * ctx->Ch * ctx->Hm * ctx->Wm;
   const double copy = (double)ctx->frame_bytes / 50e9, fixed = 45e-6, stream = ops / (ctx->bf16 ? 1.3e15 : 25e12);
+  int on_host[TT_MAX_STREAMS + 1] = {};   // of the first n frames
+  for (int n = 0; n < K; ++n) on_host[n + 1] = on_host[n] + (frames[n].on_device ? 0 : 1);
   int best = K;
-  double best_t = 0.95 * (K * copy + fixed + K * stream);
+  double best_t = 0.95 * (on_host[K] * copy + fixed + K * stream);
   for (int k = 1; k < K; ++k) {
     double arrived = 0, done = 0;
     for (int n0 = 0, n1; n0 < K; n0 = n1) {
       n1 = n0 == 0 && K % k ? K % k : n0 + k;
-      arrived += (n1 - n0) * copy;
+      arrived = on_host[n1] * copy;
       done = std::max(done, arrived) + fixed + (n1 - n0) * stream;
     }
     if (done < best_t) { best_t = done; best = k; }
@@ -1266,7 +1268,7 @@ tt_status tt_submit_frames(tt_ctx* ctx, int32_t K, const tt_frame* frames, tt_st
   const uint8_t* const* const table = ctx->frame_tab_dev[slot] + tab * TT_MAX_STREAMS;
   // With nothing else in flight a tick of host frames is cut into parts, each launched when its frames have arrived (submits behind
   // others need no cut: their copies run while those compute).  A stream's results do not depend on what shares its launches.
-  const int part = any_h2d && !ctx->profiling && ctx->q_count == 0 ? part_size(ctx, K) : K;
+  const int part = any_h2d && !ctx->profiling && ctx->q_count == 0 ? part_size(ctx, K, frames) : K;
   const auto part_end = [&](int n0) { return n0 == 0 && K % part ? K % part : n0 + part; };   // the odd part first
   ctx->n_stepped = 0;
   bool launching = false;

@@ -174,3 +174,23 @@ def test_the_first_layers_blocks_fit_and_its_grid_is_theirs(fake, src, net, cout
     ho, wo = ((n - 1) // stride + 1 for n in (net[1], net[0]))
     assert grid == min(2 * ((wo + 31) // 32) * ((ho + 7) // 8), fits * 148)
     s.sync()
+
+
+def _parts(log):
+    """Launch sequences of a tick that ran plainly: each begins with the resize (or the first layer that contains it)."""
+    return sum(bool(re.match(r"launch \S*(preprocess|conv_first_fused)", line)) for line in log)
+
+
+@pytest.mark.parametrize("on_device,parts", [
+    ((), 8),                                  # 8 x (124 + 31) us one behind the other, or compute under the copies
+    ((0, 1, 2, 3, 4, 5, 6), 2),               # one copy of 124 us, under 45 + 4 x 31 us of the first part
+    ((0, 1, 2, 4, 5, 6, 7), 2),
+    ((1, 2, 3, 4, 5, 6, 7), 1),               # nothing to compute before it has arrived
+    ((0, 1, 2, 3, 4, 5, 6, 7), 1),
+])
+def test_a_tick_is_cut_by_the_frames_that_have_to_be_copied(fake, on_device, parts):
+    """Frames that are on the device already do not arrive one behind the other."""
+    s = Streams(fake, 8, plain_launches=True)
+    status, log = s.submit(on_device)
+    assert status == binding.TT_OK and _parts(log) == parts and len(_copies(log)) == 8 - len(on_device)
+    s.sync()
