@@ -998,11 +998,10 @@ int part_size(const tt_ctx* ctx, int K, const tt_frame* frames) {
 
 // Launches batch positions n0 .. n0 + K - 1 of the tick being submitted (fp, table and states are the whole tick's).
 //
-// The launch sequence is replayed from a CUDA graph.  Which kernel variants it launches depends
-// on the stream count and the frames' alignment alone, so the first launch of such a family runs as plain
-// launches (modules load, attributes are set outside any capture); after it, every new (positions, slot, pointer
-// table, state placement) of the family is captured the first time it shows up.  With stage events
-// requested the tick always runs as plain launches.
+// The launch sequence is replayed from a CUDA graph.  Which kernel variants it launches depends on the stream count and on the alignment
+// of frames and overlay alone, so the first launch of such a family runs as plain launches (modules load, attributes are set outside any capture); after
+// it, every new (positions, slot, pointer table, state placement) of the family is captured the first time it shows up.  With stage
+// events requested the tick always runs as plain launches.
 template <typename Refresh>
 tt_status launch_part(tt_ctx* ctx, int slot, int tab, int n0, int K, const FramePtrs& tick_fp, const uint8_t* const* table, tt_state* const* tick_states,
                       Refresh refresh_table) {
@@ -1015,8 +1014,9 @@ tt_status launch_part(tt_ctx* ctx, int slot, int tab, int n0, int K, const Frame
   tt_ctx::TickGraph* tg = nullptr;
   bool family_warm = false;
   if (!ctx->graphs_off && !ctx->profiling) {
-    int flat = 1;
-    // the overlay launch picks its word-wise variant from the frames' 4-byte alignment: part of the key
+    // the overlay launch picks its word-wise variant by the 4-byte alignment of the frames and the 16-byte alignment of its output, which in a part
+    // begins behind n0 images: part of the key
+    int flat = !ctx->overlay || ((uintptr_t)(ctx->overlay + (size_t)n0 * ctx->cfg.src_w * ctx->cfg.src_h * 4) & 15) == 0 ? 1 : 0;
     for (int n = 0; n < K; ++n) flat &= (((uintptr_t)fp.p[n] & 3) == 0) ? 1 : 0;
     for (auto& g : ctx->graphs) {
       family_warm |= g.K == K && g.flat == flat && (g.seen >= 1 || g.exec);

@@ -194,3 +194,29 @@ def test_a_tick_is_cut_by_the_frames_that_have_to_be_copied(fake, on_device, par
     status, log = s.submit(on_device)
     assert status == binding.TT_OK and _parts(log) == parts and len(_copies(log)) == 8 - len(on_device)
     s.sync()
+
+
+@pytest.mark.parametrize("src,on_device,shift", [
+    ((1917, 1081), (1,), 0),               # an aligned device frame whose overlay begins between 16-byte boundaries, in a part of its own
+    ((1917, 1081), (1,), 1),
+    ((1918, 1081), (), 0),
+])
+def test_no_kernel_runs_for_the_first_time_inside_a_capture(fake, src, on_device, shift):
+    """Neither a tick nor a part of one is captured with a variant that has not run plainly before."""
+    s = Streams(fake, 4, workload=dict(WORKLOAD, src_w=src[0], src_h=src[1]), overlay=True)
+    for k in on_device:
+        s.addr[k] += shift - s.addr[k] % 4
+        fake.fake_pinned(s.addr[k], s.bytes)
+    ran, captured = set(), set()
+    for _ in range(9):
+        status, log = s.submit(on_device)
+        assert status == binding.TT_OK
+        for line in log:
+            if line.startswith("launch"):
+                ran.add(line.split()[1])
+            if line.startswith("capture"):
+                assert line.split()[1] in ran
+                captured.add(line.split()[1])
+        s.sync()
+    assert any("overlay_kernel" in k for k in captured)
+    assert len([k for k in ran if "overlay_kernel" in k]) == 2      # word by word where frames and output allow it, byte by byte elsewhere
