@@ -38,6 +38,8 @@ void fake_pinned(void* p, size_t n) {
   pinned[n_pinned++ % 64].hi = (uintptr_t)p + n;
 }
 
+void fake_unpin(void) { n_pinned = 0; }
+
 void** __cudaRegisterFatBinary(void* f) { (void)f; static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void** h) { (void)h; }
 void __cudaUnregisterFatBinary(void** h) { (void)h; }

@@ -165,17 +165,17 @@ def test_stride2_layer_kernels_give_the_same_bits_at_small_and_large_batches(cud
         ctx.destroy()
 
 
-# units on 148, 128, 100 and 78 multiprocessors (0, 20, 48 and 70 reserved); "full": the kernel of full rounds
+# groups of columns on 148, 128, 100 and 78 multiprocessors (0, 20, 48 and 70 reserved); single blocks, pairs of blocks beyond one round of units of 256
 @pytest.mark.parametrize("hidden,net", [
-    (64, (640, 840)),      # 70 tiles of one group of 256: cut into halves on 148, else full
-    (128, (640, 480)),     # 40 tiles x 512 columns: 192, 192 and 128, but full on 100
+    (64, (640, 840)),      # 70 tiles of one group of 256: cut into halves on 148, else whole
+    (128, (640, 480)),     # 40 tiles x 512 columns: 192, 192 and 128, whole on 100, on pairs again 192, 192 and 128 on 78
     (128, (400, 300)),     # 21 ragged tiles x 512: halves, but 192, 192 and 128 on 78
-    (256, (1280, 720)),    # 120 tiles x 1024: several rounds of 256, the last cut into halves; full on 128 and 100
-    (256, (368, 480)),     # 24 ragged tiles x 1024: five groups of 192 and one of 64 on 148 and 78, else full
+    (256, (1280, 720)),    # 120 tiles x 1024, on pairs: several rounds of 256, the last cut into halves on 148 and 78, whole on 128 and 100
+    (256, (368, 480)),     # 24 ragged tiles x 1024: five groups of 192 and one of 64 on 148 and, on pairs, on 78; whole on 128 and 100
 ])
 def test_convlstm_column_groups_change_no_bit(cuda_device, hidden, net):
-    """How many multiprocessors there are decides how the gates' columns are grouped into units (or that the kernel of full rounds
-    runs): every grouping adds up the same products in the same order, so probabilities, confidences and state are the same bits."""
+    """How many multiprocessors there are decides how the gates' columns are grouped into units, and whether these run on pairs of
+    blocks: every form adds up the same products in the same order, so probabilities, confidences and state are the same bits."""
     wl = tt_synth.workload("cfg1-gain").with_(name="groups", src_w=net[0] + 30, src_h=net[1] + 20, net_w=net[0], net_h=net[1], hidden=hidden)
     host = _frames(wl, 1, 2)[0]
     w = tt_synth.make_weights(wl)
@@ -196,9 +196,11 @@ def test_convlstm_column_groups_change_no_bit(cuda_device, hidden, net):
 
 
 @pytest.mark.parametrize("hidden,net,K", [
-    (128, (400, 300), 5),     # 105 tiles: the last pair has no second tile
+    (128, (400, 300), 5),     # 105 tiles: the last pair has no second tile; the second round cut into halves
     (64, (400, 300), 8),      # one group of columns
-    (256, (368, 480), 3),     # 72 ragged tiles x 1024 columns: several rounds, the last cut into halves
+    (256, (368, 480), 3),     # 72 ragged tiles x 1024 columns: two rounds of whole groups
+    (256, (368, 480), 2),     # 48: five groups of 192 and one of 64
+    (512, (160, 120), 8),     # 24 tiles x 2048: ten groups of 192 and one of 128
 ])
 def test_convlstm_on_pairs_of_blocks_changes_no_bit(cuda_device, hidden, net, K):
     """Beyond one round of units the ConvLSTM runs on pairs of blocks: every stream must get the bits it gets alone, on single blocks."""

@@ -220,3 +220,47 @@ def test_no_kernel_runs_for_the_first_time_inside_a_capture(fake, src, on_device
         s.sync()
     assert any("overlay_kernel" in k for k in captured)
     assert len([k for k in ran if "overlay_kernel" in k]) == 2      # word by word where frames and output allow it, byte by byte elsewhere
+
+
+@pytest.mark.parametrize("K,pad,layout,on_device,expected", [
+    (3, 0, "one", (), [(0, 3)]),                     # one buffer: one copy
+    (3, 10, "one", (), [(0, 3)]),                    # rows padded to another pitch
+    (4, 0, "one", (2,), [(0, 2), (3, 1)]),           # a frame in between that is on the device
+    (3, 0, "gap", (), [(0, 1), (1, 1), (2, 1)]),     # 64 bytes between the frames
+    (3, 0, "backwards", (), [(0, 1), (1, 1), (2, 1)]),
+    (3, 0, "neighbours", (), [(0, 2), (2, 1)]),      # two page-locked ranges, one right behind the other
+    (3, 0, "pageable", (), [(0, 1), (1, 1), (2, 1)]),
+])
+@pytest.mark.parametrize("cut", [False, True])
+def test_frames_that_lie_one_behind_the_other_travel_as_one_copy(fake, K, pad, layout, on_device, expected, cut):
+    """Every frame arrives in its place of the staging buffer, whatever travels together; no copy reaches over the edge of a part or out of a
+    page-locked range, and none takes a frame that is on the device."""
+    small = dict(WORKLOAD, src_w=340, src_h=250)
+    s = Streams(fake, K, pad=pad, workload=WORKLOAD if cut else small, plain_launches=True)     # cut: parts of one stream
+    fake.fake_unpin()
+    step = s.bytes + (64 if layout == "gap" else 0)
+    buf = np.repeat(np.arange(1, K + 1, dtype=np.uint8), step)
+    base = buf.ctypes.data
+    if layout == "neighbours":
+        fake.fake_pinned(base, 2 * step)
+        fake.fake_pinned(base + 2 * step, step)
+    elif layout != "pageable":
+        fake.fake_pinned(base, buf.size)
+    order = range(K)[::-1] if layout == "backwards" else range(K)
+    s.addr = [base + i * step for i in order]
+    status, log = s.submit(on_device)
+    assert status == binding.TT_OK
+    assert _parts(log) == (K if cut else 1)
+    copies = _copies(log)
+    staging = copies[0][2] - next(n for n in range(K) if n not in on_device) * s.bytes
+    got = [((to - staging) // s.bytes, size // s.bytes) for _, size, to in copies]
+    assert all((to - staging) % s.bytes == 0 and size % s.bytes == 0 for _, size, to in copies)
+    if cut:
+        assert got == [(n, 1) for n in range(K) if n not in on_device]
+    else:
+        assert got == expected
+    for n in range(K):
+        if n not in on_device:
+            staged = np.ctypeslib.as_array((C.c_uint8 * s.bytes).from_address(staging + n * s.bytes))
+            assert np.array_equal(staged, buf[order[n] * step:order[n] * step + s.bytes])
+    s.sync()
