@@ -19,6 +19,7 @@ using namespace pre;
 constexpr int PRE_THREADS = 256, PRE_PER_SM = 4;   // four full-HD frames: 20.5, 18.4, 18.5, 20.5, 22.5, 24.6 us with 2, 3, 4, 5, 6, 8 blocks
 constexpr int PRE_MAX_ROWS = 32;             // output rows of a tile
 constexpr int PRE_STAGE_BYTES = 26 * 1024;   // staged rows of a tile; two tiles of four blocks fit a multiprocessor
+constexpr int PRE_STATIC_BYTES = 2 * PRE_MAX_ROWS * 16;   // the kernel's row tables
 
 struct PreprocessArgs {
   PreprocessParams p;
@@ -215,7 +216,7 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   a.tiles_left = (int)(total % grid);
   const size_t smem = (size_t)2 * a.rows_cap * a.row_cap;
   auto kern = p.src_h == p.net_h ? preprocess_staged_kernel<COLS, true> : preprocess_staged_kernel<COLS, false>;
-  if (smem > 48 * 1024) {
+  if (smem + PRE_STATIC_BYTES > 48 * 1024) {   // what a kernel may have of both without asking
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * PRE_STAGE_BYTES);
     if (e != cudaSuccess) return e;
   }

@@ -11,7 +11,8 @@ static char log_text[1 << 20];
 static size_t log_len;
 static int capturing, captured, fail_in;
 static char fail_name[64];
-static struct { const void* host; const char* name; } kernels[512];
+static cudaError_t last_error;
+static struct { const void* host; const char* name; size_t max_smem; } kernels[512];
 static int n_kernels;
 static struct { uintptr_t lo, hi; } pinned[64];
 static int n_pinned;
@@ -46,7 +47,11 @@ void __cudaUnregisterFatBinary(void** h) { (void)h; }
 void __cudaRegisterVar(void** h, char* v, char* a, const char* n, int e, size_t s, int c, int g) { (void)h; (void)v; (void)a; (void)n; (void)e; (void)s; (void)c; (void)g; }
 void __cudaRegisterFunction(void** h, const char* host, char* dev, const char* name, int lim, uint3* t, uint3* b, dim3* bd, dim3* gd, int* w) {
   (void)h; (void)dev; (void)lim; (void)t; (void)b; (void)bd; (void)gd; (void)w;
-  if (n_kernels < 512) { kernels[n_kernels].host = host; kernels[n_kernels++].name = name; }
+  if (n_kernels < 512) {
+    kernels[n_kernels].host = host;
+    kernels[n_kernels].max_smem = 47 * 1024;   /* 48 KB without asking, static variables (up to 1 KB here) included */
+    kernels[n_kernels++].name = name;
+  }
 }
 static struct { dim3 grid, block; size_t smem; void* stream; } pushed;
 unsigned __cudaPushCallConfiguration(dim3 grid, dim3 block, size_t smem, void* s) {
@@ -61,7 +66,11 @@ static cudaError_t launch(const char* call, const void* func, dim3 grid, size_t 
   cudaError_t e = done(call);
   const char* name = "?";
   for (int i = 0; i < n_kernels; ++i)
-    if (kernels[i].host == func) name = kernels[i].name;
+    if (kernels[i].host == func) {
+      name = kernels[i].name;
+      if (smem > kernels[i].max_smem) e = cudaErrorInvalidValue;
+    }
+  if (e != cudaSuccess) last_error = e;
   if (e == cudaSuccess) {
     captured += capturing;
     note("%s %s grid %u %u %u smem %zu\n", capturing ? "capture" : "launch", name, grid.x, grid.y, grid.z, smem);
@@ -111,7 +120,11 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t s) {
 }
 cudaError_t cudaGraphDestroy(cudaGraph_t g) { free(g); return cudaSuccess; }
 cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { free(x); return cudaSuccess; }
-cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) { (void)f; (void)a; (void)v; return cudaSuccess; }
+cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) {
+  for (int i = 0; i < n_kernels; ++i)
+    if (kernels[i].host == f && a == cudaFuncAttributeMaxDynamicSharedMemorySize) kernels[i].max_smem = (size_t)v;
+  return v <= 227 * 1024 ? cudaSuccess : cudaErrorInvalidValue;
+}
 cudaError_t cudaGetSymbolAddress(void** p, const void* s) { *p = (void*)s; return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { (void)d; return cudaSuccess; }
@@ -126,7 +139,11 @@ cudaError_t cudaGetDeviceProperties(struct cudaDeviceProp* p, int d) {
 }
 cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void* f, const cudaLaunchConfig_t* c) { (void)f; (void)c; *n = 74; return cudaSuccess; }
 const char* cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "made by the test"; }
-cudaError_t cudaGetLastError(void) { return cudaSuccess; }
+cudaError_t cudaGetLastError(void) {
+  const cudaError_t e = last_error;
+  last_error = cudaSuccess;
+  return e;
+}
 
 static int encode_tiled(void) { return 0; }
 static int pointer_attribute(void* out, int what, uintptr_t p) {

@@ -244,6 +244,16 @@ def test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, K):
         assert np.max(np.abs(out[k] - oracle.preprocess(frames[k], nw, nh))) < 2e-5
 
 
+@pytest.mark.parametrize("src,net,K", [
+    ((504, 738), (224, 378), 8),         # 47.1 KB staged with wide tiles, beside 1 KB of tables
+    ((534, 716), (297, 310), 8),         # ... with narrow tiles
+    ((1920, 1080), (520, 292), 1),       # exactly 48 KB
+])
+def test_preprocess_whose_staging_takes_almost_48_kilobytes(cuda_device, src, net, K):
+    """More than a kernel gets unasked, static variables included.  Bound as above."""
+    test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, 3, K)
+
+
 @pytest.mark.parametrize("shape,K", [
     (dict(src_w=854, src_h=480, net_w=640, net_h=480, hidden=128), 5),                        # parts of 2 and 3 streams
     (dict(src_w=854, src_h=480, net_w=642, net_h=480, hidden=128), 6),                        # parts of 3; first layer on the fp32 kernel

@@ -2,6 +2,7 @@
 import ctypes as C
 import glob
 import os
+import random
 import re
 import subprocess
 
@@ -264,3 +265,16 @@ def test_frames_that_lie_one_behind_the_other_travel_as_one_copy(fake, K, pad, l
             staged = np.ctypeslib.as_array((C.c_uint8 * s.bytes).from_address(staging + n * s.bytes))
             assert np.array_equal(staged, buf[order[n] * step:order[n] * step + s.bytes])
     s.sync()
+
+
+def test_preprocessing_is_refused_at_no_size(fake):
+    """However the tile and its staging come out, the launch asks for the shared memory that it takes."""
+    rng, at = random.Random(3), 0x7F0000000000        # addresses that nothing reads
+    sizes = [(1920, 1080, 520, 292, 1), (504, 738, 224, 378, 8), (534, 716, 297, 310, 8)]
+    for _ in range(1500):
+        nw, nh = rng.randint(16, 1280), rng.randint(16, 960)
+        sizes.append((max(2, int(nw * rng.uniform(0.3, 4.0))), max(2, int(nh * rng.uniform(0.3, 4.0))), nw, nh, rng.randint(1, 8)))
+    for sw, sh, nw, nh, K in sizes:
+        fake.fake_reset()
+        assert fake.tt_preprocess(at, K, 3 * sw * sh, sw, sh, 3 * sw, at + 0x10000000, nw, nh, 255.0, 0.5, 0.25, None) == 0, (sw, sh, nw, nh, K)
+        assert b"launch" in fake.fake_log()
