@@ -192,23 +192,37 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   a.scale = pre::norm_scale(p.inv_div, p.inv_std);
   a.shift = pre::norm_shift(p.mean, p.inv_std);
   a.tiles_x = (p.net_w + COLS - 1) / COLS;
-  // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least.
+  // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least, and the higher tile of
+  // two that come out alike; another height where by it the busiest multiprocessor has at least a tenth less to do, a tile's latency counted as twelve
+  // rows.  Device time of frames from memory, us, by rows: four 1280x960 to 640x480 6 11.7, 8 10.3, 10 10.6, 12 9.3*, 14 9.3; four 1920x1080 to 1280x720 16 19.1, 20 18.8,
+  // 24 18.1, 26 17.8*; one 320x240 to 1280x960 18 7.4, 22 6.9*, 24 7.0, 28 7.6 (* chosen).  Of 140 sizes and batches one is 4 % slower by the second rule, the mean 3 % faster.
   const long slots = (long)PRE_PER_SM * sms;
-  long best = -1;
+  struct Height {
+    int rows = 0;
+    long cap_r = 0, cap_b = 0, tiles = 0, busiest_sm = 0, cost = 0;
+  } by_round, by_sm, tallest;
   for (int rows = GROUPS; rows <= PRE_MAX_ROWS; rows += GROUPS) {
-    long cap_r, cap_b;
-    staging(p, COLS, rows, &cap_r, &cap_b);
-    if (cap_r * cap_b > PRE_STAGE_BYTES) break;
-    const long tiles = (long)p.K * a.tiles_x * ((p.net_h + rows - 1) / rows);
-    const long cost = (tiles + slots - 1) / slots * (rows + 2);
-    if (best >= 0 && cost >= best) continue;
-    best = cost;
-    a.tile_rows = rows;
-    a.rows_cap = (int)cap_r;
-    a.row_cap = (int)cap_b;
+    Height h;
+    h.rows = rows;
+    staging(p, COLS, rows, &h.cap_r, &h.cap_b);
+    if (h.cap_r * h.cap_b > PRE_STAGE_BYTES) break;
+    h.tiles = (long)p.K * a.tiles_x * ((p.net_h + rows - 1) / rows);
+    h.busiest_sm = (h.tiles / slots * PRE_PER_SM + (h.tiles % slots + sms - 1) / sms) * (rows + 12);
+    h.cost = (h.tiles + slots - 1) / slots * (rows + 2);
+    if (!by_round.rows || h.cost <= by_round.cost) by_round = h;
+    if (!by_sm.rows || h.busiest_sm <= by_sm.busiest_sm) by_sm = h;
+    tallest = h;
   }
-  *fits = best >= 0;
+  // A tile of few rows is mostly halo and latency (resize factors from about three on): there taps straight from memory are faster once there are several
+  // rounds of such tiles, and of two rows always.  Staged / direct, us, one and eight frames: 1920x1080 to 480x270 (2 rows) 4.9 / 4.4 and 19.3 / 15.4; to 608x342 (4) 5.0 / 5.4
+  // and 20.1 / 18.9; to 400x225 (4) 4.5 / 4.6 and 16.9 / 14.1; to 640x360 (6) 5.4 / 5.5 and 18.4 / 19.1.
+  *fits = tallest.rows >= 6 && tallest.rows >= 2 * GROUPS;
+  if (!*fits) *fits = tallest.rows >= 4 && tallest.tiles <= 3 * slots;
   if (!*fits) return cudaSuccess;
+  const Height& h = 10 * by_sm.busiest_sm < 9 * by_round.busiest_sm ? by_sm : by_round;
+  a.tile_rows = h.rows;
+  a.rows_cap = (int)h.cap_r;
+  a.row_cap = (int)h.cap_b;
   a.tiles_y = (p.net_h + a.tile_rows - 1) / a.tile_rows;
   const long total = (long)p.K * a.tiles_x * a.tiles_y;
   const int grid = (int)(total < slots ? total : slots);

@@ -248,9 +248,12 @@ def test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, K):
     ((504, 738), (224, 378), 8),         # 47.1 KB staged with wide tiles, beside 1 KB of tables
     ((534, 716), (297, 310), 8),         # ... with narrow tiles
     ((1920, 1080), (520, 292), 1),       # exactly 48 KB
+    ((1280, 720), (320, 180), 1),        # tiles of four rows, the fewest that are staged ...
+    ((1280, 720), (320, 180), 8),        # ... and the same frames without staging, beyond three rounds of them
+    ((1280, 960), (640, 480), 4),        # two tiles of a block of different heights
 ])
 def test_preprocess_whose_staging_takes_almost_48_kilobytes(cuda_device, src, net, K):
-    """More than a kernel gets unasked, static variables included.  Bound as above."""
+    """More than a kernel gets unasked, static variables included; and the largest resize factors that are staged.  Bound as above."""
     test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, 3, K)
 
 

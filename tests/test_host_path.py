@@ -278,3 +278,22 @@ def test_preprocessing_is_refused_at_no_size(fake):
         fake.fake_reset()
         assert fake.tt_preprocess(at, K, 3 * sw * sh, sw, sh, 3 * sw, at + 0x10000000, nw, nh, 255.0, 0.5, 0.25, None) == 0, (sw, sh, nw, nh, K)
         assert b"launch" in fake.fake_log()
+
+
+@pytest.mark.parametrize("src,net,K,cols,smem", [                  # smem: two tiles of staged rows x bytes a row; 0: taps straight from memory
+    ((1920, 1080), (1280, 720), 4, 128, 2 * 41 * 640),             # 26 output rows a tile
+    ((1280, 960), (640, 480), 4, 128, 2 * 30 * 832),               # 14, where rounds of tiles alone would have 6 or 10
+    ((320, 240), (1280, 960), 1, 128, 2 * 8 * 160),                # 22 instead of 18
+    ((1920, 1080), (640, 360), 8, 128, 2 * 20 * 1216),             # 6, the fewest at any batch
+    ((1920, 1080), (480, 270), 1, 128, 0),                         # 2 would fit
+    ((1920, 1080), (608, 342), 1, 128, 2 * 15 * 1280),             # 4 in up to three rounds
+    ((1920, 1080), (608, 342), 8, 128, 0),
+    ((1280, 720), (320, 180), 4, 64, 2 * 18 * 832),
+    ((1280, 720), (320, 180), 8, 64, 0),
+    ((2400, 1300), (40, 20), 8, 64, 0),                            # none fits
+])
+def test_tiles_of_the_preprocessing_and_where_it_stages_none(fake, src, net, K, cols, smem):
+    at = 0x7F0000000000
+    assert fake.tt_preprocess(at, K, 3 * src[0] * src[1], *src, 3 * src[0], at + 0x10000000, *net, 255.0, 0.5, 0.25, None) == 0
+    (line,) = [x for x in fake.fake_log().decode().splitlines() if x.startswith("launch")]
+    assert line.endswith(f" smem {smem}") and (f"preprocess_staged_kernelILi{cols}E" if smem else "preprocess_direct_kernel") in line
