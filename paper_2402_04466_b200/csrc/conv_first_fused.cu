@@ -3,10 +3,10 @@
 // The resized fp32 image is an observable tensor of the context and is still written (unless the caller does not
 // want it), but nothing reads it back, and one launch with its start-up and drain is gone.
 //
-// Bound by the load/store pipe (at two full-HD frames 72 % of the active cycles, of which 72 % passes through shared memory, against 30 % of
-// the issue slots), the chain of phases below, and by HBM (8 full-HD frames: 50 MB in, 88 + 236 MB out).  A block of 8 warps takes tiles of 32 x 8 outputs in
+// Bound by the load/store pipe (at two full-HD frames 61 % of the active cycles, 89 % of it through shared memory; 58 % of the issue
+// slots), the chain of phases below, and by HBM (8 full-HD frames: 50 MB in, 88 + 236 MB out).  A block of 8 warps takes tiles of 32 x 8 outputs in
 // turn, down a column of tiles, and every warp takes part in every phase, so the sampling has all the warps of
-// the multiprocessor (three blocks) at its disposal and the phases of different blocks overlap:
+// the multiprocessor (three blocks, two at the largest resize factors) at its disposal and the phases of different blocks overlap:
 //   stage    the 16-byte aligned byte range of every frame row under the tile's input patch, by bulk copies two
 //            tiles ahead;
 //   sample   the patch (with halo; zero outside the image = the convolution's padding): a lane per column, a warp per row,
@@ -35,7 +35,7 @@ using namespace tc;
 using namespace pre;
 
 constexpr int FF_THREADS = 256, FF_WARPS = 8;
-constexpr int FF_PER_SM = 3;                         // blocks per multiprocessor at 80 registers; with four at 64, 8 full-HD frames take 107 us instead of 97
+constexpr int FF_PER_SM = 3;                         // most blocks per multiprocessor; before the tile stores (80 registers) 8 full-HD frames took 97 us with three, 107 with four
 constexpr int FF_TW = 32, FF_TH = 8;                 // output tile
 constexpr int FF_SRC_BUDGET = 48 * 1024;             // shared memory the two buffers of frame rows may take
 
