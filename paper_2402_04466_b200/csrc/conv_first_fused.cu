@@ -43,13 +43,6 @@ __host__ __device__ constexpr int ff_patch_w(int stride) { return (FF_TW - 1) * 
 __host__ __device__ constexpr int ff_patch_h(int stride) { return (FF_TH - 1) * stride + 3; }
 __host__ __device__ constexpr int ff_pitch(int stride) { return stride == 2 ? 68 : 36; }   // bf16 values per patch row
 
-// bulk copy of `bytes` (a multiple of 16, both addresses too) that completes on the barrier, and its announcement
-__device__ __forceinline__ void copy_row(uint32_t dst, uintptr_t src, uint32_t bytes, uint32_t bar) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
-}
-
 struct Tile {
   int img, tx, ty;
 };
@@ -123,7 +116,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
     for (int r = warp + FF_WARPS * lane; r < rows; r += FF_WARPS * 32) {
       const uintptr_t first = (uintptr_t)frame + (size_t)(r_lo + r) * p.src_pitch + b_lo;
       const int bytes = min((int)((((uint32_t)first & 15u) + span) & ~15u) + 16, p.src_row_cap);
-      copy_row(smem_u32(s_src + buf * src_bytes) + r * p.src_row_cap, first & ~(uintptr_t)15, (uint32_t)bytes, bar);
+      bulk_copy(smem_u32(s_src + buf * src_bytes) + r * p.src_row_cap, first & ~(uintptr_t)15, (uint32_t)bytes, bar);
     }
     __syncwarp();
     if (lane == 0) mbar_arrive(bar);

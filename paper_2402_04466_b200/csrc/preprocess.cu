@@ -1,25 +1,41 @@
 // S1: uint8 RGB interleaved frame -> bilinear resize -> normalise -> planar fp32.
 //
-// Bound by instruction issue (78 % of the slots at four full-HD frames, about 117 instructions per pixel of three channels) and by HBM.  A block
-// works down a column of tiles of COLS output columns and `tile_rows` rows.  A thread keeps one output column, so the horizontal
-// sample position stays in its registers, neighbouring lanes read neighbouring bytes of a staged row (few bank conflicts; with
-// four neighbouring outputs per thread every fetch took four to five passes), and a warp's store is 128 contiguous bytes.
-// The frame rows under a tile are staged as a byte stream (row pitch 3*W is in general not a multiple of 16) by asynchronous 16-byte
-// copies of the aligned range that covers them, while the tile before is sampled.  A bilinear tap pair (two neighbouring RGB pixels = 6
-// bytes) is fetched as three 32-bit shared loads plus funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
-// Four full-HD frames to 1280x720: 24.4 -> 18.45 us a call against a block per 128 x 16 tile (2.8 -> 3.75 TB/s); eight, alone under the profiler: 37.6 -> 34.1.
+// A block works down a column of tiles of TILE_W output columns and `tile_rows` rows.  A ninth warp works out where the tiles lie and has the frame rows under a tile
+// staged as a byte stream (row pitch 3*W is in general not a multiple of 16) by one bulk copy a row of the aligned range that covers it, a tile ahead; per-thread copies and
+// every warp's index arithmetic had been a third of the instructions.  A sampling thread keeps two output columns half a tile apart and goes down a run of rows: the two are one
+// packed fp32 instruction each step, neighbouring lanes read neighbouring bytes of a staged row (few bank conflicts), a warp's store is 128 contiguous bytes, and a frame row
+// that the row above has already blended horizontally is not fetched again.  A bilinear tap pair (two neighbouring RGB pixels = 6 bytes) is three 32-bit shared loads plus
+// funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
+// Bound by issue and by the start: every block's first tile comes before anything can be sampled (four full-HD frames: launch 2, first rows 3, two tiles 9 us).  Instructions per
+// pixel of three channels 117 -> 80.  Device time, us, of frames in L2 before / now: four full-HD frames to 1280x720 17.7 / 14.6, eight 33.0 / 27.0, one 6.1 / 5.8, eight to
+// 768x432 19.5 / 15.2, four 1280x960 to 640x480 9.0 / 8.3, two 960x540 to 1280x720 9.3 / 8.6; a call with frames from memory: 18.5 / 16.4, 34.8 / 29.5, 8.2 / 8.0, 20.5 / 17.8, 10.3 / 10.3.
+// Not kept: per-thread asynchronous copies by the ninth warp (25 us), three and four tiles in flight of 8 to 16 rows (16.6 to 18.8), five or six blocks with smaller tiles.
 #include "tt_internal.h"
 #include "pre_math.cuh"
+#include "tc_ptx.cuh"
 
 namespace tt {
 namespace {
 
 using namespace pre;
+using tc::pack2;
+using tc::unpack2;
+typedef unsigned long long f32x2;   // two fp32 values
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
 
-constexpr int PRE_THREADS = 256, PRE_PER_SM = 4;   // four full-HD frames: 20.5, 18.4, 18.5, 20.5, 22.5, 24.6 us with 2, 3, 4, 5, 6, 8 blocks
+constexpr int PRE_SAMPLERS = 256, PRE_THREADS = PRE_SAMPLERS + 32, PRE_WARPS = PRE_THREADS / 32, PRE_PER_SM = 4;
 constexpr int PRE_MAX_ROWS = 32;             // output rows of a tile
 constexpr int PRE_STAGE_BYTES = 26 * 1024;   // staged rows of a tile; two tiles of four blocks fit a multiprocessor
-constexpr int PRE_STATIC_BYTES = 2 * PRE_MAX_ROWS * 16;   // the kernel's row tables
+constexpr int PRE_STATIC_BYTES = 2 * (PRE_MAX_ROWS * 16 + 64) + 16;   // the kernel's tables and barriers
 
 struct PreprocessArgs {
   PreprocessParams p;
@@ -29,119 +45,193 @@ struct PreprocessArgs {
   int32_t tiles_per_block, tiles_left;       // the first tiles_left blocks take one tile more
 };
 
-struct Tile {
-  int img, tx, ty;
+// What the sampling warps are told of a tile.
+struct alignas(16) TileInfo {
+  int32_t img, y0, rows, tx;
 };
 
+// Where a tile lies: image, tile column, first output row and their number, frame, first frame column, last byte of a staged row counted from its first, first frame
+// row and their number; sy: of the lane's output row.
+struct Place {
+  int img, tx, y0, rows;
+  const uint8_t* src;
+  int left, span, first, src_rows;
+  AxisSample sy;
+};
+// as `count` arrivals at once
+__device__ __forceinline__ void mbar_arrive_n(uint32_t bar, uint32_t count) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(count) : "memory");
+}
+
+// Three channels of a frame row between two of its pixels, for a thread's two columns.  The loads are volatile: a row that is at hand already is not
+// fetched all the same.
+struct Blend {
+  f32x2 r, g, b;
+};
+struct Taps {
+  uint32_t lo, hi;   // bytes R0 G0 B0 R1, G1 B1 . .
+};
+__device__ __forceinline__ Taps fetch_taps(uint32_t addr) {
+  uint32_t w0, w1, w2;
+  const uint32_t word = addr & ~3u, sh = addr << 3;   // a funnel shift takes its shift modulo 32
+  asm volatile("ld.shared.u32 %0, [%3];\n\tld.shared.u32 %1, [%3+4];\n\tld.shared.u32 %2, [%3+8];" : "=r"(w0), "=r"(w1), "=r"(w2) : "r"(word));
+  return {__funnelshift_r(w0, w1, sh), __funnelshift_r(w1, w2, sh)};
+}
+__device__ __forceinline__ f32x2 magic2(uint32_t a, uint32_t b, uint32_t selector) { return pack2(byte_to_magic(a, selector), byte_to_magic(b, selector)); }
+__device__ __forceinline__ Blend blend_row(uint32_t addr_a, uint32_t addr_b, f32x2 fx) {
+  const Taps a = fetch_taps(addr_a), b = fetch_taps(addr_b);
+  const f32x2 magic = pack2(8388608.0f, 8388608.0f);
+  const f32x2 l0 = magic2(a.lo, b.lo, 0x7440), l1 = magic2(a.lo, b.lo, 0x7441), l2 = magic2(a.lo, b.lo, 0x7442);
+  return {fma2(fx, sub2(magic2(a.lo, b.lo, 0x7443), l0), sub2(l0, magic)), fma2(fx, sub2(magic2(a.hi, b.hi, 0x7440), l1), sub2(l1, magic)),
+          fma2(fx, sub2(magic2(a.hi, b.hi, 0x7441), l2), sub2(l2, magic))};
+}
+
 // ONE_ROW: the height is not resized, so every sample sits on a source row (weight zero for the next one).
-template <int COLS, bool ONE_ROW>
+template <int TILE_W, bool ONE_ROW>
 __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_kernel(const __grid_constant__ PreprocessArgs a) {
-  constexpr int GROUPS = PRE_THREADS / COLS;         // rows sampled at a time
+  constexpr int COLS = TILE_W / 2;                   // a thread's columns are COLS apart
+  constexpr int GROUPS = PRE_SAMPLERS / COLS;        // runs of rows sampled at a time
   extern __shared__ __align__(16) uint8_t s_mem[];   // [2][rows_cap][row_cap]
-  __shared__ __align__(16) int4 s_row[2][PRE_MAX_ROWS];   // per tile row: byte offsets of its two source rows in the buffer, bits of the lower one's weight
+  __shared__ TileInfo s_tile[2];
+  __shared__ __align__(16) int4 s_row[2][PRE_MAX_ROWS];   // per tile row: byte offsets of its two source rows in the buffer, bits of the lower one's weight, whether the upper one is the row above's lower one
+  __shared__ __align__(8) uint64_t s_full[2];             // a buffer's frame rows have landed
   // the next kernel of the stream, if it was launched as a programmatic dependent, may start its set-up now;
   // it waits for this grid to finish before it reads the output
   pdl_launch_dependents();
   const PreprocessParams& p = a.p;
-  const int tid = threadIdx.x, col = tid % COLS, grp = tid / COLS;
-  const int buf_bytes = a.rows_cap * a.row_cap, vecs = a.row_cap >> 4;
+  const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+  const int buf_bytes = a.rows_cap * a.row_cap;
   const int t_begin = (int)blockIdx.x * a.tiles_per_block + min((int)blockIdx.x, a.tiles_left);
   const int n = a.tiles_per_block + ((int)blockIdx.x < a.tiles_left ? 1 : 0);
-  const int step_r = PRE_THREADS / vecs, step_v = PRE_THREADS - step_r * vecs;   // from one of a thread's copies to its next
-  const int r_first = tid / vecs, v_first = tid - r_first * vecs;
-  // tiles in order of (image, tile column, tile row)
-  auto advance = [&](Tile& t) {
-    if (++t.ty == a.tiles_y) {
-      t.ty = 0;
-      if (++t.tx == a.tiles_x) { t.tx = 0; ++t.img; }
-    }
-  };
-  auto left_column = [&](int tx) { return axis_sample(tx * COLS, p.src_w, p.net_w).i0; };
-
-  // Byte b of a staged row is the frame's byte (aligned start of that row's range) + b.
-  auto stage = [&](const Tile& t, int buf, int sx_lo, int sx_hi) {
-    const uint8_t* src = p.src_tab ? p.src_tab[t.img] : p.src.p[t.img];
-    const int y0 = t.ty * a.tile_rows, y_last = min(y0 + a.tile_rows, p.net_h) - 1;
-    const int r_lo = axis_sample(y0, p.src_h, p.net_h).i0, rows = axis_sample(y_last, p.src_h, p.net_h).i1 - r_lo + 1;
-    if (tid < a.tile_rows) {
-      const AxisSample sy = axis_sample(min(y0 + tid, p.net_h - 1), p.src_h, p.net_h);
-      // low bits of the address of column sx_lo in source row 0: (that + row * pitch) & 15 is its position in the staged row
-      const uint32_t base_lo = (uint32_t)(uintptr_t)src + 3u * (uint32_t)sx_lo;
-      s_row[buf][tid] = make_int4((sy.i0 - r_lo) * a.row_cap + (int)((base_lo + (uint32_t)(sy.i0 * p.src_pitch)) & 15u),
-                                  (sy.i1 - r_lo) * a.row_cap + (int)((base_lo + (uint32_t)(sy.i1 * p.src_pitch)) & 15u), __float_as_int(sy.f), 0);
-    }
-    const uintptr_t first = (uintptr_t)src + (size_t)r_lo * p.src_pitch + 3 * sx_lo;
-    const int span = 3 * (sx_hi - sx_lo) + 2;          // last byte of a row, counted from its first
-    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(s_mem + buf * buf_bytes);
-    for (int r = r_first, v = v_first; r < rows;) {
-      const uintptr_t g = first + (size_t)r * p.src_pitch;
-      if (v * 16 <= (int)(g & 15) + span)
-        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + r * a.row_cap + v * 16), "l"((g & ~(uintptr_t)15) + v * 16) : "memory");
-      r += step_r;
-      v += step_v;
-      if (v >= vecs) { v -= vecs; ++r; }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-
-  Tile cur, ahead;
-  {
-    const int tiles_per_img = a.tiles_x * a.tiles_y;
-    cur.img = t_begin / tiles_per_img;
-    const int rem = t_begin - cur.img * tiles_per_img;
-    cur.tx = rem / a.tiles_y;
-    cur.ty = rem - cur.tx * a.tiles_y;
+  if (tid == 0) {
+    tc::mbar_init(tc::smem_u32(&s_full[0]), PRE_WARPS);
+    tc::mbar_init(tc::smem_u32(&s_full[1]), PRE_WARPS);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  ahead = cur;
-  auto stage_ahead = [&](int buf) {
-    const int sx_lo = left_column(ahead.tx), sx_hi = axis_sample(min((ahead.tx + 1) * COLS, p.net_w) - 1, p.src_w, p.net_w).i1;
-    stage(ahead, buf, sx_lo, sx_hi);
-    advance(ahead);
-  };
-  if (n > 0) stage_ahead(0);
+  __syncthreads();
 
-  const size_t plane = (size_t)p.net_h * p.net_w;
-  int tx = -1, x = 0, xo = 0;
-  float fx = 0.f;
-  for (int i = 0; i < n; ++i) {
-    if (i + 1 < n) {
-      stage_ahead((i + 1) & 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
+  // Worked out by a whole warp, a lane per row: the i-th tile's place (tiles in order of image, tile column, tile row) ...
+  auto place_of = [&](int i) {
+    Place t;
+    const int tile = t_begin + i, col_tiles = tile / a.tiles_y;
+    t.img = col_tiles / a.tiles_x;
+    t.tx = col_tiles - t.img * a.tiles_x;
+    t.y0 = (tile - col_tiles * a.tiles_y) * a.tile_rows;
+    t.rows = min(a.tile_rows, p.net_h - t.y0);
+    t.src = p.src_tab ? p.src_tab[t.img] : p.src.p[t.img];
+    const AxisSample sx = axis_sample(lane == 0 ? t.tx * TILE_W : min((t.tx + 1) * TILE_W, p.net_w) - 1, p.src_w, p.net_w);
+    t.left = __shfl_sync(0xffffffffu, sx.i0, 0);
+    t.span = 3 * (__shfl_sync(0xffffffffu, sx.i1, 1) - t.left) + 2;
+    t.sy = axis_sample(t.y0 + min(lane, t.rows - 1), p.src_h, p.net_h);
+    t.first = __shfl_sync(0xffffffffu, t.sy.i0, 0);
+    t.src_rows = __shfl_sync(0xffffffffu, t.sy.i1, t.rows - 1) - t.first + 1;
+    return t;
+  };
+  // ... copies of its frame rows r, r + step, ...: byte b of a staged row is the frame's byte (aligned start of that row's range) + b ...
+  auto copy_rows = [&](const Place& t, int buf, int r, int step) {
+    const uint32_t bar = tc::smem_u32(&s_full[buf]), dst = tc::smem_u32(s_mem) + (uint32_t)(buf * buf_bytes);
+    for (; r < t.src_rows; r += step) {
+      const uintptr_t g = (uintptr_t)t.src + (size_t)(t.first + r) * p.src_pitch + 3 * t.left;
+      tc::bulk_copy(dst + (uint32_t)(r * a.row_cap), g & ~(uintptr_t)15, ((((uint32_t)g & 15u) + t.span) & ~15u) + 16u, bar);
     }
-    if (cur.tx != tx) {
-      tx = cur.tx;
-      x = tx * COLS + col;
-      const AxisSample sx = axis_sample(min(x, p.net_w - 1), p.src_w, p.net_w);
-      xo = 3 * (sx.i0 - left_column(tx));
-      fx = sx.f;
-    }
-    __syncthreads();                                   // this tile's rows and row table are complete
-    const uint32_t* words = reinterpret_cast<const uint32_t*>(s_mem + (i & 1) * buf_bytes);
-    const int y0 = cur.ty * a.tile_rows, rows = min(a.tile_rows, p.net_h - y0);
-    if (x < p.net_w) {
-      float* d = p.dst + (size_t)cur.img * 3 * plane + (size_t)(y0 + grp) * p.net_w + x;
-#pragma unroll 2
-      for (int r = grp; r < rows; r += GROUPS, d += GROUPS * p.net_w) {
-        const int4 e = s_row[i & 1][r];
-        float o0, o1, o2;
-        uint32_t lo0, hi0;
-        fetch_pair(words, e.x + xo, lo0, hi0);
-        if (ONE_ROW) {
-          sample_row(lo0, hi0, fx, a.scale, a.shift, o0, o1, o2);
-        } else {
-          uint32_t lo1, hi1;
-          fetch_pair(words, e.y + xo, lo1, hi1);
-          sample_rows(lo0, hi0, lo1, hi1, fx, __int_as_float(e.z), a.scale, a.shift, o0, o1, o2);
-        }
-        d[0] = o0;
-        d[plane] = o1;
-        d[2 * plane] = o2;
+    __syncwarp();
+  };
+  // ... and what the sampling warps are told of it.
+  auto tell = [&](const Place& t, int buf) {
+    const int above = __shfl_up_sync(0xffffffffu, t.sy.i1, 1);
+    // low bits of the address of the tile's first column in source row 0: (that + row * pitch) & 15 is its position in the staged row
+    const uint32_t base_lo = (uint32_t)(uintptr_t)t.src + 3u * (uint32_t)t.left;
+    if (lane < a.tile_rows)
+      s_row[buf][lane] = make_int4((t.sy.i0 - t.first) * a.row_cap + (int)((base_lo + (uint32_t)(t.sy.i0 * p.src_pitch)) & 15u),
+                                   (t.sy.i1 - t.first) * a.row_cap + (int)((base_lo + (uint32_t)(t.sy.i1 * p.src_pitch)) & 15u), __float_as_int(t.sy.f), above == t.sy.i0);
+    if (lane == 0) s_tile[buf] = {t.img, t.y0, t.rows, t.tx};
+  };
+
+  // A warp issues its copies one behind the other: those of the first tile, which everything waits for, are shared out.
+  const Place first = place_of(0);
+  copy_rows(first, 0, warp + PRE_WARPS * lane, PRE_WARPS * 32);
+  if (lane == 0) tc::mbar_arrive(tc::smem_u32(&s_full[0]));
+
+  if (warp == PRE_WARPS - 1) {
+    // ------------------------------------------------------------------------ frame rows
+    tell(first, 0);
+    __syncthreads();
+    for (int i = 1; i <= n; ++i) {
+      if (i < n) {
+        const Place t = place_of(i);
+        copy_rows(t, i & 1, lane, 32);
+        if (lane == 0) mbar_arrive_n(tc::smem_u32(&s_full[i & 1]), PRE_WARPS);
+        tell(t, i & 1);
+      }
+      if (__syncthreads_or(0)) {                       // tile i - 1 has been sampled; or a wait has run out: let what is in flight land
+        for (int w = 0; w < 64; ++w) __nanosleep(16000);
+        break;
       }
     }
-    __syncthreads();                                   // the buffer has been read
-    advance(cur);
+    return;
+  }
+
+  // -------------------------------------------------------------------------- samples
+  const int col = tid % COLS, grp = tid / COLS;
+  const uint32_t plane = (uint32_t)(p.net_h * p.net_w);
+  const f32x2 scale = pack2(a.scale, a.scale), shift = pack2(a.shift, a.shift);
+  int tx, x, xo_a, xo_b;
+  f32x2 fx;
+  auto column = [&](int tile_x) {
+    tx = tile_x;
+    x = tx * TILE_W + col;
+    const int left = axis_sample(tx * TILE_W, p.src_w, p.net_w).i0;
+    const AxisSample sa = axis_sample(min(x, p.net_w - 1), p.src_w, p.net_w), sb = axis_sample(min(x + COLS, p.net_w - 1), p.src_w, p.net_w);
+    xo_a = 3 * (sa.i0 - left);
+    xo_b = 3 * (sb.i0 - left);
+    fx = pack2(sa.f, sb.f);
+  };
+  column(first.tx);                                    // while the first rows are on their way
+  __syncthreads();                                     // the first tile has been told of
+  for (int i = 0; i < n; ++i) {
+    const TileInfo& t = s_tile[i & 1];
+    const int img = __shfl_sync(0xffffffffu, t.img, 0), rows = __shfl_sync(0xffffffffu, t.rows, 0);
+    if (t.tx != tx) column(t.tx);
+    const bool ok = tc::mbar_wait_limit(tc::smem_u32(&s_full[i & 1]), (uint32_t)(i >> 1) & 1u, tc::WAIT_LIMIT_CYCLES);
+    if (ok && x < p.net_w) {
+      const uint32_t buf = tc::smem_u32(s_mem) + (uint32_t)((i & 1) * buf_bytes), buf_a = buf + (uint32_t)xo_a, buf_b = buf + (uint32_t)xo_b;
+      const bool two = x + COLS < p.net_w;
+      float* out = p.dst + (size_t)img * 3 * plane;
+      const int share = (rows + GROUPS - 1) / GROUPS, r_begin = grp * share, r_end = min(r_begin + share, rows);
+      const int4* e_tab = s_row[i & 1];
+      uint32_t o = (uint32_t)((t.y0 + r_begin) * p.net_w + x);
+      Blend bot{};
+#pragma unroll 1
+      for (int r = r_begin; r < r_end; ++r, o += (uint32_t)p.net_w) {
+        const int4 e = e_tab[r];
+        Blend top = bot;
+        if (ONE_ROW || e.w == 0 || r == r_begin) top = blend_row(buf_a + e.x, buf_b + e.x, fx);
+        if (!ONE_ROW) {
+          bot = blend_row(buf_a + e.y, buf_b + e.y, fx);
+          const float f = __int_as_float(e.z);
+          const f32x2 fy = pack2(f, f);
+          top.r = fma2(fy, sub2(bot.r, top.r), top.r);
+          top.g = fma2(fy, sub2(bot.g, top.g), top.g);
+          top.b = fma2(fy, sub2(bot.b, top.b), top.b);
+        }
+        float v[3][2];
+        unpack2(fma2(top.r, scale, shift), v[0][0], v[0][1]);
+        unpack2(fma2(top.g, scale, shift), v[1][0], v[1][1]);
+        unpack2(fma2(top.b, scale, shift), v[2][0], v[2][1]);
+        // streaming stores: the image is written once (four frames to 1103x1103, whose rows do not fill whole sectors, 24.4 -> 23.4 us; to 1279x719 16.5 -> 14.9; whole lines the same)
+        float* d = out + o;
+        __stcs(d, v[0][0]);
+        __stcs(d + plane, v[1][0]);
+        __stcs(d + 2 * (size_t)plane, v[2][0]);
+        if (two) {
+          __stcs(d + COLS, v[0][1]);
+          __stcs(d + plane + COLS, v[1][1]);
+          __stcs(d + 2 * (size_t)plane + COLS, v[2][1]);
+        }
+      }
+    }
+    if (!ok && p.status) atomicCAS(p.status, 0, tc::WAIT_PREPROCESS + (i & 1));
+    if (__syncthreads_or(!ok)) break;                  // the buffer has been read
   }
 }
 
@@ -173,7 +263,7 @@ __global__ void __launch_bounds__(DIR_TX * DIR_TY) preprocess_direct_kernel(cons
   }
 }
 
-// Staged rows and bytes per row of a tile in the worst case: rows = ceil(tile_rows * sh/nh) + 2; bytes = 3 * (ceil(COLS * sw/nw) + 2) + 15
+// Staged rows and bytes per row of a tile in the worst case: rows = ceil(tile_rows * sh/nh) + 2; bytes = 3 * (ceil(cols * sw/nw) + 2) + 15
 // (alignment at the front) + 15 (at the end) + 12 (the tap fetch reads three whole words from its first byte), rounded up to 16.
 void staging(const PreprocessParams& p, int cols, int tile_rows, long* rows, long* row_cap) {
   *rows = ((long)tile_rows * p.src_h + p.net_h - 1) / p.net_h + 2;
@@ -181,9 +271,9 @@ void staging(const PreprocessParams& p, int cols, int tile_rows, long* rows, lon
   *row_cap = ((3 * c + 48 + 15) / 16) * 16;
 }
 
-template <int COLS>
+template <int TILE_W>
 cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits) {
-  constexpr int GROUPS = PRE_THREADS / COLS;
+  constexpr int STEP = 256 / TILE_W;
   int sms = 0;
   cudaError_t e = post_sm_count(&sms);
   if (e != cudaSuccess) return e;
@@ -191,20 +281,20 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   a.p = p;
   a.scale = pre::norm_scale(p.inv_div, p.inv_std);
   a.shift = pre::norm_shift(p.mean, p.inv_std);
-  a.tiles_x = (p.net_w + COLS - 1) / COLS;
+  a.tiles_x = (p.net_w + TILE_W - 1) / TILE_W;
   // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least, and the higher tile of
   // two that come out alike; another height where by it the busiest multiprocessor has at least a tenth less to do, a tile's latency counted as twelve
-  // rows.  Device time of frames from memory, us, by rows: four 1280x960 to 640x480 6 11.7, 8 10.3, 10 10.6, 12 9.3*, 14 9.3; four 1920x1080 to 1280x720 16 19.1, 20 18.8,
-  // 24 18.1, 26 17.8*; one 320x240 to 1280x960 18 7.4, 22 6.9*, 24 7.0, 28 7.6 (* chosen).  Of 140 sizes and batches one is 4 % slower by the second rule, the mean 3 % faster.
+  // rows.  Device time of frames in L2, us, by rows: four 1280x960 to 640x480 6 10.4, 8 9.3, 10 9.5, 12 8.4, 14 8.4*; four 1920x1080 to 1280x720 16 15.4, 20 15.2,
+  // 24 15.1, 26 14.7*; one 320x240 to 1280x960 18 7.7, 22 7.0*, 24 7.2, 28 7.7 (* chosen).
   const long slots = (long)PRE_PER_SM * sms;
   struct Height {
     int rows = 0;
     long cap_r = 0, cap_b = 0, tiles = 0, busiest_sm = 0, cost = 0;
   } by_round, by_sm, tallest;
-  for (int rows = GROUPS; rows <= PRE_MAX_ROWS; rows += GROUPS) {
+  for (int rows = STEP; rows <= PRE_MAX_ROWS; rows += STEP) {
     Height h;
     h.rows = rows;
-    staging(p, COLS, rows, &h.cap_r, &h.cap_b);
+    staging(p, TILE_W, rows, &h.cap_r, &h.cap_b);
     if (h.cap_r * h.cap_b > PRE_STAGE_BYTES) break;
     h.tiles = (long)p.K * a.tiles_x * ((p.net_h + rows - 1) / rows);
     h.busiest_sm = (h.tiles / slots * PRE_PER_SM + (h.tiles % slots + sms - 1) / sms) * (rows + 12);
@@ -213,10 +303,10 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
     if (!by_sm.rows || h.busiest_sm <= by_sm.busiest_sm) by_sm = h;
     tallest = h;
   }
-  // A tile of few rows is mostly halo and latency (resize factors from about three on): there taps straight from memory are faster once there are several
-  // rounds of such tiles, and of two rows always.  Staged / direct, us, one and eight frames: 1920x1080 to 480x270 (2 rows) 4.9 / 4.4 and 19.3 / 15.4; to 608x342 (4) 5.0 / 5.4
-  // and 20.1 / 18.9; to 400x225 (4) 4.5 / 4.6 and 16.9 / 14.1; to 640x360 (6) 5.4 / 5.5 and 18.4 / 19.1.
-  *fits = tallest.rows >= 6 && tallest.rows >= 2 * GROUPS;
+  // A tile of few rows is mostly halo and latency (resize factors from about three on): taps straight from memory where two rows are the most that fit, and of four beyond three
+  // rounds.  Staged / direct, us, one, four and eight frames: 1920x1080 to 480x270 (2 rows) 4.6 / 3.8, 8.3 / 8.4, 11.8 / 13.9; to 608x342 (4) 4.4 / 4.6, 8.9 / 10.0,
+  // 13.6 / 17.1; to 640x360 (6) 5.2 / 4.8, 9.0 / 10.7, 13.5 / 17.5; 1280x720 to 320x180 (4, narrow) 3.2 / 3.7, 5.6 / 5.0, 7.6 / 7.8.
+  *fits = tallest.rows >= 6 && tallest.rows >= 2 * STEP;
   if (!*fits) *fits = tallest.rows >= 4 && tallest.tiles <= 3 * slots;
   if (!*fits) return cudaSuccess;
   const Height& h = 10 * by_sm.busiest_sm < 9 * by_round.busiest_sm ? by_sm : by_round;
@@ -229,7 +319,7 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   a.tiles_per_block = (int)(total / grid);
   a.tiles_left = (int)(total % grid);
   const size_t smem = (size_t)2 * a.rows_cap * a.row_cap;
-  auto kern = p.src_h == p.net_h ? preprocess_staged_kernel<COLS, true> : preprocess_staged_kernel<COLS, false>;
+  auto kern = p.src_h == p.net_h ? preprocess_staged_kernel<TILE_W, true> : preprocess_staged_kernel<TILE_W, false>;
   if (smem + PRE_STATIC_BYTES > 48 * 1024) {   // what a kernel may have of both without asking
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * PRE_STAGE_BYTES);
     if (e != cudaSuccess) return e;

@@ -17,7 +17,7 @@ constexpr uint32_t TRY_WAIT_SUSPEND_NS = 20000u;
 // What a kernel writes to the status word when one of its waits runs out: its own hundreds, in them the wait (its tens) and
 // the stage, buffer or view (ones).  The host prints the code.
 constexpr int WAIT_CONV_TC = 0x100, WAIT_CONV_LSTM = 0x200, WAIT_CONV_FIRST = 0x300, WAIT_CONV_FIRST_FUSED = 0x400, WAIT_CONV_S2 = 0x500,
-              WAIT_POST_TC = 0x600, WAIT_POST_STREAM = 0x700, WAIT_PROBE = 0xA00;
+              WAIT_POST_TC = 0x600, WAIT_POST_STREAM = 0x700, WAIT_PREPROCESS = 0x800, WAIT_PROBE = 0xA00;
 
 // ------------------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -64,6 +64,25 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
       }
     }
   }
+}
+
+// A wait bounded by its own limit alone, for kernels without an abort flag: false when it ran out.
+__device__ __forceinline__ bool mbar_wait_limit(uint32_t bar, uint32_t parity, long long limit) {
+  long long t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((it & 63u) == 63u) {
+      const long long now = clock64();
+      if (t0 == 0) t0 = now;
+      else if (now - t0 > limit) return false;
+    }
+  }
+}
+// Bulk copy of `bytes` (a multiple of 16, both addresses too) that completes on the barrier, and its announcement.
+__device__ __forceinline__ void bulk_copy(uint32_t dst, uintptr_t src, uint32_t bytes, uint32_t bar) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+               ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
 
 // The same wait for a whole warp whose control flow has to stay uniform: the usual case, the phase completing within a few

@@ -784,6 +784,7 @@ PreprocessParams preprocess_params(const tt_ctx* ctx, int n0, int K, const Frame
   pp.net_w = c.net_w; pp.net_h = c.net_h;
   pp.inv_div = 1.0f / c.norm_div; pp.mean = c.norm_mean; pp.inv_std = 1.0f / c.norm_std;
   pp.dst = ctx->pre + (size_t)n0 * 3 * c.net_h * c.net_w;
+  pp.status = ctx->status_dev;
   return pp;
 }
 

@@ -59,6 +59,7 @@ struct PreprocessParams {
   int32_t K, src_w, src_h, src_pitch, net_w, net_h;
   float inv_div, mean, inv_std;
   float* dst;  // [K][3][net_h][net_w]
+  int32_t* status = nullptr;   // optional device word: set non-zero when a bounded wait ran out
 };
 cudaError_t launch_preprocess(const PreprocessParams& p, cudaStream_t s);
 

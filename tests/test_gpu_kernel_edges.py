@@ -257,6 +257,24 @@ def test_preprocess_whose_staging_takes_almost_48_kilobytes(cuda_device, src, ne
     test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, 3, K)
 
 
+@pytest.mark.parametrize("src,net,pad,K", [
+    ((300, 200), (64, 5), 0, 3),         # a thread's second column lies outside; fewer rows than runs of them
+    ((300, 200), (127, 33), 1, 2),       # ... of the last lane alone
+    ((97, 61), (191, 95), 2, 8),         # narrow tiles beside a full one, frame rows used by several output rows
+    ((640, 360), (427, 241), 5, 5),      # rows that share a frame row with the one above, and rows that do not
+    ((1280, 960), (1000, 562), 0, 8),    # several tiles a block, the copies of all but the first by one warp
+    ((320, 240), (321, 240), 0, 8),      # the height not resized
+])
+def test_preprocess_of_a_frame_is_the_same_whatever_shares_its_launch(cuda_device, src, net, pad, K):
+    """Tile heights, runs of rows and the blocks' shares depend on the batch; the bits of a frame do not.  Bound against the oracle as above."""
+    test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, min(K, 2))
+    (sw, sh), (nw, nh) = src, net
+    frames = torch.from_numpy(np.random.default_rng(6).integers(0, 256, (K, sh * (3 * sw + pad)), dtype=np.uint8)).to(cuda_device)
+    batch = binding.preprocess(frames, sw, sh, 3 * sw + pad, nw, nh)
+    for k in range(K):
+        assert torch.equal(binding.preprocess(frames[k:k + 1], sw, sh, 3 * sw + pad, nw, nh)[0], batch[k])
+
+
 @pytest.mark.parametrize("shape,K", [
     (dict(src_w=854, src_h=480, net_w=640, net_h=480, hidden=128), 5),                        # parts of 2 and 3 streams
     (dict(src_w=854, src_h=480, net_w=642, net_h=480, hidden=128), 6),                        # parts of 3; first layer on the fp32 kernel
