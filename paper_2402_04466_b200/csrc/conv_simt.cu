@@ -14,7 +14,9 @@
 // Against one pixel x 16/32 channels per thread, 32 x 8 pixels per block and synchronous staging (stage times with
 // their event): ConvLSTM of one 64x64 map with 16 channels 51 -> 15 us, of three 80x60 maps with 32 channels 135 -> 70 us.  With single FMAs those took
 // 16.2 and 69.9 us (80 % of the issue slots, a quarter of them for other things than FMAs), in pairs 14.4 and 67.8.  Pairs of
-// pixels instead of channels lost (94 us): they need register moves for every shifted pair.
+// pixels instead of channels lost (94 us), with register moves for every shifted pair and with every weight twice in shared memory alike: a 128-bit load takes the
+// load/store unit four cycles whether its lanes read one address or 32, so that weights are what it is busy with (6 loads for 96 FMA instructions: 75 % of it with
+// the inputs').  4 x 4 pixels of 4 channels per thread halve those loads and were slower all the same (75 us).
 #include <algorithm>
 
 #include "tt_internal.h"
@@ -62,6 +64,13 @@ struct SimtCfg {
   static constexpr int W_VECS = CB * 9 * WO * (OC / 4);                 // 16-byte vectors of weights per chunk
   static_assert((KS - 1) * WY * WO * 32 * OC * PX <= BUFS * BUF_FLOATS, "the channel groups' partial sums reuse the staging buffers");
 };
+
+// the six input columns under a run of four pixels
+__device__ __forceinline__ void load_row(const float* r, float (&x)[6]) {
+  const float4 a = *reinterpret_cast<const float4*>(r);
+  const float2 b = *reinterpret_cast<const float2*>(r + 4);
+  x[0] = a.x; x[1] = a.y; x[2] = a.z; x[3] = a.w; x[4] = b.x; x[5] = b.y;
+}
 
 template <int STRIDE, int EPI, int WY, int WO, int KS, int PX>
 __global__ void __launch_bounds__(32 * WY * WO * KS) conv3x3_simt_kernel(const __grid_constant__ ConvSimtParams p) {
@@ -160,48 +169,93 @@ __global__ void __launch_bounds__(32 * WY * WO * KS) conv3x3_simt_kernel(const _
     copies_commit();                                 // also where there is nothing left to copy, so that the wait above counts alike
     buf = buf == 2 ? 0 : buf + 1;
     const int c_end = min(CB, cin - c0);
+    if constexpr (STRIDE == 1) {
+      // One row of taps after the other, the inputs and weights of the next one fetched while this one's products run: two or three warps to a scheduler
+      // do not hide a shared-memory load.  Ticks, us: two 200x150 maps, ConvLSTM of 24, 154 -> 145; eight 80x60, ConvLSTM of 32, 201.5 -> 199.5, three 112.6 -> 112.0.
+      const float* in_c = cur + (ks * IN_H + ly) * PITCH + lx;
+      const float* w_c = cur + Cfg::IN_FLOATS + (ks * 9 * WO + wo) * OC;
+      float xn[RUNS][6];
+      ulonglong2 wn[3][OC / 4];
+      auto fetch = [&](const float* in, const float* w) {
+#pragma unroll
+        for (int g = 0; g < RUNS; ++g) load_row(in + g * RUN_STEP, xn[g]);
+#pragma unroll
+        for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+          for (int o = 0; o < OC / 4; ++o) wn[kx][o] = *reinterpret_cast<const ulonglong2*>(w + kx * WO * OC + 4 * o);
+      };
+      if (ks < c_end) fetch(in_c, w_c);
 #pragma unroll 1
-    for (int c = ks; c < c_end; c += KS) {
-      const float* in_c = cur + (c * IN_H + ly * STRIDE) * PITCH + lx;
-      const float* w_c = cur + Cfg::IN_FLOATS + (c * 9 * WO + wo) * OC;
+      for (int c = ks; c < c_end; c += KS) {
+        const bool more = c + KS < c_end;
+        const float* in_next = in_c + (more ? KS * IN_H * PITCH : 0);     // behind the last channel: that one again, unused
+        const float* w_next = w_c + (more ? KS * 9 * WO * OC : 0);
 #pragma unroll
-      for (int ky = 0; ky < 3; ++ky) {
-        // x[g][i]: input column (lx + 8 g) * STRIDE + i of this row
-        float x[RUNS][3 * STRIDE + 3];
+        for (int ky = 0; ky < 3; ++ky) {
+          unsigned long long x2[RUNS][6];               // each value twice
 #pragma unroll
-        for (int g = 0; g < RUNS; ++g) {
-          const float* r = in_c + ky * PITCH + g * RUN_STEP;
-          if (STRIDE == 1) {
-            const float4 a = *reinterpret_cast<const float4*>(r);
-            const float2 b = *reinterpret_cast<const float2*>(r + 4);
-            x[g][0] = a.x; x[g][1] = a.y; x[g][2] = a.z; x[g][3] = a.w; x[g][4] = b.x; x[g][5] = b.y;
-          } else {
-            const float4 e = *reinterpret_cast<const float4*>(r);
-            const float4 o = *reinterpret_cast<const float4*>(r + Cfg::ODD);
-            x[g][0] = e.x; x[g][2] = e.y; x[g][4] = e.z; x[g][6] = e.w; x[g][8] = r[4];
-            x[g][1] = o.x; x[g][3] = o.y; x[g][5] = o.z; x[g][7] = o.w;
-          }
-          if (EPI == EPI_RELU_BF16_NHWC) {
+          for (int g = 0; g < RUNS; ++g)
 #pragma unroll
-            for (int i = 0; i < 3 * STRIDE + 3; ++i) x[g][i] = round_bf16(x[g][i]);
+            for (int i = 0; i < 6; ++i) {
+              const float v = EPI == EPI_RELU_BF16_NHWC ? round_bf16(xn[g][i]) : xn[g][i];
+              x2[g][i] = tc::pack2(v, v);
+            }
+          ulonglong2 w[3][OC / 4];
+#pragma unroll
+          for (int kx = 0; kx < 3; ++kx)
+#pragma unroll
+            for (int o = 0; o < OC / 4; ++o) w[kx][o] = wn[kx][o];
+          if (ky < 2) fetch(in_c + (ky + 1) * PITCH, w_c + (ky + 1) * 3 * WO * OC);
+          else fetch(in_next, w_next);
+#pragma unroll
+          for (int kx = 0; kx < 3; ++kx) {
+#pragma unroll
+            for (int o = 0; o < OC; o += 4) {
+#pragma unroll
+              for (int i = 0; i < PX; ++i) {
+                const unsigned long long v = x2[i >> 2][(i & 3) + kx];
+                tc::fma2(acc2[o / 2][i], v, w[kx][o >> 2].x);
+                tc::fma2(acc2[o / 2 + 1][i], v, w[kx][o >> 2].y);
+              }
+            }
           }
         }
-        unsigned long long x2[RUNS][3 * STRIDE + 3];   // each value twice
+        in_c = in_next;
+        w_c = w_next;
+      }
+    } else {
+      // The compiler's own order: fetched ahead, the registers cost blocks (six 480x360 inputs 80 -> 85 us a tick).
+#pragma unroll 1
+      for (int c = ks; c < c_end; c += KS) {
+        const float* in_c = cur + (c * IN_H + ly * 2) * PITCH + lx;
+        const float* w_c = cur + Cfg::IN_FLOATS + (c * 9 * WO + wo) * OC;
 #pragma unroll
-        for (int g = 0; g < RUNS; ++g)
+        for (int ky = 0; ky < 3; ++ky) {
+          // x[i]: input column lx * 2 + i of this row
+          const float* r = in_c + ky * PITCH;
+          float x[9];
+          const float4 e = *reinterpret_cast<const float4*>(r);
+          const float4 o = *reinterpret_cast<const float4*>(r + Cfg::ODD);
+          x[0] = e.x; x[2] = e.y; x[4] = e.z; x[6] = e.w; x[8] = r[4];
+          x[1] = o.x; x[3] = o.y; x[5] = o.z; x[7] = o.w;
+          if (EPI == EPI_RELU_BF16_NHWC) {
 #pragma unroll
-          for (int i = 0; i < 3 * STRIDE + 3; ++i) x2[g][i] = tc::pack2(x[g][i], x[g][i]);
+            for (int i = 0; i < 9; ++i) x[i] = round_bf16(x[i]);
+          }
+          unsigned long long x2[9];                      // each value twice
 #pragma unroll
-        for (int kx = 0; kx < 3; ++kx) {
-          const ulonglong2* w = reinterpret_cast<const ulonglong2*>(w_c + (ky * 3 + kx) * WO * OC);
+          for (int i = 0; i < 9; ++i) x2[i] = tc::pack2(x[i], x[i]);
 #pragma unroll
-          for (int o = 0; o < OC; o += 4) {
-            const ulonglong2 w4 = w[o >> 2];
+          for (int kx = 0; kx < 3; ++kx) {
+            const ulonglong2* w = reinterpret_cast<const ulonglong2*>(w_c + (ky * 3 + kx) * WO * OC);
 #pragma unroll
-            for (int i = 0; i < PX; ++i) {
-              const unsigned long long v = x2[i >> 2][(i & 3) * STRIDE + kx];
-              tc::fma2(acc2[o / 2][i], v, w4.x);
-              tc::fma2(acc2[o / 2 + 1][i], v, w4.y);
+            for (int o4 = 0; o4 < OC; o4 += 4) {
+              const ulonglong2 w4 = w[o4 >> 2];
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                tc::fma2(acc2[o4 / 2][i], x2[i * 2 + kx], w4.x);
+                tc::fma2(acc2[o4 / 2 + 1][i], x2[i * 2 + kx], w4.y);
+              }
             }
           }
         }
