@@ -900,13 +900,16 @@ cudaError_t post_sm_count(int* out) {
 }
 
 cudaError_t post_prepare() {
-  cudaError_t e = cudaFuncSetAttribute(post_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)post_smem_bytes(512));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(post_stream_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<1>::SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(post_stream_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<2>::SMEM_BYTES);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(post_stream_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<4>::SMEM_BYTES);
+  static OncePerDevice once;
+  return once([]() {
+    cudaError_t e = cudaFuncSetAttribute(post_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)post_smem_bytes(512));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(post_stream_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<1>::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(post_stream_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<2>::SMEM_BYTES);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(post_stream_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, StreamCfg<4>::SMEM_BYTES);
+  });
 }
 
 cudaError_t launch_postprocess(const PostParams& p, cudaStream_t s) {

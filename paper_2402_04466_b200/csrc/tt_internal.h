@@ -5,6 +5,8 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "tt.h"
 
 namespace tt {
@@ -41,6 +43,22 @@ inline cudaError_t launch_kernel(void (*kern)(const Params), dim3 grid, int bloc
   cfg.numAttrs = (unsigned)n;
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
+
+// Runs what has to be done once on every device (kernel attributes: 0.9 us each on every call otherwise) until it has succeeded there.
+struct OncePerDevice {
+  std::atomic<uint64_t> done{0};
+  template <typename F>
+  cudaError_t operator()(F&& f) {
+    int dev = -1;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
+    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+    e = f();
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    return e;
+  }
+};
 
 // Maps batch position n (0..K-1) of a launch to an image index inside a tensor that holds
 // more images than the batch (state slots, ping-pong halves).
