@@ -2,8 +2,8 @@
 //
 // A block works down a column of tiles of TILE_W output columns and `tile_rows` rows.  A ninth warp works out where the tiles lie and has the frame rows under a tile
 // staged as a byte stream (row pitch 3*W is in general not a multiple of 16) by one bulk copy a row of the aligned range that covers it, a tile ahead; per-thread copies and
-// every warp's index arithmetic had been a third of the instructions.  A sampling thread keeps two output columns half a tile apart and goes down a run of rows: the two are one
-// packed fp32 instruction each step, neighbouring lanes read neighbouring bytes of a staged row (few bank conflicts), a warp's store is 128 contiguous bytes, and a frame row
+// every warp's index arithmetic had been a third of the instructions.  A sampling thread keeps two output columns 32 apart and goes down a run of rows: the two are one
+// packed fp32 instruction each step, neighbouring lanes read neighbouring bytes of a staged row (few bank conflicts), a warp's stores are 256 contiguous bytes, and a frame row
 // that the row above has already blended horizontally is not fetched again.  A bilinear tap pair (two neighbouring RGB pixels = 6 bytes) is three 32-bit shared loads plus
 // funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
 // Bound by issue and by the start: every block's first tile comes before anything can be sampled (four full-HD frames: launch 2, first rows 3, two tiles 9 us).  Instructions per
@@ -89,7 +89,7 @@ __device__ __forceinline__ Blend blend_row(uint32_t addr_a, uint32_t addr_b, f32
 // ONE_ROW: the height is not resized, so every sample sits on a source row (weight zero for the next one).
 template <int TILE_W, bool ONE_ROW>
 __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_kernel(const __grid_constant__ PreprocessArgs a) {
-  constexpr int COLS = TILE_W / 2;                   // a thread's columns are COLS apart
+  constexpr int COLS = TILE_W / 2;                   // threads to a row; a thread's two columns are 32 apart
   constexpr int GROUPS = PRE_SAMPLERS / COLS;        // runs of rows sampled at a time
   extern __shared__ __align__(16) uint8_t s_mem[];   // [2][rows_cap][row_cap]
   __shared__ TileInfo s_tile[2];
@@ -179,9 +179,9 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
   f32x2 fx;
   auto column = [&](int tile_x) {
     tx = tile_x;
-    x = tx * TILE_W + col;
+    x = tx * TILE_W + 2 * (col & ~31) + (col & 31);
     const int left = axis_sample(tx * TILE_W, p.src_w, p.net_w).i0;
-    const AxisSample sa = axis_sample(min(x, p.net_w - 1), p.src_w, p.net_w), sb = axis_sample(min(x + COLS, p.net_w - 1), p.src_w, p.net_w);
+    const AxisSample sa = axis_sample(min(x, p.net_w - 1), p.src_w, p.net_w), sb = axis_sample(min(x + 32, p.net_w - 1), p.src_w, p.net_w);
     xo_a = 3 * (sa.i0 - left);
     xo_b = 3 * (sb.i0 - left);
     fx = pack2(sa.f, sb.f);
@@ -195,7 +195,7 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
     const bool ok = tc::mbar_wait_limit(tc::smem_u32(&s_full[i & 1]), (uint32_t)(i >> 1) & 1u, tc::WAIT_LIMIT_CYCLES);
     if (ok && x < p.net_w) {
       const uint32_t buf = tc::smem_u32(s_mem) + (uint32_t)((i & 1) * buf_bytes), buf_a = buf + (uint32_t)xo_a, buf_b = buf + (uint32_t)xo_b;
-      const bool two = x + COLS < p.net_w;
+      const bool two = x + 32 < p.net_w;
       float* out = p.dst + (size_t)img * 3 * plane;
       const int share = (rows + GROUPS - 1) / GROUPS, r_begin = grp * share, r_end = min(r_begin + share, rows);
       const int4* e_tab = s_row[i & 1];
@@ -218,15 +218,16 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
         unpack2(fma2(top.r, scale, shift), v[0][0], v[0][1]);
         unpack2(fma2(top.g, scale, shift), v[1][0], v[1][1]);
         unpack2(fma2(top.b, scale, shift), v[2][0], v[2][1]);
-        // streaming stores: the image is written once (four frames to 1103x1103, whose rows do not fill whole sectors, 24.4 -> 23.4 us; to 1279x719 16.5 -> 14.9; whole lines the same)
+        // streaming stores: the image is written once (four frames to 1103x1103, whose rows do not fill
+        // whole sectors, 24.4 -> 23.3 us, and with the two columns side by side 21.1; to 1279x719 16.5 -> 15.0 -> 14.4; whole lines the same)
         float* d = out + o;
         __stcs(d, v[0][0]);
         __stcs(d + plane, v[1][0]);
         __stcs(d + 2 * (size_t)plane, v[2][0]);
         if (two) {
-          __stcs(d + COLS, v[0][1]);
-          __stcs(d + plane + COLS, v[1][1]);
-          __stcs(d + 2 * (size_t)plane + COLS, v[2][1]);
+          __stcs(d + 32, v[0][1]);
+          __stcs(d + plane + 32, v[1][1]);
+          __stcs(d + 2 * (size_t)plane + 32, v[2][1]);
         }
       }
     }
