@@ -21,7 +21,9 @@
 // 7.2 + 9.2 us for one stream, 100 against 38 + 61 us for 8 full-HD streams, where only the second launch's gap is won.  All that with the
 // output read back from shared memory and stored by the warps, and the resized image stored one column off its 128-byte lines; with tile
 // stores and whole lines (both sides in one call): a tick of eight full-HD streams 1049 -> 1034 us, of one 168.4 -> 166.9, of five 854x480 streams
-// 111.6 -> 110.7, of one 64.15 -> 63.9.
+// 111.6 -> 110.7, of one 64.15 -> 63.9.  The biases are operands in the constant bank: from shared memory they took the load/store unit 512 of a tile's 1800 cycles at 64 channels
+// (a 128-bit load four cycles, whether its lanes read one address or 32).  This launch in a tick, one, five 854x480 streams 7.44 -> 7.39, 17.0 -> 16.9 us, one, eight full-HD 15.35 -> 15.0,
+// 84.8 -> 82.2.
 #include <type_traits>
 
 #include "tt_internal.h"
@@ -58,8 +60,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
   uint8_t* s_a = smem;                                        // operand: two tiles of [128 rows][32] bf16
   uint8_t* s_out = s_a + A_BYTES;                             // OWN_OUT: per warp 32 pixels x 32 channels on their way out
   uint8_t* s_b = s_out + (OWN_OUT ? FF_WARPS * 2048 : 0);     // weights in operand layout
-  float* s_bias = reinterpret_cast<float*>(s_b + COUT * 64);
-  __nv_bfloat16* s_patch = reinterpret_cast<__nv_bfloat16*>(s_bias + COUT);      // [3][PH][PITCH]
+  __nv_bfloat16* s_patch = reinterpret_cast<__nv_bfloat16*>(s_b + COUT * 64);    // [3][PH][PITCH]
   uint8_t* s_src = reinterpret_cast<uint8_t*>(s_patch) + ((3 * PH * PITCH * 2 + 15) & ~15);   // [2][src_rows_cap][src_row_cap]
   // per buffer: of every patch row {offsets of its two frame rows in the buffer, bits of the lower one's weight, row of the
   // resized image or -1 outside it}, and the first staged byte column
@@ -253,9 +254,10 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
         uint32_t u[4];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
-          const float4 b = *reinterpret_cast<const float4*>(s_bias + ck * 32 + i + 4 * q);
-          u[2 * q] = pack_relu_bf16(__uint_as_float(v[i + 4 * q]) + b.x, __uint_as_float(v[i + 4 * q + 1]) + b.y);
-          u[2 * q + 1] = pack_relu_bf16(__uint_as_float(v[i + 4 * q + 2]) + b.z, __uint_as_float(v[i + 4 * q + 3]) + b.w);
+          const int c = i + 4 * q;
+          const float* b = p.bias_v + ck * 32 + c;
+          u[2 * q] = pack_relu_bf16(__uint_as_float(v[c]) + b[0], __uint_as_float(v[c + 1]) + b[1]);
+          u[2 * q + 1] = pack_relu_bf16(__uint_as_float(v[c + 2]) + b[2], __uint_as_float(v[c + 3]) + b[3]);
         }
         *reinterpret_cast<uint4*>(mine + lane * 64 + (((i >> 3) ^ ((lane >> 1) & 3)) << 4)) = make_uint4(u[0], u[1], u[2], u[3]);
       }
@@ -295,9 +297,8 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
 #pragma unroll
   for (int i = 0; i < 2; ++i)
     if (i < n) { stage(ahead, i); advance(ahead); }
-  // weights and biases while the first rows are on their way
+  // weights while the first rows are on their way
   for (int i = tid; i < COUT * 4; i += FF_THREADS) reinterpret_cast<uint4*>(s_b)[i] = __ldg(reinterpret_cast<const uint4*>(p.w_packed) + i);
-  if (tid < COUT) s_bias[tid] = __ldg(p.bias + tid);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -357,7 +358,7 @@ __global__ void __launch_bounds__(FF_THREADS, FF_PER_SM) conv_first_fused_kernel
 // Dynamic shared memory of a block whose two buffers of frame rows take src_bytes.
 template <int COUT, int STRIDE, bool OWN_OUT>
 constexpr int ff_smem(int src_bytes) {
-  return 2 * 128 * 64 + (OWN_OUT ? FF_WARPS * 2048 : 0) + COUT * 64 + COUT * 4 + ((3 * ff_patch_h(STRIDE) * ff_pitch(STRIDE) * 2 + 15) & ~15) + src_bytes;
+  return 2 * 128 * 64 + (OWN_OUT ? FF_WARPS * 2048 : 0) + COUT * 64 + ((3 * ff_patch_h(STRIDE) * ff_pitch(STRIDE) * 2 + 15) & ~15) + src_bytes;
 }
 
 // Blocks of a form that a multiprocessor holds, by shared memory: a block takes 1 KB beside its own, and its static variables' up to the

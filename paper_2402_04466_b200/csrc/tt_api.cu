@@ -614,6 +614,7 @@ tt_status build(tt_ctx* ctx, const tt_weights* w) {
       f.in = ctx->pre; f.out = reinterpret_cast<__nv_bfloat16*>(ctx->enc_out[0]);
       f.H = c.net_h; f.W = c.net_w; f.Ho = ctx->lay_h[1]; f.Wo = ctx->lay_w[1]; f.stride = c.enc_stride[0]; f.cout = co;
       f.tiles_x = (f.Wo + 15) / 16; f.tiles_y = (f.Ho + 7) / 8;
+      std::copy(hb.begin(), hb.end(), f.bias_v);   // 32 or 64 channels
       f.w_packed = dw; f.bias = db; f.status = ctx->status_dev; f.wait_limit = ctx->wait_limit;
       {
         const cuuint64_t dims[4] = {(cuuint64_t)co, (cuuint64_t)f.Wo, (cuuint64_t)f.Ho, (cuuint64_t)S};

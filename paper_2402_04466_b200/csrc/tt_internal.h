@@ -128,6 +128,7 @@ struct ConvFirstTcParams {
   int32_t pdl;                // launch as a programmatic dependent of the previous kernel in the stream
   const uint16_t* w_packed;   // device, cout*32 bf16 in the MMA operand layout
   const float* bias;          // device, [cout]
+  float bias_v[64];           // the same by value: operands in the constant bank (conv_first_fused)
   int32_t* status;
   long long wait_limit;       // SM cycles after which a barrier wait gives up
   TensorMap128 map_rows;      // conv_first_fused: output again, box [32][32][1][1], 64B swizzle
