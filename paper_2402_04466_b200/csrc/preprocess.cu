@@ -37,17 +37,16 @@ constexpr int PRE_MAX_ROWS = 32;             // output rows of a tile
 constexpr int PRE_STAGE_BYTES = 26 * 1024;   // staged rows of a tile; two tiles of four blocks fit a multiprocessor
 constexpr int PRE_STATIC_BYTES = 2 * (PRE_MAX_ROWS * 16 + 64) + 16;   // the kernel's tables and barriers
 
-struct PreprocessArgs {
+struct alignas(32) PreprocessArgs {
   PreprocessParams p;
-  float scale, shift;
   int32_t tile_rows, tiles_x, tiles_y;
   int32_t rows_cap, row_cap;                 // staged rows of a tile, bytes of one (a multiple of 16)
   int32_t tiles_per_block, tiles_left;       // the first tiles_left blocks take one tile more
 };
-
 // What the sampling warps are told of a tile.
 struct alignas(16) TileInfo {
   int32_t img, y0, rows, tx;
+  int32_t left;              // first frame column
 };
 
 // Where a tile lies: image, tile column, first output row and their number, frame, first frame column, last byte of a staged row counted from its first, first frame
@@ -144,7 +143,7 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
     if (lane < a.tile_rows)
       s_row[buf][lane] = make_int4((t.sy.i0 - t.first) * a.row_cap + (int)((base_lo + (uint32_t)(t.sy.i0 * p.src_pitch)) & 15u),
                                    (t.sy.i1 - t.first) * a.row_cap + (int)((base_lo + (uint32_t)(t.sy.i1 * p.src_pitch)) & 15u), __float_as_int(t.sy.f), above == t.sy.i0);
-    if (lane == 0) s_tile[buf] = {t.img, t.y0, t.rows, t.tx};
+    if (lane == 0) s_tile[buf] = {t.img, t.y0, t.rows, t.tx, t.left};
   };
 
   // A warp issues its copies one behind the other: those of the first tile, which everything waits for, are shared out.
@@ -174,24 +173,23 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
   // -------------------------------------------------------------------------- samples
   const int col = tid % COLS, grp = tid / COLS;
   const uint32_t plane = (uint32_t)(p.net_h * p.net_w);
-  const f32x2 scale = pack2(a.scale, a.scale), shift = pack2(a.shift, a.shift);
+  const f32x2 scale = pack2(p.scale, p.scale), shift = pack2(p.shift, p.shift);
   int tx, x, xo_a, xo_b;
   f32x2 fx;
-  auto column = [&](int tile_x) {
+  auto column = [&](int tile_x, int left) {
     tx = tile_x;
     x = tx * TILE_W + 2 * (col & ~31) + (col & 31);
-    const int left = axis_sample(tx * TILE_W, p.src_w, p.net_w).i0;
     const AxisSample sa = axis_sample(min(x, p.net_w - 1), p.src_w, p.net_w), sb = axis_sample(min(x + 32, p.net_w - 1), p.src_w, p.net_w);
     xo_a = 3 * (sa.i0 - left);
     xo_b = 3 * (sb.i0 - left);
     fx = pack2(sa.f, sb.f);
   };
-  column(first.tx);                                    // while the first rows are on their way
+  column(first.tx, first.left);                                    // while the first rows are on their way
   __syncthreads();                                     // the first tile has been told of
   for (int i = 0; i < n; ++i) {
     const TileInfo& t = s_tile[i & 1];
     const int img = __shfl_sync(0xffffffffu, t.img, 0), rows = __shfl_sync(0xffffffffu, t.rows, 0);
-    if (t.tx != tx) column(t.tx);
+    if (t.tx != tx) column(t.tx, t.left);
     const bool ok = tc::mbar_wait_limit(tc::smem_u32(&s_full[i & 1]), (uint32_t)(i >> 1) & 1u, tc::WAIT_LIMIT_CYCLES);
     if (ok && x < p.net_w) {
       const uint32_t buf = tc::smem_u32(s_mem) + (uint32_t)((i & 1) * buf_bytes), buf_a = buf + (uint32_t)xo_a, buf_b = buf + (uint32_t)xo_b;
@@ -240,7 +238,7 @@ constexpr int DIR_TX = 32, DIR_TY = 8, DIR_OUT_W = DIR_TX * 4;   // threads of a
 
 // Fallback for extreme down-scaling factors whose footprint does not fit in shared memory:
 // taps are read straight from global memory (L1-cached byte loads).
-__global__ void __launch_bounds__(DIR_TX * DIR_TY) preprocess_direct_kernel(const __grid_constant__ PreprocessParams p, float scale, float shift) {
+__global__ void __launch_bounds__(DIR_TX * DIR_TY) preprocess_direct_kernel(const __grid_constant__ PreprocessParams p) {
   const int n = blockIdx.z;
   const uint8_t* __restrict__ src = p.src_tab ? p.src_tab[n] : p.src.p[n];
   const int yo = blockIdx.y * DIR_TY + threadIdx.y;
@@ -259,7 +257,7 @@ __global__ void __launch_bounds__(DIR_TX * DIR_TY) preprocess_direct_kernel(cons
       const float p10 = (float)__ldg(r1 + 3 * sx.i0 + c), p11 = (float)__ldg(r1 + 3 * sx.i1 + c);
       const float top = p00 + sx.f * (p01 - p00);
       const float bot = p10 + sx.f * (p11 - p10);
-      dst[c * plane + j] = fmaf(top + sy.f * (bot - top), scale, shift);
+      dst[c * plane + j] = fmaf(top + sy.f * (bot - top), p.scale, p.shift);
     }
   }
 }
@@ -280,8 +278,6 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   if (e != cudaSuccess) return e;
   PreprocessArgs a;
   a.p = p;
-  a.scale = pre::norm_scale(p.inv_div, p.inv_std);
-  a.shift = pre::norm_shift(p.mean, p.inv_std);
   a.tiles_x = (p.net_w + TILE_W - 1) / TILE_W;
   // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least, and the higher tile of
   // two that come out alike; another height where by it the busiest multiprocessor has at least a tenth less to do, a tile's latency counted as twelve
@@ -342,7 +338,7 @@ cudaError_t launch_preprocess(const PreprocessParams& p, cudaStream_t s) {
   cudaError_t e = over > 0 && over <= 64 ? launch_staged<64>(p, s, &fits) : launch_staged<128>(p, s, &fits);
   if (e != cudaSuccess || fits) return e;
   dim3 grid((p.net_w + DIR_OUT_W - 1) / DIR_OUT_W, (p.net_h + DIR_TY - 1) / DIR_TY, p.K);
-  preprocess_direct_kernel<<<grid, dim3(DIR_TX, DIR_TY), 0, s>>>(p, pre::norm_scale(p.inv_div, p.inv_std), pre::norm_shift(p.mean, p.inv_std));
+  preprocess_direct_kernel<<<grid, dim3(DIR_TX, DIR_TY), 0, s>>>(p);
   return cudaGetLastError();
 }
 

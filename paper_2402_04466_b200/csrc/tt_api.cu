@@ -783,7 +783,8 @@ PreprocessParams preprocess_params(const tt_ctx* ctx, int n0, int K, const Frame
   PreprocessParams pp;
   pp.src = frames; pp.src_tab = tab; pp.K = K; pp.src_w = c.src_w; pp.src_h = c.src_h; pp.src_pitch = c.src_pitch;
   pp.net_w = c.net_w; pp.net_h = c.net_h;
-  pp.inv_div = 1.0f / c.norm_div; pp.mean = c.norm_mean; pp.inv_std = 1.0f / c.norm_std;
+  pp.scale = pre::norm_scale(1.0f / c.norm_div, 1.0f / c.norm_std);
+  pp.shift = pre::norm_shift(c.norm_mean, 1.0f / c.norm_std);
   pp.dst = ctx->pre + (size_t)n0 * 3 * c.net_h * c.net_w;
   pp.status = ctx->status_dev;
   return pp;
@@ -1529,7 +1530,9 @@ tt_status tt_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_str
   PreprocessParams p{};
   for (int n = 0; n < K; ++n) p.src.p[n] = src_dev + (size_t)n * src_frame_stride;
   p.K = K; p.src_w = src_w; p.src_h = src_h; p.src_pitch = src_pitch; p.net_w = net_w; p.net_h = net_h;
-  p.inv_div = 1.0f / norm_div; p.mean = norm_mean; p.inv_std = 1.0f / norm_std; p.dst = dst_dev;
+  p.scale = pre::norm_scale(1.0f / norm_div, 1.0f / norm_std);
+  p.shift = pre::norm_shift(norm_mean, 1.0f / norm_std);
+  p.dst = dst_dev;
   cudaError_t e = launch_preprocess(p, reinterpret_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return fail(nullptr, TT_ERR_CUDA, "tt_preprocess: %s", cudaGetErrorString(e));
   return TT_OK;
