@@ -3,7 +3,7 @@
 // The resized fp32 image is an observable tensor of the context and is still written (unless the caller does not
 // want it), but nothing reads it back, and one launch with its start-up and drain is gone.
 //
-// Bound by the load/store pipe (at two full-HD frames 61 % of the active cycles, 89 % of it through shared memory; 58 % of the issue
+// Bound by the load/store pipe (at two full-HD frames 53 % of the active cycles, most of it through shared memory; 58 % of the issue
 // slots), the chain of phases below, and by HBM (8 full-HD frames: 50 MB in, 88 + 236 MB out).  A block of 8 warps takes tiles of 32 x 8 outputs in
 // turn, down a column of tiles, and every warp takes part in every phase, so the sampling has all the warps of
 // the multiprocessor (three blocks, two at the largest resize factors) at its disposal and the phases of different blocks overlap:

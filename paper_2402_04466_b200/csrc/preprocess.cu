@@ -7,8 +7,8 @@
 // that the row above has already blended horizontally is not fetched again.  A bilinear tap pair (two neighbouring RGB pixels = 6 bytes) is three 32-bit shared loads plus
 // funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
 // Bound by issue and by the start: every block's first tile comes before anything can be sampled (four full-HD frames: launch 2, first rows 3, two tiles 9 us).  Instructions per
-// pixel of three channels 117 -> 80.  Device time, us, of frames in L2 before / now: four full-HD frames to 1280x720 17.7 / 14.6, eight 33.0 / 27.0, one 6.1 / 5.8, eight to
-// 768x432 19.5 / 15.2, four 1280x960 to 640x480 9.0 / 8.3, two 960x540 to 1280x720 9.3 / 8.6; a call with frames from memory: 18.5 / 16.4, 34.8 / 29.5, 8.2 / 8.0, 20.5 / 17.8, 10.3 / 10.3.
+// pixel of three channels 117 -> 82, 78 -> 68 % of the issue slots.  Device time, us, of frames in L2 before / now: four full-HD frames to 1280x720 17.7 / 14.3, eight 33.0 / 27.0, one 6.1 / 5.8, eight to
+// 768x432 19.5 / 15.2, four 1280x960 to 640x480 9.0 / 8.3, two 960x540 to 1280x720 9.3 / 8.6 (launches of 3 to 4 us, one tile a block, up to 0.3 longer: three 428x240 to 320x240 3.0 / 3.2); a call with frames from memory: 18.5 / 16.4, 34.8 / 29.0, 8.2 / 7.2, 20.5 / 17.8, 10.3 / 10.3.
 // Not kept: per-thread asynchronous copies by the ninth warp (25 us), three and four tiles in flight of 8 to 16 rows (16.6 to 18.8), five or six blocks with smaller tiles.
 #include "tt_internal.h"
 #include "pre_math.cuh"
