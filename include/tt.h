@@ -307,7 +307,7 @@ tt_status tt_get_counters(const tt_ctx* ctx, uint64_t* kernel_launches, uint64_t
 
 /*
  * tt_debug_expire_wait — failure-path probe, for tests.  Every barrier wait inside the kernels is
- * bounded: when one runs out the kernel records a code in the context's status word and returns,
+ * bounded: when one runs out the kernel records a code in the context's status word and gives up,
  * and the tt_sync of that tick answers TT_ERR_DEVICE_STATUS (the paper's systems have no such
  * path; it is this library's reading of "a failed client must not take the GPU down with it",
  * Section IV-A).  This call enqueues, on the context's stream, one warp that waits through that
@@ -331,10 +331,20 @@ tt_status tt_debug_expire_wait(tt_ctx* ctx, uint64_t limit_cycles);
  * (16-byte alignment with net_w a multiple of 4 lets the kernel use 128-bit stores).  For output sample o of
  * an axis resized from `in` to `out`: s = clamp((o+1/2)*in/out - 1/2, 0, in-1) evaluated in
  * exact integer arithmetic, i0 = floor(s), i1 = min(i0+1, in-1), weight s - i0.
+ * The kernel's wait for staged frame rows is bounded.  Should one run out (which no healthy device produces), the rest is
+ * sampled from memory directly: the image is whole and the same bits, so this call needs no status word.
  */
 tt_status tt_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_stride, int32_t src_w,
                         int32_t src_h, int32_t src_pitch, float* dst_dev, int32_t net_w, int32_t net_h,
                         float norm_div, float norm_mean, float norm_std, void* cuda_stream);
+
+/*
+ * tt_debug_preprocess_expired — tt_preprocess in which every block gives up its waits for frame rows at once from its
+ * from_tile-th tile on (0: all of them), for tests of the path behind such a wait.  Same output.
+ */
+tt_status tt_debug_preprocess_expired(const uint8_t* src_dev, int32_t K, int64_t src_frame_stride, int32_t src_w,
+                                      int32_t src_h, int32_t src_pitch, float* dst_dev, int32_t net_w, int32_t net_h,
+                                      float norm_div, float norm_mean, float norm_std, int32_t from_tile, void* cuda_stream);
 
 /*
  * tt_postprocess — S4+S5, the tool-tracking post-processing operator of Section III-A.
@@ -346,10 +356,9 @@ tt_status tt_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_str
  * scratch_dev: tt_postprocess_scratch_bytes(...) bytes of device memory, 8-byte aligned; the call
  * clears it first, contents on entry are ignored.
  * hidden must be a multiple of 4 and at most 512; hm, wm at most 16384.  A misaligned or null
- * pointer is answered with TT_ERR_INVALID_ARG before anything is launched.  The stage-level calls
- * have no status word: a bounded device-side wait that ran out inside them (which no healthy
- * device produces) leaves the outputs incomplete without an error code; contexts report it
- * through tt_sync.
+ * pointer is answered with TT_ERR_INVALID_ARG before anything is launched.  This call has no
+ * status word: a bounded device-side wait that ran out inside it (which no healthy device
+ * produces) leaves its outputs incomplete without an error code; contexts report it through tt_sync.
  */
 size_t tt_postprocess_scratch_bytes(int32_t K, int32_t hm, int32_t wm, int32_t hidden, int32_t n_tools);
 tt_status tt_postprocess(const float* h_dev, int32_t channels_last, int32_t K, int32_t hm, int32_t wm,

@@ -30,7 +30,7 @@ TENSOR_IDS = {"pre": 0, "enc0": 1, "enc1": 2, "enc2": 3, "enc3": 4, "h": 8, "c":
 EXPORTED_SYMBOLS = [
     "tt_abi_version", "tt_create", "tt_destroy", "tt_last_error", "tt_map_size", "tt_state_create",
     "tt_state_reset", "tt_state_export", "tt_state_import", "tt_submit_frames", "tt_sync", "tt_debug_tensor",
-    "tt_set_profiling", "tt_get_stage_times", "tt_get_counters", "tt_query", "tt_debug_expire_wait",
+    "tt_set_profiling", "tt_get_stage_times", "tt_get_counters", "tt_query", "tt_debug_expire_wait", "tt_debug_preprocess_expired",
     "tt_sched_create", "tt_sched_destroy", "tt_sched_admit", "tt_sched_release", "tt_sched_arrive", "tt_sched_next",
     "tt_sched_complete", "tt_sched_predict_ms", "tt_sched_stats",
     "tt_preprocess", "tt_postprocess_scratch_bytes", "tt_postprocess", "tt_postprocess_static", "tt_overlay", "tt_render_layers",
@@ -133,6 +133,7 @@ def load_library(build_if_missing: bool = True) -> C.CDLL:
     lib.tt_sched_predict_ms.argtypes = [vp, i32, C.POINTER(f32)]
     lib.tt_sched_stats.argtypes = [vp, u64p, u64p, u64p, u64p]
     lib.tt_preprocess.argtypes = [vp, i32, i64, i32, i32, i32, vp, i32, i32, f32, f32, f32, vp]
+    lib.tt_debug_preprocess_expired.argtypes = [vp, i32, i64, i32, i32, i32, vp, i32, i32, f32, f32, f32, i32, vp]
     lib.tt_postprocess_scratch_bytes.argtypes = [i32, i32, i32, i32, i32]
     lib.tt_postprocess_scratch_bytes.restype = C.c_size_t
     lib.tt_postprocess.argtypes = [vp, i32, i32, i32, i32, i32, i32, vp, vp, vp, vp, i32, f32, vp, vp, vp, vp, vp, vp]

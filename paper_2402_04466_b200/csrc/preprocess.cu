@@ -35,12 +35,14 @@ __device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
 constexpr int PRE_SAMPLERS = 256, PRE_THREADS = PRE_SAMPLERS + 32, PRE_WARPS = PRE_THREADS / 32, PRE_PER_SM = 4;
 constexpr int PRE_MAX_ROWS = 32;             // output rows of a tile
 constexpr int PRE_STAGE_BYTES = 26 * 1024;   // staged rows of a tile; two tiles of four blocks fit a multiprocessor
+constexpr long long PRE_LAND_CYCLES = 2000000;   // how long a block that has given up a wait stays for copies in flight: about a millisecond
 constexpr int PRE_STATIC_BYTES = 2 * (PRE_MAX_ROWS * 16 + 64) + 16;   // the kernel's tables and barriers
 
 struct alignas(32) PreprocessArgs {
   PreprocessParams p;
   int32_t tile_rows, tiles_x, tiles_y;
   int32_t rows_cap, row_cap;                 // staged rows of a tile, bytes of one (a multiple of 16)
+  int32_t expire_from = 0x7fffffff;          // the first tile of a block whose wait gives up at once (tests)
   int32_t tiles_per_block, tiles_left;       // the first tiles_left blocks take one tile more
 };
 // What the sampling warps are told of a tile.
@@ -83,6 +85,37 @@ __device__ __forceinline__ Blend blend_row(uint32_t addr_a, uint32_t addr_b, f32
   const f32x2 l0 = magic2(a.lo, b.lo, 0x7440), l1 = magic2(a.lo, b.lo, 0x7441), l2 = magic2(a.lo, b.lo, 0x7442);
   return {fma2(fx, sub2(magic2(a.lo, b.lo, 0x7443), l0), sub2(l0, magic)), fma2(fx, sub2(magic2(a.hi, b.hi, 0x7440), l1), sub2(l1, magic)),
           fma2(fx, sub2(magic2(a.hi, b.hi, 0x7441), l2), sub2(l2, magic))};
+}
+
+// One output pixel from taps straight in memory, with the frame's rows r0 and r1: the same bits as from staged rows.
+__device__ __forceinline__ void direct_pixel(const PreprocessParams& p, const uint8_t* __restrict__ r0, const uint8_t* __restrict__ r1, float fy, float* dst, size_t plane, int x) {
+  const AxisSample sx = axis_sample(x, p.src_w, p.net_w);
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float p00 = (float)__ldg(r0 + 3 * sx.i0 + c), p01 = (float)__ldg(r0 + 3 * sx.i1 + c);
+    const float p10 = (float)__ldg(r1 + 3 * sx.i0 + c), p11 = (float)__ldg(r1 + 3 * sx.i1 + c);
+    const float top = p00 + sx.f * (p01 - p00);
+    const float bot = p10 + sx.f * (p11 - p10);
+    dst[c * plane] = fmaf(top + fy * (bot - top), p.scale, p.shift);
+  }
+}
+
+// A block's tiles from the i-th on, by one warp and without staging: where a wait for frame rows has run out.  In the copying warp, for the sampling warps' code is as fast
+// as without it only there (four full-HD frames 14.6 us; with the call behind their loop 15.3).
+template <int TILE_W>
+__device__ __noinline__ void sample_unstaged(const PreprocessArgs& a, int t_begin, int i, int n) {
+  const PreprocessParams& p = a.p;
+  const size_t plane = (size_t)p.net_h * p.net_w;
+  for (; i < n; ++i) {
+    const int col_tiles = (t_begin + i) / a.tiles_y, img = col_tiles / a.tiles_x, x0 = (col_tiles - img * a.tiles_x) * TILE_W;
+    const int y0 = (t_begin + i - col_tiles * a.tiles_y) * a.tile_rows, rows = min(a.tile_rows, p.net_h - y0), cols = min(TILE_W, p.net_w - x0);
+    const uint8_t* src = p.src_tab ? p.src_tab[img] : p.src.p[img];
+    for (int k = threadIdx.x & 31; k < rows * cols; k += 32) {
+      const int y = y0 + k / cols, x = x0 + k % cols;
+      const AxisSample sy = axis_sample(y, p.src_h, p.net_h);
+      direct_pixel(p, src + (size_t)sy.i0 * p.src_pitch, src + (size_t)sy.i1 * p.src_pitch, sy.f, p.dst + (size_t)img * 3 * plane + (size_t)y * p.net_w + x, plane, x);
+    }
+  }
 }
 
 // ONE_ROW: the height is not resized, so every sample sits on a source row (weight zero for the next one).
@@ -162,8 +195,10 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
         if (lane == 0) mbar_arrive_n(tc::smem_u32(&s_full[i & 1]), PRE_WARPS);
         tell(t, i & 1);
       }
-      if (__syncthreads_or(0)) {                       // tile i - 1 has been sampled; or a wait has run out: let what is in flight land
-        for (int w = 0; w < 64; ++w) __nanosleep(16000);
+      if (__syncthreads_or(0)) {                       // tile i - 1 has been sampled; or a wait has run out: what is in flight may still land, then the rest by this warp
+        tc::mbar_wait_limit(tc::smem_u32(&s_full[(i - 1) & 1]), (uint32_t)((i - 1) >> 1) & 1u, PRE_LAND_CYCLES);
+        if (i < n) tc::mbar_wait_limit(tc::smem_u32(&s_full[i & 1]), (uint32_t)(i >> 1) & 1u, PRE_LAND_CYCLES);
+        sample_unstaged<TILE_W>(a, t_begin, i - 1, n);
         break;
       }
     }
@@ -190,7 +225,7 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
     const TileInfo& t = s_tile[i & 1];
     const int img = __shfl_sync(0xffffffffu, t.img, 0), rows = __shfl_sync(0xffffffffu, t.rows, 0);
     if (t.tx != tx) column(t.tx, t.left);
-    const bool ok = tc::mbar_wait_limit(tc::smem_u32(&s_full[i & 1]), (uint32_t)(i >> 1) & 1u, tc::WAIT_LIMIT_CYCLES);
+    const bool ok = i < a.expire_from && tc::mbar_wait_limit(tc::smem_u32(&s_full[i & 1]), (uint32_t)(i >> 1) & 1u, p.wait_limit);
     if (ok && x < p.net_w) {
       const uint32_t buf = tc::smem_u32(s_mem) + (uint32_t)((i & 1) * buf_bytes), buf_a = buf + (uint32_t)xo_a, buf_b = buf + (uint32_t)xo_b;
       const bool two = x + 32 < p.net_w;
@@ -249,17 +284,7 @@ __global__ void __launch_bounds__(DIR_TX * DIR_TY) preprocess_direct_kernel(cons
   const uint8_t* r1 = src + (size_t)sy.i1 * p.src_pitch;
   const size_t plane = (size_t)p.net_h * p.net_w;
   float* dst = p.dst + (size_t)n * 3 * plane + (size_t)yo * p.net_w + xo0;
-  for (int j = 0; j < 4 && xo0 + j < p.net_w; ++j) {
-    const AxisSample sx = axis_sample(xo0 + j, p.src_w, p.net_w);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float p00 = (float)__ldg(r0 + 3 * sx.i0 + c), p01 = (float)__ldg(r0 + 3 * sx.i1 + c);
-      const float p10 = (float)__ldg(r1 + 3 * sx.i0 + c), p11 = (float)__ldg(r1 + 3 * sx.i1 + c);
-      const float top = p00 + sx.f * (p01 - p00);
-      const float bot = p10 + sx.f * (p11 - p10);
-      dst[c * plane + j] = fmaf(top + sy.f * (bot - top), p.scale, p.shift);
-    }
-  }
+  for (int j = 0; j < 4 && xo0 + j < p.net_w; ++j) direct_pixel(p, r0, r1, sy.f, dst + j, plane, xo0 + j);
 }
 
 // Staged rows and bytes per row of a tile in the worst case: rows = ceil(tile_rows * sh/nh) + 2; bytes = 3 * (ceil(cols * sw/nw) + 2) + 15
@@ -278,6 +303,8 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   if (e != cudaSuccess) return e;
   PreprocessArgs a;
   a.p = p;
+  a.p.wait_limit = p.wait_limit > 0 ? p.wait_limit : tc::WAIT_LIMIT_CYCLES;
+  if (p.wait_limit < 0) a.expire_from = (int)~p.wait_limit;
   a.tiles_x = (p.net_w + TILE_W - 1) / TILE_W;
   // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least, and the higher tile of
   // two that come out alike; another height where by it the busiest multiprocessor has at least a tenth less to do, a tile's latency counted as twelve

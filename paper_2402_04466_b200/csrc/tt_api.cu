@@ -786,7 +786,7 @@ PreprocessParams preprocess_params(const tt_ctx* ctx, int n0, int K, const Frame
   pp.scale = pre::norm_scale(1.0f / c.norm_div, 1.0f / c.norm_std);
   pp.shift = pre::norm_shift(c.norm_mean, 1.0f / c.norm_std);
   pp.dst = ctx->pre + (size_t)n0 * 3 * c.net_h * c.net_w;
-  pp.status = ctx->status_dev;
+  pp.status = ctx->status_dev; pp.wait_limit = ctx->wait_limit;
   return pp;
 }
 
@@ -1436,7 +1436,9 @@ tt_status tt_debug_tensor(tt_ctx* ctx, tt_state* st, int32_t which, float* host_
     n = (size_t)3 * ctx->cfg.net_h * ctx->cfg.net_w;
     if (ctx->fuse_pre) {
       // the resized image never reached memory: make it now, from the frame buffers of that submit
-      TT_CUDA(ctx, launch_preprocess(preprocess_params(ctx, 0, ctx->K_inflight, ctx->fp_inflight, nullptr), s));
+      PreprocessParams pp = preprocess_params(ctx, 0, ctx->K_inflight, ctx->fp_inflight, nullptr);
+      pp.status = nullptr;   // no tick's report
+      TT_CUDA(ctx, launch_preprocess(pp, s));
     }
     src = ctx->pre + (size_t)pos * n;
   } else if (which >= TT_TENSOR_ENC0 && which < TT_TENSOR_ENC0 + ctx->n_enc) {
@@ -1519,9 +1521,9 @@ tt_status check_post_args(const char* who, const float* h_dev, int32_t channels_
 }
 }  // namespace
 
-tt_status tt_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_stride, int32_t src_w, int32_t src_h,
-                        int32_t src_pitch, float* dst_dev, int32_t net_w, int32_t net_h, float norm_div,
-                        float norm_mean, float norm_std, void* cuda_stream) {
+static tt_status run_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_stride, int32_t src_w, int32_t src_h,
+                                int32_t src_pitch, float* dst_dev, int32_t net_w, int32_t net_h, float norm_div,
+                                float norm_mean, float norm_std, long long wait_limit, void* cuda_stream) {
   if (!src_dev || !dst_dev || K < 1 || K > TT_MAX_STREAMS || src_w < 1 || src_h < 1 || net_w < 1 || net_h < 1 ||
       src_w > 16384 || src_h > 16384 || net_w > 16384 || net_h > 16384 || src_pitch < 3 * src_w || norm_div == 0.f ||
       norm_std == 0.f)
@@ -1532,10 +1534,23 @@ tt_status tt_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_str
   p.K = K; p.src_w = src_w; p.src_h = src_h; p.src_pitch = src_pitch; p.net_w = net_w; p.net_h = net_h;
   p.scale = pre::norm_scale(1.0f / norm_div, 1.0f / norm_std);
   p.shift = pre::norm_shift(norm_mean, 1.0f / norm_std);
-  p.dst = dst_dev;
+  p.dst = dst_dev; p.wait_limit = wait_limit;
   cudaError_t e = launch_preprocess(p, reinterpret_cast<cudaStream_t>(cuda_stream));
   if (e != cudaSuccess) return fail(nullptr, TT_ERR_CUDA, "tt_preprocess: %s", cudaGetErrorString(e));
   return TT_OK;
+}
+
+tt_status tt_preprocess(const uint8_t* src_dev, int32_t K, int64_t src_frame_stride, int32_t src_w, int32_t src_h,
+                        int32_t src_pitch, float* dst_dev, int32_t net_w, int32_t net_h, float norm_div,
+                        float norm_mean, float norm_std, void* cuda_stream) {
+  return run_preprocess(src_dev, K, src_frame_stride, src_w, src_h, src_pitch, dst_dev, net_w, net_h, norm_div, norm_mean, norm_std, 0, cuda_stream);
+}
+
+tt_status tt_debug_preprocess_expired(const uint8_t* src_dev, int32_t K, int64_t src_frame_stride, int32_t src_w, int32_t src_h,
+                                      int32_t src_pitch, float* dst_dev, int32_t net_w, int32_t net_h, float norm_div,
+                                      float norm_mean, float norm_std, int32_t from_tile, void* cuda_stream) {
+  if (from_tile < 0) return fail(nullptr, TT_ERR_INVALID_ARG, "tt_debug_preprocess_expired: from_tile must not be negative");
+  return run_preprocess(src_dev, K, src_frame_stride, src_w, src_h, src_pitch, dst_dev, net_w, net_h, norm_div, norm_mean, norm_std, ~(long long)from_tile, cuda_stream);
 }
 
 size_t tt_postprocess_scratch_bytes(int32_t K, int32_t hm, int32_t wm, int32_t hidden, int32_t n_tools) {

@@ -79,7 +79,8 @@ struct PreprocessParams {
   int32_t K, src_w, src_h, src_pitch, net_w, net_h;
   float scale, shift;              // v * scale + shift normalises (pre::norm_scale, pre::norm_shift)
   float* dst;  // [K][3][net_h][net_w]
-  int32_t* status = nullptr;   // optional device word: set non-zero when a bounded wait ran out
+  int32_t* status = nullptr;   // optional device word: set non-zero when a bounded wait ran out (the image is whole all the same)
+  long long wait_limit = 0;    // SM cycles after which a wait for frame rows gives up (0: the default); ~t below zero: at once from a block's t-th tile on (tests)
 };
 cudaError_t launch_preprocess(const PreprocessParams& p, cudaStream_t s);
 

@@ -275,6 +275,24 @@ def test_preprocess_of_a_frame_is_the_same_whatever_shares_its_launch(cuda_devic
         assert torch.equal(binding.preprocess(frames[k:k + 1], sw, sh, 3 * sw + pad, nw, nh)[0], batch[k])
 
 
+@pytest.mark.parametrize("from_tile", [0, 1, 2])
+@pytest.mark.parametrize("src,net,pad,K", [
+    ((97, 61), (191, 95), 2, 8),         # one tile a block
+    ((1920, 1080), (1279, 717), 1, 4),   # two or three
+    ((854, 720), (1216, 720), 3, 8),     # five or six narrow ones, the height not resized
+])
+def test_preprocess_whose_waits_run_out_still_makes_the_whole_image(cuda_device, src, net, pad, K, from_tile):
+    """Behind a wait that gave up (here at once, the rows on their way) a block takes the rest of its tiles from memory: every float, the same bits."""
+    (sw, sh), (nw, nh) = src, net
+    frames = torch.from_numpy(np.random.default_rng(8).integers(0, 256, (K, sh * (3 * sw + pad)), dtype=np.uint8)).to(cuda_device)
+    whole = binding.preprocess(frames, sw, sh, 3 * sw + pad, nw, nh)
+    got = torch.full_like(whole, float("nan"))
+    assert binding.load_library().tt_debug_preprocess_expired(frames.data_ptr(), K, frames.stride(0), sw, sh, 3 * sw + pad, got.data_ptr(), nw, nh,
+                                                              255.0, 0.5, 0.25, from_tile, None) == 0
+    torch.cuda.synchronize()
+    assert torch.equal(got, whole)
+
+
 @pytest.mark.parametrize("shape,K", [
     (dict(src_w=854, src_h=480, net_w=640, net_h=480, hidden=128), 5),                        # parts of 2 and 3 streams
     (dict(src_w=854, src_h=480, net_w=642, net_h=480, hidden=128), 6),                        # parts of 3; first layer on the fp32 kernel

@@ -53,6 +53,12 @@ def test_status_codes_name_the_kernel():
             m = re.fullmatch(r"(?:tc::)?(WAIT_[A-Z0-9_]+)((?: \+ .*)?)", w)
             assert m and m.group(1) in bases, (name, w)
             of_file.setdefault(m.group(1), {}).setdefault(name, []).append(m.group(2))
+        # kernels without an abort flag wait by a limit of their own, which the host gives them too, and report behind the wait
+        calls = re.sub(r"bool sw_wait\([^{]*\{", "", code)
+        own = re.findall(r"\b(?:mbar_wait_limit|sw_wait)\([^;]*?, (?:p\.)?(\w+)\)[;,)]", calls)
+        assert len(own) == calls.count("mbar_wait_limit(") + calls.count("sw_wait(") and set(own) <= {"wait_limit", "PRE_LAND_CYCLES"}
+        if own:
+            assert "p.wait_limit > 0 ? p.wait_limit :" in code and "atomicCAS(p.status" in code
     for base, files in of_file.items():
         assert len(files) == 1, f"{base} is used by {sorted(files)}"
     assert set(of_file) == set(bases) - {"WAIT_PROBE"}
@@ -94,3 +100,11 @@ def test_a_turn_of_the_ring_waits_for_each_stages_last_use_once(producers, stage
                     if stage >= stages:
                         stage, phase = stage - stages, phase ^ 1
             assert sorted(waited) == list(range(total - stages, total))     # negative: never used, the wait returns at once
+
+
+def test_every_kernel_that_waits_is_given_the_contexts_limit():
+    """A context's ticks pass its limit and its status word to every kernel that has both."""
+    lines = [line for line in SOURCES["tt_api.cu"].splitlines() if ".status = ctx->status_dev" in line]
+    assert len(lines) == 7
+    for line in lines:
+        assert re.search(r"(\w+)\.status = ctx->status_dev;.* \1\.wait_limit = ctx->wait_limit;", line), line
