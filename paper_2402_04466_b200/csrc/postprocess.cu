@@ -900,7 +900,7 @@ cudaError_t post_sm_count(int* out) {
 }
 
 cudaError_t post_prepare() {
-  static OncePerDevice once;
+  static OncePerContext once;
   return once([]() {
     cudaError_t e = cudaFuncSetAttribute(post_tile_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)post_smem_bytes(512));
     if (e != cudaSuccess) return e;

@@ -345,7 +345,7 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   const size_t smem = (size_t)2 * a.rows_cap * a.row_cap;
   auto kern = p.src_h == p.net_h ? preprocess_staged_kernel<TILE_W, true> : preprocess_staged_kernel<TILE_W, false>;
   if (smem + PRE_STATIC_BYTES > 48 * 1024) {   // what a kernel may have of both without asking
-    static OncePerDevice once;
+    static OncePerContext once;
     e = once([]() {
       const cudaError_t r = cudaFuncSetAttribute(preprocess_staged_kernel<TILE_W, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * PRE_STAGE_BYTES);
       return r != cudaSuccess ? r : cudaFuncSetAttribute(preprocess_staged_kernel<TILE_W, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * PRE_STAGE_BYTES);

@@ -71,6 +71,24 @@ EncodeTiledFn get_encode_fn() {
   return fn;
 }
 
+}  // namespace
+
+uint64_t tt::context_number() {
+  typedef CUresult (*IdFn)(CUcontext, unsigned long long*);
+  static IdFn fn = nullptr;
+  static std::once_flag once;
+  std::call_once(once, [] {
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint("cuCtxGetId", &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess)
+      fn = reinterpret_cast<IdFn>(p);
+  });
+  unsigned long long id = 0;
+  return fn && fn(nullptr, &id) == CUDA_SUCCESS ? (uint64_t)id : 0;
+}
+
+namespace {
+
 // Whether two host pointers lie in one pinned allocation (pageable memory: no).
 bool same_pinned_range(const void* a, const void* b) {
   typedef CUresult (*AttributeFn)(void*, CUpointer_attribute, CUdeviceptr);

@@ -44,18 +44,20 @@ inline cudaError_t launch_kernel(void (*kern)(const Params), dim3 grid, int bloc
   return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
-// Runs what has to be done once on every device (kernel attributes: 0.9 us each on every call otherwise) until it has succeeded there.
-struct OncePerDevice {
-  std::atomic<uint64_t> done{0};
+// The current context's number: no other context of the process, before it or after it, has the same.  0 where none is current yet.
+uint64_t context_number();
+
+// Runs what has to be done once in every context (kernel attributes: 0.9 us each on every call otherwise) until it has succeeded there.  A kernel's attributes are
+// its context's: a device reset takes them along, and a second context on the device has its own.  Contexts whose numbers meet in one entry run it again.
+struct OncePerContext {
+  std::atomic<uint64_t> done[64] = {};
   template <typename F>
   cudaError_t operator()(F&& f) {
-    int dev = -1;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e != cudaSuccess) return e;
-    const uint64_t bit = dev >= 0 && dev < 64 ? 1ull << dev : 0;
-    if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
-    e = f();
-    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+    const uint64_t ctx = context_number();
+    std::atomic<uint64_t>& at = done[ctx % 64];
+    if (ctx != 0 && at.load(std::memory_order_acquire) == ctx) return cudaSuccess;
+    const cudaError_t e = f();
+    if (e == cudaSuccess) at.store(ctx, std::memory_order_release);
     return e;
   }
 };

@@ -152,9 +152,16 @@ static int pointer_attribute(void* out, int what, uintptr_t p) {
     if (p >= pinned[i].lo && p < pinned[i].hi) { *(uintptr_t*)out = pinned[i].lo; return 0; }
   return 1;
 }
+/* A context is gone and another current: kernels are as they were loaded.  No two have the same number. */
+static unsigned long long context_id = 7;
+void fake_new_context(void) {
+  ++context_id;
+  for (int i = 0; i < n_kernels; ++i) kernels[i].max_smem = 47 * 1024;
+}
+static int context_number(void* ctx, unsigned long long* id) { (void)ctx; *id = context_id; return 0; }
 cudaError_t cudaGetDriverEntryPoint(const char* name, void** f, unsigned long long flags, enum cudaDriverEntryPointQueryResult* q) {
   (void)flags;
-  *f = !strcmp(name, "cuPointerGetAttribute") ? (void*)pointer_attribute : (void*)encode_tiled;
+  *f = !strcmp(name, "cuPointerGetAttribute") ? (void*)pointer_attribute : !strcmp(name, "cuCtxGetId") ? (void*)context_number : (void*)encode_tiled;
   if (q) *q = cudaDriverEntryPointSuccess;
   return cudaSuccess;
 }

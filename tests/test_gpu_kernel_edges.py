@@ -1,4 +1,8 @@
 """Sizes at which a kernel's tiles, remainders or dispatch rules could go wrong, against the CPU oracle."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 import torch
@@ -291,6 +295,47 @@ def test_preprocess_whose_waits_run_out_still_makes_the_whole_image(cuda_device,
                                                               255.0, 0.5, 0.25, from_tile, None) == 0
     torch.cuda.synchronize()
     assert torch.equal(got, whole)
+
+
+_TWO_CONTEXTS = """
+import ctypes as C, sys
+import numpy as np
+from paper_2402_04466_b200 import binding
+cu, lib = C.CDLL("libcuda.so.1"), binding.load_library()
+def do(name, *args):
+    assert getattr(cu, name)(*args) == 0, name
+def alloc(n):
+    p = C.c_void_p()
+    do("cuMemAlloc_v2", C.byref(p), C.c_size_t(n))
+    return p
+frame, out = np.random.default_rng(9).integers(0, 256, 1920 * 1080 * 3, dtype=np.uint8), []
+def stage():
+    src, dst, got = alloc(frame.size), alloc(3 * 520 * 292 * 4), np.zeros(3 * 520 * 292, np.float32)
+    do("cuMemcpyHtoD_v2", src, frame.ctypes.data_as(C.c_void_p), C.c_size_t(frame.size))
+    for _ in range(2):
+        assert lib.tt_preprocess(src, 1, 0, 1920, 1080, 3 * 1920, dst, 520, 292, 255.0, 0.5, 0.25, None) == 0, lib.tt_last_error(None)
+    do("cuCtxSynchronize")
+    do("cuMemcpyDtoH_v2", got.ctypes.data_as(C.c_void_p), dst, C.c_size_t(got.nbytes))
+    out.append(got)
+do("cuInit", 0)
+dev, first, second, popped = C.c_int(), C.c_void_p(), C.c_void_p(), C.c_void_p()
+do("cuDeviceGet", C.byref(dev), 0)
+do("cuDevicePrimaryCtxRetain", C.byref(first), dev)
+do("cuCtxPushCurrent_v2", first)
+stage()
+do("cuCtxCreate_v2", C.byref(second), 0, dev)
+stage()
+do("cuCtxPopCurrent_v2", C.byref(popped))
+stage()
+assert out[0].any() and all(np.array_equal(out[0], x) for x in out[1:])
+print("three alike")
+"""
+
+
+def test_calls_in_a_second_context_of_the_device(cuda_device):
+    """More shared memory than a kernel gets unasked, in a context of its own that knows nothing of what the first one's kernels were given."""
+    r = subprocess.run([sys.executable, "-c", _TWO_CONTEXTS], capture_output=True, text=True, timeout=240, cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0 and "three alike" in r.stdout, r.stderr[-2000:]
 
 
 @pytest.mark.parametrize("shape,K", [

@@ -297,3 +297,20 @@ def test_tiles_of_the_preprocessing_and_where_it_stages_none(fake, src, net, K, 
     assert fake.tt_preprocess(at, K, 3 * src[0] * src[1], *src, 3 * src[0], at + 0x10000000, *net, 255.0, 0.5, 0.25, None) == 0
     (line,) = [x for x in fake.fake_log().decode().splitlines() if x.startswith("launch")]
     assert line.endswith(f" smem {smem}") and (f"preprocess_staged_kernelILi{cols}E" if smem else "preprocess_direct_kernel") in line
+
+
+def test_kernel_attributes_are_set_in_every_context(fake):
+    """Kernels of a context that came after another one (a device reset, a second context on the device) know nothing of what the first one's were given."""
+    at = 0x7F0000000000
+    wl = dict(WORKLOAD, src_w=854, src_h=480, net_w=640, net_h=480, enc_cout=(32, 64), hidden=128, precision="bf16")
+    for _ in range(3):
+        for _ in range(2):
+            assert fake.tt_preprocess(at, 1, 3 * 1920 * 1080, 1920, 1080, 3 * 1920, at + 0x10000000, 520, 292, 255.0, 0.5, 0.25, None) == 0
+            for hidden in (16, 128, 256, 512):
+                args = (at, 1, 2, 9, 16, hidden, 3, at, at, None, None, 0, 0.5, at, at, at, at)
+                assert fake.tt_postprocess_static(*args, None) == 0
+        s = Streams(fake, 1, workload=wl, post_tc=False)
+        assert s.submit(on_device=(0,))[0] == binding.TT_OK
+        s.sync()
+        s.ctx.destroy()
+        fake.fake_new_context()
