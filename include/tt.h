@@ -374,7 +374,7 @@ tt_status tt_postprocess(const float* h_dev, int32_t channels_last, int32_t K, i
  * that promised its host application a fixed memory footprint, plug-ins that are handed their
  * buffers by a framework's own allocator, and callers that keep a whole device reserved by
  * another pool.  Nothing is allocated or freed here, neither through CUDA nor through any
- * library (one exception: the very first call on a device makes the CUDA runtime load the
+ * library (one exception: the very first call in a context makes the CUDA runtime load the
  * library's device code, which the runtime does with allocations of its own; see below): the partial sums that tt_postprocess keeps in caller-provided scratch live in a
  * fixed array of TT_POSTPROCESS_STATIC_SCRATCH_BYTES that is part of the library image (each
  * GPU that loads the library holds that much memory until the process ends).  Inputs and
@@ -386,8 +386,8 @@ tt_status tt_postprocess(const float* h_dev, int32_t channels_last, int32_t K, i
  *     (32 KiB: 256 + K * 8 * (hidden + 32) bytes rounded up to 256, so 8 streams fit with up to 476
  *     hidden channels whatever the grid size; 8 streams of 512 hidden channels need 35 KB and are
  *     refused, 7 such streams fit);
- *   - the first call on a device looks up the array's device address and sets the kernels'
- *     shared-memory attributes (with that device current); make that first call, once, in a
+ *   - the first call in a CUDA context looks up the array's device address and sets the kernels'
+ *     shared-memory attributes (with that context current); make that first call, once, in a
  *     set-up phase and before starting any stream capture;
  *   - all calls on a device share the one array.  It keeps whatever the previous call left; the
  *     accumulators in it must start at zero, so every call clears the part it uses (a memset on

@@ -858,24 +858,24 @@ size_t post_smem_bytes(int ch) {
 
 size_t post_scratch_bytes(int K, int hm, int wm, int ch, int T) { return scratch_layout(K, hm * wm, ch, T).total; }
 
-// In host code the array's name is only a handle; the device address has to be asked for,
-// once per device, with that device current.
+// In host code the array's name is only a handle; the device address has to be asked for, once in every
+// context: each loads the array for itself, and a reset device's next context may have it elsewhere.
 cudaError_t post_static_scratch(void** ptr) {
-  constexpr int MAX_DEV = 64;
-  static void* addr[MAX_DEV] = {};
+  struct Loaded {
+    uint64_t ctx = 0;
+    void* addr = nullptr;
+  };
+  static Loaded loaded[64];
   static std::mutex mu;
-  int dev = -1;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  if (dev < 0 || dev >= MAX_DEV) return cudaErrorInvalidDevice;
+  const uint64_t ctx = context_number();
   std::lock_guard<std::mutex> lk(mu);
-  if (!addr[dev]) {
-    void* p = nullptr;
-    e = cudaGetSymbolAddress(&p, g_static_post_scratch);
+  Loaded& l = loaded[ctx % 64];
+  if (ctx == 0 || l.ctx != ctx) {
+    const cudaError_t e = cudaGetSymbolAddress(&l.addr, g_static_post_scratch);
+    l.ctx = e == cudaSuccess ? ctx : 0;
     if (e != cudaSuccess) return e;
-    addr[dev] = p;
   }
-  *ptr = addr[dev];
+  *ptr = l.addr;
   return cudaSuccess;
 }
 

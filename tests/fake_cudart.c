@@ -96,7 +96,7 @@ cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, enum cudaMemcpyKin
   note("copy %s %zu from %p to %p\n", k == cudaMemcpyHostToDevice ? "in" : "out", n, s, d);
   return e;
 }
-cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t s) { (void)s; memset(d, v, n); return cudaSuccess; }
+cudaError_t cudaMemsetAsync(void* d, int v, size_t n, cudaStream_t s) { (void)s; memset(d, v, n); note("clear %p %zu\n", d, n); return cudaSuccess; }
 static cudaError_t handle(void* out) { *(void**)out = malloc(8); return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { return handle(e); }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned f) { (void)f; return handle(e); }
@@ -125,7 +125,6 @@ cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v)
     if (kernels[i].host == f && a == cudaFuncAttributeMaxDynamicSharedMemorySize) kernels[i].max_smem = (size_t)v;
   return v <= 227 * 1024 ? cudaSuccess : cudaErrorInvalidValue;
 }
-cudaError_t cudaGetSymbolAddress(void** p, const void* s) { *p = (void*)s; return cudaSuccess; }
 cudaError_t cudaGetDevice(int* d) { *d = 0; return cudaSuccess; }
 cudaError_t cudaSetDevice(int d) { (void)d; return cudaSuccess; }
 cudaError_t cudaGetDeviceCount(int* n) { *n = 1; return cudaSuccess; }
@@ -152,11 +151,18 @@ static int pointer_attribute(void* out, int what, uintptr_t p) {
     if (p >= pinned[i].lo && p < pinned[i].hi) { *(uintptr_t*)out = pinned[i].lo; return 0; }
   return 1;
 }
+static unsigned char symbols[4][1 << 16] __attribute__((aligned(256)));   /* where a context keeps the library's one array */
 /* A context is gone and another current: kernels are as they were loaded.  No two have the same number. */
 static unsigned long long context_id = 7;
 void fake_new_context(void) {
   ++context_id;
   for (int i = 0; i < n_kernels; ++i) kernels[i].max_smem = 47 * 1024;
+}
+cudaError_t cudaGetSymbolAddress(void** p, const void* s) {
+  (void)s;
+  *p = symbols[context_id % 4];
+  note("symbol %p\n", *p);
+  return cudaSuccess;
 }
 static int context_number(void* ctx, unsigned long long* id) { (void)ctx; *id = context_id; return 0; }
 cudaError_t cudaGetDriverEntryPoint(const char* name, void** f, unsigned long long flags, enum cudaDriverEntryPointQueryResult* q) {

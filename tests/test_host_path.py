@@ -314,3 +314,17 @@ def test_kernel_attributes_are_set_in_every_context(fake):
         s.sync()
         s.ctx.destroy()
         fake.fake_new_context()
+
+
+def test_the_static_scratch_is_looked_up_in_every_context(fake):
+    """An address of a context that is gone is never handed to a kernel."""
+    at, seen = 0x7F0000000000, []
+    for _ in range(3):
+        fake.fake_new_context()
+        for again in range(2):
+            fake.fake_reset()
+            assert fake.tt_postprocess_static(at, 0, 1, 9, 16, 16, 3, at, at, None, None, 0, 0.5, at, at, at, at, None) == 0
+            asked, cleared = (re.findall(rf"^{word} (0x\w+)", fake.fake_log().decode(), re.M) for word in ("symbol", "clear"))
+            assert len(asked) == 1 - again
+            seen.append(cleared[0])
+    assert seen[0::2] == seen[1::2] and len(set(seen)) == 3
