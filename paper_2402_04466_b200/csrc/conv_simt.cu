@@ -361,10 +361,12 @@ cudaError_t launch_one(const ConvSimtParams& p, cudaStream_t s) {
   const int tiles = ((p.Wo + Cfg::TW - 1) / Cfg::TW) * ((p.Ho + Cfg::TH - 1) / Cfg::TH), groups = p.cout_packed / (WO * OC);
   // As a dependent the grid starts while its predecessor still holds some multiprocessors, and the others would be filled with as many blocks
   // as fit (three ConvLSTM maps of 80x60: 90 us instead of 67).  So a block asks for enough shared memory that one more than the busiest
-  // multiprocessor's even share does not fit.  Not where that share is one block: two kernels' blocks could not be resident side by side.
+  // multiprocessor's even share does not fit.  An encoder layer of one block to a multiprocessor asks for no more than it takes, so that it can lie beside its
+  // predecessor's blocks; a ConvLSTM of one block asks for its half all the same: its blocks ran in piles of up to four, how many depending on the registers of the layer
+  // before it (one and three maps of 40x30, 64 channels behind 64: 120, 161 -> 49, 69 us; of 80x60, 64 behind 32: 55, 127 -> 38, 60).
   constexpr int SMEM_SM = 228 * 1024, SMEM_RESERVED = 1024;      // of a multiprocessor, and per block beside its own
   const long share = ((long)tiles * groups * p.K + p.sm_count - 1) / p.sm_count;
-  const int smem = share == 1 ? Cfg::SMEM_BYTES : std::max<int>(Cfg::SMEM_BYTES, (int)(SMEM_SM / (std::min<long>(share, 15) + 1)) - SMEM_RESERVED + 16);
+  const int smem = share == 1 && EPI != EPI_LSTM_F32_NCHW ? Cfg::SMEM_BYTES : std::max<int>(Cfg::SMEM_BYTES, (int)(SMEM_SM / (std::min<long>(share, 15) + 1)) - SMEM_RESERVED + 16);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_SM - SMEM_RESERVED);
   if (e != cudaSuccess) return e;
   return launch_kernel(kern, dim3(tiles, groups, p.K), Cfg::THREADS, smem, s, p, p.pdl != 0);

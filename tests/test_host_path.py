@@ -328,3 +328,19 @@ def test_the_static_scratch_is_looked_up_in_every_context(fake):
             assert len(asked) == 1 - again
             seen.append(cleared[0])
     assert seen[0::2] == seen[1::2] and len(set(seen)) == 3
+
+
+@pytest.mark.parametrize("net,enc,stride,hidden,K", [
+    ((40, 30), (32, 64), (1, 1), 64, 1), ((40, 30), (32, 64), (1, 1), 64, 2), ((40, 30), (32, 64), (1, 1), 64, 3),
+    ((160, 120), (16, 32), (2, 2), 64, 3), ((64, 64), (16,), (1,), 16, 1), ((320, 240), (16, 32), (2, 2), 32, 3), ((200, 150), (16,), (2,), 24, 2),
+])
+def test_a_multiprocessor_holds_no_more_blocks_of_an_fp32_convlstm_than_its_even_share(fake, net, enc, stride, hidden, K):
+    """As a dependent it is placed where its predecessor leaves room, and blocks in a pile take as long as the pile is high."""
+    s = Streams(fake, K, workload=dict(src_w=net[0], src_h=net[1], net_w=net[0], net_h=net[1], enc_cout=enc, enc_stride=stride, hidden=hidden, n_tools=3))
+    log = s.submit(on_device=range(K))[1]
+    lstm = [re.search(r"grid (\d+) (\d+) (\d+) smem (\d+)", line) for line in log if re.match(r"launch \S*conv3x3_simt_kernelILi1ELi2E", line)]
+    assert len(lstm) == 1
+    x, y, z, smem = (int(v) for v in lstm[0].groups())
+    share = -(-x * y * z // 148)
+    assert (share + 1) * (smem + 1024) > 228 * 1024 >= share * (smem + 1024)
+    s.sync()
