@@ -75,6 +75,15 @@ __device__ __forceinline__ void load_row(const float* r, float (&x)[6]) {
 template <int STRIDE, int EPI, int WY, int WO, int KS, int PX>
 __global__ void __launch_bounds__(32 * WY * WO * KS) conv3x3_simt_kernel(const __grid_constant__ ConvSimtParams p) {
   using Cfg = SimtCfg<STRIDE, WY, WO, KS, PX>;
+  // Whether a row of taps is fetched while the one before it is multiplied: two or three warps to a scheduler do not hide a shared-memory load.  Only where that
+  // pays for its registers (blocks, or spills of more than a word); us without / with it: not at stride 2 (a tick of six 480x360 inputs 80 / 85), not with bf16 outputs of four pixels a thread (eight 502x374
+  // images to 32 channels 97 / 115; eight pixels, eight 320x240 to 96 channels 111 / 107), not in encoder layers of four channel groups to a tile (eight 320x240 images to 64 channels
+  // 73.5 / 78.2; two groups 28.5 / 27.9; channels shared out by four warps 8.3 / 7.6), nor in a ConvLSTM whose channels four warps share (two 32x32 maps of 32 channels 17.9 / 18.7) or
+  // with eight pixels a thread and two groups to a tile (eight 320x240 maps of 12 channels 313 / 320).  The other ConvLSTMs: eight 320x240 maps of 16 channels 486 / 449, three 80x60 of 32
+  // 69.2 / 68.3.
+  constexpr bool AHEAD = STRIDE == 1 && (EPI == EPI_LSTM_F32_NCHW    ? KS <= 2 && !(WO == 2 && PX == 8)
+                                         : EPI == EPI_RELU_F32_NCHW ? WO < 4
+                                                                    : PX == 8);
   constexpr int CB = Cfg::CB, IN_H = Cfg::IN_H, IN_W = Cfg::IN_W, PITCH = Cfg::PITCH, NT = Cfg::THREADS, TW = Cfg::TW;
   constexpr int RUNS = PX / 4, RUN_STEP = 8;         // runs of 4 pixels of a thread, and columns from one to the next
   extern __shared__ __align__(16) float smem[];
@@ -169,9 +178,7 @@ __global__ void __launch_bounds__(32 * WY * WO * KS) conv3x3_simt_kernel(const _
     copies_commit();                                 // also where there is nothing left to copy, so that the wait above counts alike
     buf = buf == 2 ? 0 : buf + 1;
     const int c_end = min(CB, cin - c0);
-    if constexpr (STRIDE == 1) {
-      // One row of taps after the other, the inputs and weights of the next one fetched while this one's products run: two or three warps to a scheduler
-      // do not hide a shared-memory load.  Ticks, us: two 200x150 maps, ConvLSTM of 24, 154 -> 145; eight 80x60, ConvLSTM of 32, 201.5 -> 199.5, three 112.6 -> 112.0.
+    if constexpr (AHEAD) {
       const float* in_c = cur + (ks * IN_H + ly) * PITCH + lx;
       const float* w_c = cur + Cfg::IN_FLOATS + (ks * 9 * WO + wo) * OC;
       float xn[RUNS][6];
@@ -224,37 +231,46 @@ __global__ void __launch_bounds__(32 * WY * WO * KS) conv3x3_simt_kernel(const _
         w_c = w_next;
       }
     } else {
-      // The compiler's own order: fetched ahead, the registers cost blocks (six 480x360 inputs 80 -> 85 us a tick).
 #pragma unroll 1
       for (int c = ks; c < c_end; c += KS) {
-        const float* in_c = cur + (c * IN_H + ly * 2) * PITCH + lx;
+        const float* in_c = cur + (c * IN_H + ly * STRIDE) * PITCH + lx;
         const float* w_c = cur + Cfg::IN_FLOATS + (c * 9 * WO + wo) * OC;
 #pragma unroll
         for (int ky = 0; ky < 3; ++ky) {
-          // x[i]: input column lx * 2 + i of this row
-          const float* r = in_c + ky * PITCH;
-          float x[9];
-          const float4 e = *reinterpret_cast<const float4*>(r);
-          const float4 o = *reinterpret_cast<const float4*>(r + Cfg::ODD);
-          x[0] = e.x; x[2] = e.y; x[4] = e.z; x[6] = e.w; x[8] = r[4];
-          x[1] = o.x; x[3] = o.y; x[5] = o.z; x[7] = o.w;
-          if (EPI == EPI_RELU_BF16_NHWC) {
+          // x[g][i]: input column (lx + 8 g) * STRIDE + i of this row
+          float x[RUNS][3 * STRIDE + 3];
 #pragma unroll
-            for (int i = 0; i < 9; ++i) x[i] = round_bf16(x[i]);
+          for (int g = 0; g < RUNS; ++g) {
+            const float* r = in_c + ky * PITCH + g * RUN_STEP;
+            if constexpr (STRIDE == 1) {
+              load_row(r, x[g]);
+            } else {
+              const float4 e = *reinterpret_cast<const float4*>(r);
+              const float4 o = *reinterpret_cast<const float4*>(r + Cfg::ODD);
+              x[g][0] = e.x; x[g][2] = e.y; x[g][4] = e.z; x[g][6] = e.w; x[g][8] = r[4];
+              x[g][1] = o.x; x[g][3] = o.y; x[g][5] = o.z; x[g][7] = o.w;
+            }
+            if (EPI == EPI_RELU_BF16_NHWC) {
+#pragma unroll
+              for (int i = 0; i < 3 * STRIDE + 3; ++i) x[g][i] = round_bf16(x[g][i]);
+            }
           }
-          unsigned long long x2[9];                      // each value twice
+          unsigned long long x2[RUNS][3 * STRIDE + 3];   // each value twice
 #pragma unroll
-          for (int i = 0; i < 9; ++i) x2[i] = tc::pack2(x[i], x[i]);
+          for (int g = 0; g < RUNS; ++g)
+#pragma unroll
+            for (int i = 0; i < 3 * STRIDE + 3; ++i) x2[g][i] = tc::pack2(x[g][i], x[g][i]);
 #pragma unroll
           for (int kx = 0; kx < 3; ++kx) {
             const ulonglong2* w = reinterpret_cast<const ulonglong2*>(w_c + (ky * 3 + kx) * WO * OC);
 #pragma unroll
-            for (int o4 = 0; o4 < OC; o4 += 4) {
-              const ulonglong2 w4 = w[o4 >> 2];
+            for (int o = 0; o < OC; o += 4) {
+              const ulonglong2 w4 = w[o >> 2];
 #pragma unroll
-              for (int i = 0; i < 4; ++i) {
-                tc::fma2(acc2[o4 / 2][i], x2[i * 2 + kx], w4.x);
-                tc::fma2(acc2[o4 / 2 + 1][i], x2[i * 2 + kx], w4.y);
+              for (int i = 0; i < PX; ++i) {
+                const unsigned long long v = x2[i >> 2][(i & 3) * STRIDE + kx];
+                tc::fma2(acc2[o / 2][i], v, w4.x);
+                tc::fma2(acc2[o / 2 + 1][i], v, w4.y);
               }
             }
           }
