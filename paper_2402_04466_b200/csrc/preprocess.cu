@@ -8,7 +8,7 @@
 // funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
 // Bound by issue and by the start: every block's first tile comes before anything can be sampled (four full-HD frames: launch 2, first rows 3, two tiles 9 us).  Instructions per
 // pixel of three channels 117 -> 82, 78 -> 68 % of the issue slots.  Device time, us, of frames in L2 before / now: four full-HD frames to 1280x720 17.7 / 14.3, eight 33.0 / 27.0, one 6.1 / 5.8, eight to
-// 768x432 19.5 / 15.2, four 1280x960 to 640x480 9.0 / 8.3, two 960x540 to 1280x720 9.3 / 8.6 (launches of 3 to 4 us, one tile a block, up to 0.3 longer: three 428x240 to 320x240 3.0 / 3.2); a call with frames from memory: 18.5 / 16.4, 34.8 / 29.0, 8.2 / 7.2, 20.5 / 17.8, 10.3 / 10.3.
+// 768x432 19.5 / 15.2, four 1280x960 to 640x480 9.0 / 8.3, two 960x540 to 1280x720 9.3 / 8.6 (launches of 2.5 to 3.5 us, one tile a block, up to 0.15 longer, for a bulk copy arrives later than a thread's own: three 428x240 to 320x240 3.30 / 3.36); a call with frames from memory: 18.5 / 16.4, 34.8 / 29.0, 8.2 / 7.2, 20.5 / 17.8, 10.3 / 10.3.
 // Not kept: per-thread asynchronous copies by the ninth warp (25 us), three and four tiles in flight of 8 to 16 rows (16.6 to 18.8), five or six blocks with smaller tiles.
 #include "tt_internal.h"
 #include "pre_math.cuh"
@@ -140,7 +140,6 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
     tc::mbar_init(tc::smem_u32(&s_full[1]), PRE_WARPS);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  __syncthreads();
 
   // Worked out by a whole warp, a lane per row: the i-th tile's place (tiles in order of image, tile column, tile row) ...
   auto place_of = [&](int i) {
@@ -179,8 +178,10 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
     if (lane == 0) s_tile[buf] = {t.img, t.y0, t.rows, t.tx, t.left};
   };
 
-  // A warp issues its copies one behind the other: those of the first tile, which everything waits for, are shared out.
+  // A warp issues its copies one behind the other: those of the first tile, which everything waits for, are shared out.  Its place
+  // is worked out while the barriers are set up (three 428x240 to 320x240 3.44 -> 3.36 us, four full-HD frames 14.57 -> 14.45).
   const Place first = place_of(0);
+  __syncthreads();
   copy_rows(first, 0, warp + PRE_WARPS * lane, PRE_WARPS * 32);
   if (lane == 0) tc::mbar_arrive(tc::smem_u32(&s_full[0]));
 
