@@ -327,9 +327,8 @@ tt_status tt_debug_expire_wait(tt_ctx* ctx, uint64_t limit_cycles);
 /*
  * tt_preprocess — S1, the format-conversion operator of Section III-A.
  * src_dev: K frames, frame k at src_dev + k*src_frame_stride bytes, uint8 RGB interleaved,
- * row pitch src_pitch bytes (any alignment).  dst_dev: fp32 [K][3][net_h][net_w], 4-byte aligned
- * (16-byte alignment with net_w a multiple of 4 lets the kernel use 128-bit stores).  For output sample o of
- * an axis resized from `in` to `out`: s = clamp((o+1/2)*in/out - 1/2, 0, in-1) evaluated in
+ * row pitch src_pitch bytes (any alignment).  dst_dev: fp32 [K][3][net_h][net_w], 4-byte aligned.
+ * For output sample o of an axis resized from `in` to `out`: s = clamp((o+1/2)*in/out - 1/2, 0, in-1) evaluated in
  * exact integer arithmetic, i0 = floor(s), i1 = min(i0+1, in-1), weight s - i0.
  * The kernel's wait for staged frame rows is bounded.  Should one run out (which no healthy device produces), the rest is
  * sampled from memory directly: the image is whole and the same bits, so this call needs no status word.

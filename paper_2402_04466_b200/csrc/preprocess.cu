@@ -38,13 +38,14 @@ constexpr int PRE_STAGE_BYTES = 26 * 1024;   // staged rows of a tile; two tiles
 constexpr long long PRE_LAND_CYCLES = 2000000;   // how long a block that has given up a wait stays for copies in flight: about a millisecond
 constexpr int PRE_STATIC_BYTES = 2 * (PRE_MAX_ROWS * 16 + 64) + 16;   // the kernel's tables and barriers
 
-struct alignas(32) PreprocessArgs {
+struct PreprocessArgs {
   PreprocessParams p;
   int32_t tile_rows, tiles_x, tiles_y;
   int32_t rows_cap, row_cap;                 // staged rows of a tile, bytes of one (a multiple of 16)
   int32_t expire_from = 0x7fffffff;          // the first tile of a block whose wait gives up at once (tests)
   int32_t tiles_per_block, tiles_left;       // the first tiles_left blocks take one tile more
 };
+static_assert(whole_arguments<PreprocessArgs> && whole_arguments<PreprocessParams>, "kernel arguments");
 // What the sampling warps are told of a tile.
 struct alignas(16) TileInfo {
   int32_t img, y0, rows, tx;

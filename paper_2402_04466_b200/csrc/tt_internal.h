@@ -19,9 +19,14 @@ namespace tt {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
+// Kernel arguments are whole runs of 32 bytes: a launch copies them, and any other size takes the host 0.4 us more a launch (160 bytes 4.5, 152 or 168 4.9 us a call).
+template <typename Params>
+constexpr bool whole_arguments = sizeof(Params) % 32 == 0;
+
 template <typename Params>
 inline cudaError_t launch_kernel(void (*kern)(const Params), dim3 grid, int block, size_t smem, cudaStream_t s, const Params& p,
                                  bool pdl, int cluster = 1) {
+  static_assert(whole_arguments<Params>, "kernel arguments");
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
@@ -62,8 +67,6 @@ struct OncePerContext {
   }
 };
 
-// Kernel arguments are whole runs of 32 bytes: a launch copies them, and any other size takes the host 0.4 us more a launch (160 bytes 4.5, 152 or 168 4.9 us a call).
-
 // Maps batch position n (0..K-1) of a launch to an image index inside a tensor that holds
 // more images than the batch (state slots, ping-pong halves).
 struct IdxMap {
@@ -75,7 +78,7 @@ struct FramePtrs {
 };
 
 // ------------------------------------------------------------------------- S1 preprocess
-struct PreprocessParams {
+struct alignas(32) PreprocessParams {
   FramePtrs src;                   // frame pointers by value (also used for host-side decisions)
   const uint8_t* const* src_tab;   // if non-null the kernel reads the pointers from this device table instead
   int32_t K, src_w, src_h, src_pitch, net_w, net_h;
