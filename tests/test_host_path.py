@@ -344,3 +344,18 @@ def test_a_multiprocessor_holds_no_more_blocks_of_an_fp32_convlstm_than_its_even
     share = -(-x * y * z // 148)
     assert (share + 1) * (smem + 1024) > 228 * 1024 >= share * (smem + 1024)
     s.sync()
+
+
+@pytest.mark.parametrize("missing", [(), ("_cuda_getCurrentRawStream",), ("_cuda_getDevice",)])
+def test_the_current_streams_handle_with_and_without_torchs_own_shortcut(monkeypatch, missing):
+    """Names of torch that begin with an underscore may go; the public way to the handle stays."""
+    import torch
+
+    class Stream:
+        cuda_stream = 77
+
+    shortcut = {"_cuda_getDevice": lambda: 3, "_cuda_getCurrentRawStream": lambda device: 70 + device}
+    monkeypatch.setattr(torch, "_C", type("C", (), {k: staticmethod(v) for k, v in shortcut.items() if k not in missing}))
+    monkeypatch.setattr(torch.cuda, "current_stream", Stream)
+    assert binding._stream_ptr(None) == (77 if missing else 73)
+    assert binding._stream_ptr(Stream()) == 77 and binding._stream_ptr(5) == 5
