@@ -233,7 +233,7 @@ def test_convlstm_on_pairs_of_blocks_changes_no_bit(cuda_device, hidden, net, K)
     ((200, 150), (192, 90), 7, 3),       # half of the last wide tile: narrow tiles
     ((200, 150), (193, 90), 1, 1),       # more than half: wide tiles
     ((64, 40), (1, 1), 0, 8),
-    ((1600, 900), (160, 90), 2, 2),      # ten source rows and columns per output: few rows of a tile fit
+    ((1600, 900), (160, 90), 2, 2),      # ten source rows and columns per output: no tile of four rows fits
     ((2400, 1300), (40, 20), 0, 1),      # sixty: no tile fits, the kernel without staging
     ((90, 700), (300, 700), 5, 2),       # height not resized
 ])
@@ -261,14 +261,17 @@ def test_preprocess_whose_staging_takes_almost_48_kilobytes(cuda_device, src, ne
     test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, 3, K)
 
 
-@pytest.mark.parametrize("src,net,pad,K", [
-    ((300, 200), (64, 5), 0, 3),         # a thread's second column lies outside; fewer rows than runs of them
-    ((300, 200), (127, 33), 1, 2),       # ... of the last lane alone
-    ((97, 61), (191, 95), 2, 8),         # narrow tiles beside a full one, frame rows used by several output rows
+STAGED_SIZES = [                         # with the kernel that stages frame rows, whatever the batch (test_host_path.py asks the dispatch)
+    ((40, 8), (20, 5), 0, 3),            # every thread's second column lies outside; fewer rows than runs of them
+    ((300, 200), (127, 33), 1, 2),       # the second column of the last lane alone lies outside
+    ((97, 61), (191, 95), 2, 8),         # narrow tiles, the last a column short; frame rows used by several output rows
     ((640, 360), (427, 241), 5, 5),      # rows that share a frame row with the one above, and rows that do not
     ((1280, 960), (1000, 562), 0, 8),    # several tiles a block, the copies of all but the first by one warp
     ((320, 240), (321, 240), 0, 8),      # the height not resized
-])
+]
+
+
+@pytest.mark.parametrize("src,net,pad,K", STAGED_SIZES + [((300, 200), (64, 5), 0, 3)])     # the last: forty frame rows to an output row, none staged
 def test_preprocess_of_a_frame_is_the_same_whatever_shares_its_launch(cuda_device, src, net, pad, K):
     """Tile heights, runs of rows and the blocks' shares depend on the batch; the bits of a frame do not.  Bound against the oracle as above."""
     test_preprocess_at_the_edges_of_its_tiles(cuda_device, src, net, pad, min(K, 2))

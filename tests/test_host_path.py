@@ -12,6 +12,7 @@ import pytest
 import tt_synth
 from paper_2402_04466_b200 import binding
 from paper_2402_04466_b200 import build as build_mod
+from test_gpu_kernel_edges import STAGED_SIZES
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 
@@ -297,6 +298,15 @@ def test_tiles_of_the_preprocessing_and_where_it_stages_none(fake, src, net, K, 
     assert fake.tt_preprocess(at, K, 3 * src[0] * src[1], *src, 3 * src[0], at + 0x10000000, *net, 255.0, 0.5, 0.25, None) == 0
     (line,) = [x for x in fake.fake_log().decode().splitlines() if x.startswith("launch")]
     assert line.endswith(f" smem {smem}") and (f"preprocess_staged_kernelILi{cols}E" if smem else "preprocess_direct_kernel") in line
+
+
+@pytest.mark.parametrize("src,net,pad,K", STAGED_SIZES)
+def test_sizes_that_are_there_for_the_staged_preprocessing_reach_it(fake, src, net, pad, K):
+    at = 0x7F0000000000
+    for batch in (1, K):
+        fake.fake_reset()
+        assert fake.tt_preprocess(at, batch, src[1] * (3 * src[0] + pad), *src, 3 * src[0] + pad, at + 0x10000000, *net, 255.0, 0.5, 0.25, None) == 0
+        assert b"preprocess_staged_kernel" in fake.fake_log()
 
 
 def test_kernel_attributes_are_set_in_every_context(fake):
