@@ -1,6 +1,7 @@
-// Arithmetic of the preprocessing stage (bilinear resize of a uint8 RGB frame + normalisation), shared by
-// the stand-alone preprocess kernel and by the first encoder layer when it samples the frame itself.
-// Both must give the same fp32 bits, so both evaluate exactly these expressions.
+// Arithmetic of the preprocessing stage (bilinear resize of a uint8 RGB frame + normalisation): sample positions, bytes as
+// floats and the normalisation for the stand-alone preprocess kernel and for the first encoder layer when it samples the frame
+// itself.  fetch_pair, blend_magic, sample_row and sample_rows are the first layer's; the preprocess kernel evaluates the same
+// expressions on pairs of columns.  Both give the same fp32 bits, which the GPU tests of the fused against the separate launches compare.
 #pragma once
 #include <cstdint>
 #include <cuda_runtime.h>
