@@ -7,8 +7,10 @@
 // that the row above has already blended horizontally is not fetched again.  A bilinear tap pair (two neighbouring RGB pixels = 6 bytes) is three 32-bit shared loads plus
 // funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
 // Bound by issue and by the start: every block's first tile comes before anything can be sampled (four full-HD frames: launch 2, first rows 3, two tiles 9 us).  Instructions per
-// pixel of three channels 117 -> 82, 78 -> 68 % of the issue slots.  Device time, us, of frames in L2 before / now: four full-HD frames to 1280x720 17.7 / 14.3, eight 33.0 / 27.0, one 6.1 / 5.8, eight to
-// 768x432 19.5 / 15.2, four 1280x960 to 640x480 9.0 / 8.3, two 960x540 to 1280x720 9.3 / 8.6 (launches of 2.5 to 3.5 us, one tile a block, up to 0.15 longer, for a bulk copy arrives later than a thread's own: three 428x240 to 320x240 3.30 / 3.36); a call with frames from memory: 18.5 / 16.4, 34.8 / 29.0, 8.2 / 7.2, 20.5 / 17.8, 10.3 / 10.3.
+// pixel of three channels 117 -> 82, 78 -> 68 % of the issue slots.  Device time, us, of frames in L2, with a column a thread and every thread's own copies / now: four full-HD frames to
+// 1280x720 17.6 / 14.4, eight 32.9 / 27.8, one 6.1 / 5.7, eight to 768x432 19.6 / 15.8, four 1280x960 to 640x480 9.2 / 8.2, two 960x540 to 1280x720 9.3 / 8.3 (launches of 2.5 to 3.5 us, one
+// tile a block, up to 0.15 longer, for a bulk copy arrives later than a thread's own: three 428x240 to 320x240 3.30 / 3.36); a call among others, frames from memory, in the same order:
+// 18.5 / 16.4, 34.8 / 29.1, 8.2 / 8.2, 20.5 / 17.9, 10.3 / 10.3, 10.3 / 10.3 (4.2 / 4.2).
 // Not kept: per-thread asynchronous copies by the ninth warp (25 us), three and four tiles in flight of 8 to 16 rows (16.6 to 18.8), five or six blocks with smaller tiles.
 #include "tt_internal.h"
 #include "pre_math.cuh"
@@ -253,8 +255,8 @@ __global__ void __launch_bounds__(PRE_THREADS, PRE_PER_SM) preprocess_staged_ker
         unpack2(fma2(top.r, scale, shift), v[0][0], v[0][1]);
         unpack2(fma2(top.g, scale, shift), v[1][0], v[1][1]);
         unpack2(fma2(top.b, scale, shift), v[2][0], v[2][1]);
-        // streaming stores: the image is written once (four frames to 1103x1103, whose rows do not fill
-        // whole sectors, 24.4 -> 23.3 us, and with the two columns side by side 21.1; to 1279x719 16.5 -> 15.0 -> 14.4; whole lines the same)
+        // streaming stores: the image is written once (four 1134x907 frames to 1103x1103, whose rows do not fill whole sectors, 20.3 -> 19.7 us, four full-HD ones to
+        // 1280x720 14.9 -> 14.4, eight 27.6 -> 27.8)
         float* d = out + o;
         __stcs(d, v[0][0]);
         __stcs(d + plane, v[1][0]);
@@ -310,8 +312,10 @@ cudaError_t launch_staged(const PreprocessParams& p, cudaStream_t s, bool* fits)
   a.tiles_x = (p.net_w + TILE_W - 1) / TILE_W;
   // Rows per tile: the busiest block's tiles x (rows to sample, and about two rows' worth for its halo and barriers) is least, and the higher tile of
   // two that come out alike; another height where by it the busiest multiprocessor has at least a tenth less to do, a tile's latency counted as twelve
-  // rows.  Device time of frames in L2, us, by rows: four 1280x960 to 640x480 6 10.4, 8 9.3, 10 9.5, 12 8.4, 14 8.4*; four 1920x1080 to 1280x720 16 15.4, 20 15.2,
-  // 24 15.1, 26 14.7*; one 320x240 to 1280x960 18 7.7, 22 7.0*, 24 7.2, 28 7.7 (* chosen).
+  // rows.  Device time of frames in L2, us, by rows: four 1280x960 to 640x480 6 10.1, 8 9.0, 10 9.3, 12 8.1, 14 8.2*; four 1920x1080 to 1280x720 16 15.1, 20 14.7,
+  // 24 14.3, 26 14.4*; one 320x240 to 1280x960 18 7.5, 22 6.8*, 24 7.0, 28 7.4; heights that leave a run of rows idle are no worse for it, one 640x360 to 427x241 8 3.44,
+  // 12 3.18*, 16 3.25 (* chosen).  Of 31 sizes and batches 29 are within 1.5 % of their best height; five 854x480 to 640x480 and three 1280x720 to 700x390 are 8 % from it (one tile a
+  // block of 30 and 32 rows 6.25, 22* and 24* 6.7).
   const long slots = (long)PRE_PER_SM * sms;
   struct Height {
     int rows = 0;
