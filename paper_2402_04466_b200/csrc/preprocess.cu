@@ -7,7 +7,7 @@
 // that the row above has already blended horizontally is not fetched again.  A bilinear tap pair (two neighbouring RGB pixels = 6 bytes) is three 32-bit shared loads plus
 // funnel shifts; bytes become floats by a byte permute into the mantissa of 2^23.
 // Bound by issue and by the start: every block's first tile comes before anything can be sampled (four full-HD frames: launch 2, first rows 3, two tiles 9 us).  Instructions per
-// pixel of three channels 117 -> 82, 78 -> 68 % of the issue slots.  Device time, us, of frames in L2, with a column a thread and every thread's own copies / now: four full-HD frames to
+// pixel of three channels 117 -> 82, 78 -> 69 % of the issue slots.  Device time, us, of frames in L2, with a column a thread and every thread's own copies / now: four full-HD frames to
 // 1280x720 17.6 / 14.4, eight 32.9 / 27.8, one 6.1 / 5.7, eight to 768x432 19.6 / 15.8, four 1280x960 to 640x480 9.2 / 8.2, two 960x540 to 1280x720 9.3 / 8.3 (launches of 2.5 to 3.5 us, one
 // tile a block, up to 0.15 longer, for a bulk copy arrives later than a thread's own: three 428x240 to 320x240 3.30 / 3.36); a call among others, frames from memory, in the same order:
 // 18.5 / 16.4, 34.8 / 29.1, 8.2 / 8.2, 20.5 / 17.9, 10.3 / 10.3, 10.3 / 10.3 (4.2 / 4.2).
